@@ -561,7 +561,7 @@ def run_ours(args):
                    "l2": "flushed between timed iterations (%d MiB write)" % (L2_FLUSH_BYTES >> 20),
                    "parallelism": "replicas only" if world > 1 else "single GPU"},
         "plan_ms": plan1["plan_ms"], "plan_workload": PLAN_WORKLOAD,
-        "plan_greedy_loop": {"kernel": "k_plan_one", "bound": "latency", "ms": plan1.get("greedy_loop_ms"),
+        "plan_greedy_loop": {"kernel": "k_plan_chip", "bound": "latency", "ms": plan1.get("greedy_loop_ms"),
                              "us_per_iteration": plan1.get("greedy_loop_us_per_iteration"), "iterations": plan1["iterations"],
                              "note": "the planner state of this workload lives in the shared memory of one SM: a chain of dependent "
                                      "iterations (search, rescore, commit); reported per iteration, an HBM fraction would mean nothing"},

@@ -297,15 +297,15 @@ int32_t g10_emit_instructions(int64_t num_kernels, int64_t num_tensors, const in
    in the next iteration).  Same arguments, outputs and workspace (G10_WS_PLAN) as g10_plan_migrations; of the
    options only host_capacity_bytes and max_iterations are used.  g10_schedule_prefetch and g10_emit_instructions take
    the records as they are.
-   A trace whose pressure, clock, bookings and periods fit the shared memory of one SM (K <= 32000) is planned by one
-   thread block; a larger one by the multi-block formulation of Algorithm 1 as printed (every live period rescored
+   A trace whose pressure, clock and periods fit the shared memory of one thread-block cluster is planned there; a larger
+   one by the multi-block formulation of Algorithm 1 as printed (every live period rescored
    every iteration: the same plan, slower). */
 int32_t g10_plan_cyclic(const g10_trace *trace, uint64_t gpu_capacity_bytes, uint64_t host_bw, uint64_t ssd_bw,
                         const g10_options *options /* NULL = defaults */, g10_plan_out *out,
                         void *ws, size_t ws_bytes, void *stream);
 
 /* Section 5's sensitivity studies seen from the planner: the same trace planned under V variants at once -- other
-   kernel durations (profiling error), SSD / host bandwidths, GPU capacity, host capacity -- one thread block per
+   kernel durations (profiling error), SSD / host bandwidths, GPU capacity, host capacity -- one thread-block cluster per
    variant, all variants running concurrently.  Every variant's result is exactly what g10_plan_migrations gives for
    the trace with that variant's durations and parameters.  `variants` is a HOST array (copied before the call
    returns); its kernel_ns pointers are DEVICE pointers.  Outputs are DEVICE pointers: migrations [V][migrations_cap],
@@ -313,8 +313,7 @@ int32_t g10_plan_cyclic(const g10_trace *trace, uint64_t gpu_capacity_bytes, uin
    stability [V][2] = (|M_v & M_0|, |M_v | M_0|) over the sets of migrated periods of variant v and variant 0 (their
    quotient is the Jaccard index; (-1, -1) when a plan is missing).
    Limits: the trace has to be device resident (G10_MEM_DEVICE); 1 <= V <= 1024.
-   One block per variant requires that pressure, clock, bookings and the periods of the trace fit the shared memory of
-   one SM (the DNN-shaped traces of a few thousand kernels do).  Only the device can tell, so the call reads variant
+   One cluster per variant requires that pressure, clock, bookings and the periods of the trace fit its shared memory (the DNN-shaped traces of a few thousand kernels do).  Only the device can tell, so the call reads variant
    0's summary back (one small copy and a synchronisation of `stream`: unlike the other calls this one returns with
    its kernels finished); if the trace did not fit, the variants are then planned one after the other by the planners
    that use the whole GPU -- the same results, V times the time of one plan.

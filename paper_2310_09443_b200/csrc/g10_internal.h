@@ -16,6 +16,7 @@ typedef unsigned long long ull;
 extern ull g_launch_count;
 inline void count_launch() { __atomic_fetch_add(&g_launch_count, 1ull, __ATOMIC_RELAXED); }
 }  // namespace g10
+#define cudaLaunchKernelExC(...) (g10::count_launch(), ::cudaLaunchKernelExC(__VA_ARGS__))
 #define cudaLaunchKernelEx(...) (g10::count_launch(), ::cudaLaunchKernelEx(__VA_ARGS__))
 #define cudaLaunchCooperativeKernel(...) (g10::count_launch(), ::cudaLaunchCooperativeKernel(__VA_ARGS__))
 namespace g10 {
@@ -93,12 +94,11 @@ struct Workspace {
     int64_t *hocc;               // [K] host-memory occupancy per slot
     unsigned char *dead;         // [E] period erased
     unsigned *wl_count;          // [2] lengths of the two DIRTY work lists
-    unsigned *one_done;          // [1] the single-block planner produced the plan
+    unsigned *one_done;          // [1] the on-chip planner produced the plan
     ull *event_budget;           // [1] events booked by the blocks of the first / last pass (at most E for a valid trace)
     unsigned *bk_count, *bk_cursor;   // [4096] events per tensor bucket, scatter cursors
     ull *bk_words;               // [2 * 4096] tagged per-bucket totals
     long long *bk_carry;         // [4] distinct uses and periods of all tensors before the current pass (two copies used in turn)
-    ull *xwords;                 // [2][kSmallMaxBlocks][16] tagged words of the proposal exchange
     ull *seg_words, *seg_words2; // [blocks * 16] each: tagged segment sums of the slot-clock scan and of the pressure scan, one 128-byte line per block
     // --- uninitialised region ---
     int32_t *raw_ptr;            // [N+1]
@@ -132,7 +132,7 @@ struct Workspace {
     int2 *c_rng;                 // [E] absent range of the current destination
     int *worklist;               // [2*E]
     ull *bk_pairs;               // [E] events as (tensor in bucket, kernel) keys, bucket after bucket
-    int64_t *busy_rep, *hocc_rep; // per-block copies of the channel bookings / host occupancy (small-trace planner)
+    int64_t *busy_rep, *hocc_rep; // per-block copies of the channel bookings / host occupancy (on-chip planner)
     int64_t *peak_part;          // [max blocks]
     g10_migration *migrations;   // host mode only
     int64_t *summary;            // [8]
@@ -182,8 +182,8 @@ struct PlanParams {
 };
 
 constexpr int kMaxPlanBlocks = 1024;
-constexpr int kSmallMaxBlocks = 160;       // blocks of the small-trace planner (one per SM, at most)
-constexpr int64_t kSmallMaxSlots = 12000;  // largest K whose pressure + clock fit in shared memory
+constexpr int kChipMaxCluster = 16;        // blocks of the on-chip planner's cluster, at most
+constexpr int64_t kChipMaxSlots = 13000;   // no larger timeline fits shared memory
 
 // passes (g10_passes.cu)
 // (zero_diff [K + 1], zero_point [K]: arrays the kernel clears on its way, for a later kernel of the same call)
@@ -257,12 +257,13 @@ cudaError_t launch_characterize(int64_t K, int64_t N, const int64_t *use_ptr, co
 cudaError_t launch_plan_loop(const DeviceTrace &t, const Workspace &w, const PlanParams &p, cudaStream_t s);
 cudaError_t launch_cyclic_prepare(const DeviceTrace &t, const Workspace &w, cudaStream_t s);
 cudaError_t launch_plan_cyclic(const DeviceTrace &t, const Workspace &w, const PlanParams &p, cudaStream_t s);
-cudaError_t launch_plan_variants(const DeviceTrace &t, const Workspace &w, const PlanParams &p, int V, int64_t *stability, cudaStream_t s);
+// C: blocks per variant, a power of two up to kChipMaxCluster
+cudaError_t launch_plan_variants(const DeviceTrace &t, const Workspace &w, const PlanParams &p, int V, int C, int64_t *stability, cudaStream_t s);
 // stability pairs of V finished plans against plan 0; ORs *status_word into every plan's summary[7]
 cudaError_t launch_batch_finish(const DeviceTrace &t, const Workspace &w, const PlanParams &p, int V, int64_t *stability, const ull *status_word,
                                 cudaStream_t s);
 int plan_loop_max_blocks();
-bool plan_keeps_state_on_chip(int64_t K, int64_t E, uint32_t flags);   // true: the small-trace planner will run
+bool plan_keeps_state_on_chip(int64_t K, int64_t E, bool host_cap, uint32_t flags, bool cyclic);   // true: no other planner will be needed
 cudaError_t launch_publish_status(const Workspace &w, int64_t *dst, cudaStream_t s);
 cudaError_t launch_publish_status_or(const Workspace &w, int64_t *dst, cudaStream_t s);
 

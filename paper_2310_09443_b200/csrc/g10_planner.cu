@@ -7,13 +7,13 @@
 namespace g10 {
 
 // kCyclic: steady-state planning (period and geometry arrays hold slots unrolled over two iterations, A.start is the
-// unrolled clock; see phys_slot) for traces too large for the single-block planner, which runs first: when it has
+// unrolled clock; see phys_slot) for traces too large for the on-chip planner, which runs first: when it has
 // produced the plan (`done`), this grid returns at once.
 template <bool kCyclic>
 __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_loop(PlanArgs A, const unsigned *done)
 {
     if (kCyclic && *done) return;          // (same answer in every thread of the grid: written by an earlier launch)
-    if (kCyclic && blockIdx.x == 0 && threadIdx.x == 0) A.summary[7] = 0;      // (the single-block planner left "does not fit" there)
+    if (kCyclic && blockIdx.x == 0 && threadIdx.x == 0) A.summary[7] = 0;      // (the on-chip planner may have left "does not fit" there)
     __shared__ Cand s_cand[kPlanWarps + 1];
     __shared__ long long s_max[kPlanWarps + 1];
     const int G = gridDim.x, c = blockIdx.x;
@@ -122,44 +122,41 @@ static int blocks_for(const void *kernel)
 
 cudaError_t launch_plan_lazy(const PlanArgs &A, const Workspace &w, int G, cudaStream_t s);
 int plan_lazy_blocks();
-cudaError_t launch_plan_small(const PlanArgs &A, const Workspace &w, int G, int cand_cap, size_t smem, cudaStream_t s);
-int plan_small_blocks();
-bool plan_small_fits(int64_t K, int64_t E, int G, int *cand_cap_out, size_t *smem_out);
-bool plan_one_possible(int64_t K, int64_t E, bool host_cap);
-cudaError_t launch_plan_one(const PlanArgs &A, const Workspace &w, cudaStream_t s);
+int plan_chip_blocks(int64_t E, bool several);
+int plan_chip_possible(int64_t K, int64_t E, int C, bool host_cap, bool cyclic);
+cudaError_t launch_plan_chip(const PlanArgs &A, const Workspace &w, int C, bool cyclic, cudaStream_t s);
 
-bool plan_keeps_state_on_chip(int64_t K, int64_t E, uint32_t flags)
+static int chip_blocks(int64_t E, uint32_t flags) { return plan_chip_blocks(E, (flags & G10_FLAG_MULTI_BLOCK) != 0); }
+
+bool plan_keeps_state_on_chip(int64_t K, int64_t E, bool host_cap, uint32_t flags, bool cyclic)
 {
-    if ((flags & (G10_FLAG_RESCORE_ALL | G10_FLAG_GLOBAL_STATE)) || K > kSmallMaxSlots) return false;
-    int Gs = plan_small_blocks();
-    if (Gs > kSmallMaxBlocks) Gs = kSmallMaxBlocks;
-    int cand_cap = 0;
-    size_t smem = 0;
-    return Gs >= 1 && plan_small_fits(K, E, Gs, &cand_cap, &smem);
+    if (flags & (G10_FLAG_RESCORE_ALL | G10_FLAG_GLOBAL_STATE)) return false;
+    return plan_chip_possible(K, E, chip_blocks(E, flags), host_cap, cyclic) == 2;
 }
 
-cudaError_t launch_plan_batch(const PlanArgs &A, const Workspace &w, int V, const BatchArgs &B, int64_t *stability, cudaStream_t s);
+cudaError_t launch_plan_batch(const PlanArgs &A, const Workspace &w, int V, int C, const BatchArgs &B, int64_t *stability, cudaStream_t s);
 
-cudaError_t launch_plan_variants(const DeviceTrace &t, const Workspace &w, const PlanParams &p, int V, int64_t *stability, cudaStream_t s)
+cudaError_t launch_plan_variants(const DeviceTrace &t, const Workspace &w, const PlanParams &p, int V, int C, int64_t *stability, cudaStream_t s)
 {
     PlanArgs A;
     fill_plan_args(t, w, p, A);
     BatchArgs B;
     B.variants = w.batch_variants; B.P0 = w.pressure; B.P_out = p.final_pressure;
-    return launch_plan_batch(A, w, V, B, stability, s);
+    return launch_plan_batch(A, w, V, C, B, stability, s);
 }
-
-cudaError_t launch_plan_one_cyclic(const PlanArgs &A, const Workspace &w, cudaStream_t s);
 
 cudaError_t launch_plan_cyclic(const DeviceTrace &t, const Workspace &w, const PlanParams &p, cudaStream_t s)
 {
     PlanArgs A;
     fill_plan_args(t, w, p, A);
     A.start = w.start2;
-    // one block plans when everything fits its shared memory (decided on the device); the multi-block planner queued
-    // behind it does the work otherwise
-    cudaError_t e = launch_plan_one_cyclic(A, w, s);
-    if (e != cudaSuccess) return e;
+    // one cluster plans when everything fits its shared memory; where only the device can tell, the planner that uses the whole
+    // GPU is queued behind it and does the work otherwise
+    const int C = chip_blocks(t.E, 0), fits = plan_chip_possible(t.K, t.E, C, p.host_capacity_bytes != 0, true);
+    if (fits) {
+        const cudaError_t e = launch_plan_chip(A, w, C, true, s);
+        if (e != cudaSuccess || fits == 2) return e;
+    }
     const int G = blocks_for((const void *)k_plan_loop<true>);
     if (G < 1) return cudaErrorLaunchFailure;
     const unsigned *done = w.one_done;
@@ -187,19 +184,12 @@ cudaError_t launch_plan_loop(const DeviceTrace &t, const Workspace &w, const Pla
         void *args[] = {&A, &done};
         return cudaLaunchCooperativeKernel((const void *)k_plan_loop<false>, dim3(G), dim3(kPlanThreads), args, 0, s);
     }
-    if (plan_keeps_state_on_chip(t.K, t.E, p.flags)) {
-        int Gs = plan_small_blocks();
-        if (Gs > kSmallMaxBlocks) Gs = kSmallMaxBlocks;
-        int cand_cap = 0;
-        size_t smem = 0;
-        if (Gs >= 1 && plan_small_fits(t.K, t.E, Gs, &cand_cap, &smem)) {
-            // one block does the whole loop when the device finds that everything fits its shared memory; the
-            // multi-block planner queued behind it returns at once in that case and does the work otherwise
-            if (!(p.flags & G10_FLAG_MULTI_BLOCK) && plan_one_possible(t.K, t.E, p.host_capacity_bytes != 0)) {
-                const cudaError_t e = launch_plan_one(A, w, s);
-                if (e != cudaSuccess) return e;
-            }
-            return launch_plan_small(A, w, Gs, cand_cap, smem, s);
+    if (!(p.flags & G10_FLAG_GLOBAL_STATE)) {
+        // (as in launch_plan_cyclic)
+        const int C = chip_blocks(t.E, p.flags), fits = plan_chip_possible(t.K, t.E, C, p.host_capacity_bytes != 0, false);
+        if (fits) {
+            const cudaError_t e = launch_plan_chip(A, w, C, false, s);
+            if (e != cudaSuccess || fits == 2) return e;
         }
     }
     const int G = plan_lazy_blocks();

@@ -35,6 +35,7 @@ struct LazyArgs {
     ull *partials;              // [3][kRoundM][2] 128-bit sums of the benefits rescored together (three buffers in turn)
     int64_t *tmin, *tmax;       // [tiles of kSlotTile slots] smallest / largest pressure of each tile
     int64_t stride;
+    const unsigned *done;       // non-zero: the on-chip planner already produced the plan
 };
 
 __device__ __forceinline__ u128 benefit_partial(const PlanArgs &A, int ap, int bp, int64_t s, int tid, int nthreads)
@@ -562,6 +563,7 @@ __device__ __forceinline__ bool may_beat(double key, const Cand &t)
 // All decisions are taken from data every block has, so the control flow is the same in every block.
 __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_lazy(PlanArgs A, LazyArgs L)
 {
+    if (*L.done) return;                       // (same answer in every thread of the grid: written by an earlier launch)
     __shared__ Cand s_cand[kPlanWarps + 1];
     __shared__ BestScratch s_best;
     __shared__ long long s_max[2 * kPlanWarps + 1];
@@ -948,7 +950,7 @@ cudaError_t launch_plan_lazy(const PlanArgs &A_in, const Workspace &w, int G, cu
     LazyArgs L;
     L.c_state = w.c_state; L.c_ben_lo = w.c_ben_lo; L.c_ben_hi = w.c_ben_hi; L.c_cost = w.c_cost; L.c_key = w.c_key;
     L.c_rng = w.c_rng; L.worklist = w.worklist; L.wl_count = w.wl_count; L.props = w.lazy_props; L.partials = w.lazy_partials; L.stride = A.geo_stride;
-    L.tmin = w.lazy_tmin; L.tmax = w.lazy_tmax;
+    L.tmin = w.lazy_tmin; L.tmax = w.lazy_tmax; L.done = w.one_done;
     void *args[] = {&A, &L};
     const cudaError_t e = cudaFuncSetAttribute(k_plan_lazy, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLazyDynBytes);
     if (e != cudaSuccess) return e;

@@ -936,3 +936,34 @@ def test_analysis_call_in_a_cuda_graph(gpu, oracle):
         assert np.array_equal(_np(v.first_use), ov.first_use) and np.array_equal(_np(v.last_use), ov.last_use)
         assert np.array_equal(_np(v.period_tensor)[:pn], ov.period_tensor)
         assert np.array_equal(_np(v.timeline.pressure)[:tr.K], P0) and int(v.timeline.peak_bytes.item()) == peak
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("K,chains", [(31, 3), (32, 40), (33, 40), (64, 300), (97, 1040), (200, 2100), (1025, 700)])
+def test_on_chip_planner_edges(gpu, oracle, K, chains):
+    """The on-chip planner where its layouts change: timelines around whole tiles of 32 slots; one block, a cluster of 16;
+    groups of 32, 64 and 128 periods per lane-look (a block's 1024 / 2048 periods); finite host memory; the cycle.  Every
+    tensor is used at a few random kernels.  Bit for bit against the oracle."""
+    rng = np.random.default_rng(K * 10007 + chains)
+    lists = [[] for _ in range(K)]
+    for i in range(chains * 4):
+        for k in sorted(set(int(x) for x in rng.integers(0, K, size=int(rng.integers(2, 6))))):
+            lists[k].append(i)
+    n = chains * 4
+    tr = traces.from_lists("edges", lists, rng.integers(1 << 16, 1 << 24, size=n), rng.integers(10_000, 3_000_000, size=K),
+                           (rng.random(n) < 0.2).astype(np.uint8), capacity_frac=(2, 5))
+    tb = gpu.upload(tr)
+    start, P0, peak, slot = oracle.timeline(tr)
+    cap = tr.capacity_from_peak(peak)
+    for host in (0, 3 << 24):
+        ref = oracle.plan(tr, cap, lazy=True, host_capacity_bytes=host)
+        for flags in (0, gpu.FLAG_MULTI_BLOCK):
+            check_plan(gpu, tr, tb, cap, ref, host_capacity=host, flags=flags)
+    check_cyclic(gpu, oracle, tr, cap)
+    variants = [dict(gpu_capacity_bytes=cap, host_bw=tr.host_bw, ssd_bw=tr.ssd_bw)] * 2
+    ref = oracle.plan(tr, cap, lazy=True)
+    for V in (2, 80):                                    # a cluster per variant, one block per variant
+        out = gpu.g10_plan_batch(tb, variants * (V // 2))
+        for v in (0, V - 1):
+            assert np.array_equal(gpu.batch_migrations_numpy(out, v), ref.migrations) and int(out.summary[v, 7].item()) == 0
+            assert np.array_equal(_np(out.final_pressure)[v], ref.final_pressure)
