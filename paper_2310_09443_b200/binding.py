@@ -397,9 +397,16 @@ def g10_plan_batch(tb: TraceBuffers, variants, max_iterations=0, migrations_cap=
 
 
 def batch_migrations_numpy(batch, v) -> np.ndarray:
-    """Committed migration records of variant v of a finished batch (synchronises)."""
-    n = min(int(batch.summary[v, 0].item()), batch.migrations_cap)
-    return batch.migrations[v, : n * 48].cpu().numpy().view(MIGRATION_DTYPE).copy()
+    """Committed migration records of variant v of a finished batch (synchronises).  The first call brings the records of all
+    variants over in two copies: a study reads them all, and a copy each costs some 40 us."""
+    host = getattr(batch, "_host", None)
+    if host is None:
+        counts = batch.summary[:, 0].cpu().numpy().clip(0, batch.migrations_cap)
+        most = int(counts.max()) if counts.size else 0
+        records = torch.empty((counts.size, most * 48), dtype=torch.uint8, pin_memory=True)
+        records.copy_(batch.migrations[:, : most * 48])
+        host = batch._host = (counts, records.numpy())
+    return host[1][v, : int(host[0][v]) * 48].view(MIGRATION_DTYPE).copy()
 
 
 def g10_schedule_prefetch(K, num_migrations, migrations, kernel_start_ns, tensor_bytes, gpu_capacity_bytes, pressure,
