@@ -176,13 +176,13 @@ int32_t check_ws(int32_t which, const g10_trace *t, void *ws, size_t ws_bytes)
     } while (0)
 
 // Prepares the workspace and returns the device view of the trace (staging it first in host mode).
-enum { kZeroCounts = 1, kZeroDiff = 2, kZeroState = 4, kZeroPairs = 8, kZeroDiffPoint = 16 };
+enum { kZeroCounts = 1, kZeroDiff = 2, kZeroState = 4, kZeroPairs = 8, kZeroDiffPoint = 16, kZeroNothing = 32 };
 
 int32_t begin_call(int32_t which, const g10_trace *t, void *ws, Workspace &w, DeviceTrace &d, cudaStream_t s, int zero_mask)
 {
     Sizes z{t->num_kernels, t->num_tensors, t->num_events, t->mem == G10_MEM_HOST};
     carve(ws, z, w, which);
-    {
+    if (!(zero_mask & kZeroNothing)) {
         size_t head = w.zero_bytes;
         if (zero_mask & kZeroDiff) head = (size_t)((char *)(w.diff + z.K + 1) - w.zero_begin);
         if (zero_mask & kZeroPairs) head = (size_t)((char *)(w.tl_pair + 2 * z.N) - w.zero_begin);
@@ -213,6 +213,54 @@ cudaError_t d2h(T *dst, const T *src, size_t count, cudaStream_t s)
 {
     if (count == 0 || dst == nullptr) return cudaSuccess;
     return cudaMemcpyAsync(dst, src, sizeof(T) * count, cudaMemcpyDeviceToHost, s);
+}
+
+// The device's address of pinned host memory (null if `p` is not pinned; a null p with nothing behind it stays null).
+template <typename T>
+bool pinned(T *p, size_t count, T **out)
+{
+    *out = nullptr;
+    if (p == nullptr || count == 0) return true;
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, (const void *)p) != cudaSuccess) { cudaGetLastError(); return false; }
+    if (at.type != cudaMemoryTypeHost || at.devicePointer == nullptr) return false;
+    *out = (T *)at.devicePointer;
+    return true;
+}
+
+// A host trace that fits one SM, every array pinned: the kernel reads and writes host memory itself (20 copies of 3-5 us each cost
+// more than the analysis).  False: some array is not pinned.
+bool pinned_small(const g10_trace *t, const g10_vitality_out *out, SmallArgs &A)
+{
+    const size_t K = (size_t)t->num_kernels, N = (size_t)t->num_tensors, E = (size_t)t->num_events;
+    A.t.K = t->num_kernels; A.t.N = t->num_tensors; A.t.E = t->num_events;
+    bool ok = pinned(t->kernel_ptr, K + 1, &A.t.kernel_ptr) && pinned(t->kernel_tensors, E, &A.t.kernel_tensors) &&
+              pinned(t->tensor_bytes, N, &A.t.tensor_bytes) && pinned(t->kernel_ns, K, &A.t.kernel_ns) &&
+              pinned(t->tensor_global, N, &A.t.tensor_global) && pinned(out->first_use, N, &A.v.first_use) &&
+              pinned(out->last_use, N, &A.v.last_use) && pinned(out->num_uses, N, &A.v.num_uses) && pinned(out->use_ptr, N + 1, &A.v.use_ptr) &&
+              pinned(out->uses, (size_t)out->uses_cap, &A.v.uses) && pinned(out->period_ptr, N + 1, &A.v.period_ptr) &&
+              pinned(out->period_tensor, (size_t)out->periods_cap, &A.v.period_tensor) &&
+              pinned(out->period_prev_use, (size_t)out->periods_cap, &A.v.period_prev_use) &&
+              pinned(out->period_next_use, (size_t)out->periods_cap, &A.v.period_next_use) && pinned(out->counts, 3, &A.v.counts);
+    A.v.uses_cap = out->uses_cap; A.v.periods_cap = out->periods_cap;
+    if (const g10_timeline_out *to = out->timeline)
+        ok = ok && pinned(to->kernel_start_ns, K + 1, &A.start) && pinned(to->pressure, K, &A.pressure) && pinned(to->peak_bytes, 1, &A.peak_bytes) &&
+             pinned(to->peak_slot, 1, &A.peak_slot) && pinned(to->status, 1, &A.status_timeline);
+    if (!ok) return false;
+    A.status_counts = A.v.counts + 2;
+    return true;
+}
+
+// The analysis of a planner call in one launch, into the workspace (pressure: where the planner wants it).
+SmallArgs plan_small(const DeviceTrace &d, const Workspace &w, int64_t *pressure)
+{
+    SmallArgs A;
+    A.t = d;
+    A.v = VitalityBuffers{w.first_use, w.last_use, w.num_uses, w.use_ptr, w.uses, d.E, w.period_ptr,
+                          w.period_tensor, w.period_prev_use, w.period_next_use, d.E, w.counts};
+    A.start = w.start; A.pressure = pressure; A.peak_bytes = w.peak_bytes; A.peak_slot = w.peak_slot;
+    A.status_word = w.status; A.done = w.one_done;
+    return A;
 }
 
 size_t carve_emit(void *base, int64_t N, int64_t n, EmitLaunch &L, char **zero_begin, size_t *zero_bytes)
@@ -318,6 +366,25 @@ int32_t g10_vitality(const g10_trace *trace, g10_vitality_out *out, void *ws, si
     rc = check_ws(wsk, trace, ws, ws_bytes);
     if (rc != G10_OK) return rc;
     cudaStream_t s = (cudaStream_t)stream;
+    if (small_analysis_fits(trace->num_kernels, trace->num_tensors, trace->num_events)) {
+        // (one launch, no workspace)
+        SmallArgs A;
+        if (trace->mem == G10_MEM_DEVICE) {
+            A.t = DeviceTrace{trace->num_kernels, trace->num_tensors, trace->num_events, trace->kernel_ptr, trace->kernel_tensors, trace->tensor_bytes,
+                              trace->kernel_ns, trace->tensor_global};
+            A.v = VitalityBuffers{out->first_use, out->last_use, out->num_uses, out->use_ptr, out->uses, out->uses_cap, out->period_ptr,
+                                  out->period_tensor, out->period_prev_use, out->period_next_use, out->periods_cap, out->counts};
+            if (to) { A.start = to->kernel_start_ns; A.pressure = to->pressure; A.peak_bytes = to->peak_bytes; A.peak_slot = to->peak_slot; A.status_timeline = to->status; }
+            A.status_counts = out->counts + 2;
+            CU(launch_small(A, s));
+            return G10_OK;
+        }
+        if (pinned_small(trace, out, A)) {
+            CU(launch_small(A, s));
+            CU(cudaStreamSynchronize(s));
+            return G10_OK;
+        }
+    }
     Workspace w;
     DeviceTrace d;
     const bool buckets = vitality_buckets_supported(trace->num_tensors, trace->num_events);
@@ -524,7 +591,8 @@ int32_t g10_plan_cyclic(const g10_trace *trace, uint64_t gpu_capacity_bytes, uin
     const bool buckets = vitality_buckets_supported(trace->num_tensors, trace->num_events);
     // (the planner state in global memory is cleared where a trace may be too large for the on-chip planner)
     const bool on_chip = plan_keeps_state_on_chip(trace->num_kernels, trace->num_events, options && options->host_capacity_bytes != 0, 0, true);
-    rc = begin_call(G10_WS_PLAN, trace, ws, w, d, s, (buckets ? 0 : kZeroCounts) | kZeroDiff | (on_chip ? 0 : kZeroState));
+    const bool small = small_analysis_fits(trace->num_kernels, trace->num_tensors, trace->num_events);
+    rc = begin_call(G10_WS_PLAN, trace, ws, w, d, s, small && on_chip ? (int)kZeroNothing : (buckets ? 0 : kZeroCounts) | kZeroDiff | (on_chip ? 0 : kZeroState));
     if (rc != G10_OK) return rc;
     VitalityBuffers vb{w.first_use, w.last_use, w.num_uses, w.use_ptr, w.uses, d.E, w.period_ptr,
                        w.period_tensor, w.period_prev_use, w.period_next_use, d.E, w.counts};
@@ -538,14 +606,21 @@ int32_t g10_plan_cyclic(const g10_trace *trace, uint64_t gpu_capacity_bytes, uin
     pp.migrations_cap = host ? (out->migrations_cap < d.E ? out->migrations_cap : d.E) : out->migrations_cap;
     pp.final_pressure = host ? w.pressure : out->final_pressure;
     pp.summary = host ? w.summary : out->summary;
-    CU(launch_slot_clock(d, w, w.start, s));
-    CU(buckets ? launch_vitality_buckets(d, w, vb, s) : launch_vitality(d, w, vb, s));
-    CU(launch_pressure(d, w, w.first_use, w.last_use, false, pp.final_pressure, w.peak_bytes, w.peak_slot, s));
-    CU(launch_cyclic_prepare(d, w, s));
-    CU(launch_geometry(2 * d.K, d.E, w.counts + 1, w.start2, d.tensor_bytes, w.period_tensor, w.period_prev_use, w.period_next_use,
-                       host_bw, ssd_bw, d.E > 0 ? d.E : 1, w.geo_t, w.geo_a, w.geo_b, s));
+    if (small) {
+        SmallArgs A = plan_small(d, w, pp.final_pressure);
+        A.start2 = w.start2;
+        CU(launch_small(A, s));
+    } else {
+        CU(launch_slot_clock(d, w, w.start, s));
+        CU(buckets ? launch_vitality_buckets(d, w, vb, s) : launch_vitality(d, w, vb, s));
+        CU(launch_pressure(d, w, w.first_use, w.last_use, false, pp.final_pressure, w.peak_bytes, w.peak_slot, s));
+        CU(launch_cyclic_prepare(d, w, s));
+    }
+    if (!on_chip)                                               // (the on-chip planner works the geometry out itself)
+        CU(launch_geometry(2 * d.K, d.E, w.counts + 1, w.start2, d.tensor_bytes, w.period_tensor, w.period_prev_use, w.period_next_use,
+                           host_bw, ssd_bw, d.E > 0 ? d.E : 1, w.geo_t, w.geo_a, w.geo_b, s));
     CU(launch_plan_cyclic(d, w, pp, s));
-    CU(launch_publish_status_or(w, pp.summary + 7, s));
+    if (!on_chip) CU(launch_publish_status_or(w, pp.summary + 7, s));
     if (host) {
         int64_t summary[8];
         CU(cudaMemcpyAsync(summary, w.summary, sizeof(summary), cudaMemcpyDeviceToHost, s));
@@ -581,7 +656,8 @@ int32_t g10_plan_batch(const g10_trace *trace, int32_t V, const g10_variant *var
     Workspace w;
     DeviceTrace d;
     const bool buckets = vitality_buckets_supported(trace->num_tensors, trace->num_events);
-    rc = begin_call(G10_WS_BATCH, trace, ws, w, d, s, (buckets ? 0 : kZeroCounts) | kZeroDiff);
+    const bool small = small_analysis_fits(trace->num_kernels, trace->num_tensors, trace->num_events);
+    rc = begin_call(G10_WS_BATCH, trace, ws, w, d, s, small ? (int)kZeroNothing : (buckets ? 0 : kZeroCounts) | kZeroDiff);
     if (rc != G10_OK) return rc;
     CU(cudaMemcpyAsync(w.batch_variants, bv.data(), sizeof(BatchVariant) * (size_t)V, cudaMemcpyHostToDevice, s));
     VitalityBuffers vb{w.first_use, w.last_use, w.num_uses, w.use_ptr, w.uses, d.E, w.period_ptr,
@@ -591,9 +667,12 @@ int32_t g10_plan_batch(const g10_trace *trace, int32_t V, const g10_variant *var
     pp.max_iterations = max_iterations; pp.flags = 0;
     pp.migrations = out->migrations; pp.migrations_cap = out->migrations_cap;
     pp.final_pressure = out->final_pressure; pp.summary = out->summary;
-    CU(launch_slot_clock(d, w, w.start, s));                    // validates kernel_ptr and the trace's own durations
-    CU(buckets ? launch_vitality_buckets(d, w, vb, s) : launch_vitality(d, w, vb, s));
-    CU(launch_pressure(d, w, w.first_use, w.last_use, false, w.pressure, w.peak_bytes, w.peak_slot, s));
+    if (small) CU(launch_small(plan_small(d, w, w.pressure), s));
+    else {
+        CU(launch_slot_clock(d, w, w.start, s));                // validates kernel_ptr and the trace's own durations
+        CU(buckets ? launch_vitality_buckets(d, w, vb, s) : launch_vitality(d, w, vb, s));
+        CU(launch_pressure(d, w, w.first_use, w.last_use, false, w.pressure, w.peak_bytes, w.peak_slot, s));
+    }
     // A cluster per variant: as many blocks as the SMs allow for all variants at once (measured on a ResNet-152 step: 4.4 us an
     // iteration with one block, 4.0 / 3.7 / 3.5 with 4 / 8 / 16).  It needs the trace to fit their shared memory, which only the device
     // can tell (the number of periods is counted there).  Variant 0 says so: if it could not be planned, more blocks get a try;
@@ -649,7 +728,9 @@ int32_t g10_plan_migrations(const g10_trace *trace, uint64_t gpu_capacity_bytes,
     DeviceTrace d;
     const uint32_t flags = options ? options->flags : 0;
     const bool buckets = !(flags & G10_FLAG_RESCORE_ALL) && vitality_buckets_supported(trace->num_tensors, trace->num_events);
-    rc = begin_call(G10_WS_PLAN, trace, ws, w, d, s, (buckets ? 0 : kZeroCounts) | kZeroDiff | (plan_keeps_state_on_chip(trace->num_kernels, trace->num_events, options && options->host_capacity_bytes != 0, flags, false) ? 0 : kZeroState));
+    const bool on_chip = plan_keeps_state_on_chip(trace->num_kernels, trace->num_events, options && options->host_capacity_bytes != 0, flags, false);
+    const bool small = !(flags & G10_FLAG_RESCORE_ALL) && small_analysis_fits(trace->num_kernels, trace->num_tensors, trace->num_events);
+    rc = begin_call(G10_WS_PLAN, trace, ws, w, d, s, small && on_chip ? (int)kZeroNothing : (buckets ? 0 : kZeroCounts) | kZeroDiff | (on_chip ? 0 : kZeroState));
     if (rc != G10_OK) return rc;
     const bool host = trace->mem == G10_MEM_HOST;
 #ifdef G10_TEST_HOOKS
@@ -676,17 +757,23 @@ int32_t g10_plan_migrations(const g10_trace *trace, uint64_t gpu_capacity_bytes,
         return cudaSuccess;
     };
     CU(mark(0));
-    CU(launch_slot_clock(d, w, w.start, s));
-    CU(buckets ? launch_vitality_buckets(d, w, vb, s) : launch_vitality(d, w, vb, s));
-    CU(mark(1));
-    CU(launch_pressure(d, w, w.first_use, w.last_use, false, pp.final_pressure, w.peak_bytes, w.peak_slot, s));
+    if (small) {
+        CU(launch_small(plan_small(d, w, pp.final_pressure), s));
+        CU(mark(1));
+    } else {
+        CU(launch_slot_clock(d, w, w.start, s));
+        CU(buckets ? launch_vitality_buckets(d, w, vb, s) : launch_vitality(d, w, vb, s));
+        CU(mark(1));
+        CU(launch_pressure(d, w, w.first_use, w.last_use, false, pp.final_pressure, w.peak_bytes, w.peak_slot, s));
+    }
     CU(mark(2));
-    CU(launch_geometry(d.K, d.E, w.counts + 1, w.start, d.tensor_bytes, w.period_tensor, w.period_prev_use, w.period_next_use,
-                       host_bw, ssd_bw, d.E > 0 ? d.E : 1, w.geo_t, w.geo_a, w.geo_b, s));
+    if (!on_chip)                                               // (the on-chip planner works the geometry out itself)
+        CU(launch_geometry(d.K, d.E, w.counts + 1, w.start, d.tensor_bytes, w.period_tensor, w.period_prev_use, w.period_next_use,
+                           host_bw, ssd_bw, d.E > 0 ? d.E : 1, w.geo_t, w.geo_a, w.geo_b, s));
     CU(mark(3));
     CU(launch_plan_loop(d, w, pp, s));
     CU(mark(4));
-    CU(launch_publish_status(w, pp.summary + 7, s));
+    if (!on_chip) CU(launch_publish_status(w, pp.summary + 7, s));
     if (host) {
         int64_t summary[8];
         CU(cudaMemcpyAsync(summary, w.summary, sizeof(summary), cudaMemcpyDeviceToHost, s));

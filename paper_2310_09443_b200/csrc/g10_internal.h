@@ -171,6 +171,20 @@ struct VitalityBuffers {
     int64_t tl_K = 0;
 };
 
+// The whole analysis of a trace that fits one SM, in one launch (g10_small.cu).
+struct SmallArgs {
+    DeviceTrace t;               // (device memory, or pinned host memory by its device addresses; so are the outputs)
+    VitalityBuffers v;
+    int64_t *start = nullptr, *pressure = nullptr, *peak_bytes = nullptr;     // timeline (null: vitality alone)
+    int32_t *peak_slot = nullptr;
+    int64_t *start2 = nullptr;   // unrolled clock [2K + 1] (null: not wanted); the wrap-around periods come with it
+    int64_t *status_counts = nullptr, *status_timeline = nullptr;             // receive the status word (either may be null)
+    ull *status_word = nullptr;  // planner calls: the call's own status word and "the plan is done" flag, set up here
+    unsigned *done = nullptr;
+};
+bool small_analysis_fits(int64_t K, int64_t N, int64_t E);
+cudaError_t launch_small(const SmallArgs &A, cudaStream_t s);
+
 struct PlanParams {
     uint64_t gpu_capacity_bytes, host_bw, ssd_bw, host_capacity_bytes;
     int64_t max_iterations;

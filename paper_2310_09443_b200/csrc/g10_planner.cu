@@ -103,6 +103,7 @@ void fill_plan_args(const DeviceTrace &t, const Workspace &w, const PlanParams &
     A.P = p.final_pressure; A.busy = w.busy; A.hocc = w.hocc; A.dead = w.dead;
     A.fits_always = p.gpu_capacity_bytes >= ((uint64_t)1 << 63) ? 1 : 0;
     A.cap = A.fits_always ? INT64_MAX : (int64_t)p.gpu_capacity_bytes;
+    A.bw[G10_DEST_SSD] = p.ssd_bw; A.bw[G10_DEST_HOST] = p.host_bw;
     A.host_capacity = p.host_capacity_bytes;
     A.max_iterations = p.max_iterations;
     A.out = p.migrations; A.out_cap = p.migrations_cap; A.summary = p.summary;
@@ -124,7 +125,7 @@ cudaError_t launch_plan_lazy(const PlanArgs &A, const Workspace &w, int G, cudaS
 int plan_lazy_blocks();
 int plan_chip_blocks(int64_t E, bool several);
 int plan_chip_possible(int64_t K, int64_t E, int C, bool host_cap, bool cyclic);
-cudaError_t launch_plan_chip(const PlanArgs &A, const Workspace &w, int C, bool cyclic, cudaStream_t s);
+cudaError_t launch_plan_chip(const PlanArgs &A, const Workspace &w, int C, bool cyclic, bool alone, cudaStream_t s);
 
 static int chip_blocks(int64_t E, uint32_t flags) { return plan_chip_blocks(E, (flags & G10_FLAG_MULTI_BLOCK) != 0); }
 
@@ -154,7 +155,7 @@ cudaError_t launch_plan_cyclic(const DeviceTrace &t, const Workspace &w, const P
     // GPU is queued behind it and does the work otherwise
     const int C = chip_blocks(t.E, 0), fits = plan_chip_possible(t.K, t.E, C, p.host_capacity_bytes != 0, true);
     if (fits) {
-        const cudaError_t e = launch_plan_chip(A, w, C, true, s);
+        const cudaError_t e = launch_plan_chip(A, w, C, true, fits == 2, s);
         if (e != cudaSuccess || fits == 2) return e;
     }
     const int G = blocks_for((const void *)k_plan_loop<true>);
@@ -188,7 +189,7 @@ cudaError_t launch_plan_loop(const DeviceTrace &t, const Workspace &w, const Pla
         // (as in launch_plan_cyclic)
         const int C = chip_blocks(t.E, p.flags), fits = plan_chip_possible(t.K, t.E, C, p.host_capacity_bytes != 0, false);
         if (fits) {
-            const cudaError_t e = launch_plan_chip(A, w, C, false, s);
+            const cudaError_t e = launch_plan_chip(A, w, C, false, fits == 2, s);
             if (e != cudaSuccess || fits == 2) return e;
         }
     }

@@ -24,6 +24,7 @@ struct PlanArgs {
     unsigned char *dead;                   // period erased (committed, or no destination can ever take it)
     int64_t cap;
     int fits_always;
+    uint64_t bw[2];                        // bytes per second: SSD, host link
     uint64_t host_capacity;
     int64_t max_iterations;
     g10_migration *out;

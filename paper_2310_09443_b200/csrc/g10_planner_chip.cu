@@ -42,6 +42,7 @@ struct ChipArgs {
     int smem_bytes;          // dynamic shared memory the launch provides
     int64_t *busy_global;    // [cluster size][4][K], hocc_global [cluster size][K]: used when they do not fit shared memory
     int64_t *hocc_global;    // (null in batch mode: everything has to fit)
+    int alone;               // the only planner of the call: works the geometry out itself and hands the status word over
 };
 
 // The best period of a block, as the blocks of the cluster tell each other.
@@ -334,7 +335,7 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_plan_chip(PlanArgs A, ChipA
     const int K = (int)A.K;
     const int64_t Pn64 = *A.Pn_dev < A.geo_stride ? *A.Pn_dev : A.geo_stride;
     const int64_t *P_src = A.P;
-    uint64_t bw0 = 0, bw1 = 0;
+    uint64_t bw0 = A.bw[G10_DEST_SSD], bw1 = A.bw[G10_DEST_HOST];
     const int64_t *var_dur = nullptr;
     if (kBatch) {
         const int v = blockIdx.x / C;
@@ -509,7 +510,7 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_plan_chip(PlanArgs A, ChipA
         for (int X = 1; X >= 0; --X) {
             int ap, bp;
             int64_t tx;
-            if (kBatch) period_geometry(T.start, u, v, s, X ? bw1 : bw0, &tx, &ap, &bp);
+            if (kBatch || O.alone) period_geometry(T.start, u, v, s, X ? bw1 : bw0, &tx, &ap, &bp);
             else { ap = A.geo_a[X * A.geo_stride + p]; bp = A.geo_b[X * A.geo_stride + p]; tx = A.geo_t[X * A.geo_stride + p]; }
             if (X == G10_DEST_HOST && host_cap && (uint64_t)s > A.host_capacity) ap = -1;            // (never fits there)
             if (ap < 0) continue;
@@ -850,12 +851,13 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_plan_chip(PlanArgs A, ChipA
 #pragma unroll 1
         for (int j = 1; j < kChipWarps; ++j)
             if (s_ps[j] >= 0 && (ps < 0 || s_pk[j] > pk || (s_pk[j] == pk && s_ps[j] < ps))) { pk = s_pk[j]; ps = s_ps[j]; }
-        if (status == -2) raise_status(A.status, G10_DEV_TIMEOUT);
+        if (status == -2) { raise_status(A.status, G10_DEV_TIMEOUT); s_bits |= G10_DEV_TIMEOUT; }
         A.summary[0] = n_mig; A.summary[1] = rounds; A.summary[2] = status == -2 ? -1 : status;
         A.summary[3] = ps < 0 ? 0 : pk; A.summary[4] = ps;
         A.summary[5] = s_moved[0]; A.summary[6] = s_moved[1];
         // status bits found by this plan: the batch keeps them per variant, a single plan in the call's status word
-        if (kBatch || kCyclic) A.summary[7] = s_bits;        // (the call-wide status word is folded in afterwards)
+        if (O.alone) A.summary[7] = (int64_t)(s_bits | (unsigned)*(volatile ull *)A.status);
+        else if (kBatch || kCyclic) A.summary[7] = s_bits;   // (the call-wide status word is folded in afterwards)
         else if (s_bits) raise_status(A.status, s_bits);
         if (!kBatch) *O.done = 1u;
     }
@@ -894,6 +896,7 @@ static ChipArgs chip_args(const void *kernel, const Workspace &w)
     ChipArgs O;
     O.done = w.one_done; O.smem_bytes = chip_smem_budget(kernel);
     O.busy_global = w.busy_rep; O.hocc_global = w.hocc_rep;
+    O.alone = 0;
     return O;
 }
 
@@ -914,13 +917,15 @@ int plan_chip_possible(int64_t K, int64_t E, int C, bool host_cap, bool cyclic)
     return (int64_t)chip_smem_core(K, most < 64 ? most : 64, C, host_cap, cyclic) <= room ? 1 : 0;
 }
 
-// cyclic (steady-state planning): A.start is the unrolled clock [2K + 1], the period and geometry arrays hold unrolled slots.
-cudaError_t launch_plan_chip(const PlanArgs &A, const Workspace &w, int C, bool cyclic, cudaStream_t s)
+// alone: no other planner is queued behind (plan_chip_possible == 2).  cyclic (steady-state planning): A.start is the unrolled clock [2K + 1], the period and geometry arrays hold unrolled slots.
+cudaError_t launch_plan_chip(const PlanArgs &A, const Workspace &w, int C, bool cyclic, bool alone, cudaStream_t s)
 {
     const void *kernel = chip_kernel(cyclic);
     BatchArgs B;
     B.variants = nullptr; B.P0 = nullptr; B.P_out = nullptr;
-    return launch_chip(kernel, A, chip_args(kernel, w), B, 1, C, s);
+    ChipArgs O = chip_args(kernel, w);
+    O.alone = alone ? 1 : 0;
+    return launch_chip(kernel, A, O, B, 1, C, s);
 }
 
 // ---------------------------------------------------------------------------------------------

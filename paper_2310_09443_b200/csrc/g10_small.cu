@@ -1,0 +1,422 @@
+// All of the analysis -- slot clock, tensor vitality, pressure timeline, and for the steady-state planner the unrolled clock and
+// the wrap-around periods -- of a trace that fits the shared memory of one SM, by ONE block in one launch.  The general passes are
+// five launches of a few microseconds each on such a trace, every one a chain of latencies on a nearly idle GPU; here a step hands
+// over to the next through shared memory and a block barrier.  Inputs are read once and outputs written once, both coalesced, so
+// that the pointers may also be those of pinned host memory: no copies, no staging.
+// Kernels, tensors and positions in the use lists are 16-bit numbers in shared memory (K, N, E < 65535).
+#include "g10_device.cuh"
+#include "g10_internal.h"
+
+namespace g10 {
+
+constexpr int kSmThreads = 1024;
+constexpr int kSmWarps = kSmThreads / 32;
+constexpr int kSmMid = 32;                          // longer segments are sorted by a warp or by the block
+constexpr int kSmWarpSort = 1024;                   // ... up to this length by a warp
+typedef unsigned short u16;
+
+struct SmallLayout {
+    size_t r1, r2, r3, off, dp, total;              // byte offsets of the regions
+};
+__host__ __device__ inline SmallLayout small_layout(int64_t K, int64_t N, int64_t E)
+{
+    auto up = [](size_t x) { return (x + 15) / 16 * 16; };
+    const size_t ev = up((size_t)E * 2), slots = up((size_t)(K + 1) * 8), a = ev > slots ? ev : slots;
+    SmallLayout l;
+    l.r1 = 0; l.r2 = a; l.r3 = 2 * a; l.off = l.r3 + ev; l.dp = l.off + up((size_t)(N + 1) * 4); l.total = l.dp + up((size_t)(N + 1) * 4);
+    return l;
+}
+
+// Exclusive sum over the block (one value per thread); *total gets the sum of all.
+template <typename T>
+__device__ __forceinline__ T small_scan(T v, T *s_w /* [kSmWarps] */, T *total)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    T incl = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) { const T y = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += y; }
+    __syncthreads();                                // (s_w free)
+    if (lane == 31) s_w[warp] = incl;
+    __syncthreads();
+    const T x = s_w[lane];
+    T xi = x;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) { const T y = __shfl_up_sync(0xffffffffu, xi, o); if (lane >= o) xi += y; }
+    *total = __shfl_sync(0xffffffffu, xi, 31);
+    return __shfl_sync(0xffffffffu, xi - x, warp) + incl - v;
+}
+
+// In-place exclusive prefix of n entries in shared memory: a run of consecutive entries per thread (an odd number, so that the
+// threads of a warp meet in different banks).  Returns the total; ends without a barrier.
+template <typename T>
+__device__ __forceinline__ T small_prefix(T *a, int n, T *s_w)
+{
+    const int c = ((n + kSmThreads - 1) / kSmThreads) | 1, lo = (int)threadIdx.x * c < n ? (int)threadIdx.x * c : n, hi = lo + c < n ? lo + c : n;
+    T sum = 0, total;
+#pragma unroll 4
+    for (int k = lo; k < hi; ++k) sum += a[k];
+    T run = small_scan<T>(sum, s_w, &total);
+#pragma unroll 4
+    for (int k = lo; k < hi; ++k) { const T v = a[k]; a[k] = run; run += v; }
+    return total;
+}
+
+// Adds to a 64-bit word of shared memory: two 32-bit atomics with a carry (a 64-bit one is a compare-and-swap loop).
+__device__ __forceinline__ void small_add64(long long *p, long long v)
+{
+    unsigned *w = reinterpret_cast<unsigned *>(p);
+    const unsigned lo = (unsigned)v, old = atomicAdd(&w[0], lo);
+    const unsigned up = (unsigned)((ull)v >> 32) + (old + lo < old ? 1u : 0u);
+    if (up) atomicAdd(&w[1], up);
+}
+
+// Bitonic sort of n entries by `nt` threads (a warp or the block); arbitrary n: the network only moves values up.
+template <bool kBlock>
+__device__ void small_sort(u16 *a, int n, int me, int nt)
+{
+    int n2 = 1;
+    while (n2 < n) n2 <<= 1;
+    for (int k = 2; k <= n2; k <<= 1)
+        for (int j = k >> 1, lj = 31 - __clz(k >> 1); j > 0; j >>= 1, --lj) {
+            const bool mirror = j == (k >> 1);
+            for (int t = me; t < n2 / 2; t += nt) {
+                const int blk = t >> lj, f = t & (j - 1), i = blk * 2 * j + f, p = mirror ? blk * 2 * j + 2 * j - 1 - f : i + j;
+                if (p < n) {
+                    const u16 x = a[i], y = a[p];
+                    if (x > y) { a[i] = y; a[p] = x; }
+                }
+            }
+            if (kBlock) __syncthreads(); else __syncwarp();
+        }
+}
+
+// Removes the repeats of a sorted segment and counts its periods (one warp); distinct uses | periods << 16.
+__device__ unsigned small_compact_warp(u16 *seg, int m, int lane)
+{
+    int d = 0, pp = 0, prev = -1;                   // prev: last use kept so far
+    for (int c0 = 0; c0 < m; c0 += 32) {
+        const int t = c0 + lane;
+        const int x = t < m ? seg[t] : 0x10000;
+        int before = __shfl_up_sync(0xffffffffu, x, 1);
+        if (lane == 0) before = prev;
+        const bool keep = t < m && x != before, per = keep && before >= 0 && x - before >= 2;
+        const unsigned mk = __ballot_sync(0xffffffffu, keep), mp = __ballot_sync(0xffffffffu, per);
+        if (keep) seg[d + __popc(mk & ((1u << lane) - 1u))] = (u16)x;        // (never overtakes an unread entry)
+        d += __popc(mk); pp += __popc(mp);
+        const int last = (m - c0 < 32 ? m - c0 : 32) - 1;
+        prev = __shfl_sync(0xffffffffu, x, last);
+        __syncwarp();
+    }
+    return (unsigned)d | (unsigned)pp << 16;
+}
+
+__global__ void __launch_bounds__(kSmThreads, 1) k_small(SmallArgs A)
+{
+    extern __shared__ __align__(16) unsigned char s_mem[];
+    __shared__ long long s_w64[kSmWarps];
+    __shared__ unsigned s_w32[kSmWarps];
+    __shared__ int s_sl[kSmWarps];
+    __shared__ unsigned s_bits;
+    __shared__ int s_nmid, s_nheavy;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int K = (int)A.t.K, N = (int)A.t.N, E = (int)A.t.E;
+    const SmallLayout l = small_layout(K, N, E);
+    u16 *s_id = (u16 *)(s_mem + l.r1), *s_krel = (u16 *)(s_mem + l.r2), *ks = (u16 *)(s_mem + l.r3);
+    long long *s_diff = (long long *)(s_mem + l.r1), *s_ns = (long long *)(s_mem + l.r2);
+    unsigned *off = (unsigned *)(s_mem + l.off), *dp = (unsigned *)(s_mem + l.dp);
+    const bool clock = A.start != nullptr;
+    unsigned bad = 0;
+
+    // ---- tensor ids, durations, kernels of the events
+    if (tid == 0) { s_bits = 0; s_nmid = 0; s_nheavy = 0; }
+#pragma unroll 4
+    for (int t = tid; t <= N; t += kSmThreads) off[t] = 0;
+    if (clock)
+#pragma unroll 4
+        for (int k = tid; k < K; k += kSmThreads) {
+            long long d = A.t.kernel_ns[k];
+            if (d < 1 || d >= ((long long)1 << 44)) { bad |= G10_DEV_BAD_DURATION; d = 1; }
+            s_ns[k] = d;
+        }
+    __syncthreads();
+#pragma unroll 8
+    for (int e = tid; e < E; e += kSmThreads) {
+        const int id = A.t.kernel_tensors[e];
+        const bool ok = id >= 0 && id < N;
+        if (ok) atomicAdd(&off[id], 1u); else bad |= G10_DEV_BAD_TENSOR_ID;
+        s_id[e] = ok ? (u16)id : (u16)0xffff;
+    }
+    if (clock) {
+        // slot clock
+        const long long total = small_prefix<long long>(s_ns, K, s_w64);
+        if (total >= ((long long)1 << 44)) bad |= G10_DEV_BAD_DURATION;
+        __syncthreads();
+        for (int k = tid; k < K; k += kSmThreads) {
+            const long long s = s_ns[k];
+            A.start[k] = s;
+            if (A.start2 != nullptr) { A.start2[k] = s; A.start2[K + k] = s + total; }
+        }
+        if (tid == 0) { A.start[K] = total; if (A.start2 != nullptr) A.start2[2 * K] = 2 * total; }
+        __syncthreads();
+    }
+    // (a kernel_ptr that is no monotone map onto [0, E] leaves every tensor unused; the walk stays inside the events in any case)
+#pragma unroll 2
+    for (int k0 = warp * 32; k0 < K; k0 += kSmThreads) {
+        const int k = k0 + lane;
+        const int64_t p0 = k < K ? A.t.kernel_ptr[k] : 0, p1 = k < K ? A.t.kernel_ptr[k + 1] : 0;
+        if (k < K && (p0 > p1 || p0 < 0 || p1 > E || (k == 0 && p0 != 0) || (k == K - 1 && p1 != E))) bad |= G10_DEV_BAD_KERNEL_PTR;
+        const int a = p0 < 0 ? 0 : p0 > E ? E : (int)p0, b = p1 < 0 ? 0 : p1 > E ? E : (int)p1;
+        const bool wide = b - a > 64;
+        if (!wide) for (int p = a; p < b; ++p) s_krel[p] = (u16)k;
+        unsigned m = __ballot_sync(0xffffffffu, wide);
+        while (m) {
+            const int src = __ffs(m) - 1;
+            m &= m - 1;
+            const int wa = __shfl_sync(0xffffffffu, a, src), wb = __shfl_sync(0xffffffffu, b, src);
+            for (int p = wa + lane; p < wb; p += 32) s_krel[p] = (u16)(k0 + src);
+        }
+    }
+    {
+        const unsigned w = __reduce_or_sync(0xffffffffu, bad);
+        if (lane == 0 && w) atomicOr(&s_bits, w);
+    }
+    // ---- events into per-tensor segments of ks (off[t]: first the start of t's segment, after the scatter its end)
+    __syncthreads();
+    small_prefix<unsigned>(off, N, s_w32);
+    __syncthreads();
+    const bool none = (s_bits & G10_DEV_BAD_KERNEL_PTR) != 0;
+    if (!none)
+#pragma unroll 4
+        for (int e = tid; e < E; e += kSmThreads) {
+            const unsigned id = s_id[e];
+            if (id != 0xffffu) ks[atomicAdd(&off[id], 1u)] = s_krel[e];
+        }
+    __syncthreads();
+    u16 *s_mid = s_krel;                            // tensors with three to kSmMid raw uses; with more, from the other end
+    auto segment = [&](int t, int *m) {
+        const int o = t > 0 ? (int)off[t - 1] : 0;
+        *m = none ? 0 : (int)off[t] - o;
+        return ks + o;
+    };
+#pragma unroll 2
+    for (int t = tid; t < N; t += kSmThreads) {
+        int m;
+        u16 *seg = segment(t, &m);
+        unsigned r = m > 0 ? 1u : 0u;
+        if (m == 2) {
+            const int x = seg[0], y = seg[1], lo = x < y ? x : y, hi = x < y ? y : x;
+            if (lo != hi) { seg[0] = (u16)lo; seg[1] = (u16)hi; r = 2u | (hi - lo >= 2 ? 1u << 16 : 0u); }
+        } else if (m > kSmMid) s_mid[E - 1 - atomicAdd(&s_nheavy, 1)] = (u16)t;
+        else if (m > 2) s_mid[atomicAdd(&s_nmid, 1)] = (u16)t;
+        dp[t] = r;
+    }
+    __syncthreads();
+    const int nmid = s_nmid, nheavy = s_nheavy;
+    for (int q = tid; q < nmid; q += kSmThreads) {
+        const int t = s_mid[q];
+        int m;
+        u16 *seg = segment(t, &m);
+        int d = 1, pp = 0, prev;
+        if (m <= 8) {
+            // put in order by a network in registers, the padding to the end: one round trip to shared memory
+            int v[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) v[j] = j < m ? seg[j] : 0x10000;
+#define G10_CE(a, b) { const int lo = min(v[a], v[b]), hi = max(v[a], v[b]); v[a] = lo; v[b] = hi; }
+            G10_CE(0, 1) G10_CE(2, 3) G10_CE(4, 5) G10_CE(6, 7) G10_CE(0, 2) G10_CE(1, 3) G10_CE(4, 6) G10_CE(5, 7) G10_CE(1, 2) G10_CE(5, 6)
+            G10_CE(0, 4) G10_CE(1, 5) G10_CE(2, 6) G10_CE(3, 7) G10_CE(2, 4) G10_CE(3, 5) G10_CE(1, 2) G10_CE(3, 4) G10_CE(5, 6)
+#undef G10_CE
+            prev = v[0];
+            seg[0] = (u16)prev;
+#pragma unroll
+            for (int a = 1; a < 8; ++a) {
+                const int x = v[a];
+                if (a < m && x != prev) { if (x - prev >= 2) ++pp; seg[d++] = (u16)x; prev = x; }
+            }
+        } else {
+            // (the scatter took the events nearly in order: hardly anything moves)
+            for (int a = 1; a < m; ++a) {
+                const u16 x = seg[a];
+                int c = a - 1;
+                while (c >= 0 && seg[c] > x) { seg[c + 1] = seg[c]; --c; }
+                seg[c + 1] = x;
+            }
+            prev = seg[0];
+            for (int a = 1; a < m; ++a) {
+                const int x = seg[a];
+                if (x != prev) { if (x - prev >= 2) ++pp; seg[d++] = (u16)x; prev = x; }
+            }
+        }
+        dp[t] = (unsigned)d | (unsigned)pp << 16;
+    }
+    for (int q = warp; q < nheavy; q += kSmWarps) {
+        const int t = s_mid[E - 1 - q];
+        int m;
+        u16 *seg = segment(t, &m);
+        if (m > kSmWarpSort) continue;
+        small_sort<false>(seg, m, lane, 32);
+        const unsigned r = small_compact_warp(seg, m, lane);
+        if (lane == 0) dp[t] = r;
+    }
+    for (int q = 0; q < nheavy; ++q) {              // (the few that a block sorts better)
+        const int t = s_mid[E - 1 - q];
+        int m;
+        u16 *seg = segment(t, &m);
+        if (m <= kSmWarpSort) continue;
+        small_sort<true>(seg, m, tid, kSmThreads);
+        if (warp == 0) { const unsigned r = small_compact_warp(seg, m, lane); if (lane == 0) dp[t] = r; }
+    }
+    __syncthreads();
+    // ---- offsets of every tensor's uses and periods (16 bits each: both sums are at most E)
+    const unsigned total = small_prefix<unsigned>(dp, N, s_w32);
+    if (tid == 0) dp[N] = total;
+    __syncthreads();
+    const int D = (int)(total & 0xffffu), PC = (int)(total >> 16);
+    const VitalityBuffers &out = A.v;
+    bad = 0;
+    if (D > out.uses_cap) bad |= G10_DEV_USES_OVERFLOW;
+    if (PC > out.periods_cap) bad |= G10_DEV_PERIODS_OVERFLOW;
+    const int raw = none ? 0 : (int)off[N - 1];
+    const bool dense = D == raw;                    // no repeats: ks is the use list as it stands
+    u16 *s_pos = s_id, *s_ten = s_krel;             // of every period: where its first use stands in ks, its tensor
+#pragma unroll 2
+    for (int t = tid; t < N; t += kSmThreads) {
+        int m;
+        const u16 *seg = segment(t, &m);
+        const unsigned x = dp[t], y = dp[t + 1];
+        const int d = (int)((y - x) & 0xffffu), uo = (int)(x & 0xffffu);
+        int po = (int)(x >> 16);
+        out.first_use[t] = d > 0 ? (int)seg[0] : -1;
+        out.last_use[t] = d > 0 ? (int)seg[d - 1] : -1;
+        out.num_uses[t] = d;
+        out.use_ptr[t] = uo; out.period_ptr[t] = po;
+        const int o = (int)(seg - ks);
+        for (int a = 0; a < d; ++a) {
+            if (!dense && uo + a < out.uses_cap) out.uses[uo + a] = seg[a];
+            if (a + 1 < d && seg[a + 1] - seg[a] >= 2) { s_pos[po] = (u16)(o + a); s_ten[po] = (u16)t; ++po; }
+        }
+    }
+    if (tid == 0) { out.use_ptr[N] = D; out.period_ptr[N] = PC; out.counts[0] = D; out.counts[1] = PC; }
+    if (dense)
+        for (int j = tid; j < D && j < out.uses_cap; j += kSmThreads) out.uses[j] = ks[j];
+    __syncthreads();
+#pragma unroll 4
+    for (int p = tid; p < PC; p += kSmThreads) {
+        const int i = s_pos[p];
+        if (p < out.periods_cap) { out.period_tensor[p] = s_ten[p]; out.period_prev_use[p] = ks[i]; out.period_next_use[p] = ks[i + 1]; }
+    }
+    if (clock) {
+        __syncthreads();
+        for (int k = tid; k <= K; k += kSmThreads) s_diff[k] = 0;
+        __syncthreads();
+        // ---- pressure: sizes where the tensors are born and where they die, prefix sum, peak and its lowest slot
+        long long everywhere = 0;                   // bytes of the global tensors
+        int wrap_base = PC;
+        const uint8_t *glob = A.t.tensor_global;
+        for (int t0 = 0; t0 < N; t0 += kSmThreads) {
+            const int t = t0 + tid;
+            bool wrap = false;
+            int f = 0, la = 0;
+            if (t < N) {
+                const long long b = A.t.tensor_bytes[t];
+                const bool g = glob != nullptr && glob[t] != 0;
+                int m;
+                const u16 *seg = segment(t, &m);
+                const int d = (int)((dp[t + 1] - dp[t]) & 0xffffu);
+                if (b < 1 || b >= ((long long)1 << 40)) bad |= G10_DEV_BAD_BYTES;
+                if (d > 0) {
+                    f = seg[0]; la = seg[d - 1];
+                    if (g) { everywhere += b; wrap = f + K - la >= 2; }
+                    else { small_add64(&s_diff[f], b); small_add64(&s_diff[la + 1], -b); }
+                }
+            }
+            if (A.start2 != nullptr) {
+                // steady state: the period of a global tensor that spans two iterations, behind the ordinary ones in tensor order
+                unsigned n;
+                const unsigned at = small_scan<unsigned>(wrap ? 1u : 0u, s_w32, &n);
+                const int64_t p = (int64_t)wrap_base + at;
+                if (wrap) {
+                    if (p < out.periods_cap) { out.period_tensor[p] = t; out.period_prev_use[p] = la; out.period_next_use[p] = f + K; }
+                    else bad |= G10_DEV_PERIODS_OVERFLOW;
+                }
+                wrap_base += (int)n;
+            }
+        }
+        if (A.start2 != nullptr && tid == 0) out.counts[1] = wrap_base;
+        everywhere = warp_sum_i64(everywhere);
+        if (lane == 0 && everywhere != 0) small_add64(&s_diff[0], everywhere);
+        __syncthreads();
+        const int c = ((K + kSmThreads - 1) / kSmThreads) | 1, lo = tid * c < K ? tid * c : K, hi = lo + c < K ? lo + c : K;
+        long long sum = 0, all, mx = 0;
+        int sl = -1;
+#pragma unroll 4
+        for (int k = lo; k < hi; ++k) sum += s_diff[k];
+        long long run = small_scan<long long>(sum, s_w64, &all);
+#pragma unroll 4
+        for (int k = lo; k < hi; ++k) {
+            run += s_diff[k];
+            s_diff[k] = run;
+            if (sl < 0 || run > mx) { mx = run; sl = k; }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const long long ym = __shfl_down_sync(0xffffffffu, mx, o);
+            const int ys = __shfl_down_sync(0xffffffffu, sl, o);
+            if (ys >= 0 && (sl < 0 || ym > mx || (ym == mx && ys < sl))) { mx = ym; sl = ys; }
+        }
+        __syncthreads();
+        if (lane == 0) { s_w64[warp] = mx; s_sl[warp] = sl; }
+#pragma unroll 4
+        for (int k = tid; k < K; k += kSmThreads) A.pressure[k] = s_diff[k];
+        __syncthreads();
+        if (warp == 0) {
+            mx = s_w64[lane]; sl = s_sl[lane];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const long long ym = __shfl_down_sync(0xffffffffu, mx, o);
+                const int ys = __shfl_down_sync(0xffffffffu, sl, o);
+                if (ys >= 0 && (sl < 0 || ym > mx || (ym == mx && ys < sl))) { mx = ym; sl = ys; }
+            }
+            if (lane == 0) { *A.peak_bytes = mx; *A.peak_slot = sl; }
+        }
+    }
+    {
+        const unsigned w = __reduce_or_sync(0xffffffffu, bad);
+        if (lane == 0 && w) atomicOr(&s_bits, w);
+    }
+    __syncthreads();
+    if (tid == 0) {
+        const int64_t st = (int64_t)s_bits;
+        if (A.status_counts != nullptr) *A.status_counts = st;
+        if (A.status_timeline != nullptr) *A.status_timeline = st;
+        if (A.status_word != nullptr) *A.status_word = (ull)st;
+        if (A.done != nullptr) *A.done = 0u;
+    }
+}
+
+// Shared memory the kernel may use: the most that a block can opt in to, minus its static part.
+static size_t small_budget()
+{
+    int dev = 0, optin = 0;
+    cudaFuncAttributes fa;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) return 0;
+    if (cudaFuncGetAttributes(&fa, (const void *)k_small) != cudaSuccess) return 0;
+    return optin > (int)fa.sharedSizeBytes ? (size_t)optin - fa.sharedSizeBytes : 0;
+}
+
+bool small_analysis_fits(int64_t K, int64_t N, int64_t E)
+{
+    if (K < 1 || N < 1 || E < 1 || K >= 65535 || N >= 65535 || E >= 65535) return false;
+    return small_layout(K, N, E).total <= small_budget();
+}
+
+cudaError_t launch_small(const SmallArgs &A, cudaStream_t s)
+{
+    const size_t smem = small_layout(A.t.K, A.t.N, A.t.E).total;
+    const cudaError_t e = cudaFuncSetAttribute((const void *)k_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k_small<<<1, kSmThreads, smem, s>>>(A); count_launch();
+    return cudaGetLastError();
+}
+
+}  // namespace g10

@@ -967,3 +967,29 @@ def test_on_chip_planner_edges(gpu, oracle, K, chains):
         for v in (0, V - 1):
             assert np.array_equal(gpu.batch_migrations_numpy(out, v), ref.migrations) and int(out.summary[v, 7].item()) == 0
             assert np.array_equal(_np(out.final_pressure)[v], ref.final_pressure)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("K,N,E", [(1, 1, 1), (1023, 1025, 2048), (1024, 33, 9000), (37, 3, 30000), (2049, 20000, 20001), (9000, 9000, 30000)])
+def test_one_launch_analysis_edges(gpu, oracle, K, N, E):
+    """The one-block analysis around its block size, with segments for one thread, a warp and the block (repeats in all),
+    near the most that fits shared memory; results in device memory, in pinned host memory and (staged) in pageable memory."""
+    rng = np.random.default_rng(K + 7 * N + 11 * E)
+    ptr = np.sort(np.concatenate([[0, E], rng.integers(0, E + 1, size=K - 1)])).astype(np.int64)
+    tr = traces.Trace(name="edges", kernel_ptr=ptr, kernel_tensors=rng.integers(0, N, size=E).astype(np.int32),
+                      tensor_bytes=rng.integers(1, 1 << 39, size=N).astype(np.int64), kernel_ns=rng.integers(1, 1 << 20, size=K).astype(np.int64),
+                      tensor_global=(rng.random(N) < 0.3).astype(np.uint8), capacity_frac=(1, 2))
+    tb = gpu.upload(tr)
+    v, ov = check_vitality(gpu, oracle, tr, tb)
+    check_timeline(gpu, oracle, tr, tb)
+    ref = gpu.g10_vitality(tb, timeline=True)
+    pinned = gpu.pin(tr)
+    pageable = gpu.TraceBuffers(*(t.clone() for t in (pinned.kernel_ptr, pinned.kernel_tensors, pinned.tensor_bytes, pinned.kernel_ns, pinned.tensor_global)))
+    nu, npd = len(ov.uses), len(ov.period_tensor)
+    for host in (pinned, pageable):
+        h = gpu.g10_vitality(host, timeline=True)
+        for a, b, n in ((h.first_use, ref.first_use, N), (h.last_use, ref.last_use, N), (h.use_ptr, ref.use_ptr, N + 1), (h.uses, ref.uses, nu),
+                        (h.period_tensor, ref.period_tensor, npd), (h.period_prev_use, ref.period_prev_use, npd), (h.counts, ref.counts, 3),
+                        (h.timeline.pressure, ref.timeline.pressure, K), (h.timeline.kernel_start_ns, ref.timeline.kernel_start_ns, K + 1),
+                        (h.timeline.peak_bytes, ref.timeline.peak_bytes, 1), (h.timeline.status, ref.timeline.status, 1)):
+            assert np.array_equal(a[:n].numpy(), _np(b)[:n])
