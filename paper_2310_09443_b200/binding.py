@@ -7,6 +7,7 @@ raise.
 from __future__ import annotations
 
 import ctypes as C
+import functools
 import os
 from types import SimpleNamespace
 
@@ -154,13 +155,14 @@ def _check(rc):
 
 
 def _ptr(t):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream):
+    # (the raw handle of the current device's current stream: building a Stream object around it costs a microsecond)
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return C.c_void_p(stream.cuda_stream)
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return stream.cuda_stream
 
 
 class TraceBuffers:
@@ -211,6 +213,7 @@ def g10_launch_count() -> int:
     return int(load_library().g10_launch_count())
 
 
+@functools.lru_cache(maxsize=256)
 def g10_workspace_bytes(which, K, N, E, mem=MEM_DEVICE) -> int:
     out = C.c_size_t(0)
     _check(load_library().g10_workspace_bytes(which, K, N, E, mem, C.byref(out)))

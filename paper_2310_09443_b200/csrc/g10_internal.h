@@ -22,6 +22,7 @@ inline void count_launch() { __atomic_fetch_add(&g_launch_count, 1ull, __ATOMIC_
 namespace g10 {
 
 constexpr size_t kAlign = 256;
+constexpr int kMaxDevices = 64;          // devices whose attributes are remembered
 constexpr int kHeavyThreshold = 32;      // tensors with more raw uses than this are sorted by a whole block
 
 // Multiprocessors of the current device (0 if the query fails).  Asked every time: a process may use several devices.

@@ -863,24 +863,34 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_plan_chip(PlanArgs A, ChipA
     }
 }
 
-// Shared memory a launch can offer (opt-in maximum minus the kernel's static part); 0 if a query fails.
-static int chip_smem_budget(const void *kernel)
+enum { kOnePlan, kOneCycle, kManyPlans };
+static const void *chip_kernel(int which)
 {
+    return which == kOnePlan ? (const void *)k_plan_chip<false, false> : which == kOneCycle ? (const void *)k_plan_chip<false, true> : (const void *)k_plan_chip<true, false>;
+}
+
+// Shared memory a launch can offer (opt-in maximum minus the kernel's static part; 0 if a query fails), and that and the largest
+// cluster allowed on the current device: asked once per kernel and device.
+static int chip_smem_budget(int which)
+{
+    static int known[3][kMaxDevices];
     int dev = 0, optin = 0;
     cudaFuncAttributes fa;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    const void *kernel = chip_kernel(which);
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return 0;
+    if (dev < kMaxDevices) if (const int b = __atomic_load_n(&known[which][dev], __ATOMIC_ACQUIRE)) return b;
     if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) return 0;
     if (cudaFuncGetAttributes(&fa, kernel) != cudaSuccess) return 0;
     const int room = optin - (int)fa.sharedSizeBytes;
-    return room > 0 ? room : 0;
+    if (room <= 0 || cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, room) != cudaSuccess ||
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return 0;
+    if (dev < kMaxDevices) __atomic_store_n(&known[which][dev], room, __ATOMIC_RELEASE);
+    return room;
 }
 
 // Launches `plans` clusters of C blocks (one per plan).
-static cudaError_t launch_chip(const void *kernel, PlanArgs A, ChipArgs O, BatchArgs B, int plans, int C, cudaStream_t s)
+static cudaError_t launch_chip(int which, PlanArgs A, ChipArgs O, BatchArgs B, int plans, int C, cudaStream_t s)
 {
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, O.smem_bytes);
-    if (e == cudaSuccess && C > 8) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(plans * C)); cfg.blockDim = dim3(kChipThreads); cfg.dynamicSmemBytes = (size_t)O.smem_bytes; cfg.stream = s;
     cudaLaunchAttribute at[1];
@@ -888,19 +898,17 @@ static cudaError_t launch_chip(const void *kernel, PlanArgs A, ChipArgs O, Batch
     at[0].val.clusterDim.x = (unsigned)C; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
     cfg.attrs = at; cfg.numAttrs = 1;
     void *args[] = {&A, &O, &B};
-    return cudaLaunchKernelExC(&cfg, kernel, args);
+    return cudaLaunchKernelExC(&cfg, chip_kernel(which), args);
 }
 
-static ChipArgs chip_args(const void *kernel, const Workspace &w)
+static ChipArgs chip_args(int which, const Workspace &w)
 {
     ChipArgs O;
-    O.done = w.one_done; O.smem_bytes = chip_smem_budget(kernel);
+    O.done = w.one_done; O.smem_bytes = chip_smem_budget(which);
     O.busy_global = w.busy_rep; O.hocc_global = w.hocc_rep;
     O.alone = 0;
     return O;
 }
-
-static const void *chip_kernel(bool cyclic) { return cyclic ? (const void *)k_plan_chip<false, true> : (const void *)k_plan_chip<false, false>; }
 
 // Blocks of the cluster.  Measured (ms): 96-kernel chain 0.18 with one block, 0.21 with 16; ResNet-152 step (1652 kernels, 2020
 // periods) 3.7 / 3.1 / 2.9 with 1 / 8 / 16; four ViT-H steps (6692 kernels, 13 875 periods) do not fit fewer than 16.  A block
@@ -912,7 +920,7 @@ int plan_chip_blocks(int64_t E, bool several) { return E <= 1024 && !several ? 1
 int plan_chip_possible(int64_t K, int64_t E, int C, bool host_cap, bool cyclic)
 {
     if (E < 1 || K > kChipMaxSlots || (cyclic ? 2 * K : K) >= (int64_t)kSlotTop) return 0;
-    const int64_t room = chip_smem_budget(chip_kernel(cyclic)), most = (E + C - 1) / C;
+    const int64_t room = chip_smem_budget(cyclic ? kOneCycle : kOnePlan), most = (E + C - 1) / C;
     if (most <= kChipMaxPeriods && (int64_t)chip_smem_core(K, most, C, host_cap, cyclic) <= room) return 2;
     return (int64_t)chip_smem_core(K, most < 64 ? most : 64, C, host_cap, cyclic) <= room ? 1 : 0;
 }
@@ -920,12 +928,12 @@ int plan_chip_possible(int64_t K, int64_t E, int C, bool host_cap, bool cyclic)
 // alone: no other planner is queued behind (plan_chip_possible == 2).  cyclic (steady-state planning): A.start is the unrolled clock [2K + 1], the period and geometry arrays hold unrolled slots.
 cudaError_t launch_plan_chip(const PlanArgs &A, const Workspace &w, int C, bool cyclic, bool alone, cudaStream_t s)
 {
-    const void *kernel = chip_kernel(cyclic);
+    const int which = cyclic ? kOneCycle : kOnePlan;
     BatchArgs B;
     B.variants = nullptr; B.P0 = nullptr; B.P_out = nullptr;
-    ChipArgs O = chip_args(kernel, w);
+    ChipArgs O = chip_args(which, w);
     O.alone = alone ? 1 : 0;
-    return launch_chip(kernel, A, O, B, 1, C, s);
+    return launch_chip(which, A, O, B, 1, C, s);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -987,10 +995,9 @@ cudaError_t launch_batch_finish(const DeviceTrace &t, const Workspace &w, const 
 
 cudaError_t launch_plan_batch(const PlanArgs &A, const Workspace &w, int V, int C, const BatchArgs &B, int64_t *stability, cudaStream_t s)
 {
-    const void *kernel = (const void *)k_plan_chip<true, false>;
-    ChipArgs O = chip_args(kernel, w);
+    ChipArgs O = chip_args(kManyPlans, w);
     O.busy_global = nullptr; O.hocc_global = nullptr;      // (the workspace has no room per variant)
-    cudaError_t e = launch_chip(kernel, A, O, B, V, C, s);
+    cudaError_t e = launch_chip(kManyPlans, A, O, B, V, C, s);
     if (e != cudaSuccess) return e;
     return run_batch_finish(A.geo_stride, A.Pn_dev, A.out, A.out_cap, A.summary, V, stability, A.status, s);
 }

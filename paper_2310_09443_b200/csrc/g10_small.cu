@@ -131,21 +131,37 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(SmallArgs A)
     if (tid == 0) { s_bits = 0; s_nmid = 0; s_nheavy = 0; }
 #pragma unroll 4
     for (int t = tid; t <= N; t += kSmThreads) off[t] = 0;
-    if (clock)
-#pragma unroll 4
-        for (int k = tid; k < K; k += kSmThreads) {
-            long long d = A.t.kernel_ns[k];
-            if (d < 1 || d >= ((long long)1 << 44)) { bad |= G10_DEV_BAD_DURATION; d = 1; }
-            s_ns[k] = d;
-        }
     __syncthreads();
-#pragma unroll 8
-    for (int e = tid; e < E; e += kSmThreads) {
-        const int id = A.t.kernel_tensors[e];
+    // (loads in batches, all of a batch before the first use: the stores in between would keep the compiler from doing that, and
+    // from host memory a load takes 1.5 us)
+    if (clock)
+        for (int k0 = tid; k0 < K; k0 += 4 * kSmThreads) {
+            long long d[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) d[q] = k0 + q * kSmThreads < K ? A.t.kernel_ns[k0 + q * kSmThreads] : 1;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                if (d[q] < 1 || d[q] >= ((long long)1 << 44)) { bad |= G10_DEV_BAD_DURATION; d[q] = 1; }
+                if (k0 + q * kSmThreads < K) s_ns[k0 + q * kSmThreads] = d[q];
+            }
+        }
+    auto event = [&](int e, int id) {
         const bool ok = id >= 0 && id < N;
         if (ok) atomicAdd(&off[id], 1u); else bad |= G10_DEV_BAD_TENSOR_ID;
         s_id[e] = ok ? (u16)id : (u16)0xffff;
+    };
+    const int E4 = ((uintptr_t)A.t.kernel_tensors & 15) == 0 ? E / 4 : 0;        // events taken four at a time
+    for (int e0 = tid; e0 < E4; e0 += 4 * kSmThreads) {
+        int4 id[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) id[q] = e0 + q * kSmThreads < E4 ? reinterpret_cast<const int4 *>(A.t.kernel_tensors)[e0 + q * kSmThreads] : make_int4(0, 0, 0, 0);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int e = 4 * (e0 + q * kSmThreads);
+            if (e < 4 * E4) { event(e, id[q].x); event(e + 1, id[q].y); event(e + 2, id[q].z); event(e + 3, id[q].w); }
+        }
     }
+    for (int e = 4 * E4 + tid; e < E; e += kSmThreads) event(e, A.t.kernel_tensors[e]);
     if (clock) {
         // slot clock
         const long long total = small_prefix<long long>(s_ns, K, s_w64);
@@ -160,20 +176,30 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(SmallArgs A)
         __syncthreads();
     }
     // (a kernel_ptr that is no monotone map onto [0, E] leaves every tensor unused; the walk stays inside the events in any case)
-#pragma unroll 2
-    for (int k0 = warp * 32; k0 < K; k0 += kSmThreads) {
-        const int k = k0 + lane;
-        const int64_t p0 = k < K ? A.t.kernel_ptr[k] : 0, p1 = k < K ? A.t.kernel_ptr[k + 1] : 0;
-        if (k < K && (p0 > p1 || p0 < 0 || p1 > E || (k == 0 && p0 != 0) || (k == K - 1 && p1 != E))) bad |= G10_DEV_BAD_KERNEL_PTR;
-        const int a = p0 < 0 ? 0 : p0 > E ? E : (int)p0, b = p1 < 0 ? 0 : p1 > E ? E : (int)p1;
-        const bool wide = b - a > 64;
-        if (!wide) for (int p = a; p < b; ++p) s_krel[p] = (u16)k;
-        unsigned m = __ballot_sync(0xffffffffu, wide);
-        while (m) {
-            const int src = __ffs(m) - 1;
-            m &= m - 1;
-            const int wa = __shfl_sync(0xffffffffu, a, src), wb = __shfl_sync(0xffffffffu, b, src);
-            for (int p = wa + lane; p < wb; p += 32) s_krel[p] = (u16)(k0 + src);
+    for (int k0 = warp * 32; k0 < K; k0 += 4 * kSmThreads) {
+        int64_t first[4], next[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int k = k0 + q * kSmThreads + lane;
+            first[q] = k <= K ? A.t.kernel_ptr[k] : E;
+            next[q] = lane == 31 && k < K ? A.t.kernel_ptr[k + 1] : E;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int kq = k0 + q * kSmThreads, k = kq + lane;
+            if (kq >= K) break;
+            const int64_t p0 = first[q], down = __shfl_down_sync(0xffffffffu, first[q], 1), p1 = lane == 31 ? next[q] : down;
+            if (k < K && (p0 > p1 || p0 < 0 || p1 > E || (k == 0 && p0 != 0) || (k == K - 1 && p1 != E))) bad |= G10_DEV_BAD_KERNEL_PTR;
+            const int a = p0 < 0 ? 0 : p0 > E ? E : (int)p0, b = k >= K || p1 < 0 ? 0 : p1 > E ? E : (int)p1;
+            const bool wide = b - a > 64;
+            if (!wide) for (int p = a; p < b; ++p) s_krel[p] = (u16)k;
+            unsigned m = __ballot_sync(0xffffffffu, wide);
+            while (m) {
+                const int src = __ffs(m) - 1;
+                m &= m - 1;
+                const int wa = __shfl_sync(0xffffffffu, a, src), wb = __shfl_sync(0xffffffffu, b, src);
+                for (int p = wa + lane; p < wb; p += 32) s_krel[p] = (u16)(kq + src);
+            }
         }
     }
     {
@@ -279,21 +305,36 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(SmallArgs A)
     const int raw = none ? 0 : (int)off[N - 1];
     const bool dense = D == raw;                    // no repeats: ks is the use list as it stands
     u16 *s_pos = s_id, *s_ten = s_krel;             // of every period: where its first use stands in ks, its tensor
-#pragma unroll 2
-    for (int t = tid; t < N; t += kSmThreads) {
-        int m;
-        const u16 *seg = segment(t, &m);
-        const unsigned x = dp[t], y = dp[t + 1];
-        const int d = (int)((y - x) & 0xffffu), uo = (int)(x & 0xffffu);
-        int po = (int)(x >> 16);
-        out.first_use[t] = d > 0 ? (int)seg[0] : -1;
-        out.last_use[t] = d > 0 ? (int)seg[d - 1] : -1;
-        out.num_uses[t] = d;
-        out.use_ptr[t] = uo; out.period_ptr[t] = po;
-        const int o = (int)(seg - ks);
-        for (int a = 0; a < d; ++a) {
-            if (!dense && uo + a < out.uses_cap) out.uses[uo + a] = seg[a];
-            if (a + 1 < d && seg[a + 1] - seg[a] >= 2) { s_pos[po] = (u16)(o + a); s_ten[po] = (u16)t; ++po; }
+    for (int t0 = tid; t0 < N; t0 += 2 * kSmThreads) {
+        unsigned x[2], y[2];
+        int o[2], f[2], la[2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int t = t0 + q * kSmThreads;
+            const bool in = t < N;
+            x[q] = in ? dp[t] : 0u; y[q] = in ? dp[t + 1] : 0u;
+            o[q] = in && t > 0 ? (int)off[t - 1] : 0;
+        }
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int d = (int)((y[q] - x[q]) & 0xffffu);
+            f[q] = d > 0 ? (int)ks[o[q]] : -1; la[q] = d > 0 ? (int)ks[o[q] + d - 1] : -1;
+        }
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int t = t0 + q * kSmThreads;
+            if (t >= N) break;
+            const int d = (int)((y[q] - x[q]) & 0xffffu), uo = (int)(x[q] & 0xffffu), p0 = (int)(x[q] >> 16);
+            out.first_use[t] = f[q]; out.last_use[t] = la[q]; out.num_uses[t] = d;
+            out.use_ptr[t] = uo; out.period_ptr[t] = p0;
+            if (!dense) for (int a = 0; a < d && uo + a < out.uses_cap; ++a) out.uses[uo + a] = ks[o[q] + a];
+            if (y[q] >> 16 == (unsigned)p0) continue;         // (no period: nearly all)
+            int po = p0, prev = f[q];
+            for (int a = 1; a < d; ++a) {
+                const int v = ks[o[q] + a];
+                if (v - prev >= 2) { s_pos[po] = (u16)(o[q] + a - 1); s_ten[po] = (u16)t; ++po; }
+                prev = v;
+            }
         }
     }
     if (tid == 0) { out.use_ptr[N] = D; out.period_ptr[N] = PC; out.counts[0] = D; out.counts[1] = PC; }
@@ -307,39 +348,53 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(SmallArgs A)
     }
     if (clock) {
         __syncthreads();
-        for (int k = tid; k <= K; k += kSmThreads) s_diff[k] = 0;
-        __syncthreads();
         // ---- pressure: sizes where the tensors are born and where they die, prefix sum, peak and its lowest slot
         long long everywhere = 0;                   // bytes of the global tensors
         int wrap_base = PC;
         const uint8_t *glob = A.t.tensor_global;
-        for (int t0 = 0; t0 < N; t0 += kSmThreads) {
-            const int t = t0 + tid;
-            bool wrap = false;
-            int f = 0, la = 0;
-            if (t < N) {
-                const long long b = A.t.tensor_bytes[t];
-                const bool g = glob != nullptr && glob[t] != 0;
-                int m;
-                const u16 *seg = segment(t, &m);
-                const int d = (int)((dp[t + 1] - dp[t]) & 0xffffu);
-                if (b < 1 || b >= ((long long)1 << 40)) bad |= G10_DEV_BAD_BYTES;
-                if (d > 0) {
-                    f = seg[0]; la = seg[d - 1];
-                    if (g) { everywhere += b; wrap = f + K - la >= 2; }
-                    else { small_add64(&s_diff[f], b); small_add64(&s_diff[la + 1], -b); }
-                }
+        constexpr int kBook = 4;
+        for (int t00 = 0; t00 < N; t00 += kBook * kSmThreads) {
+            long long size[kBook];
+            bool global[kBook];
+#pragma unroll
+            for (int q = 0; q < kBook; ++q) {
+                const int t = t00 + q * kSmThreads + tid;
+                size[q] = t < N ? A.t.tensor_bytes[t] : 1;
+                global[q] = t < N && glob != nullptr && glob[t] != 0;
             }
-            if (A.start2 != nullptr) {
-                // steady state: the period of a global tensor that spans two iterations, behind the ordinary ones in tensor order
-                unsigned n;
-                const unsigned at = small_scan<unsigned>(wrap ? 1u : 0u, s_w32, &n);
-                const int64_t p = (int64_t)wrap_base + at;
-                if (wrap) {
-                    if (p < out.periods_cap) { out.period_tensor[p] = t; out.period_prev_use[p] = la; out.period_next_use[p] = f + K; }
-                    else bad |= G10_DEV_PERIODS_OVERFLOW;
+            if (t00 == 0) {                         // (cleared while the first sizes come in)
+                for (int k = tid; k <= K; k += kSmThreads) s_diff[k] = 0;
+                __syncthreads();
+            }
+#pragma unroll
+            for (int q = 0; q < kBook; ++q) {
+                const int t = t00 + q * kSmThreads + tid;
+                if (t00 + q * kSmThreads >= N) break;
+                const long long b = size[q];
+                bool wrap = false;
+                int f = 0, la = 0;
+                if (t < N) {
+                    int m;
+                    const u16 *seg = segment(t, &m);
+                    const int d = (int)((dp[t + 1] - dp[t]) & 0xffffu);
+                    if (b < 1 || b >= ((long long)1 << 40)) bad |= G10_DEV_BAD_BYTES;
+                    if (d > 0) {
+                        f = seg[0]; la = seg[d - 1];
+                        if (global[q]) { everywhere += b; wrap = f + K - la >= 2; }
+                        else { small_add64(&s_diff[f], b); small_add64(&s_diff[la + 1], -b); }
+                    }
                 }
-                wrap_base += (int)n;
+                if (A.start2 != nullptr) {
+                    // steady state: the period of a global tensor that spans two iterations, behind the ordinary ones in tensor order
+                    unsigned n;
+                    const unsigned at = small_scan<unsigned>(wrap ? 1u : 0u, s_w32, &n);
+                    const int64_t p = (int64_t)wrap_base + at;
+                    if (wrap) {
+                        if (p < out.periods_cap) { out.period_tensor[p] = t; out.period_prev_use[p] = la; out.period_next_use[p] = f + K; }
+                        else bad |= G10_DEV_PERIODS_OVERFLOW;
+                    }
+                    wrap_base += (int)n;
+                }
             }
         }
         if (A.start2 != nullptr && tid == 0) out.counts[1] = wrap_base;
@@ -394,14 +449,21 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(SmallArgs A)
     }
 }
 
-// Shared memory the kernel may use: the most that a block can opt in to, minus its static part.
+// Shared memory the kernel may use (the most that a block can opt in to, minus its static part), allowed on the current device:
+// asked once per device.
 static size_t small_budget()
 {
+    static int known[kMaxDevices];                  // 0: not asked yet
     int dev = 0, optin = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return 0;
+    if (dev < kMaxDevices) if (const int b = __atomic_load_n(&known[dev], __ATOMIC_ACQUIRE)) return (size_t)b;
     cudaFuncAttributes fa;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) return 0;
+    if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) return 0;
     if (cudaFuncGetAttributes(&fa, (const void *)k_small) != cudaSuccess) return 0;
-    return optin > (int)fa.sharedSizeBytes ? (size_t)optin - fa.sharedSizeBytes : 0;
+    const int room = optin - (int)fa.sharedSizeBytes;
+    if (room <= 0 || cudaFuncSetAttribute((const void *)k_small, cudaFuncAttributeMaxDynamicSharedMemorySize, room) != cudaSuccess) return 0;
+    if (dev < kMaxDevices) __atomic_store_n(&known[dev], room, __ATOMIC_RELEASE);
+    return (size_t)room;
 }
 
 bool small_analysis_fits(int64_t K, int64_t N, int64_t E)
@@ -413,8 +475,6 @@ bool small_analysis_fits(int64_t K, int64_t N, int64_t E)
 cudaError_t launch_small(const SmallArgs &A, cudaStream_t s)
 {
     const size_t smem = small_layout(A.t.K, A.t.N, A.t.E).total;
-    const cudaError_t e = cudaFuncSetAttribute((const void *)k_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
     k_small<<<1, kSmThreads, smem, s>>>(A); count_launch();
     return cudaGetLastError();
 }
