@@ -465,10 +465,9 @@ def g10_characterize(K, N, use_ptr, uses, tensor_bytes, kernel_start_ns, num_per
     """Section 3 statistics (Figures 2-4) from the vitality results and the slot clock (device tensors)."""
     lib = load_library()
     dev = kernel_start_ns.device
-    r = SimpleNamespace(active_bytes=torch.empty(max(K, 1), dtype=torch.int64, device=dev),
-                        len_hist=torch.empty(64, dtype=torch.int64, device=dev),
-                        size_len_hist=torch.empty(41 * 45, dtype=torch.int64, device=dev),
-                        hide=torch.empty(2, dtype=torch.int64, device=dev), summary=torch.empty(2, dtype=torch.int64, device=dev))
+    n = max(K, 1)                                                     # (one allocation for the five results)
+    active, lens, sizes, hide, summary = torch.empty(n + 64 + 41 * 45 + 4, dtype=torch.int64, device=dev).split((n, 64, 41 * 45, 2, 2))
+    r = SimpleNamespace(active_bytes=active, len_hist=lens, size_len_hist=sizes, hide=hide, summary=summary)
     out = _StatsOut(_ptr(r.active_bytes), _ptr(r.len_hist), _ptr(r.size_len_hist), _ptr(r.hide), _ptr(r.summary))
     _check(lib.g10_characterize(K, N, _ptr(use_ptr), _ptr(uses), _ptr(tensor_bytes), _ptr(kernel_start_ns), int(num_periods),
                                 _ptr(period_tensor), _ptr(period_prev_use), _ptr(period_next_use), host_bw, ssd_bw, C.byref(out),
