@@ -164,6 +164,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(SmallArgs A)
     for (int e = 4 * E4 + tid; e < E; e += kSmThreads) event(e, A.t.kernel_tensors[e]);
     if (clock) {
         // slot clock
+        __syncthreads();
         const long long total = small_prefix<long long>(s_ns, K, s_w64);
         if (total >= ((long long)1 << 44)) bad |= G10_DEV_BAD_DURATION;
         __syncthreads();
