@@ -15,7 +15,7 @@ CSRC = os.path.join(HERE, "csrc")
 OBJ_PLAIN, OBJ_HOOKS = os.path.join(HERE, "build"), os.path.join(HERE, "build_hooks")
 LIB_PLAIN, LIB_HOOKS = os.path.join(HERE, "libg10.so"), os.path.join(HERE, "libg10_hooks.so")
 LIB = LIB_PLAIN
-SOURCES = ["g10_api.cu", "g10_passes.cu", "g10_planner.cu", "g10_planner_lazy.cu",
+SOURCES = ["g10_api.cu", "g10_passes.cu", "g10_planner.cu", "g10_planner_lazy.cu", "g10_planner_spread.cu",
            "g10_planner_chip.cu", "g10_small.cu", "g10_vitality_buckets.cu", "g10_prefetch.cu", "g10_emit.cu", "g10_stats.cu", "g10_cyclic.cu",
            "g10_static.cu"]
 HEADERS = ["g10_device.cuh", "g10_internal.h", "g10_planner.cuh"]

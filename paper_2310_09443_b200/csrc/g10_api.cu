@@ -56,6 +56,8 @@ size_t carve(void *base, const Sizes &z, Workspace &w, int32_t which)
     w.heavy_count = c.take<unsigned>(1);
     w.peak_key = c.take<int>(1);
     w.barrier = c.take<unsigned>(4);
+    w.barrier2 = c.take<unsigned>(4);
+    w.spread_flag = c.take<unsigned>(1);
     carve_scan(c, w.clock_scan, ktiles, 1);
     carve_scan(c, w.count_scan, vit ? ntiles : 1, 1);
     carve_scan(c, w.emit_scan, vit ? etiles : 1, 2);
@@ -116,7 +118,7 @@ size_t carve(void *base, const Sizes &z, Workspace &w, int32_t which)
     w.geo_b = c.take<int32_t>(plan ? 2 * E : 1);
     w.proposals = c.take<Proposal>(plan ? kMaxPlanBlocks : 1);
     w.prop_stale = c.take<Proposal>(plan ? kMaxPlanBlocks : 1);
-    w.lazy_props = c.take<LazyProp>(plan ? 2 * kLazyMaxBlocks : 1);
+    w.lazy_props = c.take<LazyProp>(plan ? 4 * kLazyMaxBlocks : 1);
     w.lazy_partials = c.take<ull>(plan ? (size_t)2 * kRoundM * kLazyMaxBlocks * 2 : 1);
     w.lazy_tmin = c.take<int64_t>(plan ? (size_t)tiles_of(z.K, 1024) : 1);
     w.lazy_tmax = c.take<int64_t>(plan ? (size_t)tiles_of(z.K, 1024) : 1);

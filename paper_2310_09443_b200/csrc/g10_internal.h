@@ -87,7 +87,8 @@ struct Workspace {
     ull *status;                 // device status word
     unsigned *heavy_count;
     int *peak_key;               // K - lowest peak slot (0 = none), reduced with atomicMax
-    void *barrier;               // GridBarrier
+    void *barrier, *barrier2;    // GridBarrier (two: a planner that gives up leaves the other one fresh)
+    unsigned *spread_flag;       // [1] the spread planner cannot keep the trace after all
     ScanSlot clock_scan, count_scan, emit_scan, pressure_scan;
     int32_t *cnt;                // [N] raw use counts, then scatter cursor, then heavy slot index
     int64_t *diff;               // [K+1] signed-size difference array
@@ -124,7 +125,7 @@ struct Workspace {
     int32_t *geo_a, *geo_b;      // [2*E]
     Proposal *proposals;         // [max blocks]
     Proposal *prop_stale;        // [max blocks]
-    LazyProp *lazy_props;        // [2][kLazyMaxBlocks]
+    LazyProp *lazy_props;        // [4][kLazyMaxBlocks]
     ull *lazy_partials;          // [2][kRoundM][kLazyMaxBlocks][2]
     int64_t *lazy_tmin, *lazy_tmax; // [tiles of 1024 slots]
     unsigned char *c_state;      // [E] per-period state of the lazy planner

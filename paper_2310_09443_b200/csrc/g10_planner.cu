@@ -123,6 +123,8 @@ static int blocks_for(const void *kernel)
 
 cudaError_t launch_plan_lazy(const PlanArgs &A, const Workspace &w, int G, cudaStream_t s);
 int plan_lazy_blocks();
+bool plan_spread_possible(int64_t K, int64_t E);
+cudaError_t launch_plan_spread(const PlanArgs &A, const Workspace &w, cudaStream_t s);
 int plan_chip_blocks(int64_t E, bool several);
 int plan_chip_possible(int64_t K, int64_t E, int C, bool host_cap, bool cyclic);
 cudaError_t launch_plan_chip(const PlanArgs &A, const Workspace &w, int C, bool cyclic, bool alone, cudaStream_t s);
@@ -192,6 +194,11 @@ cudaError_t launch_plan_loop(const DeviceTrace &t, const Workspace &w, const Pla
             const cudaError_t e = launch_plan_chip(A, w, C, false, fits == 2, s);
             if (e != cudaSuccess || fits == 2) return e;
         }
+    }
+    // state spread over the shared memory of all SMs if it fits (the device knows), else in global memory
+    if (plan_spread_possible(t.K, t.E)) {
+        const cudaError_t e = launch_plan_spread(A, w, s);
+        if (e != cudaSuccess) return e;
     }
     const int G = plan_lazy_blocks();
     if (G < 1) return cudaErrorLaunchFailure;

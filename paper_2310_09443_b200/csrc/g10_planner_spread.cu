@@ -1,0 +1,838 @@
+// Algorithm 1 for long timelines whose state fits the shared memory of the whole GPU (about 150 SMs, 30 MB: a million slots and a
+// million periods): the lazy evaluation of g10_planner_lazy.cu with every piece of hot state in some SM's shared memory.
+//   - The timeline is cut into tiles of 64 slots, tile t in block t mod G: pressure above capacity and duration per slot; smallest
+//     and largest value, a pending offset and the total duration per tile.  A range of slots, however long, is thus spread evenly
+//     over all blocks, and so are the tiles that have to be read slot by slot, which cluster where the pressure is near capacity.
+//   - Runs of 32 periods are dealt out the same way.  A period is 16 bytes: rounded score, inactive and absent slots, destination,
+//     and whether the score is FRESH (exact) or a bound (pressure only falls, so an earlier score is one).
+// Per iteration:
+//  A  every block applies the last commit to its tiles, compares its periods with it (absent ranges that meet: no longer FRESH;
+//     transfer windows on the same channel that meet: is the destination still possible?  Channels only fill up: SSD -> host ->
+//     erased) and publishes its best FRESH score and its four best bounds; grid barrier;
+//  R  rounds: the published bounds that may beat the best exact score are rescored by all blocks together, each over its own
+//     tiles, with the shares added into grid-wide sums; grid barrier; the best exact score is updated.  A block whose published
+//     bounds are used up while the last may still beat the best score publishes more;
+//  D  no bound left that may beat it: commit.
+// All decisions are taken from data every block has, so the control flow is the same in every block.  Rounded scores steer the
+// search; anything within kNear of a decision is settled by exact 128-bit comparison.
+// What bounds it: grid barriers (three to four an iteration) and waiting in them for the block with the most to rescore.
+// periods in global memory (g10_planner_lazy.cu) an iteration on a million kernels read 140 MB through the L2: 1.02 s for its plan,
+// 0.90 s here (200 k kernels: 1.4 to 1.5 times faster).
+#include "g10_planner.cuh"
+
+namespace g10 {
+
+constexpr int kSpTile = 64;                     // slots per tile
+constexpr int kSpRound = 256;                   // periods rescored together, at most
+constexpr int kSpMix = 1024;                    // (period, tile) pairs of one round that need more than the tile's summary, listed
+constexpr int kSpEdge = 2 * kSpRound;           // pairs in which the period covers the tile in part
+constexpr int kSpSort = 12;                     // tiles sorted together (one warp each)
+constexpr float kFirst = 0.97f;
+constexpr double kNear = 1e-6;                  // (scores are kept as floats, rounded up: 2^-23)
+constexpr int kSpTop = 8;                       // bounds a block publishes
+constexpr int kSpPool = kLazyMaxBlocks * kSpTop;
+static_assert(kPlanWarps == 16, "two chunks of warp counts per 32 lanes");
+constexpr int kSpLimbs = 6;                     // a benefit (below 2^84) as 16-bit limbs
+
+// What a block tells the grid: its best exactly scored period, its best bounds (descending; anything it did not list is no larger
+// than the last), its largest pressure above capacity.
+struct __align__(16) SpProp {
+    ull ben_lo, ben_hi, cost;
+    int idx;                                    // period << 1 | destination, -1 = none
+    unsigned key;                               // its rounded score
+    unsigned skey[kSpTop];
+    int sidx[kSpTop];                           // period << 1 | destination, -1 = none
+    long long peak, pad;
+};
+static_assert(sizeof(SpProp) % 16 == 0 && 2 * sizeof(LazyProp) >= sizeof(SpProp), "workspace for two LazyProp a block");
+
+struct SpreadArgs {
+    ull *c_ben_lo, *c_ben_hi, *c_cost;          // [periods] last computed benefit (exact or a bound), cost of the current destination
+    SpProp *props;                              // [2][kLazyMaxBlocks]
+    ull *partials;                              // [3][2][kSpRound] sums of the low 44 bits and of the rest (three buffers in turn)
+    unsigned *flag;                             // raised by a block that cannot keep its part (a duration of 2^32 ns or more)
+    unsigned *done;                             // set to 1 when this kernel produced the plan
+    int smem_bytes;
+};
+
+// A period: x = score (float bits, rounded up; 0 = no benefit), y, z, w = inactive slots [a, b], absent slots [ap, bp] of the
+// current destination (21 bits each), destination + 1 (0 = erased), FRESH.
+struct SpPeriod { int a, b, ap, bp, dest; bool fresh; };
+__device__ __forceinline__ uint4 sp_pack(unsigned key, int a, int b, int ap, int bp, int dest, bool fresh)
+{
+    return make_uint4(key, (unsigned)a | (unsigned)b << 21, (unsigned)b >> 11 | (unsigned)ap << 10, (unsigned)bp | (unsigned)(dest + 1) << 21 | (fresh ? 1u << 23 : 0u));
+}
+__device__ __forceinline__ SpPeriod sp_unpack(uint4 q)
+{
+    SpPeriod r;
+    r.a = (int)(q.y & 0x1fffffu); r.b = (int)(q.y >> 21 | (q.z & 0x3ffu) << 11); r.ap = (int)(q.z >> 10 & 0x1fffffu);
+    r.bp = (int)(q.w & 0x1fffffu); r.dest = (int)(q.w >> 21 & 3u) - 1; r.fresh = (q.w >> 23 & 1u) != 0u;
+    return r;
+}
+constexpr int kSpMaxSlots = (1 << 21) - 1;
+
+__device__ __forceinline__ unsigned sp_key(u128 ben, ull cost)
+{
+    if (ben == 0) return 0u;
+    Cand c;
+    c.ben = ben; c.cost = cost; c.idx = 0; c.dest = 0;
+    return __float_as_uint(__double2float_ru(cand_key(c) * (1.0 + 1e-14)));     // (positive floats compare like integers)
+}
+__device__ __forceinline__ double sp_val(unsigned key) { return (double)__uint_as_float(key); }
+
+// Could a period with rounded score `key` (an upper bound) beat t?  Clear cases by the rounded scores, close ones exactly.
+__device__ __forceinline__ bool sp_may_beat(const SpreadArgs &S, int p, unsigned key, double t_key, const Cand &t)
+{
+    if (key == 0u) return false;
+    if (t.idx < 0) return true;
+    const double k = sp_val(key);
+    if (k > t_key * (1.0 + kNear)) return true;
+    if (k < t_key * (1.0 - kNear)) return false;
+    Cand x;
+    x.ben = ((u128)__ldcg(&S.c_ben_hi[p]) << 64) | __ldcg(&S.c_ben_lo[p]); x.cost = __ldcg(&S.c_cost[p]); x.idx = p; x.dest = 0;
+    return cand_beats(x, t);
+}
+
+// Largest of the lanes' (key, idx), lowest idx on equal keys; uniform.  idx < 0: nothing.
+__device__ __forceinline__ void sp_warp_max(unsigned &key, int &idx)
+{
+    const unsigned m = __reduce_max_sync(0xffffffffu, idx >= 0 ? key : 0u);
+    const unsigned i = __reduce_min_sync(0xffffffffu, idx >= 0 && key == m ? (unsigned)idx : 0xffffffffu);
+    key = m; idx = i == 0xffffffffu ? -1 : (int)i;
+}
+
+// A tile's slots in order of their pressure, for the periods of a round that cover it all and find some of its slots less than their
+// size above capacity: with prefix sums of the durations and of pressure x duration, a period's benefit is a binary search
+// instead of 64 slots (a round's periods mostly overlap: the same few tiles near capacity are wanted a hundred times).
+struct SpSorted {
+    long long v[kSpTile];                       // pressure above capacity, at least 0 and at most 2^40 (tensors are smaller), ascending
+    ull lo[kSpTile + 1], hi[kSpTile + 1];       // sums of (v mod 2^20) x duration and of (v >> 20) x duration over the first n
+    unsigned d[kSpTile + 1];                    // sums of the durations (a tile's total is below 2^32 ns)
+    int n;
+};
+
+__host__ __device__ inline size_t sp_round16(size_t x) { return (x + 15) / 16 * 16; }
+__host__ __device__ inline size_t sp_smem(int64_t K, int64_t Pn, int G)
+{
+    const size_t tiles = (size_t)(((K + kSpTile - 1) / kSpTile + G - 1) / G), runs = (size_t)(((Pn + 31) / 32 + G - 1) / G);
+    return tiles * kSpTile * 8 + tiles * 40 + runs * 32 * 16 + kSpSort * sizeof(SpSorted) + kSpEdge * 4 +                                     // slots, tiles, periods
+           sp_round16((size_t)G * kSpTop * 4) * 2 + sp_round16((size_t)G * kSpTop) +                              // published bounds
+           (size_t)kSpRound * (4 * kSpLimbs + 8 + 8 + 4 * 4) + (size_t)kSpMix * 4 + 128;                      // a round
+}
+
+__global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, SpreadArgs S)
+{
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    __shared__ Cand s_cand[kPlanWarps + 1];
+    __shared__ BestScratch s_best;
+    __shared__ long long s_max[kPlanWarps + 1];
+    __shared__ unsigned s_wk[kPlanWarps * kSpTop], s_tk[kSpTop], s_fk[kPlanWarps];
+    __shared__ int s_wi[kPlanWarps * kSpTop], s_ti[kSpTop];
+    constexpr int kChunks = (kSpPool + kPlanThreads - 1) / kPlanThreads;        // entries of the pool a thread looks at
+    __shared__ int s_fin[32], s_nfin, s_nmix, s_nedge, s_ndist, s_wcnt[kChunks * kPlanWarps];
+    __shared__ Cand s_one;
+    __shared__ unsigned char s_refresh[kLazyMaxBlocks];
+    if (*S.done) return;                                     // (same answer in every thread of the grid: written by an earlier launch)
+    const int G = gridDim.x, c = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t Pn64 = *A.Pn_dev < A.geo_stride ? *A.Pn_dev : A.geo_stride;
+    if (A.K < 1 || A.K > kSpMaxSlots || Pn64 > 0x3fffffff || sp_smem(A.K, Pn64, G) > (size_t)S.smem_bytes) return;     // (the same answer in all blocks)
+    const int K = (int)A.K, Pn = (int)Pn64;
+    const int64_t limit = (A.max_iterations <= 0 || A.max_iterations > Pn64) ? Pn64 : A.max_iterations;
+    const int NT = (K + kSpTile - 1) / kSpTile, tiles = (NT + G - 1) / G, NR = (Pn + 31) / 32, runs = (NR + G - 1) / G;
+    const int my_tiles = NT > c ? (NT - c + G - 1) / G : 0, my_runs = NR > c ? (NR - c + G - 1) / G : 0;
+    unsigned char *at = s_raw;
+    auto take = [&](size_t bytes) { unsigned char *p = at; at += sp_round16(bytes); return p; };
+    longlong2 *mm = (longlong2 *)take((size_t)tiles * 16);                      // [tiles] smallest / largest, offset included
+    uint4 *hot = (uint4 *)take((size_t)runs * 32 * 16);
+    unsigned *r_acc = (unsigned *)take((size_t)kSpRound * 4 * kSpLimbs);        // [limb][period] (sums of at most 2^16 16-bit limbs)
+    long long *r_s = (long long *)take((size_t)kSpRound * 8);
+    ull *r_cost = (ull *)take((size_t)kSpRound * 8);
+    int *r_p = (int *)take((size_t)kSpRound * 4), *r_e = (int *)take((size_t)kSpRound * 4);      // period << 1 | destination; pool entry
+    int *r_ap = (int *)take((size_t)kSpRound * 4), *r_bp = (int *)take((size_t)kSpRound * 4);
+    unsigned *s_mix = (unsigned *)take((size_t)kSpMix * 4), *s_edge = (unsigned *)take((size_t)kSpEdge * 4);      // period of the round << 20 | local tile
+    SpSorted *sorted = (SpSorted *)take(kSpSort * sizeof(SpSorted));
+    int *t_no = (int *)take((size_t)tiles * 4), *t_at = (int *)take((size_t)tiles * 4);      // distinct tiles of the pairs: number of a tile (-1: none), tile of a number
+    unsigned *pkey = (unsigned *)take((size_t)G * kSpTop * 4);                 // published bounds, [rank in the list][block]
+    int *pidx = (int *)take((size_t)G * kSpTop * 4);                               // period << 1 | destination, -1 = none
+    unsigned char *pdone = take((size_t)G * kSpTop);
+    long long *ex = (long long *)take((size_t)tiles * kSpTile * 8);
+    long long *off = (long long *)take((size_t)tiles * 8);
+    ull *tsum = (ull *)take((size_t)tiles * 8);
+    auto owner_entry = [&](int p) { return (p >> 5) % G == c ? ((p >> 5) / G) * 32 + (p & 31) : -1; };
+
+    unsigned gen = 0;
+    int64_t n_mig = 0, rounds = 0, bytes_ssd = 0, bytes_host = 0;
+    int status = -1;
+    long long peak = 0;
+    int pbuf = 0, pp = 0;
+
+    // ---- own slots, tiles and periods
+    bool bad = false;
+    for (int x = tid; x < my_tiles * kSpTile; x += kPlanThreads) {
+        const int64_t k = ((int64_t)(x / kSpTile) * G + c) * kSpTile + x % kSpTile;
+        ex[x] = k < K ? A.P[k] - A.cap : 0;
+    }
+    for (int lt = tid; lt < my_tiles; lt += kPlanThreads) {
+        const int t = lt * G + c;
+        const long long d = A.start[t * kSpTile + kSpTile < K ? t * kSpTile + kSpTile : K] - A.start[t * kSpTile];
+        if (d >> 32) bad = true;
+        off[lt] = 0; tsum[lt] = (ull)d; t_no[lt] = -1;
+    }
+    if (c == 0) for (int j = tid; j < 3 * kSpRound * 2; j += kPlanThreads) S.partials[j] = 0;
+    __syncthreads();
+    // smallest and largest value of local tile lt (one warp)
+    auto refresh_tile = [&](int lt) {
+        const int t = lt * G + c, n = K - t * kSpTile < kSpTile ? K - t * kSpTile : kSpTile;
+        long long mn = 0x7fffffffffffffffll, mx = -0x7fffffffffffffffll - 1;
+#pragma unroll
+        for (int j = 0; j < kSpTile; j += 32)
+            if (j + lane < n) {
+                const long long v = ex[lt * kSpTile + j + lane];
+                mn = v < mn ? v : mn; mx = v > mx ? v : mx;
+            }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const long long a = __shfl_xor_sync(0xffffffffu, mn, o), b = __shfl_xor_sync(0xffffffffu, mx, o);
+            mn = a < mn ? a : mn; mx = b > mx ? b : mx;
+        }
+        if (lane == 0) mm[lt] = make_longlong2(mn + off[lt], mx + off[lt]);
+    };
+    for (int lt = warp; lt < my_tiles; lt += kPlanWarps) refresh_tile(lt);
+    // (re)starts a period on destination X: its first bound is the benefit it would have if its whole absent range were at least s
+    // above capacity
+    auto begin_period = [&](int p, int e, int X, int a, int b) {
+        const int ap = A.geo_a[X * A.geo_stride + p], bp = A.geo_b[X * A.geo_stride + p];
+        const u128 ben = (u128)(ull)A.bytes[A.per_t[p]] * (u128)(ull)(A.start[bp + 1] - A.start[ap]);
+        const ull cost = 2ull * (ull)A.geo_t[X * A.geo_stride + p];
+        S.c_ben_lo[p] = (ull)ben; S.c_ben_hi[p] = (ull)(ben >> 64); S.c_cost[p] = cost;
+        hot[e] = sp_pack(sp_key(ben, cost), a, b, ap, bp, X, false);
+    };
+    for (int e = tid; e < my_runs * 32; e += kPlanThreads) {
+        const int64_t p = ((int64_t)(e >> 5) * G + c) * 32 + (e & 31);
+        hot[e] = make_uint4(0, 0, 0, 0);
+        if (p >= Pn) continue;
+        // nothing is booked yet: the first usable destination it is
+        const bool room = A.host_capacity == 0 || (uint64_t)A.bytes[A.per_t[p]] <= A.host_capacity;
+        const int X = A.geo_a[p] >= 0 ? 0 : A.geo_a[A.geo_stride + p] >= 0 && room ? 1 : -1;
+        if (X >= 0) begin_period((int)p, e, X, A.per_u[p] + 1, A.per_v[p] - 1);
+    }
+    if (bad) atomicOr(S.flag, 1u);
+    __syncthreads();
+    if (!grid_barrier(A.bar, G, gen)) status = -2;
+    else if (__ldcg(S.flag) != 0u) return;                   // (nothing changed: the planner queued behind this one takes over)
+
+    struct { int idx, dest, a, ap, bp, b; int64_t s, t, t_r, t_end; } w = {-1, -1, 0, 0, -1, -1, 0, 0, 0, 0};     // the pending commit
+    unsigned likely = 0;                                     // bounds below this (four fifths of the last winner's score) are not listed at first
+    float last_key = 0.0f;                                   // the last winner's score
+    bool pending = false;
+    Cand gBest;                                              // best exactly scored period known to the grid
+    gBest.ben = 0; gBest.cost = 1; gBest.idx = -1; gBest.dest = -1;
+
+    // One pass of the block over its periods.  With `classify` the pending commit is applied to them first (its bookings are not in
+    // A.busy yet).  With a floor only bounds that may beat it are listed.  Publishes into buffer pbuf.
+    auto scan = [&](bool classify, bool with_floor) {
+        unsigned fk = 0, tk[kSpTop];
+        int ti[kSpTop];
+#pragma unroll
+        for (int j = 0; j < kSpTop; ++j) { tk[j] = 0; ti[j] = -1; }
+        const int64_t *bo = A.busy + (size_t)(2 * (w.dest < 0 ? 0 : w.dest)) * A.K, *bi = bo + A.K;
+        const unsigned least = with_floor ? 0u : likely;
+        const double floor_key = with_floor && gBest.idx >= 0 ? cand_key(gBest) : -1.0;
+        if (tid == 0) s_nfin = 0;
+        constexpr int kAhead = 4;                                   // runs whose periods are read together
+#pragma unroll 1
+        for (int r0 = warp; r0 < my_runs; r0 += kAhead * kPlanWarps) {
+          uint4 ahead[kAhead];
+#pragma unroll
+          for (int h = 0; h < kAhead; ++h) ahead[h] = r0 + h * kPlanWarps < my_runs ? hot[(r0 + h * kPlanWarps) * 32 + lane] : make_uint4(0, 0, 0, 0);
+#pragma unroll
+          for (int h = 0; h < kAhead; ++h) {
+            const int r = r0 + h * kPlanWarps, e = r * 32 + lane, p = (r * G + c) * 32 + lane;
+            if (r >= my_runs) break;
+            uint4 q = ahead[h];
+            if (classify) {
+                const SpPeriod P = sp_unpack(q);
+                bool lost = false;
+                if (P.dest >= 0 && P.a <= w.b && w.a <= P.b) {
+                    if (p == w.idx) { q = make_uint4(0, 0, 0, 0); hot[e] = q; }
+                    else {
+                        if (P.dest == w.dest) {
+                            const bool meet_out = P.a <= w.ap - 1 && w.a <= P.ap - 1, meet_in = P.bp + 1 <= w.b && w.bp + 1 <= P.b;
+                            if (meet_out || meet_in) {
+                                const int64_t tq = (int64_t)(S.c_cost[p] >> 1), q_r = A.start[P.a], q_end = A.start[P.b + 1];
+                                lost = (meet_out && window_conflict<false, true>(A.start, bo, w.a, w.ap - 1, w.t_r, w.t_r + w.t, q_r, q_r + tq, P.a, P.ap - 1)) ||
+                                       (meet_in && window_conflict<false, true>(A.start, bi, w.bp + 1, w.b, w.t_end - w.t, w.t_end, q_end - tq, q_end, P.bp + 1, P.b));
+                            }
+                        }
+                        if (P.fresh && P.ap <= w.bp && w.ap <= P.bp) { q.w &= ~(1u << 23); hot[e] = q; }
+                    }
+                }
+                // host memory of these slots has filled up (finite capacity): is there still room?
+                const bool room = A.host_capacity != 0 && w.dest == G10_DEST_HOST && P.dest == G10_DEST_HOST && p != w.idx && P.a <= w.b && w.a <= P.b;
+                unsigned todo = __ballot_sync(0xffffffffu, lost || room);
+                __syncwarp();
+#pragma unroll 1
+                while (todo) {                              // the whole warp, one period after the other
+                    const int src = __ffs(todo) - 1;
+                    todo &= todo - 1;
+                    const int p2 = (r * G + c) * 32 + src, e2 = r * 32 + src;
+                    const bool gone = __shfl_sync(0xffffffffu, lost, src);
+                    const SpPeriod Q = sp_unpack(hot[e2]);
+                    const int64_t s2 = A.bytes[A.per_t[p2]];
+                    auto host_room = [&]() {
+                        if (A.host_capacity == 0) return true;
+                        bool ok = true;
+                        for (int k = Q.a + lane; k <= Q.b; k += 32) {
+                            const uint64_t more = w.dest == G10_DEST_HOST && k >= w.a && k <= w.b ? (uint64_t)w.s : 0u;
+                            if ((uint64_t)__ldcg(&A.hocc[k]) + more + (uint64_t)s2 > A.host_capacity) ok = false;
+                        }
+                        return __all_sync(0xffffffffu, ok) != 0;
+                    };
+                    if (!gone && host_room()) continue;
+                    // SSD -> host -> erased.  (A period that leaves the SSD does so because of a commit to the SSD: nothing is pending
+                    // on the host's channels.)
+                    bool to_host = false;
+                    if (Q.dest == G10_DEST_SSD) {
+                        const int ap = A.geo_a[A.geo_stride + p2];
+                        if (ap >= 0) {
+                            const int bp = A.geo_b[A.geo_stride + p2];
+                            const int64_t t2 = A.geo_t[A.geo_stride + p2], q_r = A.start[Q.a], q_end = A.start[Q.b + 1];
+                            to_host = window_free(A, A.busy + (size_t)(2 * G10_DEST_HOST) * A.K, q_r, q_r + t2, Q.a, ap - 1, lane) &&
+                                      window_free(A, A.busy + (size_t)(2 * G10_DEST_HOST + 1) * A.K, q_end - t2, q_end, bp + 1, Q.b, lane) && host_room();
+                        }
+                    }
+                    if (lane == 0) { if (to_host) begin_period(p2, e2, G10_DEST_HOST, Q.a, Q.b); else hot[e2] = make_uint4(0, 0, 0, 0); }
+                }
+                __syncwarp();
+                q = hot[e];
+            }
+            if (q.x == 0u) continue;
+            if (q.w >> 23 & 1u) { if (q.x > fk) fk = q.x; }
+            else if (q.x > tk[kSpTop - 1] && q.x >= least && (!with_floor || sp_may_beat(S, p, q.x, floor_key, gBest))) {
+                unsigned k = q.x;
+                int i = p << 1 | (int)((q.w >> 21 & 3u) - 1u);
+#pragma unroll
+                for (int j = 0; j < kSpTop; ++j)
+                    if (k > tk[j]) { const unsigned a = tk[j]; const int b = ti[j]; tk[j] = k; ti[j] = i; k = a; i = b; }
+            }
+          }
+        }
+        long long top = -0x7fffffffffffffffll - 1;                  // largest pressure above capacity of the own tiles
+        for (int lt = tid; lt < my_tiles; lt += kPlanThreads) { const long long v = mm[lt].y; top = v > top ? v : top; }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) { const long long y = __shfl_xor_sync(0xffffffffu, top, o); top = y > top ? y : top; }
+        const unsigned wf = __reduce_max_sync(0xffffffffu, fk);
+#pragma unroll 1
+        for (int j = 0; j < kSpTop; ++j) {
+            unsigned k = tk[0];
+            int i = ti[0];
+            sp_warp_max(k, i);
+            if (i >= 0 && i == ti[0]) {                             // this lane's head was taken: the next one moves up
+#pragma unroll
+                for (int q = 0; q < kSpTop - 1; ++q) { tk[q] = tk[q + 1]; ti[q] = ti[q + 1]; }
+                tk[kSpTop - 1] = 0; ti[kSpTop - 1] = -1;
+            }
+            if (lane == 0) { s_wk[warp * kSpTop + j] = i >= 0 ? k : 0u; s_wi[warp * kSpTop + j] = i; }
+            if (i < 0) { if (lane == 0) for (int x = j + 1; x < kSpTop; ++x) { s_wk[warp * kSpTop + x] = 0u; s_wi[warp * kSpTop + x] = -1; } break; }
+        }
+        if (lane == 0) { s_fk[warp] = wf; s_max[warp] = top; }
+        __syncthreads();
+        const unsigned bf = __reduce_max_sync(0xffffffffu, lane < kPlanWarps ? s_fk[lane] : 0u);
+        // the exactly scored periods that may be the best of them
+        const unsigned thr = bf ? __float_as_uint((float)(sp_val(bf) * (1.0 - kNear))) : 0u;
+        if (wf != 0u && wf >= thr)
+#pragma unroll 1
+            for (int r = warp; r < my_runs; r += kPlanWarps) {
+                const uint4 q = hot[r * 32 + lane];
+                if (q.x >= thr && (q.w >> 23 & 1u)) {
+                    const int n = atomicAdd(&s_nfin, 1);
+                    if (n < 32) s_fin[n] = (r * G + c) * 32 + lane;
+                }
+            }
+        if (warp == 0) {
+            // (every warp's list is in order: lane w has warp w's, and moves on in it when its head is taken)
+            int at = 0;
+            unsigned hk = lane < kPlanWarps ? s_wk[lane * kSpTop] : 0u;
+            int hi = lane < kPlanWarps ? s_wi[lane * kSpTop] : -1;
+#pragma unroll 1
+            for (int j = 0; j < kSpTop; ++j) {
+                unsigned k = hk;
+                int i = hi;
+                sp_warp_max(k, i);
+                if (i >= 0 && i == hi) {
+                    ++at;
+                    hk = at < kSpTop ? s_wk[lane * kSpTop + at] : 0u; hi = at < kSpTop ? s_wi[lane * kSpTop + at] : -1;
+                }
+                if (lane == 0) { s_tk[j] = i >= 0 ? k : 0u; s_ti[j] = i; }
+                if (i < 0) { if (lane == 0) for (int x = j + 1; x < kSpTop; ++x) { s_tk[x] = 0u; s_ti[x] = -1; } break; }
+            }
+        }
+        __syncthreads();
+        auto exact = [&](int p) {
+            Cand x;
+            x.ben = ((u128)S.c_ben_hi[p] << 64) | S.c_ben_lo[p]; x.cost = S.c_cost[p]; x.idx = p;
+            x.dest = (int)(hot[owner_entry(p)].w >> 21 & 3u) - 1;
+            return x;
+        };
+        Cand best;
+        best.ben = 0; best.cost = 1; best.idx = -1; best.dest = -1;
+        const int n = s_nfin;
+        if (n <= 32) {
+            if (warp == 0) {
+                if (lane < n) best = exact(s_fin[lane]);
+                if (n > 1)
+#pragma unroll 1
+                    for (int o = 16; o > 0; o >>= 1) { const Cand y = cand_shfl_down(best, o); if (cand_beats(y, best)) best = y; }
+            }
+        } else {                                                    // very many close scores
+#pragma unroll 1
+            for (int r = warp; r < my_runs; r += kPlanWarps) {
+                const uint4 q = hot[r * 32 + lane];
+                if (q.x >= thr && (q.w >> 23 & 1u)) { const Cand y = exact((r * G + c) * 32 + lane); if (cand_beats(y, best)) best = y; }
+            }
+            best = block_best(best, s_cand);
+        }
+        if (tid == 0) {
+            SpProp o;
+            o.ben_lo = (ull)best.ben; o.ben_hi = (ull)(best.ben >> 64); o.cost = best.cost; o.idx = best.idx < 0 ? -1 : best.idx << 1 | best.dest; o.key = best.idx < 0 ? 0u : sp_key(best.ben, best.cost);
+#pragma unroll
+            for (int j = 0; j < kSpTop; ++j) { o.skey[j] = s_tk[j]; o.sidx[j] = s_ti[j]; }
+            long long m = s_max[0];
+            for (int x = 1; x < kPlanWarps; ++x) m = s_max[x] > m ? s_max[x] : m;
+            o.peak = m; o.pad = 0;
+            S.props[(size_t)pbuf * kLazyMaxBlocks + c] = o;
+        }
+    };
+    // The exactly best of the threads' candidates (at most one each, with its rounded score): the block's threads all get it.
+    auto best_of = [&](const Cand &x, unsigned key) {
+        const unsigned wk = __reduce_max_sync(0xffffffffu, key);
+        if (lane == 0) s_fk[warp] = wk;
+        __syncthreads();
+        const unsigned m = __reduce_max_sync(0xffffffffu, lane < kPlanWarps ? s_fk[lane] : 0u);
+        const bool near = key != 0u && sp_val(key) >= sp_val(m) * (1.0 - kNear);
+        if (near) s_one = x;                                 // (usually one thread)
+        if (m == 0u && tid == 0) s_one = x;
+        if (__syncthreads_count(near) <= 1) return s_one;    // (nobody: thread 0's, which is none)
+        return block_best_fast(x, &s_best, s_cand);
+    };
+    // Reads publications of buffer `buf` into the pool of bounds (all, or those of the blocks that published again); returns the best
+    // exactly scored one, and whether anything is above capacity.
+    auto load = [&](int buf, bool only_flagged, bool *over) {
+        Cand x;
+        x.ben = 0; x.cost = 1; x.idx = -1; x.dest = -1;
+        unsigned key = 0;
+        bool above = false;
+        for (int j = tid; j < G; j += kPlanThreads) {        // (G <= kPlanThreads: one block's values per thread)
+            if (only_flagged && !s_refresh[j]) continue;
+            const uint4 *src = (const uint4 *)&S.props[(size_t)buf * kLazyMaxBlocks + j];
+            union { uint4 v[sizeof(SpProp) / 16]; SpProp o; } u;
+#pragma unroll
+            for (int q = 0; q < (int)sizeof(SpProp) / 16; ++q) u.v[q] = __ldcg(src + q);
+            if (u.o.idx >= 0) { x.ben = ((u128)u.o.ben_hi << 64) | u.o.ben_lo; x.cost = u.o.cost; x.idx = u.o.idx >> 1; x.dest = u.o.idx & 1; key = u.o.key; }
+            above = u.o.peak > 0;
+#pragma unroll
+            for (int q = 0; q < kSpTop; ++q) { pkey[q * G + j] = u.o.skey[q]; pidx[q * G + j] = u.o.sidx[q]; pdone[q * G + j] = 0; }
+        }
+        if (over != nullptr) *over = __syncthreads_or(above) != 0;
+        const Cand b = best_of(x, key);
+        __syncthreads();
+        return b;
+    };
+
+#pragma unroll 1
+    for (int64_t it = 0; status == -1; ++it) {
+        bool barrier_since_booking = true;
+        // ---------------- A: the pending commit on the own tiles: whole ones by their offset, the two at the ends slot by slot
+        if (pending) {
+            const int ta = w.ap / kSpTile, tb = w.bp / kSpTile;
+            const int l0 = ta > c ? (ta - c + G - 1) / G : 0, l1 = tb >= c ? (tb - c) / G : -1;
+#pragma unroll 1
+            for (int lt = l0 + tid; lt <= l1; lt += kPlanThreads) {
+                const int t = lt * G + c;
+                if (t * kSpTile < w.ap || (t * kSpTile + kSpTile - 1 > w.bp && w.bp != K - 1)) continue;
+                longlong2 m = mm[lt];
+                m.x -= w.s; m.y -= w.s;
+                mm[lt] = m; off[lt] -= w.s;
+            }
+#pragma unroll 1
+            for (int end = 0; end < 2; ++end) {
+                const int t = end ? tb : ta;
+                if (t % G != c || (end && tb == ta) || warp != kPlanWarps - 1 - end) continue;
+                if (!(t * kSpTile < w.ap || (t * kSpTile + kSpTile - 1 > w.bp && w.bp != K - 1))) continue;     // (a whole one)
+                const int lt = t / G;
+#pragma unroll
+                for (int j = 0; j < kSpTile; j += 32) {
+                    const int k = t * kSpTile + j + lane;
+                    if (k >= w.ap && k <= w.bp) ex[lt * kSpTile + j + lane] -= w.s;
+                }
+                __syncwarp();
+                refresh_tile(lt);
+            }
+            if (c == 0 && tid == 0) {
+                if (n_mig - 1 < A.out_cap) {
+                    g10_migration m;
+                    m.period = w.idx; m.tensor = A.per_t[w.idx]; m.dest = w.dest; m.absent_first = w.ap; m.absent_last = w.bp;
+                    m.iteration = (int32_t)(it - 1); m.evict_issue_ns = w.t_r; m.prefetch_issue_ns = w.t_end - w.t; m.transfer_ns = w.t;
+                    A.out[n_mig - 1] = m;
+                } else raise_status(A.status, G10_DEV_PLAN_OVERFLOW);
+            }
+        }
+        __syncthreads();
+        scan(pending, false);
+        if (!grid_barrier(A.bar, G, gen)) { status = -2; break; }
+        bool over;
+        gBest = load(pbuf, false, &over);
+        pbuf ^= 1;
+        if (A.fits_always || !over) { status = n_mig == 0 ? G10_ALREADY_FITS : G10_FIT; break; }
+        if (it >= limit) { status = limit < Pn64 ? G10_ITERATION_LIMIT : G10_EXHAUSTED; break; }
+        rounds += 1;
+        if (pending) {
+            if (c == 0) {
+                book_winner(A, w.idx, w.dest);
+                if (w.dest == G10_DEST_HOST && A.host_capacity != 0) for (int k = w.a + tid; k <= w.b; k += kPlanThreads) A.hocc[k] += w.s;
+            }
+            barrier_since_booking = false;
+        }
+        pending = false;
+        // ---------------- R: rounds of joint rescoring
+        bool failed = false;
+        int round_no = 0;
+        const int n_pool = G * kSpTop;
+#pragma unroll 1
+        for (;;) {
+            const double gkey = gBest.idx >= 0 ? cand_key(gBest) : -1.0;
+            // which published bounds are rescored now (the same choice in every block, in publication order): every unused one that
+            // may beat the best exact score -- in the first round only those within 10 % of the best bound (the winner is usually
+            // among them, and a strong exact score spares the rest)
+            int msel = 0;
+            {
+                unsigned k = 0;                               // the best unused bound
+                for (int e = tid; e < n_pool; e += kPlanThreads) if (!pdone[e] && pidx[e] >= 0 && pkey[e] > k) k = pkey[e];
+                k = __reduce_max_sync(0xffffffffu, k);
+                if (lane == 0) s_fk[warp] = k;
+                __syncthreads();
+                k = __reduce_max_sync(0xffffffffu, lane < kPlanWarps ? s_fk[lane] : 0u);
+                if (k != 0u && (gBest.idx < 0 || sp_val(k) >= gkey * (1.0 - kNear))) {
+                    const unsigned floor0 = round_no == 0 ? __float_as_uint(fminf(__uint_as_float(k), last_key > 0.0f ? last_key : __uint_as_float(k)) * kFirst) : 0u;
+                    unsigned took = 0;                        // (bit j: the thread's j-th entry)
+                    int j = 0;
+                    for (int e0 = 0; e0 < n_pool; e0 += kPlanThreads, ++j) {
+                        const int e = e0 + tid;
+                        bool take = false;
+                        if (e < n_pool && !pdone[e] && pidx[e] >= 0 && pkey[e] >= floor0) {
+                            take = sp_may_beat(S, pidx[e] >> 1, pkey[e], gkey, gBest);
+                            if (!take) pdone[e] = 2;
+                        }
+                        const unsigned mk = __ballot_sync(0xffffffffu, take);
+                        if (take) took |= 1u << j;
+                        if (lane == 0) s_wcnt[j * kPlanWarps + warp] = __popc(mk);
+                    }
+                    const int n_cnt = j * kPlanWarps;
+                    __syncthreads();
+                    // entries taken before this warp's, chunk by chunk (every warp adds them up for itself)
+                    for (int x = 0, y = 0; x < n_cnt; x += 32, y += 2) {
+                        const int v = x + lane < n_cnt ? s_wcnt[x + lane] : 0;
+                        int incl = v;
+#pragma unroll
+                        for (int o = 1; o < 32; o <<= 1) { const int z = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += z; }
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            if (y + h >= j) break;
+                            const int before = msel + __shfl_sync(0xffffffffu, incl - v, h * kPlanWarps + warp);
+                            const bool t = (took >> (y + h) & 1u) != 0u;
+                            const int pos = before + __popc(__ballot_sync(0xffffffffu, t) & ((1u << lane) - 1u));
+                            const int e = (y + h) * kPlanThreads + tid;
+                            if (t && pos < kSpRound) { r_e[pos] = e; pdone[e] = 1; }      // (beyond the cap: next round)
+                        }
+                        msel += __shfl_sync(0xffffffffu, incl, 31);
+                    }
+                    msel = msel < kSpRound ? msel : kSpRound;
+                    __syncthreads();
+                }
+            }
+            if (msel == 0) {
+                if (round_no == 0) round_no = 1;
+                // Nothing published may beat the best score.  A block whose last bound may do so could hold more; and all of them may,
+                // if bounds were left out as unlikely that it turns out may win.
+                const bool unlikely = likely != 0u && (gBest.idx < 0 || sp_val(likely) >= gkey * (1.0 - kNear));
+                bool again = false;
+                if (tid < G) {
+                    const int e = (kSpTop - 1) * G + tid;
+                    const double last = pidx[e] >= 0 ? sp_val(pkey[e]) : 0.0;
+                    again = unlikely || (last > 0.0 && (gBest.idx < 0 || last >= gkey * (1.0 - kNear)));
+                    s_refresh[tid] = again ? 1 : 0;
+                }
+                if (!__syncthreads_or(again)) break;
+                if (unlikely) likely = 0;
+                if (s_refresh[c]) scan(false, true);
+                if (!grid_barrier(A.bar, G, gen)) { failed = true; break; }
+                barrier_since_booking = true;
+                load(pbuf, true, nullptr);
+                pbuf ^= 1;
+                continue;
+            }
+            round_no += 1;
+            for (int r = tid; r < msel; r += kPlanThreads) {
+                const int i = pidx[r_e[r]], p = i >> 1, d = i & 1;
+                r_p[r] = i;
+                r_ap[r] = A.geo_a[d * A.geo_stride + p]; r_bp[r] = A.geo_b[d * A.geo_stride + p];
+                r_s[r] = A.bytes[A.per_t[p]];
+                r_cost[r] = 2ull * (ull)A.geo_t[d * A.geo_stride + p];
+#pragma unroll
+                for (int q = 0; q < kSpLimbs; ++q) r_acc[q * kSpRound + r] = 0;
+            }
+            if (tid == 0) { s_nmix = 0; s_nedge = 0; s_ndist = 0; }
+            __syncthreads();
+            auto add = [&](int r, u128 v) {
+#pragma unroll
+                for (int q = 0; q < kSpLimbs; ++q) {                                 // (a 64-bit atomic would be a compare-and-swap loop)
+                    const unsigned x = (unsigned)(v >> (16 * q)) & 0xffffu;
+                    if (x) atomicAdd(&r_acc[q * kSpRound + r], x);
+                }
+            };
+            // benefit of local tile lt for period r, slot by slot, by one warp; every lane's share
+            auto slots = [&](int r, int lt) {
+                const int t0 = (lt * G + c) * kSpTile, ap = r_ap[r], bp = r_bp[r];
+                const long long s = r_s[r], o = off[lt];
+                u128 sum = 0;
+#pragma unroll
+                for (int j = 0; j < kSpTile; j += 32) {
+                    const int k = t0 + j + lane;
+                    if (k < ap || k > bp) continue;
+                    long long e = ex[lt * kSpTile + j + lane] + o;
+                    e = e > s ? s : e;
+                    if (e > 0) sum += (u128)(ull)e * (u128)(ull)(A.start[k + 1] - A.start[k]);
+                }
+                return sum;
+            };
+            // a warp per period, a lane per own tile of its absent range: one at least the tensor's size above capacity throughout counts
+            // it for its whole time, one within capacity nothing; the others are listed
+#pragma unroll 1
+            for (int r = warp; r < msel; r += kPlanWarps) {
+                const int ap = r_ap[r], bp = r_bp[r], ta = ap / kSpTile, tb = bp / kSpTile;
+                const long long s = r_s[r];
+                const int l0 = ta > c ? (ta - c + G - 1) / G : 0, l1 = tb >= c ? (tb - c) / G : -1;
+                ull time = 0;
+#pragma unroll 1
+                for (int lb = l0; lb <= l1; lb += 32) {
+                    const int lt = lb + lane, t0 = (lt * G + c) * kSpTile;
+                    int kind = 0;                                                   // 1: part of the tile, 2: all of it, some slots near capacity
+                    if (lt <= l1) {
+                        const longlong2 m = mm[lt];
+                        const bool whole = t0 >= ap && (t0 + kSpTile - 1 <= bp || bp == K - 1);
+                        if (m.y > 0) {
+                            if (!whole) kind = 1;
+                            else if (m.x >= s) time += tsum[lt];
+                            else kind = 2;
+                        }
+                    }
+                    const unsigned b1 = __ballot_sync(0xffffffffu, kind == 1), b2 = __ballot_sync(0xffffffffu, kind == 2), below = (1u << lane) - 1u;
+                    unsigned rest = 0;
+                    if (b1 | b2) {
+                        int p1 = 0, p2 = 0;
+                        if (lane == 0) { if (b1) p1 = atomicAdd(&s_nedge, __popc(b1)); if (b2) p2 = atomicAdd(&s_nmix, __popc(b2)); }
+                        p1 = __shfl_sync(0xffffffffu, p1, 0) + __popc(b1 & below); p2 = __shfl_sync(0xffffffffu, p2, 0) + __popc(b2 & below);
+                        if (kind == 1) s_edge[p1] = (unsigned)r << 20 | (unsigned)lt;       // (two per period at most)
+                        if (kind == 2 && p2 < kSpMix) {
+                            s_mix[p2] = (unsigned)r << 20 | (unsigned)lt;
+                            if (atomicCAS(&t_no[lt], -1, -2) == -1) { const int n = atomicAdd(&s_ndist, 1); t_at[n] = lt; t_no[lt] = n; }
+                        }
+                        rest = __ballot_sync(0xffffffffu, kind == 2 && p2 >= kSpMix);
+                    }
+#pragma unroll 1
+                    while (rest) {                                                  // list full: the warp reads the tile itself
+                        const int src = __ffs(rest) - 1;
+                        rest &= rest - 1;
+                        const u128 v = warp_sum_u128(slots(r, lb + src));
+                        if (lane == 0) add(r, v);
+                    }
+                }
+                if (__any_sync(0xffffffffu, time != 0)) {
+                    const ull sum = (ull)__reduce_add_sync(0xffffffffu, (unsigned)(time & 0xffffffu)) + ((ull)__reduce_add_sync(0xffffffffu, (unsigned)(time >> 24)) << 24);
+                    if (lane == 0) add(r, (u128)sum * (u128)(ull)s);
+                }
+            }
+            __syncthreads();
+            const int nmix = s_nmix < kSpMix ? s_nmix : kSpMix, ndist = s_ndist, nedge = s_nedge;
+#pragma unroll 1
+            for (int x = kPlanWarps - 1 - warp; x < nedge; x += kPlanWarps) {
+                const int r = (int)(s_edge[x] >> 20);
+                const u128 v = warp_sum_u128(slots(r, (int)(s_edge[x] & 0xfffffu)));
+                if (lane == 0) add(r, v);
+            }
+#pragma unroll 1
+            for (int n0 = 0; n0 < ndist; n0 += kSpSort) {
+                if (n0) __syncthreads();                                            // (the sorted tiles are free)
+                if (warp < kSpSort && n0 + warp < ndist) {
+                    const int lt = t_at[n0 + warp], t0 = (lt * G + c) * kSpTile, n = K - t0 < kSpTile ? K - t0 : kSpTile;
+                    SpSorted &q = sorted[warp];
+                    const long long o = off[lt];
+                    long long v[2];
+                    ull d[2];
+                    int rank[2] = {0, 0};
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int x = h * 32 + lane;
+                        v[h] = x < n ? ex[lt * kSpTile + x] : 0x7fffffffffffffffll;
+                        d[h] = x < n ? (ull)(A.start[t0 + x + 1] - A.start[t0 + x]) : 0ull;
+                    }
+#pragma unroll 4
+                    for (int j = 0; j < n; ++j) {                                   // position of each: how many come before it
+                        const long long y = ex[lt * kSpTile + j];
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) rank[h] += y < v[h] || (y == v[h] && j < h * 32 + lane) ? 1 : 0;
+                    }
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) if (h * 32 + lane < n) {
+                        long long e = v[h] + o;
+                        e = e < 0 ? 0 : e > ((long long)1 << 40) ? (long long)1 << 40 : e;
+                        q.v[rank[h]] = e; q.d[rank[h]] = (unsigned)d[h];
+                    }
+                    __syncwarp();
+                    // prefix sums: two consecutive entries per lane
+                    const bool i0 = 2 * lane < n, i1 = 2 * lane + 1 < n;
+                    const ull v0 = i0 ? (ull)q.v[2 * lane] : 0ull, v1 = i1 ? (ull)q.v[2 * lane + 1] : 0ull;
+                    const unsigned d0 = i0 ? q.d[2 * lane] : 0u, d1 = i1 ? q.d[2 * lane + 1] : 0u;
+                    const ull a0 = (v0 & 0xfffffull) * d0, a1 = (v1 & 0xfffffull) * d1, b0 = (v0 >> 20) * d0, b1 = (v1 >> 20) * d1;
+                    unsigned sd = d0 + d1;
+                    ull sa = a0 + a1, sb = b0 + b1;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const unsigned yd = __shfl_up_sync(0xffffffffu, sd, o);
+                        const ull ya = __shfl_up_sync(0xffffffffu, sa, o), yb = __shfl_up_sync(0xffffffffu, sb, o);
+                        if (lane >= o) { sd += yd; sa += ya; sb += yb; }
+                    }
+                    __syncwarp();
+                    q.d[2 * lane] = sd - d1 - d0; q.lo[2 * lane] = sa - a1 - a0; q.hi[2 * lane] = sb - b1 - b0;
+                    q.d[2 * lane + 1] = sd - d1; q.lo[2 * lane + 1] = sa - a1; q.hi[2 * lane + 1] = sb - b1;
+                    if (lane == 31) { q.d[kSpTile] = sd; q.lo[kSpTile] = sa; q.hi[kSpTile] = sb; }
+                    if (lane == 0) q.n = n;
+                }
+                __syncthreads();
+#pragma unroll 1
+                for (int x = tid; x < nmix; x += kPlanThreads) {
+                    const int lt = (int)(s_mix[x] & 0xfffffu), r = (int)(s_mix[x] >> 20), no = t_no[lt] - n0;
+                    if (no < 0 || no >= kSpSort) continue;
+                    const SpSorted &q = sorted[no];
+                    const long long s = r_s[r];
+                    int j = 0;                                                      // slots less than s above capacity
+#pragma unroll
+                    for (int h = kSpTile / 2; h > 0; h >>= 1)
+                        if (j + h <= q.n && q.v[j + h - 1] < s) j += h;
+                    if (j < q.n && q.v[j] < s) ++j;
+                    add(r, ((u128)q.hi[j] << 20) + (u128)q.lo[j] + (u128)(ull)s * (u128)(ull)(q.d[kSpTile] - q.d[j]));
+                }
+            }
+            __syncthreads();
+            for (int x = tid; x < ndist; x += kPlanThreads) t_no[t_at[x]] = -1;
+            // this block's shares go into the grid-wide sums: the low 44 bits and the rest on their own, so that neither needs a carry
+            // and no block waits for an answer
+            for (int r = tid; r < msel; r += kPlanThreads) {
+                u128 v = 0;
+#pragma unroll
+                for (int q = 0; q < kSpLimbs; ++q) v += (u128)r_acc[q * kSpRound + r] << (16 * q);
+                ull *dst = S.partials + (size_t)pp * 2 * kSpRound + r;
+                const ull lo = (ull)v & 0xfffffffffffull, hi = (ull)(v >> 44);
+                if (lo) asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(dst), "l"(lo) : "memory");
+                if (hi) asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(dst + kSpRound), "l"(hi) : "memory");
+            }
+            if (!grid_barrier(A.bar, G, gen)) { failed = true; break; }
+            barrier_since_booking = true;
+            // (the buffer used two rounds from now was last read one round ago: block 0 clears it)
+            if (c == 0) for (int j = tid; j < kSpRound * 2; j += kPlanThreads) S.partials[(size_t)((pp + 2) % 3) * kSpRound * 2 + j] = 0;
+            Cand x;
+            x.ben = 0; x.cost = 1; x.idx = -1; x.dest = -1;
+            unsigned key = 0;
+            if (tid < msel) {
+                const int i = r_p[tid], p = i >> 1;
+                const ull *src = S.partials + (size_t)pp * 2 * kSpRound + tid;
+                const u128 tot = ((u128)__ldcg(src + kSpRound) << 44) + __ldcg(src);
+                x.ben = tot; x.cost = r_cost[tid]; x.idx = tot == 0 ? -1 : p; x.dest = i & 1;
+                key = sp_key(tot, x.cost);
+                const int e = owner_entry(p);
+                if (e >= 0) {
+                    S.c_ben_lo[p] = (ull)tot; S.c_ben_hi[p] = (ull)(tot >> 64);
+                    uint4 q = hot[e];
+                    q.x = key; q.w |= 1u << 23;
+                    hot[e] = q;
+                }
+            }
+            const Cand b = best_of(x, key);
+            if (cand_beats(b, gBest)) gBest = b;
+            pp = (pp + 1) % 3;
+            __syncthreads();
+        }
+        if (failed) { status = -2; break; }
+        if (!barrier_since_booking) { if (!grid_barrier(A.bar, G, gen)) { status = -2; break; } }
+        // ---------------- D: decide
+        if (gBest.idx < 0) { status = G10_EXHAUSTED; break; }
+        {
+            const int p = gBest.idx, X = gBest.dest;
+            w.idx = p; w.dest = X; w.a = A.per_u[p] + 1; w.b = A.per_v[p] - 1;
+            w.ap = A.geo_a[X * A.geo_stride + p]; w.bp = A.geo_b[X * A.geo_stride + p]; w.t = A.geo_t[X * A.geo_stride + p];
+            w.s = A.bytes[A.per_t[p]];
+            w.t_r = A.start[w.a]; w.t_end = A.start[w.b + 1];
+            last_key = (float)cand_key(gBest);
+            likely = __float_as_uint((float)(cand_key(gBest) * 0.8));
+            if (X == G10_DEST_SSD) bytes_ssd += w.s; else bytes_host += w.s;
+        }
+        n_mig += 1;
+        pending = true;
+    }
+    __syncthreads();
+    for (int x = tid; x < my_tiles * kSpTile; x += kPlanThreads) {
+        const int64_t k = ((int64_t)(x / kSpTile) * G + c) * kSpTile + x % kSpTile;
+        if (k < K) A.P[k] = ex[x] + off[x / kSpTile] + A.cap;
+    }
+    if (c == 0 && tid == 0) *S.done = 1u;
+    {
+        // the peak of what is left (every block's own, then all of them)
+        long long m = 0;
+        for (int x = tid; x < my_tiles; x += kPlanThreads) m = mm[x].y + A.cap > m ? mm[x].y + A.cap : m;
+        m = block_max_i64(m, s_max);
+        if (tid == 0) A.peak_part[c] = m;
+    }
+    if (status != -2 && !grid_barrier(A.bar, G, gen)) status = -2;
+    if (status != -2) {
+        long long m = 0;
+        for (int j = tid; j < G; j += kPlanThreads) { const long long x = __ldcg(&A.peak_part[j]); m = x > m ? x : m; }
+        peak = block_max_i64(m, s_max);
+    }
+    plan_epilogue(A, c, G, gen, status, peak, n_mig, rounds, bytes_ssd, bytes_host);
+}
+
+// Shared memory that the kernel may use on the current device (allowed once per device); 0 if a query fails.
+static int spread_budget()
+{
+    static int known[kMaxDevices];
+    int dev = 0, optin = 0;
+    cudaFuncAttributes fa;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return 0;
+    if (dev < kMaxDevices) if (const int b = __atomic_load_n(&known[dev], __ATOMIC_ACQUIRE)) return b;
+    if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) return 0;
+    if (cudaFuncGetAttributes(&fa, (const void *)k_plan_spread) != cudaSuccess) return 0;
+    const int room = optin - (int)fa.sharedSizeBytes;
+    if (room <= 0 || cudaFuncSetAttribute((const void *)k_plan_spread, cudaFuncAttributeMaxDynamicSharedMemorySize, room) != cudaSuccess) return 0;
+    if (dev < kMaxDevices) __atomic_store_n(&known[dev], room, __ATOMIC_RELEASE);
+    return room;
+}
+
+// Worth launching: the timeline leaves room for at least some periods (their number is counted on the device, which decides).
+bool plan_spread_possible(int64_t K, int64_t E)
+{
+    const int G = current_sm_count(), budget = spread_budget();
+    return G > 0 && G <= kLazyMaxBlocks && G <= kPlanThreads && K >= 1 && K <= kSpMaxSlots && E >= 1 && budget > 0 && sp_smem(K, E < 4096 ? E : 4096, G) <= (size_t)budget;
+}
+
+cudaError_t launch_plan_spread(const PlanArgs &A_in, const Workspace &w, cudaStream_t s)
+{
+    PlanArgs A = A_in;
+    A.bar = (GridBarrier *)(w.barrier2);
+    SpreadArgs S;
+    S.c_ben_lo = w.c_ben_lo; S.c_ben_hi = w.c_ben_hi; S.c_cost = w.c_cost; S.props = (SpProp *)w.lazy_props; S.partials = w.lazy_partials;
+    S.flag = w.spread_flag; S.done = w.one_done; S.smem_bytes = spread_budget();
+    void *args[] = {&A, &S};
+    return cudaLaunchCooperativeKernel((const void *)k_plan_spread, dim3(current_sm_count()), dim3(kPlanThreads), args, (size_t)S.smem_bytes, s);
+}
+
+}  // namespace g10

@@ -970,6 +970,28 @@ def test_on_chip_planner_edges(gpu, oracle, K, chains):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("K,n,ns", [(1, 8, 1 << 20), (63, 300, 1 << 20), (64, 3000, 1 << 12), (65, 3000, 1 << 20), (9471, 400, 1 << 20),
+                                    (9473, 3000, 1 << 10), (19000, 200, 1 << 25), (300, 400, 1 << 27)])
+def test_spread_planner_edges(gpu, oracle, K, n, ns):
+    """The planner whose state is spread over all SMs, around whole tiles of 64 slots in one block and in all of them (148 x 64),
+    long and short absent ranges, unlimited and finite host memory; at 2^27 ns a kernel a tile is longer than 2^32 ns and the
+    planner behind it takes over.  Bit for bit against the oracle."""
+    rng = np.random.default_rng(K * 10007 + n)
+    lists = [[] for _ in range(K)]
+    for i in range(n):
+        for k in sorted(set(int(x) for x in rng.integers(0, K, size=int(rng.integers(2, 6))))):
+            lists[k].append(i)
+    tr = traces.from_lists("edges", lists, rng.integers(1 << 16, 1 << 24, size=n), rng.integers(ns // 2, ns, size=K),
+                           (rng.random(n) < 0.2).astype(np.uint8), capacity_frac=(2, 5))
+    tb = gpu.upload(tr)
+    start, P0, peak, slot = oracle.timeline(tr)
+    cap = tr.capacity_from_peak(peak)
+    for host in (0, 3 << 24):
+        ref = oracle.plan(tr, cap, lazy=True, host_capacity_bytes=host)
+        check_plan(gpu, tr, tb, cap, ref, host_capacity=host, flags=gpu.FLAG_GLOBAL_STATE)
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("K,N,E", [(1, 1, 1), (1023, 1025, 2048), (1024, 33, 9000), (37, 3, 30000), (2049, 20000, 20001), (9000, 9000, 30000)])
 def test_one_launch_analysis_edges(gpu, oracle, K, N, E):
     """The one-block analysis around its block size, with segments for one thread, a warp and the block (repeats in all),
