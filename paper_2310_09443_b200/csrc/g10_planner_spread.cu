@@ -16,7 +16,7 @@
 // All decisions are taken from data every block has, so the control flow is the same in every block.  Rounded scores steer the
 // search; anything within kNear of a decision is settled by exact 128-bit comparison.
 // What bounds it: grid barriers (three to four an iteration) and waiting in them for the block with the most to rescore.
-// periods in global memory (g10_planner_lazy.cu) an iteration on a million kernels read 140 MB through the L2: 1.02 s for its plan,
+// With slots and periods in global memory (g10_planner_lazy.cu) an iteration on a million kernels read 140 MB through the L2: 1.02 s for its plan,
 // 0.90 s here (200 k kernels: 1.4 to 1.5 times faster).
 #include "g10_planner.cuh"
 
