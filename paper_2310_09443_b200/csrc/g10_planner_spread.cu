@@ -24,9 +24,9 @@ namespace g10 {
 
 constexpr int kSpTile = 64;                     // slots per tile
 constexpr int kSpRound = 256;                   // periods rescored together, at most
-constexpr int kSpMix = 1024;                    // (period, tile) pairs of one round that need more than the tile's summary, listed
 constexpr int kSpEdge = 2 * kSpRound;           // pairs in which the period covers the tile in part
-constexpr int kSpSort = 12;                     // tiles sorted together (one warp each)
+constexpr int kSpSort = kPlanWarps;             // tiles sorted together (one warp each)
+constexpr int kSpDirect = 2 * kPlanWarps;       // up to this many (period, tile) pairs are read slot by slot rather than sorted
 constexpr float kFirst = 0.97f;
 constexpr double kNear = 1e-6;                  // (scores are kept as floats, rounded up: 2^-23)
 constexpr int kSpTop = 8;                       // bounds a block publishes
@@ -108,16 +108,16 @@ struct SpSorted {
     long long v[kSpTile];                       // pressure above capacity, at least 0 and at most 2^40 (tensors are smaller), ascending
     ull lo[kSpTile + 1], hi[kSpTile + 1];       // sums of (v mod 2^20) x duration and of (v >> 20) x duration over the first n
     unsigned d[kSpTile + 1];                    // sums of the durations (a tile's total is below 2^32 ns)
-    int n;
+    int n, lt, pad;
 };
 
 __host__ __device__ inline size_t sp_round16(size_t x) { return (x + 15) / 16 * 16; }
 __host__ __device__ inline size_t sp_smem(int64_t K, int64_t Pn, int G)
 {
-    const size_t tiles = (size_t)(((K + kSpTile - 1) / kSpTile + G - 1) / G), runs = (size_t)(((Pn + 31) / 32 + G - 1) / G);
-    return tiles * kSpTile * 8 + tiles * 40 + runs * 32 * 16 + kSpSort * sizeof(SpSorted) + kSpEdge * 4 +                                     // slots, tiles, periods
+    const size_t tiles = (size_t)(((K + kSpTile - 1) / kSpTile + G - 1) / G), runs = (size_t)(((Pn + G - 1) / G + 31) / 32);
+    return tiles * kSpTile * 8 + tiles * 36 + runs * 32 * 16 + kSpSort * sizeof(SpSorted) + kSpEdge * 4 +                                     // slots, tiles, periods
            sp_round16((size_t)G * kSpTop * 4) * 2 + sp_round16((size_t)G * kSpTop) +                              // published bounds
-           (size_t)kSpRound * (4 * kSpLimbs + 8 + 8 + 4 * 4) + (size_t)kSpMix * 4 + 128;                      // a round
+           (size_t)kSpRound * (4 * kSpLimbs + 8 + 8 + 4 * 4) + 128;                      // a round
 }
 
 __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, SpreadArgs S)
@@ -129,8 +129,9 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
     __shared__ unsigned s_wk[kPlanWarps * kSpTop], s_tk[kSpTop], s_fk[kPlanWarps];
     __shared__ int s_wi[kPlanWarps * kSpTop], s_ti[kSpTop];
     constexpr int kChunks = (kSpPool + kPlanThreads - 1) / kPlanThreads;        // entries of the pool a thread looks at
-    __shared__ int s_fin[32], s_nfin, s_nmix, s_nedge, s_ndist, s_wcnt[kChunks * kPlanWarps];
+    __shared__ int s_fin[32], s_nfin, s_nmid, s_nedge, s_wcnt[kChunks * kPlanWarps];
     __shared__ Cand s_one;
+    __shared__ ull s_full[32];                                                  // [group of 32 tiles]
     __shared__ unsigned char s_refresh[kLazyMaxBlocks];
     if (*S.done) return;                                     // (same answer in every thread of the grid: written by an earlier launch)
     const int G = gridDim.x, c = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -138,8 +139,8 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
     if (A.K < 1 || A.K > kSpMaxSlots || Pn64 > 0x3fffffff || sp_smem(A.K, Pn64, G) > (size_t)S.smem_bytes) return;     // (the same answer in all blocks)
     const int K = (int)A.K, Pn = (int)Pn64;
     const int64_t limit = (A.max_iterations <= 0 || A.max_iterations > Pn64) ? Pn64 : A.max_iterations;
-    const int NT = (K + kSpTile - 1) / kSpTile, tiles = (NT + G - 1) / G, NR = (Pn + 31) / 32, runs = (NR + G - 1) / G;
-    const int my_tiles = NT > c ? (NT - c + G - 1) / G : 0, my_runs = NR > c ? (NR - c + G - 1) / G : 0;
+    const int NT = (K + kSpTile - 1) / kSpTile, tiles = (NT + G - 1) / G, runs = ((Pn + G - 1) / G + 31) / 32;
+    const int my_tiles = NT > c ? (NT - c + G - 1) / G : 0, my_runs = Pn > c ? ((Pn - c + G - 1) / G + 31) / 32 : 0;
     unsigned char *at = s_raw;
     auto take = [&](size_t bytes) { unsigned char *p = at; at += sp_round16(bytes); return p; };
     longlong2 *mm = (longlong2 *)take((size_t)tiles * 16);                      // [tiles] smallest / largest, offset included
@@ -149,16 +150,17 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
     ull *r_cost = (ull *)take((size_t)kSpRound * 8);
     int *r_p = (int *)take((size_t)kSpRound * 4), *r_e = (int *)take((size_t)kSpRound * 4);      // period << 1 | destination; pool entry
     int *r_ap = (int *)take((size_t)kSpRound * 4), *r_bp = (int *)take((size_t)kSpRound * 4);
-    unsigned *s_mix = (unsigned *)take((size_t)kSpMix * 4), *s_edge = (unsigned *)take((size_t)kSpEdge * 4);      // period of the round << 20 | local tile
+    unsigned *s_edge = (unsigned *)take((size_t)kSpEdge * 4);      // period of the round << 20 | local tile
     SpSorted *sorted = (SpSorted *)take(kSpSort * sizeof(SpSorted));
-    int *t_no = (int *)take((size_t)tiles * 4), *t_at = (int *)take((size_t)tiles * 4);      // distinct tiles of the pairs: number of a tile (-1: none), tile of a number
+    unsigned *t_mid = (unsigned *)take((size_t)tiles * 4);                      // tiles of a round that are near capacity
+    ull *t_full = (ull *)take((size_t)tiles * 8);                               // duration of the tiles of this group of 32 so far that are above it for every period of the round
     unsigned *pkey = (unsigned *)take((size_t)G * kSpTop * 4);                 // published bounds, [rank in the list][block]
     int *pidx = (int *)take((size_t)G * kSpTop * 4);                               // period << 1 | destination, -1 = none
     unsigned char *pdone = take((size_t)G * kSpTop);
     long long *ex = (long long *)take((size_t)tiles * kSpTile * 8);
     long long *off = (long long *)take((size_t)tiles * 8);
-    ull *tsum = (ull *)take((size_t)tiles * 8);
-    auto owner_entry = [&](int p) { return (p >> 5) % G == c ? ((p >> 5) / G) * 32 + (p & 31) : -1; };
+    unsigned *tsum = (unsigned *)take((size_t)tiles * 4);
+    auto owner_entry = [&](int p) { return p % G == c ? p / G : -1; };
 
     unsigned gen = 0;
     int64_t n_mig = 0, rounds = 0, bytes_ssd = 0, bytes_host = 0;
@@ -176,7 +178,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
         const int t = lt * G + c;
         const long long d = A.start[t * kSpTile + kSpTile < K ? t * kSpTile + kSpTile : K] - A.start[t * kSpTile];
         if (d >> 32) bad = true;
-        off[lt] = 0; tsum[lt] = (ull)d; t_no[lt] = -1;
+        off[lt] = 0; tsum[lt] = (unsigned)d;
     }
     if (c == 0) for (int j = tid; j < 3 * kSpRound * 2; j += kPlanThreads) S.partials[j] = 0;
     __syncthreads();
@@ -208,7 +210,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
         hot[e] = sp_pack(sp_key(ben, cost), a, b, ap, bp, X, false);
     };
     for (int e = tid; e < my_runs * 32; e += kPlanThreads) {
-        const int64_t p = ((int64_t)(e >> 5) * G + c) * 32 + (e & 31);
+        const int64_t p = (int64_t)e * G + c;
         hot[e] = make_uint4(0, 0, 0, 0);
         if (p >= Pn) continue;
         // nothing is booked yet: the first usable destination it is
@@ -247,7 +249,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
           for (int h = 0; h < kAhead; ++h) ahead[h] = r0 + h * kPlanWarps < my_runs ? hot[(r0 + h * kPlanWarps) * 32 + lane] : make_uint4(0, 0, 0, 0);
 #pragma unroll
           for (int h = 0; h < kAhead; ++h) {
-            const int r = r0 + h * kPlanWarps, e = r * 32 + lane, p = (r * G + c) * 32 + lane;
+            const int r = r0 + h * kPlanWarps, e = r * 32 + lane, p = e * G + c;
             if (r >= my_runs) break;
             uint4 q = ahead[h];
             if (classify) {
@@ -275,7 +277,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
                 while (todo) {                              // the whole warp, one period after the other
                     const int src = __ffs(todo) - 1;
                     todo &= todo - 1;
-                    const int p2 = (r * G + c) * 32 + src, e2 = r * 32 + src;
+                    const int e2 = r * 32 + src, p2 = e2 * G + c;
                     const bool gone = __shfl_sync(0xffffffffu, lost, src);
                     const SpPeriod Q = sp_unpack(hot[e2]);
                     const int64_t s2 = A.bytes[A.per_t[p2]];
@@ -346,7 +348,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
                 const uint4 q = hot[r * 32 + lane];
                 if (q.x >= thr && (q.w >> 23 & 1u)) {
                     const int n = atomicAdd(&s_nfin, 1);
-                    if (n < 32) s_fin[n] = (r * G + c) * 32 + lane;
+                    if (n < 32) s_fin[n] = (r * 32 + lane) * G + c;
                 }
             }
         if (warp == 0) {
@@ -388,7 +390,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
 #pragma unroll 1
             for (int r = warp; r < my_runs; r += kPlanWarps) {
                 const uint4 q = hot[r * 32 + lane];
-                if (q.x >= thr && (q.w >> 23 & 1u)) { const Cand y = exact((r * G + c) * 32 + lane); if (cand_beats(y, best)) best = y; }
+                if (q.x >= thr && (q.w >> 23 & 1u)) { const Cand y = exact((r * 32 + lane) * G + c); if (cand_beats(y, best)) best = y; }
             }
             best = block_best(best, s_cand);
         }
@@ -572,16 +574,19 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
                 continue;
             }
             round_no += 1;
-            for (int r = tid; r < msel; r += kPlanThreads) {
+            long long sz = 0;
+            for (int r = tid; r < msel; r += kPlanThreads) {                     // (msel <= kPlanThreads)
                 const int i = pidx[r_e[r]], p = i >> 1, d = i & 1;
                 r_p[r] = i;
                 r_ap[r] = A.geo_a[d * A.geo_stride + p]; r_bp[r] = A.geo_b[d * A.geo_stride + p];
-                r_s[r] = A.bytes[A.per_t[p]];
+                r_s[r] = sz = A.bytes[A.per_t[p]];
                 r_cost[r] = 2ull * (ull)A.geo_t[d * A.geo_stride + p];
 #pragma unroll
                 for (int q = 0; q < kSpLimbs; ++q) r_acc[q * kSpRound + r] = 0;
             }
-            if (tid == 0) { s_nmix = 0; s_nedge = 0; s_ndist = 0; }
+            // (the largest tensor of the round, rounded up: bytes are below 2^40)
+            if (const unsigned m = __reduce_max_sync(0xffffffffu, (unsigned)(sz >> 8)); lane == 0) s_fk[warp] = m;
+            if (tid == 0) { s_nmid = 0; s_nedge = 0; }
             __syncthreads();
             auto add = [&](int r, u128 v) {
 #pragma unroll
@@ -605,130 +610,137 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
                 }
                 return sum;
             };
-            // a warp per period, a lane per own tile of its absent range: one at least the tensor's size above capacity throughout counts
-            // it for its whole time, one within capacity nothing; the others are listed
-#pragma unroll 1
-            for (int r = warp; r < msel; r += kPlanWarps) {
-                const int ap = r_ap[r], bp = r_bp[r], ta = ap / kSpTile, tb = bp / kSpTile;
-                const long long s = r_s[r];
-                const int l0 = ta > c ? (ta - c + G - 1) / G : 0, l1 = tb >= c ? (tb - c) / G : -1;
-                ull time = 0;
-#pragma unroll 1
-                for (int lb = l0; lb <= l1; lb += 32) {
-                    const int lt = lb + lane, t0 = (lt * G + c) * kSpTile;
-                    int kind = 0;                                                   // 1: part of the tile, 2: all of it, some slots near capacity
-                    if (lt <= l1) {
-                        const longlong2 m = mm[lt];
-                        const bool whole = t0 >= ap && (t0 + kSpTile - 1 <= bp || bp == K - 1);
-                        if (m.y > 0) {
-                            if (!whole) kind = 1;
-                            else if (m.x >= s) time += tsum[lt];
-                            else kind = 2;
-                        }
-                    }
-                    const unsigned b1 = __ballot_sync(0xffffffffu, kind == 1), b2 = __ballot_sync(0xffffffffu, kind == 2), below = (1u << lane) - 1u;
-                    unsigned rest = 0;
-                    if (b1 | b2) {
-                        int p1 = 0, p2 = 0;
-                        if (lane == 0) { if (b1) p1 = atomicAdd(&s_nedge, __popc(b1)); if (b2) p2 = atomicAdd(&s_nmix, __popc(b2)); }
-                        p1 = __shfl_sync(0xffffffffu, p1, 0) + __popc(b1 & below); p2 = __shfl_sync(0xffffffffu, p2, 0) + __popc(b2 & below);
-                        if (kind == 1) s_edge[p1] = (unsigned)r << 20 | (unsigned)lt;       // (two per period at most)
-                        if (kind == 2 && p2 < kSpMix) {
-                            s_mix[p2] = (unsigned)r << 20 | (unsigned)lt;
-                            if (atomicCAS(&t_no[lt], -1, -2) == -1) { const int n = atomicAdd(&s_ndist, 1); t_at[n] = lt; t_no[lt] = n; }
-                        }
-                        rest = __ballot_sync(0xffffffffu, kind == 2 && p2 >= kSpMix);
-                    }
-#pragma unroll 1
-                    while (rest) {                                                  // list full: the warp reads the tile itself
-                        const int src = __ffs(rest) - 1;
-                        rest &= rest - 1;
-                        const u128 v = warp_sum_u128(slots(r, lb + src));
-                        if (lane == 0) add(r, v);
-                    }
-                }
-                if (__any_sync(0xffffffffu, time != 0)) {
-                    const ull sum = (ull)__reduce_add_sync(0xffffffffu, (unsigned)(time & 0xffffffu)) + ((ull)__reduce_add_sync(0xffffffffu, (unsigned)(time >> 24)) << 24);
-                    if (lane == 0) add(r, (u128)sum * (u128)(ull)s);
-                }
+            // Tiles above capacity by the largest tensor of the round count for their whole time for every period that covers them
+            // (prefix sums); tiles within capacity count for none.  What is left is few: listed.
+            const long long s_max_round = ((long long)__reduce_max_sync(0xffffffffu, lane < kPlanWarps ? s_fk[lane] : 0u) + 1) << 8;
+            for (int b = warp; b * 32 < my_tiles; b += kPlanWarps) {
+                const int lt = b * 32 + lane;
+                const longlong2 m = lt < my_tiles ? mm[lt] : make_longlong2(0, 0);
+                const bool full = lt < my_tiles && m.x >= s_max_round;
+                const unsigned mid = __ballot_sync(0xffffffffu, lt < my_tiles && !full && m.y > 0);
+                const ull d = full ? (ull)tsum[lt] : 0ull;
+                ull incl = d;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) { const ull y = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += y; }
+                if (lt < my_tiles) t_full[lt] = incl - d;
+                if (lane == 31) s_full[b] = incl;
+                int at = 0;
+                if (lane == 0 && mid) at = atomicAdd(&s_nmid, __popc(mid));
+                at = __shfl_sync(0xffffffffu, at, 0) + __popc(mid & ((1u << lane) - 1u));
+                if (mid >> lane & 1u) t_mid[at] = (unsigned)lt;
             }
             __syncthreads();
-            const int nmix = s_nmix < kSpMix ? s_nmix : kSpMix, ndist = s_ndist, nedge = s_nedge;
+            // two threads per period (one of them for every other listed tile): whole tiles [l0, l1]; the two at the ends, if they are
+            // covered in part, are listed for the warps
+            const int nmid = s_nmid, r_me = tid & (kSpRound - 1), half = tid / kSpRound;
+            const bool active = r_me < msel;
+            long long s_me = 0;
+            int l0 = 0, l1 = -1;
+            u128 sum_me = 0;
+            if (active) {
+                const int ap = r_ap[r_me], bp = r_bp[r_me], ta = (ap + kSpTile - 1) / kSpTile, tb = bp == K - 1 ? NT - 1 : (bp + 1) / kSpTile - 1;
+                s_me = r_s[r_me];
+                l0 = ta > c ? (ta - c + G - 1) / G : 0; l1 = tb >= c ? (tb - c) / G : -1;
+                if (half == 0) {
+                    if (l0 <= l1) {
+                        ull time = t_full[l1] + (mm[l1].x >= s_max_round ? (ull)tsum[l1] : 0ull) - t_full[l0];
+                        for (int b = l0 / 32; b < l1 / 32; ++b) time += s_full[b];
+                        sum_me = (u128)time * (u128)(ull)s_me;
+                    }
+                    const int ea = ap / kSpTile, eb = bp / kSpTile;
+                    if (ea < ta && ea % G == c && mm[ea / G].y > 0) s_edge[atomicAdd(&s_nedge, 1)] = (unsigned)r_me << 20 | (unsigned)(ea / G);
+                    if (eb > tb && (eb != ea || ea >= ta) && eb % G == c && mm[eb / G].y > 0) s_edge[atomicAdd(&s_nedge, 1)] = (unsigned)r_me << 20 | (unsigned)(eb / G);
+                }
+            }
+            const bool direct = msel * nmid <= kSpDirect;
+            if (direct) {
 #pragma unroll 1
-            for (int x = kPlanWarps - 1 - warp; x < nedge; x += kPlanWarps) {
+                for (int x = warp; x < msel * nmid; x += kPlanWarps) {
+                    const int r = x % msel, lt = (int)t_mid[x / msel], t0 = (lt * G + c) * kSpTile;
+                    if (t0 < r_ap[r] || (t0 + kSpTile - 1 > r_bp[r] && r_bp[r] != K - 1)) continue;      // (not, or in part)
+                    const u128 v = warp_sum_u128(slots(r, lt));
+                    if (lane == 0) add(r, v);
+                }
+            } else {
+#pragma unroll 1
+                for (int n0 = 0; n0 < nmid; n0 += kSpSort) {
+                    if (n0) __syncthreads();                                        // (the sorted tiles are free)
+                    if (n0 + warp < nmid) {
+                        const int lt = (int)t_mid[n0 + warp], t0 = (lt * G + c) * kSpTile, n = K - t0 < kSpTile ? K - t0 : kSpTile;
+                        SpSorted &q = sorted[warp];
+                        const long long o = off[lt];
+                        long long v[2];
+                        unsigned d[2];
+                        int rank[2] = {0, 0};
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            const int x = h * 32 + lane;
+                            d[h] = x < n ? (unsigned)(A.start[t0 + x + 1] - A.start[t0 + x]) : 0u;
+                            v[h] = x < n ? ex[lt * kSpTile + x] : 0x7fffffffffffffffll;
+                        }
+#pragma unroll 4
+                        for (int j = 0; j < n; ++j) {                               // position of each: how many come before it
+                            const long long y = ex[lt * kSpTile + j];
+#pragma unroll
+                            for (int h = 0; h < 2; ++h) rank[h] += y < v[h] || (y == v[h] && j < h * 32 + lane) ? 1 : 0;
+                        }
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) if (h * 32 + lane < n) {
+                            long long e = v[h] + o;
+                            e = e < 0 ? 0 : e > ((long long)1 << 40) ? (long long)1 << 40 : e;
+                            q.v[rank[h]] = e; q.d[rank[h]] = d[h];
+                        }
+                        __syncwarp();
+                        // prefix sums: two consecutive entries per lane
+                        const bool i0 = 2 * lane < n, i1 = 2 * lane + 1 < n;
+                        const ull v0 = i0 ? (ull)q.v[2 * lane] : 0ull, v1 = i1 ? (ull)q.v[2 * lane + 1] : 0ull;
+                        const unsigned d0 = i0 ? q.d[2 * lane] : 0u, d1 = i1 ? q.d[2 * lane + 1] : 0u;
+                        const ull a0 = (v0 & 0xfffffull) * d0, a1 = (v1 & 0xfffffull) * d1, b0 = (v0 >> 20) * d0, b1 = (v1 >> 20) * d1;
+                        unsigned sd = d0 + d1;
+                        ull sa = a0 + a1, sb = b0 + b1;
+#pragma unroll
+                        for (int o2 = 1; o2 < 32; o2 <<= 1) {
+                            const unsigned yd = __shfl_up_sync(0xffffffffu, sd, o2);
+                            const ull ya = __shfl_up_sync(0xffffffffu, sa, o2), yb = __shfl_up_sync(0xffffffffu, sb, o2);
+                            if (lane >= o2) { sd += yd; sa += ya; sb += yb; }
+                        }
+                        __syncwarp();
+                        q.d[2 * lane] = sd - d1 - d0; q.lo[2 * lane] = sa - a1 - a0; q.hi[2 * lane] = sb - b1 - b0;
+                        q.d[2 * lane + 1] = sd - d1; q.lo[2 * lane + 1] = sa - a1; q.hi[2 * lane + 1] = sb - b1;
+                        if (lane == 31) { q.d[kSpTile] = sd; q.lo[kSpTile] = sa; q.hi[kSpTile] = sb; }
+                        if (lane == 0) { q.n = n; q.lt = lt; }
+                    }
+                    __syncthreads();
+                    if (active) {
+                        const int more = nmid - n0 < kSpSort ? nmid - n0 : kSpSort;
+#pragma unroll 1
+                        for (int m = half; m < more; m += kPlanThreads / kSpRound) {
+                            const SpSorted &q = sorted[m];
+                            if (q.lt < l0 || q.lt > l1) continue;
+                            int j = 0;                                              // slots less than s above capacity
+#pragma unroll
+                            for (int h = kSpTile / 2; h > 0; h >>= 1)
+                                if (j + h <= q.n && q.v[j + h - 1] < s_me) j += h;
+                            if (j < q.n && q.v[j] < s_me) ++j;
+                            sum_me += ((u128)q.hi[j] << 20) + (u128)q.lo[j] + (u128)(ull)s_me * (u128)(ull)(q.d[kSpTile] - q.d[j]);
+                        }
+                    }
+                }
+            }
+            if (half != 0 && sum_me != 0) add(r_me, sum_me);
+            if (direct || nmid == 0) __syncthreads();                              // (the list of the ends; otherwise a barrier has passed)
+#pragma unroll 1
+            for (int x = kPlanWarps - 1 - warp, nedge = s_nedge; x < nedge; x += kPlanWarps) {
                 const int r = (int)(s_edge[x] >> 20);
                 const u128 v = warp_sum_u128(slots(r, (int)(s_edge[x] & 0xfffffu)));
                 if (lane == 0) add(r, v);
             }
-#pragma unroll 1
-            for (int n0 = 0; n0 < ndist; n0 += kSpSort) {
-                if (n0) __syncthreads();                                            // (the sorted tiles are free)
-                if (warp < kSpSort && n0 + warp < ndist) {
-                    const int lt = t_at[n0 + warp], t0 = (lt * G + c) * kSpTile, n = K - t0 < kSpTile ? K - t0 : kSpTile;
-                    SpSorted &q = sorted[warp];
-                    const long long o = off[lt];
-                    long long v[2];
-                    ull d[2];
-                    int rank[2] = {0, 0};
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const int x = h * 32 + lane;
-                        v[h] = x < n ? ex[lt * kSpTile + x] : 0x7fffffffffffffffll;
-                        d[h] = x < n ? (ull)(A.start[t0 + x + 1] - A.start[t0 + x]) : 0ull;
-                    }
-#pragma unroll 4
-                    for (int j = 0; j < n; ++j) {                                   // position of each: how many come before it
-                        const long long y = ex[lt * kSpTile + j];
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) rank[h] += y < v[h] || (y == v[h] && j < h * 32 + lane) ? 1 : 0;
-                    }
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) if (h * 32 + lane < n) {
-                        long long e = v[h] + o;
-                        e = e < 0 ? 0 : e > ((long long)1 << 40) ? (long long)1 << 40 : e;
-                        q.v[rank[h]] = e; q.d[rank[h]] = (unsigned)d[h];
-                    }
-                    __syncwarp();
-                    // prefix sums: two consecutive entries per lane
-                    const bool i0 = 2 * lane < n, i1 = 2 * lane + 1 < n;
-                    const ull v0 = i0 ? (ull)q.v[2 * lane] : 0ull, v1 = i1 ? (ull)q.v[2 * lane + 1] : 0ull;
-                    const unsigned d0 = i0 ? q.d[2 * lane] : 0u, d1 = i1 ? q.d[2 * lane + 1] : 0u;
-                    const ull a0 = (v0 & 0xfffffull) * d0, a1 = (v1 & 0xfffffull) * d1, b0 = (v0 >> 20) * d0, b1 = (v1 >> 20) * d1;
-                    unsigned sd = d0 + d1;
-                    ull sa = a0 + a1, sb = b0 + b1;
-#pragma unroll
-                    for (int o = 1; o < 32; o <<= 1) {
-                        const unsigned yd = __shfl_up_sync(0xffffffffu, sd, o);
-                        const ull ya = __shfl_up_sync(0xffffffffu, sa, o), yb = __shfl_up_sync(0xffffffffu, sb, o);
-                        if (lane >= o) { sd += yd; sa += ya; sb += yb; }
-                    }
-                    __syncwarp();
-                    q.d[2 * lane] = sd - d1 - d0; q.lo[2 * lane] = sa - a1 - a0; q.hi[2 * lane] = sb - b1 - b0;
-                    q.d[2 * lane + 1] = sd - d1; q.lo[2 * lane + 1] = sa - a1; q.hi[2 * lane + 1] = sb - b1;
-                    if (lane == 31) { q.d[kSpTile] = sd; q.lo[kSpTile] = sa; q.hi[kSpTile] = sb; }
-                    if (lane == 0) q.n = n;
-                }
-                __syncthreads();
-#pragma unroll 1
-                for (int x = tid; x < nmix; x += kPlanThreads) {
-                    const int lt = (int)(s_mix[x] & 0xfffffu), r = (int)(s_mix[x] >> 20), no = t_no[lt] - n0;
-                    if (no < 0 || no >= kSpSort) continue;
-                    const SpSorted &q = sorted[no];
-                    const long long s = r_s[r];
-                    int j = 0;                                                      // slots less than s above capacity
-#pragma unroll
-                    for (int h = kSpTile / 2; h > 0; h >>= 1)
-                        if (j + h <= q.n && q.v[j + h - 1] < s) j += h;
-                    if (j < q.n && q.v[j] < s) ++j;
-                    add(r, ((u128)q.hi[j] << 20) + (u128)q.lo[j] + (u128)(ull)s * (u128)(ull)(q.d[kSpTile] - q.d[j]));
-                }
-            }
             __syncthreads();
-            for (int x = tid; x < ndist; x += kPlanThreads) t_no[t_at[x]] = -1;
             // this block's shares go into the grid-wide sums: the low 44 bits and the rest on their own, so that neither needs a carry
             // and no block waits for an answer
-            for (int r = tid; r < msel; r += kPlanThreads) {
-                u128 v = 0;
+            if (half == 0 && active) {
+                const int r = r_me;
+                u128 v = sum_me;
 #pragma unroll
                 for (int q = 0; q < kSpLimbs; ++q) v += (u128)r_acc[q * kSpRound + r] << (16 * q);
                 ull *dst = S.partials + (size_t)pp * 2 * kSpRound + r;
