@@ -30,6 +30,7 @@ constexpr int kSpDirect = 2 * kPlanWarps;       // up to this many (period, tile
 constexpr float kFirst = 0.97f;
 constexpr double kNear = 1e-6;                  // (scores are kept as floats, rounded up: 2^-23)
 constexpr int kSpTop = 8;                       // bounds a block publishes
+constexpr int kSpSeg = 32;                      // likely bounds a warp may list (one per lane when they are ranked)
 constexpr int kSpPool = kLazyMaxBlocks * kSpTop;
 static_assert(kPlanWarps == 16, "two chunks of warp counts per 32 lanes");
 constexpr int kSpLimbs = 6;                     // a benefit (below 2^84) as 16-bit limbs
@@ -42,7 +43,7 @@ struct __align__(16) SpProp {
     unsigned key;                               // its rounded score
     unsigned skey[kSpTop];
     int sidx[kSpTop];                           // period << 1 | destination, -1 = none
-    long long peak, pad;
+    long long peak;
 };
 static_assert(sizeof(SpProp) % 16 == 0 && 2 * sizeof(LazyProp) >= sizeof(SpProp), "workspace for two LazyProp a block");
 
@@ -80,25 +81,22 @@ __device__ __forceinline__ unsigned sp_key(u128 ben, ull cost)
 }
 __device__ __forceinline__ double sp_val(unsigned key) { return (double)__uint_as_float(key); }
 
-// Could a period with rounded score `key` (an upper bound) beat t?  Clear cases by the rounded scores, close ones exactly.
-__device__ __forceinline__ bool sp_may_beat(const SpreadArgs &S, int p, unsigned key, double t_key, const Cand &t)
+// Rounded scores above `hi` beat the best exact score, those below `lo` do not; what is between is settled exactly.
+struct SpBar { unsigned lo, hi; };
+__device__ __forceinline__ SpBar sp_bar(const Cand &t)
 {
-    if (key == 0u) return false;
-    if (t.idx < 0) return true;
-    const double k = sp_val(key);
-    if (k > t_key * (1.0 + kNear)) return true;
-    if (k < t_key * (1.0 - kNear)) return false;
+    if (t.idx < 0) return {1u, 0u};
+    const double k = cand_key(t);
+    return {__float_as_uint(__double2float_rd(k * (1.0 - kNear))), __float_as_uint(__double2float_ru(k * (1.0 + kNear)))};
+}
+// Could a period with rounded score `key` (an upper bound) beat t?
+__device__ __forceinline__ bool sp_may_beat(const SpreadArgs &S, int p, unsigned key, SpBar bar, const Cand &t)
+{
+    if (key < bar.lo) return false;
+    if (key > bar.hi) return true;
     Cand x;
     x.ben = ((u128)__ldcg(&S.c_ben_hi[p]) << 64) | __ldcg(&S.c_ben_lo[p]); x.cost = __ldcg(&S.c_cost[p]); x.idx = p; x.dest = 0;
     return cand_beats(x, t);
-}
-
-// Largest of the lanes' (key, idx), lowest idx on equal keys; uniform.  idx < 0: nothing.
-__device__ __forceinline__ void sp_warp_max(unsigned &key, int &idx)
-{
-    const unsigned m = __reduce_max_sync(0xffffffffu, idx >= 0 ? key : 0u);
-    const unsigned i = __reduce_min_sync(0xffffffffu, idx >= 0 && key == m ? (unsigned)idx : 0xffffffffu);
-    key = m; idx = i == 0xffffffffu ? -1 : (int)i;
 }
 
 // A tile's slots in order of their pressure, for the periods of a round that cover it all and find some of its slots less than their
@@ -126,8 +124,9 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
     __shared__ Cand s_cand[kPlanWarps + 1];
     __shared__ BestScratch s_best;
     __shared__ long long s_max[kPlanWarps + 1];
-    __shared__ unsigned s_wk[kPlanWarps * kSpTop], s_tk[kSpTop], s_fk[kPlanWarps];
-    __shared__ int s_wi[kPlanWarps * kSpTop], s_ti[kSpTop];
+    __shared__ unsigned s_tk[kSpTop], s_fk[kPlanWarps];
+    __shared__ uint2 s_seg[kPlanWarps][kSpSeg];                                 // score, period << 1 | destination
+    __shared__ int s_ti[kSpTop], s_cnt[kPlanWarps];
     constexpr int kChunks = (kSpPool + kPlanThreads - 1) / kPlanThreads;        // entries of the pool a thread looks at
     __shared__ int s_fin[32], s_nfin, s_nmid, s_nedge, s_wcnt[kChunks * kPlanWarps];
     __shared__ Cand s_one;
@@ -233,14 +232,21 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
     // One pass of the block over its periods.  With `classify` the pending commit is applied to them first (its bookings are not in
     // A.busy yet).  With a floor only bounds that may beat it are listed.  Publishes into buffer pbuf.
     auto scan = [&](bool classify, bool with_floor) {
-        unsigned fk = 0, tk[kSpTop];
-        int ti[kSpTop];
-#pragma unroll
-        for (int j = 0; j < kSpTop; ++j) { tk[j] = 0; ti[j] = -1; }
+        unsigned fk = 0, f2 = 0;                                    // the lane's two largest exact scores
+        int fe = -1, n = 0;                                         // entry of the largest; bounds listed by this warp
         const int64_t *bo = A.busy + (size_t)(2 * (w.dest < 0 ? 0 : w.dest)) * A.K, *bi = bo + A.K;
-        const unsigned least = with_floor ? 0u : likely;
-        const double floor_key = with_floor && gBest.idx >= 0 ? cand_key(gBest) : -1.0;
+        const SpBar bar = sp_bar(gBest);
+        const unsigned least = with_floor ? bar.lo : likely ? likely : 1u;
+        const bool host_fills = A.host_capacity != 0 && w.dest == G10_DEST_HOST;
         if (tid == 0) s_nfin = 0;
+        if (tid < kSpTop) { s_tk[tid] = 0u; s_ti[tid] = -1; }
+        auto list = [&](bool take, uint4 q, int p) {
+            const unsigned m = __ballot_sync(0xffffffffu, take);
+            if (m == 0u) return;
+            const int pos = n + __popc(m & ((1u << lane) - 1u));
+            if (take && pos < kSpSeg) s_seg[warp][pos] = make_uint2(q.x, (unsigned)p << 1 | ((q.w >> 21 & 3u) - 1u));
+            n += __popc(m);
+        };
         constexpr int kAhead = 4;                                   // runs whose periods are read together
 #pragma unroll 1
         for (int r0 = warp; r0 < my_runs; r0 += kAhead * kPlanWarps) {
@@ -253,24 +259,25 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
             if (r >= my_runs) break;
             uint4 q = ahead[h];
             if (classify) {
+                // does the commit concern the period at all?  Its channel windows meet those of the commit (rarely), an exact score's
+                // absent range meets it, or it is the period itself
                 const SpPeriod P = sp_unpack(q);
+                const bool meet_out = P.dest == w.dest && P.a < w.ap && w.a < P.ap, meet_in = P.dest == w.dest && P.bp < w.b && w.bp < P.b;
+                const bool stale = P.fresh && P.ap <= w.bp && w.ap <= P.bp;
+                const bool near = (host_fills && P.dest == G10_DEST_HOST && P.a <= w.b && w.a <= P.b) || p == w.idx;
+                if (__any_sync(0xffffffffu, meet_out || meet_in || stale || near)) {
                 bool lost = false;
-                if (P.dest >= 0 && P.a <= w.b && w.a <= P.b) {
-                    if (p == w.idx) { q = make_uint4(0, 0, 0, 0); hot[e] = q; }
-                    else {
-                        if (P.dest == w.dest) {
-                            const bool meet_out = P.a <= w.ap - 1 && w.a <= P.ap - 1, meet_in = P.bp + 1 <= w.b && w.bp + 1 <= P.b;
-                            if (meet_out || meet_in) {
-                                const int64_t tq = (int64_t)(S.c_cost[p] >> 1), q_r = A.start[P.a], q_end = A.start[P.b + 1];
-                                lost = (meet_out && window_conflict<false, true>(A.start, bo, w.a, w.ap - 1, w.t_r, w.t_r + w.t, q_r, q_r + tq, P.a, P.ap - 1)) ||
-                                       (meet_in && window_conflict<false, true>(A.start, bi, w.bp + 1, w.b, w.t_end - w.t, w.t_end, q_end - tq, q_end, P.bp + 1, P.b));
-                            }
-                        }
-                        if (P.fresh && P.ap <= w.bp && w.ap <= P.bp) { q.w &= ~(1u << 23); hot[e] = q; }
+                if (p == w.idx) { q = make_uint4(0, 0, 0, 0); hot[e] = q; }
+                else {
+                    if (meet_out || meet_in) {
+                        const int64_t tq = (int64_t)(S.c_cost[p] >> 1), q_r = A.start[P.a], q_end = A.start[P.b + 1];
+                        lost = (meet_out && window_conflict<false, true>(A.start, bo, w.a, w.ap - 1, w.t_r, w.t_r + w.t, q_r, q_r + tq, P.a, P.ap - 1)) ||
+                               (meet_in && window_conflict<false, true>(A.start, bi, w.bp + 1, w.b, w.t_end - w.t, w.t_end, q_end - tq, q_end, P.bp + 1, P.b));
                     }
+                    if (stale) { q.w &= ~(1u << 23); hot[e] = q; }
                 }
                 // host memory of these slots has filled up (finite capacity): is there still room?
-                const bool room = A.host_capacity != 0 && w.dest == G10_DEST_HOST && P.dest == G10_DEST_HOST && p != w.idx && P.a <= w.b && w.a <= P.b;
+                const bool room = near && p != w.idx;
                 unsigned todo = __ballot_sync(0xffffffffu, lost || room);
                 __syncwarp();
 #pragma unroll 1
@@ -307,16 +314,13 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
                 }
                 __syncwarp();
                 q = hot[e];
+                }
             }
-            if (q.x == 0u) continue;
-            if (q.w >> 23 & 1u) { if (q.x > fk) fk = q.x; }
-            else if (q.x > tk[kSpTop - 1] && q.x >= least && (!with_floor || sp_may_beat(S, p, q.x, floor_key, gBest))) {
-                unsigned k = q.x;
-                int i = p << 1 | (int)((q.w >> 21 & 3u) - 1u);
-#pragma unroll
-                for (int j = 0; j < kSpTop; ++j)
-                    if (k > tk[j]) { const unsigned a = tk[j]; const int b = ti[j]; tk[j] = k; ti[j] = i; k = a; i = b; }
-            }
+            const bool exact = (q.w >> 23 & 1u) != 0u;
+            if (exact) { if (q.x > fk) { f2 = fk; fk = q.x; fe = e; } else if (q.x > f2) f2 = q.x; }
+            bool take = !exact && q.x >= least;
+            if (with_floor && take) take = sp_may_beat(S, p, q.x, bar, gBest);
+            list(take, q, p);
           }
         }
         long long top = -0x7fffffffffffffffll - 1;                  // largest pressure above capacity of the own tiles
@@ -324,50 +328,62 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) { const long long y = __shfl_xor_sync(0xffffffffu, top, o); top = y > top ? y : top; }
         const unsigned wf = __reduce_max_sync(0xffffffffu, fk);
-#pragma unroll 1
-        for (int j = 0; j < kSpTop; ++j) {
-            unsigned k = tk[0];
-            int i = ti[0];
-            sp_warp_max(k, i);
-            if (i >= 0 && i == ti[0]) {                             // this lane's head was taken: the next one moves up
-#pragma unroll
-                for (int q = 0; q < kSpTop - 1; ++q) { tk[q] = tk[q + 1]; ti[q] = ti[q + 1]; }
-                tk[kSpTop - 1] = 0; ti[kSpTop - 1] = -1;
-            }
-            if (lane == 0) { s_wk[warp * kSpTop + j] = i >= 0 ? k : 0u; s_wi[warp * kSpTop + j] = i; }
-            if (i < 0) { if (lane == 0) for (int x = j + 1; x < kSpTop; ++x) { s_wk[warp * kSpTop + x] = 0u; s_wi[warp * kSpTop + x] = -1; } break; }
-        }
-        if (lane == 0) { s_fk[warp] = wf; s_max[warp] = top; }
+        if (lane == 0) { s_fk[warp] = wf; s_max[warp] = top; s_cnt[warp] = n; }
         __syncthreads();
-        const unsigned bf = __reduce_max_sync(0xffffffffu, lane < kPlanWarps ? s_fk[lane] : 0u);
         // the exactly scored periods that may be the best of them
+        const unsigned bf = __reduce_max_sync(0xffffffffu, lane < kPlanWarps ? s_fk[lane] : 0u);
         const unsigned thr = bf ? __float_as_uint((float)(sp_val(bf) * (1.0 - kNear))) : 0u;
-        if (wf != 0u && wf >= thr)
+        if (wf != 0u && wf >= thr) {
+            if (!__any_sync(0xffffffffu, f2 >= thr)) {
+                if (fk >= thr) { const int x = atomicAdd(&s_nfin, 1); if (x < 32) s_fin[x] = fe * G + c; }
+            } else
 #pragma unroll 1
-            for (int r = warp; r < my_runs; r += kPlanWarps) {
-                const uint4 q = hot[r * 32 + lane];
-                if (q.x >= thr && (q.w >> 23 & 1u)) {
-                    const int n = atomicAdd(&s_nfin, 1);
-                    if (n < 32) s_fin[n] = (r * 32 + lane) * G + c;
+                for (int r = warp; r < my_runs; r += kPlanWarps) {
+                    const uint4 q = hot[r * 32 + lane];
+                    if (q.x >= thr && (q.w >> 23 & 1u)) { const int x = atomicAdd(&s_nfin, 1); if (x < 32) s_fin[x] = (r * 32 + lane) * G + c; }
                 }
-            }
-        if (warp == 0) {
-            // (every warp's list is in order: lane w has warp w's, and moves on in it when its head is taken)
-            int at = 0;
-            unsigned hk = lane < kPlanWarps ? s_wk[lane * kSpTop] : 0u;
-            int hi = lane < kPlanWarps ? s_wi[lane * kSpTop] : -1;
+        }
+        // more bounds than the lists hold: the lowest score that at least kSpTop of them reach and the lists hold, by bisection (if too
+        // many share one score, any of those: what is not listed is no larger than what is)
+        if (__any_sync(0xffffffffu, lane < kPlanWarps && s_cnt[lane] > kSpSeg)) {
+            unsigned lo = least, hi = 0x7f800000u;                  // too many; too few (or just right, which ends the search)
+            bool fits = false;
 #pragma unroll 1
-            for (int j = 0; j < kSpTop; ++j) {
-                unsigned k = hk;
-                int i = hi;
-                sp_warp_max(k, i);
-                if (i >= 0 && i == hi) {
-                    ++at;
-                    hk = at < kSpTop ? s_wk[lane * kSpTop + at] : 0u; hi = at < kSpTop ? s_wi[lane * kSpTop + at] : -1;
-                }
-                if (lane == 0) { s_tk[j] = i >= 0 ? k : 0u; s_ti[j] = i; }
-                if (i < 0) { if (lane == 0) for (int x = j + 1; x < kSpTop; ++x) { s_tk[x] = 0u; s_ti[x] = -1; } break; }
+            while (!fits && hi - lo > 1u) {
+                const unsigned mid = lo + (hi - lo) / 2;
+                unsigned m = 0;
+#pragma unroll 4
+                for (int r = warp; r < my_runs; r += kPlanWarps) { const uint4 q = hot[r * 32 + lane]; m += !(q.w >> 23 & 1u) && q.x >= mid ? 1u : 0u; }
+                m = __reduce_add_sync(0xffffffffu, m);
+                __syncthreads();
+                if (lane == 0) s_cnt[warp] = (int)m;
+                __syncthreads();
+                const unsigned z = lane < kPlanWarps ? (unsigned)s_cnt[lane] : 0u;
+                const bool many = __reduce_max_sync(0xffffffffu, z) > (unsigned)kSpSeg;
+                if (many) lo = mid;
+                else { hi = mid; fits = __reduce_add_sync(0xffffffffu, z) >= (unsigned)kSpTop; }
             }
+            n = 0;
+#pragma unroll 1
+            for (int pass = 0; pass < (fits ? 1 : 2); ++pass)
+#pragma unroll 1
+                for (int r = warp; r < my_runs; r += kPlanWarps) {
+                    const uint4 q = hot[r * 32 + lane];
+                    list(!(q.w >> 23 & 1u) && (pass == 0 ? q.x >= hi : q.x == lo), q, (r * 32 + lane) * G + c);
+                }
+            __syncthreads();
+            if (lane == 0) s_cnt[warp] = n < kSpSeg ? n : kSpSeg;
+            __syncthreads();
+        }
+        // the best kSpTop of the listed ones: everyone counts how many come before its own
+        if (lane < s_cnt[warp]) {
+            const uint2 me = s_seg[warp][lane];
+            int rank = 0;
+#pragma unroll 1
+            for (int v = 0; v < kPlanWarps; ++v)
+#pragma unroll 4
+                for (int j = 0, m = s_cnt[v]; j < m; ++j) { const uint2 q = s_seg[v][j]; rank += q.x > me.x || (q.x == me.x && q.y < me.y) ? 1 : 0; }
+            if (rank < kSpTop) { s_tk[rank] = me.x; s_ti[rank] = (int)me.y; }
         }
         __syncthreads();
         auto exact = [&](int p) {
@@ -378,11 +394,11 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
         };
         Cand best;
         best.ben = 0; best.cost = 1; best.idx = -1; best.dest = -1;
-        const int n = s_nfin;
-        if (n <= 32) {
+        const int n_fin = s_nfin;
+        if (n_fin <= 32) {
             if (warp == 0) {
-                if (lane < n) best = exact(s_fin[lane]);
-                if (n > 1)
+                if (lane < n_fin) best = exact(s_fin[lane]);
+                if (n_fin > 1)
 #pragma unroll 1
                     for (int o = 16; o > 0; o >>= 1) { const Cand y = cand_shfl_down(best, o); if (cand_beats(y, best)) best = y; }
             }
@@ -394,15 +410,13 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
             }
             best = block_best(best, s_cand);
         }
+        SpProp &o = S.props[(size_t)pbuf * kLazyMaxBlocks + c];
+        if (tid < kSpTop) { o.skey[tid] = s_tk[tid]; o.sidx[tid] = s_ti[tid]; }
         if (tid == 0) {
-            SpProp o;
             o.ben_lo = (ull)best.ben; o.ben_hi = (ull)(best.ben >> 64); o.cost = best.cost; o.idx = best.idx < 0 ? -1 : best.idx << 1 | best.dest; o.key = best.idx < 0 ? 0u : sp_key(best.ben, best.cost);
-#pragma unroll
-            for (int j = 0; j < kSpTop; ++j) { o.skey[j] = s_tk[j]; o.sidx[j] = s_ti[j]; }
             long long m = s_max[0];
             for (int x = 1; x < kPlanWarps; ++x) m = s_max[x] > m ? s_max[x] : m;
-            o.peak = m; o.pad = 0;
-            S.props[(size_t)pbuf * kLazyMaxBlocks + c] = o;
+            o.peak = m;
         }
     };
     // The exactly best of the threads' candidates (at most one each, with its rounded score): the block's threads all get it.
@@ -502,7 +516,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
         const int n_pool = G * kSpTop;
 #pragma unroll 1
         for (;;) {
-            const double gkey = gBest.idx >= 0 ? cand_key(gBest) : -1.0;
+            const SpBar bar = sp_bar(gBest);
             // which published bounds are rescored now (the same choice in every block, in publication order): every unused one that
             // may beat the best exact score -- in the first round only those within 10 % of the best bound (the winner is usually
             // among them, and a strong exact score spares the rest)
@@ -514,7 +528,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
                 if (lane == 0) s_fk[warp] = k;
                 __syncthreads();
                 k = __reduce_max_sync(0xffffffffu, lane < kPlanWarps ? s_fk[lane] : 0u);
-                if (k != 0u && (gBest.idx < 0 || sp_val(k) >= gkey * (1.0 - kNear))) {
+                if (k >= bar.lo) {
                     const unsigned floor0 = round_no == 0 ? __float_as_uint(fminf(__uint_as_float(k), last_key > 0.0f ? last_key : __uint_as_float(k)) * kFirst) : 0u;
                     unsigned took = 0;                        // (bit j: the thread's j-th entry)
                     int j = 0;
@@ -522,7 +536,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
                         const int e = e0 + tid;
                         bool take = false;
                         if (e < n_pool && !pdone[e] && pidx[e] >= 0 && pkey[e] >= floor0) {
-                            take = sp_may_beat(S, pidx[e] >> 1, pkey[e], gkey, gBest);
+                            take = sp_may_beat(S, pidx[e] >> 1, pkey[e], bar, gBest);
                             if (!take) pdone[e] = 2;
                         }
                         const unsigned mk = __ballot_sync(0xffffffffu, take);
@@ -556,12 +570,11 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
                 if (round_no == 0) round_no = 1;
                 // Nothing published may beat the best score.  A block whose last bound may do so could hold more; and all of them may,
                 // if bounds were left out as unlikely that it turns out may win.
-                const bool unlikely = likely != 0u && (gBest.idx < 0 || sp_val(likely) >= gkey * (1.0 - kNear));
+                const bool unlikely = likely >= bar.lo;
                 bool again = false;
                 if (tid < G) {
                     const int e = (kSpTop - 1) * G + tid;
-                    const double last = pidx[e] >= 0 ? sp_val(pkey[e]) : 0.0;
-                    again = unlikely || (last > 0.0 && (gBest.idx < 0 || last >= gkey * (1.0 - kNear)));
+                    again = unlikely || (pidx[e] >= 0 && pkey[e] >= bar.lo);
                     s_refresh[tid] = again ? 1 : 0;
                 }
                 if (!__syncthreads_or(again)) break;
