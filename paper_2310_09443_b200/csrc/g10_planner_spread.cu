@@ -28,6 +28,8 @@ constexpr int kSpEdge = 2 * kSpRound;           // pairs in which the period cov
 constexpr int kSpSort = kPlanWarps;             // tiles sorted together (one warp each)
 constexpr int kSpDirect = 2 * kPlanWarps;       // up to this many (period, tile) pairs are read slot by slot rather than sorted
 constexpr float kFirst = 0.97f;
+constexpr float kLikely = 0.8f;
+constexpr int kSpPast = 4;
 constexpr double kNear = 1e-6;                  // (scores are kept as floats, rounded up: 2^-23)
 constexpr int kSpTop = 8;                       // bounds a block publishes
 constexpr int kSpSeg = 32;                      // likely bounds a warp may list (one per lane when they are ranked)
@@ -224,7 +226,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
 
     struct { int idx, dest, a, ap, bp, b; int64_t s, t, t_r, t_end; } w = {-1, -1, 0, 0, -1, -1, 0, 0, 0, 0};     // the pending commit
     unsigned likely = 0;                                     // bounds below this (four fifths of the last winner's score) are not listed at first
-    float last_key = 0.0f;                                   // the last winner's score
+    float last_key = 0.0f, won[kSpPast] = {};                // the last winner's score; lowest and those of the last few
     bool pending = false;
     Cand gBest;                                              // best exactly scored period known to the grid
     gBest.ben = 0; gBest.cost = 1; gBest.idx = -1; gBest.dest = -1;
@@ -237,6 +239,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
         const int64_t *bo = A.busy + (size_t)(2 * (w.dest < 0 ? 0 : w.dest)) * A.K, *bi = bo + A.K;
         const SpBar bar = sp_bar(gBest);
         const unsigned least = with_floor ? bar.lo : likely ? likely : 1u;
+        const int w_entry = classify ? owner_entry(w.idx) : -1;
         const bool host_fills = A.host_capacity != 0 && w.dest == G10_DEST_HOST;
         if (tid == 0) s_nfin = 0;
         if (tid < kSpTop) { s_tk[tid] = 0u; s_ti[tid] = -1; }
@@ -247,37 +250,54 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
             if (take && pos < kSpSeg) s_seg[warp][pos] = make_uint2(q.x, (unsigned)p << 1 | ((q.w >> 21 & 3u) - 1u));
             n += __popc(m);
         };
+        auto look = [&](uint4 q, int e) {
+            const int p = e * G + c;
+            const bool exact = (q.w >> 23 & 1u) != 0u;
+            if (exact) { f2 = q.x > fk ? fk : q.x > f2 ? q.x : f2; fe = q.x > fk ? e : fe; fk = q.x > fk ? q.x : fk; }
+            bool take = !exact && q.x >= least;
+            if (with_floor && take) take = sp_may_beat(S, p, q.x, bar, gBest);
+            list(take, q, p);
+        };
         constexpr int kAhead = 4;                                   // runs whose periods are read together
+        unsigned touched = 0;                                       // (the warp has at most 32 runs)
 #pragma unroll 1
-        for (int r0 = warp; r0 < my_runs; r0 += kAhead * kPlanWarps) {
-          uint4 ahead[kAhead];
+        for (int r0 = 0; warp + r0 * kPlanWarps < my_runs; r0 += kAhead) {
+            uint4 ahead[kAhead];
 #pragma unroll
-          for (int h = 0; h < kAhead; ++h) ahead[h] = r0 + h * kPlanWarps < my_runs ? hot[(r0 + h * kPlanWarps) * 32 + lane] : make_uint4(0, 0, 0, 0);
+            for (int h = 0; h < kAhead; ++h) { const int r = warp + (r0 + h) * kPlanWarps; ahead[h] = r < my_runs ? hot[r * 32 + lane] : make_uint4(0, 0, 0, 0); }
 #pragma unroll
-          for (int h = 0; h < kAhead; ++h) {
-            const int r = r0 + h * kPlanWarps, e = r * 32 + lane, p = e * G + c;
-            if (r >= my_runs) break;
-            uint4 q = ahead[h];
-            if (classify) {
-                // does the commit concern the period at all?  Its channel windows meet those of the commit (rarely), an exact score's
-                // absent range meets it, or it is the period itself
-                const SpPeriod P = sp_unpack(q);
+            for (int h = 0; h < kAhead; ++h) {
+                const int e = (warp + (r0 + h) * kPlanWarps) * 32 + lane;
+                uint4 q = ahead[h];
+                if (classify) {
+                    // does the commit concern the period at all?  Its channel windows meet those of the commit, or it is the period
+                    // itself (rarely: these runs come after the others); an exact score's absent range meets it
+                    const SpPeriod P = sp_unpack(q);
+                    const bool meets = P.dest == w.dest && ((P.a < w.ap && w.a < P.ap) || (P.bp < w.b && w.bp < P.b));
+                    const bool near = (host_fills && P.dest == G10_DEST_HOST && P.a <= w.b && w.a <= P.b) || e == w_entry;
+                    if (P.fresh && P.ap <= w.bp && w.ap <= P.bp) { q.w &= ~(1u << 23); hot[e] = q; }
+                    if (__any_sync(0xffffffffu, meets || near)) { touched |= 1u << (r0 + h); continue; }
+                }
+                look(q, e);
+            }
+        }
+        if (classify) {
+            __syncwarp();
+#pragma unroll 1
+            while (touched) {
+                const int r = warp + (__ffs(touched) - 1) * kPlanWarps, e = r * 32 + lane, p = e * G + c;
+                touched &= touched - 1;
+                const SpPeriod P = sp_unpack(hot[e]);
                 const bool meet_out = P.dest == w.dest && P.a < w.ap && w.a < P.ap, meet_in = P.dest == w.dest && P.bp < w.b && w.bp < P.b;
-                const bool stale = P.fresh && P.ap <= w.bp && w.ap <= P.bp;
-                const bool near = (host_fills && P.dest == G10_DEST_HOST && P.a <= w.b && w.a <= P.b) || p == w.idx;
-                if (__any_sync(0xffffffffu, meet_out || meet_in || stale || near)) {
                 bool lost = false;
-                if (p == w.idx) { q = make_uint4(0, 0, 0, 0); hot[e] = q; }
-                else {
-                    if (meet_out || meet_in) {
-                        const int64_t tq = (int64_t)(S.c_cost[p] >> 1), q_r = A.start[P.a], q_end = A.start[P.b + 1];
-                        lost = (meet_out && window_conflict<false, true>(A.start, bo, w.a, w.ap - 1, w.t_r, w.t_r + w.t, q_r, q_r + tq, P.a, P.ap - 1)) ||
-                               (meet_in && window_conflict<false, true>(A.start, bi, w.bp + 1, w.b, w.t_end - w.t, w.t_end, q_end - tq, q_end, P.bp + 1, P.b));
-                    }
-                    if (stale) { q.w &= ~(1u << 23); hot[e] = q; }
+                if (e == w_entry) hot[e] = make_uint4(0, 0, 0, 0);
+                else if (meet_out || meet_in) {
+                    const int64_t tq = (int64_t)(S.c_cost[p] >> 1), q_r = A.start[P.a], q_end = A.start[P.b + 1];
+                    lost = (meet_out && window_conflict<false, true>(A.start, bo, w.a, w.ap - 1, w.t_r, w.t_r + w.t, q_r, q_r + tq, P.a, P.ap - 1)) ||
+                           (meet_in && window_conflict<false, true>(A.start, bi, w.bp + 1, w.b, w.t_end - w.t, w.t_end, q_end - tq, q_end, P.bp + 1, P.b));
                 }
                 // host memory of these slots has filled up (finite capacity): is there still room?
-                const bool room = near && p != w.idx;
+                const bool room = host_fills && P.dest == G10_DEST_HOST && P.a <= w.b && w.a <= P.b && e != w_entry;
                 unsigned todo = __ballot_sync(0xffffffffu, lost || room);
                 __syncwarp();
 #pragma unroll 1
@@ -313,15 +333,8 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
                     if (lane == 0) { if (to_host) begin_period(p2, e2, G10_DEST_HOST, Q.a, Q.b); else hot[e2] = make_uint4(0, 0, 0, 0); }
                 }
                 __syncwarp();
-                q = hot[e];
-                }
+                look(hot[e], e);
             }
-            const bool exact = (q.w >> 23 & 1u) != 0u;
-            if (exact) { if (q.x > fk) { f2 = fk; fk = q.x; fe = e; } else if (q.x > f2) f2 = q.x; }
-            bool take = !exact && q.x >= least;
-            if (with_floor && take) take = sp_may_beat(S, p, q.x, bar, gBest);
-            list(take, q, p);
-          }
         }
         long long top = -0x7fffffffffffffffll - 1;                  // largest pressure above capacity of the own tiles
         for (int lt = tid; lt < my_tiles; lt += kPlanThreads) { const long long v = mm[lt].y; top = v > top ? v : top; }
@@ -798,7 +811,11 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
             w.s = A.bytes[A.per_t[p]];
             w.t_r = A.start[w.a]; w.t_end = A.start[w.b + 1];
             last_key = (float)cand_key(gBest);
-            likely = __float_as_uint((float)(cand_key(gBest) * 0.8));
+            float least = last_key;
+#pragma unroll
+            for (int j = kSpPast - 1; j > 0; --j) { won[j] = won[j - 1]; least = fminf(least, won[j]); }
+            won[0] = last_key;
+            likely = __float_as_uint(least * kLikely);
             if (X == G10_DEST_SSD) bytes_ssd += w.s; else bytes_host += w.s;
         }
         n_mig += 1;
