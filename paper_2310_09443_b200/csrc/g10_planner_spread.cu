@@ -23,9 +23,9 @@
 namespace g10 {
 
 constexpr int kSpTile = 64;                     // slots per tile
-constexpr int kSpRound = 256;                   // periods rescored together, at most
+constexpr int kSpRound = 512;                   // periods rescored together, at most
 constexpr int kSpEdge = 2 * kSpRound;           // pairs in which the period covers the tile in part
-constexpr int kSpSort = kPlanWarps;             // tiles sorted together (one warp each)
+constexpr int kSpSort = 12;                     // tiles sorted together (one warp each; a round has about four in a block)
 constexpr int kSpDirect = 2 * kPlanWarps;       // up to this many (period, tile) pairs are read slot by slot rather than sorted
 constexpr float kFirst = 0.97f;
 constexpr float kLikely = 0.8f;
@@ -35,7 +35,8 @@ constexpr int kSpTop = 8;                       // bounds a block publishes
 constexpr int kSpSeg = 32;                      // likely bounds a warp may list (one per lane when they are ranked)
 constexpr int kSpPool = kLazyMaxBlocks * kSpTop;
 static_assert(kPlanWarps == 16, "two chunks of warp counts per 32 lanes");
-constexpr int kSpLimbs = 6;                     // a benefit (below 2^84) as 16-bit limbs
+static_assert(kSpRound == kPlanThreads, "one thread per period of a round");
+constexpr int kSpLimbs = 4;                     // a benefit (below 2^84) as 21-bit limbs
 
 // What a block tells the grid: its best exactly scored period, its best bounds (descending; anything it did not list is no larger
 // than the last), its largest pressure above capacity.
@@ -58,18 +59,21 @@ struct SpreadArgs {
     int smem_bytes;
 };
 
-// A period: x = score (float bits, rounded up; 0 = no benefit), y, z, w = inactive slots [a, b], absent slots [ap, bp] of the
-// current destination (21 bits each), destination + 1 (0 = erased), FRESH.
+// A period: x = score (float bits, rounded up; 0 = no benefit), inactive slots [a, b] and absent slots [ap, bp] of the current
+// destination (21 bits each), destination + 1 (0 = erased), FRESH.  a, b and ap head a word each: the pass over all periods compares
+// the words as they are.
 struct SpPeriod { int a, b, ap, bp, dest; bool fresh; };
+constexpr unsigned kSpFresh = 4u, kSpDest = 3u;
 __device__ __forceinline__ uint4 sp_pack(unsigned key, int a, int b, int ap, int bp, int dest, bool fresh)
 {
-    return make_uint4(key, (unsigned)a | (unsigned)b << 21, (unsigned)b >> 11 | (unsigned)ap << 10, (unsigned)bp | (unsigned)(dest + 1) << 21 | (fresh ? 1u << 23 : 0u));
+    return make_uint4(key, (unsigned)a << 11 | (unsigned)bp >> 10, (unsigned)b << 11 | ((unsigned)bp & 0x3ffu), (unsigned)ap << 11 | (fresh ? kSpFresh : 0u) | (unsigned)(dest + 1));
 }
+__device__ __forceinline__ int sp_bp(uint4 q) { return (int)((q.y & 0x7ffu) << 10 | (q.z & 0x3ffu)); }
 __device__ __forceinline__ SpPeriod sp_unpack(uint4 q)
 {
     SpPeriod r;
-    r.a = (int)(q.y & 0x1fffffu); r.b = (int)(q.y >> 21 | (q.z & 0x3ffu) << 11); r.ap = (int)(q.z >> 10 & 0x1fffffu);
-    r.bp = (int)(q.w & 0x1fffffu); r.dest = (int)(q.w >> 21 & 3u) - 1; r.fresh = (q.w >> 23 & 1u) != 0u;
+    r.a = (int)(q.y >> 11); r.b = (int)(q.z >> 11); r.ap = (int)(q.w >> 11); r.bp = sp_bp(q);
+    r.dest = (int)(q.w & kSpDest) - 1; r.fresh = (q.w & kSpFresh) != 0u;
     return r;
 }
 constexpr int kSpMaxSlots = (1 << 21) - 1;
@@ -117,7 +121,7 @@ __host__ __device__ inline size_t sp_smem(int64_t K, int64_t Pn, int G)
     const size_t tiles = (size_t)(((K + kSpTile - 1) / kSpTile + G - 1) / G), runs = (size_t)(((Pn + G - 1) / G + 31) / 32);
     return tiles * kSpTile * 8 + tiles * 36 + runs * 32 * 16 + kSpSort * sizeof(SpSorted) + kSpEdge * 4 +                                     // slots, tiles, periods
            sp_round16((size_t)G * kSpTop * 4) * 2 + sp_round16((size_t)G * kSpTop) +                              // published bounds
-           (size_t)kSpRound * (4 * kSpLimbs + 8 + 8 + 4 * 4) + 128;                      // a round
+           (size_t)kSpRound * (4 * kSpLimbs + 8 + 3 * 4) + 128;                      // a round
 }
 
 __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, SpreadArgs S)
@@ -126,11 +130,12 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
     __shared__ Cand s_cand[kPlanWarps + 1];
     __shared__ BestScratch s_best;
     __shared__ long long s_max[kPlanWarps + 1];
-    __shared__ unsigned s_tk[kSpTop], s_fk[kPlanWarps];
+    __shared__ unsigned s_tk[kSpTop], s_fk[kPlanWarps], s_wm[kPlanWarps];
     __shared__ uint2 s_seg[kPlanWarps][kSpSeg];                                 // score, period << 1 | destination
     __shared__ int s_ti[kSpTop], s_cnt[kPlanWarps];
     constexpr int kChunks = (kSpPool + kPlanThreads - 1) / kPlanThreads;        // entries of the pool a thread looks at
-    __shared__ int s_fin[32], s_nfin, s_nmid, s_nedge, s_wcnt[kChunks * kPlanWarps];
+    __shared__ Cand s_fin[32];
+    __shared__ int s_nfin, s_nmid, s_nedge, s_wcnt[kChunks * kPlanWarps];
     __shared__ Cand s_one;
     __shared__ ull s_full[32];                                                  // [group of 32 tiles]
     __shared__ unsigned char s_refresh[kLazyMaxBlocks];
@@ -146,10 +151,9 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
     auto take = [&](size_t bytes) { unsigned char *p = at; at += sp_round16(bytes); return p; };
     longlong2 *mm = (longlong2 *)take((size_t)tiles * 16);                      // [tiles] smallest / largest, offset included
     uint4 *hot = (uint4 *)take((size_t)runs * 32 * 16);
-    unsigned *r_acc = (unsigned *)take((size_t)kSpRound * 4 * kSpLimbs);        // [limb][period] (sums of at most 2^16 16-bit limbs)
+    unsigned *r_acc = (unsigned *)take((size_t)kSpRound * 4 * kSpLimbs);        // [limb][period] (sums of far fewer than 2^11 limbs)
     long long *r_s = (long long *)take((size_t)kSpRound * 8);
-    ull *r_cost = (ull *)take((size_t)kSpRound * 8);
-    int *r_p = (int *)take((size_t)kSpRound * 4), *r_e = (int *)take((size_t)kSpRound * 4);      // period << 1 | destination; pool entry
+    int *r_e = (int *)take((size_t)kSpRound * 4);                               // pool entry
     int *r_ap = (int *)take((size_t)kSpRound * 4), *r_bp = (int *)take((size_t)kSpRound * 4);
     unsigned *s_edge = (unsigned *)take((size_t)kSpEdge * 4);      // period of the round << 20 | local tile
     SpSorted *sorted = (SpSorted *)take(kSpSort * sizeof(SpSorted));
@@ -239,7 +243,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
         const int64_t *bo = A.busy + (size_t)(2 * (w.dest < 0 ? 0 : w.dest)) * A.K, *bi = bo + A.K;
         const SpBar bar = sp_bar(gBest);
         const unsigned least = with_floor ? bar.lo : likely ? likely : 1u;
-        const int w_entry = classify ? owner_entry(w.idx) : -1;
+        const unsigned w_tag = (unsigned)(w.dest + 1), w_ap = (unsigned)w.ap << 11, w_a1 = (unsigned)(w.a + 1) << 11, w_bp1 = (unsigned)(w.bp + 1) << 11;
         const bool host_fills = A.host_capacity != 0 && w.dest == G10_DEST_HOST;
         if (tid == 0) s_nfin = 0;
         if (tid < kSpTop) { s_tk[tid] = 0u; s_ti[tid] = -1; }
@@ -247,12 +251,12 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
             const unsigned m = __ballot_sync(0xffffffffu, take);
             if (m == 0u) return;
             const int pos = n + __popc(m & ((1u << lane) - 1u));
-            if (take && pos < kSpSeg) s_seg[warp][pos] = make_uint2(q.x, (unsigned)p << 1 | ((q.w >> 21 & 3u) - 1u));
+            if (take && pos < kSpSeg) s_seg[warp][pos] = make_uint2(q.x, (unsigned)p << 1 | ((q.w & kSpDest) - 1u));
             n += __popc(m);
         };
         auto look = [&](uint4 q, int e) {
             const int p = e * G + c;
-            const bool exact = (q.w >> 23 & 1u) != 0u;
+            const bool exact = (q.w & kSpFresh) != 0u;
             if (exact) { f2 = q.x > fk ? fk : q.x > f2 ? q.x : f2; fe = q.x > fk ? e : fe; fk = q.x > fk ? q.x : fk; }
             bool take = !exact && q.x >= least;
             if (with_floor && take) take = sp_may_beat(S, p, q.x, bar, gBest);
@@ -270,13 +274,13 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
                 const int e = (warp + (r0 + h) * kPlanWarps) * 32 + lane;
                 uint4 q = ahead[h];
                 if (classify) {
-                    // does the commit concern the period at all?  Its channel windows meet those of the commit, or it is the period
-                    // itself (rarely: these runs come after the others); an exact score's absent range meets it
-                    const SpPeriod P = sp_unpack(q);
-                    const bool meets = P.dest == w.dest && ((P.a < w.ap && w.a < P.ap) || (P.bp < w.b && w.bp < P.b));
-                    const bool near = (host_fills && P.dest == G10_DEST_HOST && P.a <= w.b && w.a <= P.b) || e == w_entry;
-                    if (P.fresh && P.ap <= w.bp && w.ap <= P.bp) { q.w &= ~(1u << 23); hot[e] = q; }
-                    if (__any_sync(0xffffffffu, meets || near)) { touched |= 1u << (r0 + h); continue; }
+                    // does the commit concern the period at all?  Its channel windows meet those of the commit (rarely: these runs come
+                    // after the others); an exact score's absent range meets it
+                    // (out: a < w.ap and w.a < ap; in: bp < w.b and w.bp < b)
+                    bool meets = (q.w & kSpDest) == w_tag && ((q.y < w_ap && q.w >= w_a1) || (q.z >= w_bp1 && sp_bp(q) < w.b));
+                    if (host_fills) meets = meets || ((q.w & kSpDest) == G10_DEST_HOST + 1 && q.y >> 11 <= (unsigned)w.b && (unsigned)w.a <= q.z >> 11);
+                    if ((q.w & kSpFresh) && q.w < w_bp1 && w.ap <= sp_bp(q)) { q.w &= ~kSpFresh; hot[e].w = q.w; }
+                    if (__any_sync(0xffffffffu, meets)) { touched |= 1u << (r0 + h); continue; }
                 }
                 look(q, e);
             }
@@ -290,14 +294,13 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
                 const SpPeriod P = sp_unpack(hot[e]);
                 const bool meet_out = P.dest == w.dest && P.a < w.ap && w.a < P.ap, meet_in = P.dest == w.dest && P.bp < w.b && w.bp < P.b;
                 bool lost = false;
-                if (e == w_entry) hot[e] = make_uint4(0, 0, 0, 0);
-                else if (meet_out || meet_in) {
+                if (meet_out || meet_in) {
                     const int64_t tq = (int64_t)(S.c_cost[p] >> 1), q_r = A.start[P.a], q_end = A.start[P.b + 1];
                     lost = (meet_out && window_conflict<false, true>(A.start, bo, w.a, w.ap - 1, w.t_r, w.t_r + w.t, q_r, q_r + tq, P.a, P.ap - 1)) ||
                            (meet_in && window_conflict<false, true>(A.start, bi, w.bp + 1, w.b, w.t_end - w.t, w.t_end, q_end - tq, q_end, P.bp + 1, P.b));
                 }
                 // host memory of these slots has filled up (finite capacity): is there still room?
-                const bool room = host_fills && P.dest == G10_DEST_HOST && P.a <= w.b && w.a <= P.b && e != w_entry;
+                const bool room = host_fills && P.dest == G10_DEST_HOST && P.a <= w.b && w.a <= P.b;
                 unsigned todo = __ballot_sync(0xffffffffu, lost || room);
                 __syncwarp();
 #pragma unroll 1
@@ -341,19 +344,27 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) { const long long y = __shfl_xor_sync(0xffffffffu, top, o); top = y > top ? y : top; }
         const unsigned wf = __reduce_max_sync(0xffffffffu, fk);
-        if (lane == 0) { s_fk[warp] = wf; s_max[warp] = top; s_cnt[warp] = n; }
+        __syncwarp();
+        uint2 mine = lane < n ? s_seg[warp][lane] : make_uint2(0, 0);
+        if (const unsigned m = __reduce_max_sync(0xffffffffu, mine.x); lane == 0) { s_fk[warp] = wf; s_wm[warp] = m; s_max[warp] = top; s_cnt[warp] = n; }
         __syncthreads();
-        // the exactly scored periods that may be the best of them
+        // the exactly scored periods that may be the best of them (their scores are on the way while the bounds are ranked)
+        auto exact = [&](int p) {
+            Cand x;
+            x.ben = ((u128)S.c_ben_hi[p] << 64) | S.c_ben_lo[p]; x.cost = S.c_cost[p]; x.idx = p;
+            x.dest = (int)(hot[owner_entry(p)].w & kSpDest) - 1;
+            return x;
+        };
         const unsigned bf = __reduce_max_sync(0xffffffffu, lane < kPlanWarps ? s_fk[lane] : 0u);
         const unsigned thr = bf ? __float_as_uint((float)(sp_val(bf) * (1.0 - kNear))) : 0u;
         if (wf != 0u && wf >= thr) {
             if (!__any_sync(0xffffffffu, f2 >= thr)) {
-                if (fk >= thr) { const int x = atomicAdd(&s_nfin, 1); if (x < 32) s_fin[x] = fe * G + c; }
+                if (fk >= thr) { const int x = atomicAdd(&s_nfin, 1); if (x < 32) s_fin[x] = exact(fe * G + c); }
             } else
 #pragma unroll 1
                 for (int r = warp; r < my_runs; r += kPlanWarps) {
                     const uint4 q = hot[r * 32 + lane];
-                    if (q.x >= thr && (q.w >> 23 & 1u)) { const int x = atomicAdd(&s_nfin, 1); if (x < 32) s_fin[x] = (r * 32 + lane) * G + c; }
+                    if (q.x >= thr && (q.w & kSpFresh)) { const int x = atomicAdd(&s_nfin, 1); if (x < 32) s_fin[x] = exact((r * 32 + lane) * G + c); }
                 }
         }
         // more bounds than the lists hold: the lowest score that at least kSpTop of them reach and the lists hold, by bisection (if too
@@ -366,7 +377,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
                 const unsigned mid = lo + (hi - lo) / 2;
                 unsigned m = 0;
 #pragma unroll 4
-                for (int r = warp; r < my_runs; r += kPlanWarps) { const uint4 q = hot[r * 32 + lane]; m += !(q.w >> 23 & 1u) && q.x >= mid ? 1u : 0u; }
+                for (int r = warp; r < my_runs; r += kPlanWarps) { const uint4 q = hot[r * 32 + lane]; m += !(q.w & kSpFresh) && q.x >= mid ? 1u : 0u; }
                 m = __reduce_add_sync(0xffffffffu, m);
                 __syncthreads();
                 if (lane == 0) s_cnt[warp] = (int)m;
@@ -382,35 +393,45 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
 #pragma unroll 1
                 for (int r = warp; r < my_runs; r += kPlanWarps) {
                     const uint4 q = hot[r * 32 + lane];
-                    list(!(q.w >> 23 & 1u) && (pass == 0 ? q.x >= hi : q.x == lo), q, (r * 32 + lane) * G + c);
+                    list(!(q.w & kSpFresh) && (pass == 0 ? q.x >= hi : q.x == lo), q, (r * 32 + lane) * G + c);
                 }
+            __syncwarp();
+            mine = lane < n ? s_seg[warp][lane] : make_uint2(0, 0);
+            const unsigned m = __reduce_max_sync(0xffffffffu, mine.x);
             __syncthreads();
-            if (lane == 0) s_cnt[warp] = n < kSpSeg ? n : kSpSeg;
+            if (lane == 0) s_wm[warp] = m;
             __syncthreads();
         }
-        // the best kSpTop of the listed ones: everyone counts how many come before its own
-        if (lane < s_cnt[warp]) {
-            const uint2 me = s_seg[warp][lane];
-            int rank = 0;
+        // the best kSpTop of the listed ones.  The kSpTop-th largest of the warps' maxima bounds them from below; of the few that
+        // reach it everyone counts how many come before its own
+        {
+            const unsigned v = lane < kPlanWarps ? s_wm[lane] : 0u;
+            int before = 0;
+#pragma unroll
+            for (int j = 0; j < kPlanWarps; ++j) { const unsigned y = __shfl_sync(0xffffffffu, v, j); before += y > v || (y == v && j < lane) ? 1 : 0; }
+            const unsigned at = __ballot_sync(0xffffffffu, before == kSpTop - 1);
+            const unsigned t = __shfl_sync(0xffffffffu, v, __ffs(at) - 1);              // (0 if fewer warps list any)
+            const bool keep = mine.x != 0u && mine.x >= t;
+            const unsigned m = __ballot_sync(0xffffffffu, keep);
+            if (keep) s_seg[warp][__popc(m & ((1u << lane) - 1u))] = mine;
+            if (lane == 0) s_cnt[warp] = __popc(m);
+            __syncthreads();
+            if (keep) {
+                int rank = 0;
 #pragma unroll 1
-            for (int v = 0; v < kPlanWarps; ++v)
-#pragma unroll 4
-                for (int j = 0, m = s_cnt[v]; j < m; ++j) { const uint2 q = s_seg[v][j]; rank += q.x > me.x || (q.x == me.x && q.y < me.y) ? 1 : 0; }
-            if (rank < kSpTop) { s_tk[rank] = me.x; s_ti[rank] = (int)me.y; }
+                for (int u = 0; u < kPlanWarps; ++u)
+#pragma unroll 1
+                    for (int j = 0, z = s_cnt[u]; j < z; ++j) { const uint2 q = s_seg[u][j]; rank += q.x > mine.x || (q.x == mine.x && q.y < mine.y) ? 1 : 0; }
+                if (rank < kSpTop) { s_tk[rank] = mine.x; s_ti[rank] = (int)mine.y; }
+            }
         }
         __syncthreads();
-        auto exact = [&](int p) {
-            Cand x;
-            x.ben = ((u128)S.c_ben_hi[p] << 64) | S.c_ben_lo[p]; x.cost = S.c_cost[p]; x.idx = p;
-            x.dest = (int)(hot[owner_entry(p)].w >> 21 & 3u) - 1;
-            return x;
-        };
         Cand best;
         best.ben = 0; best.cost = 1; best.idx = -1; best.dest = -1;
         const int n_fin = s_nfin;
         if (n_fin <= 32) {
             if (warp == 0) {
-                if (lane < n_fin) best = exact(s_fin[lane]);
+                if (lane < n_fin) best = s_fin[lane];
                 if (n_fin > 1)
 #pragma unroll 1
                     for (int o = 16; o > 0; o >>= 1) { const Cand y = cand_shfl_down(best, o); if (cand_beats(y, best)) best = y; }
@@ -419,17 +440,20 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
 #pragma unroll 1
             for (int r = warp; r < my_runs; r += kPlanWarps) {
                 const uint4 q = hot[r * 32 + lane];
-                if (q.x >= thr && (q.w >> 23 & 1u)) { const Cand y = exact((r * 32 + lane) * G + c); if (cand_beats(y, best)) best = y; }
+                if (q.x >= thr && (q.w & kSpFresh)) { const Cand y = exact((r * 32 + lane) * G + c); if (cand_beats(y, best)) best = y; }
             }
             best = block_best(best, s_cand);
         }
         SpProp &o = S.props[(size_t)pbuf * kLazyMaxBlocks + c];
         if (tid < kSpTop) { o.skey[tid] = s_tk[tid]; o.sidx[tid] = s_ti[tid]; }
         if (tid == 0) {
-            o.ben_lo = (ull)best.ben; o.ben_hi = (ull)(best.ben >> 64); o.cost = best.cost; o.idx = best.idx < 0 ? -1 : best.idx << 1 | best.dest; o.key = best.idx < 0 ? 0u : sp_key(best.ben, best.cost);
-            long long m = s_max[0];
-            for (int x = 1; x < kPlanWarps; ++x) m = s_max[x] > m ? s_max[x] : m;
-            o.peak = m;
+            o.ben_lo = (ull)best.ben; o.ben_hi = (ull)(best.ben >> 64); o.cost = best.cost; o.idx = best.idx < 0 ? -1 : best.idx << 1 | best.dest; o.key = best.idx < 0 ? 0u : hot[owner_entry(best.idx)].x;
+        }
+        if (warp == 1) {
+            long long m = lane < kPlanWarps ? s_max[lane] : s_max[0];
+#pragma unroll
+            for (int z = 16; z > 0; z >>= 1) { const long long y = __shfl_xor_sync(0xffffffffu, m, z); m = y > m ? y : m; }
+            if (lane == 0) o.peak = m;
         }
     };
     // The exactly best of the threads' candidates (at most one each, with its rounded score): the block's threads all get it.
@@ -506,6 +530,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
                 } else raise_status(A.status, G10_DEV_PLAN_OVERFLOW);
             }
         }
+        if (pending && tid == 0) { const int e = owner_entry(w.idx); if (e >= 0) hot[e] = make_uint4(0, 0, 0, 0); }
         __syncthreads();
         scan(pending, false);
         if (!grid_barrier(A.bar, G, gen)) { status = -2; break; }
@@ -601,12 +626,13 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
             }
             round_no += 1;
             long long sz = 0;
-            for (int r = tid; r < msel; r += kPlanThreads) {                     // (msel <= kPlanThreads)
-                const int i = pidx[r_e[r]], p = i >> 1, d = i & 1;
-                r_p[r] = i;
+            ull cost = 1;
+            int own = -1;                                                           // the thread's period << 1 | destination
+            if (const int r = tid; r < msel) {
+                const int i = own = pidx[r_e[r]], p = i >> 1, d = i & 1;
                 r_ap[r] = A.geo_a[d * A.geo_stride + p]; r_bp[r] = A.geo_b[d * A.geo_stride + p];
                 r_s[r] = sz = A.bytes[A.per_t[p]];
-                r_cost[r] = 2ull * (ull)A.geo_t[d * A.geo_stride + p];
+                cost = 2ull * (ull)A.geo_t[d * A.geo_stride + p];
 #pragma unroll
                 for (int q = 0; q < kSpLimbs; ++q) r_acc[q * kSpRound + r] = 0;
             }
@@ -617,7 +643,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
             auto add = [&](int r, u128 v) {
 #pragma unroll
                 for (int q = 0; q < kSpLimbs; ++q) {                                 // (a 64-bit atomic would be a compare-and-swap loop)
-                    const unsigned x = (unsigned)(v >> (16 * q)) & 0xffffu;
+                    const unsigned x = (unsigned)(v >> (21 * q)) & 0x1fffffu;
                     if (x) atomicAdd(&r_acc[q * kSpRound + r], x);
                 }
             };
@@ -656,9 +682,10 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
                 if (mid >> lane & 1u) t_mid[at] = (unsigned)lt;
             }
             __syncthreads();
-            // two threads per period (one of them for every other listed tile): whole tiles [l0, l1]; the two at the ends, if they are
-            // covered in part, are listed for the warps
-            const int nmid = s_nmid, r_me = tid & (kSpRound - 1), half = tid / kSpRound;
+            // a thread per period, two if there are enough (one of them for every other listed tile): whole tiles [l0, l1]; the two at
+            // the ends, if they are covered in part, are listed for the warps
+            const bool two = msel <= kPlanThreads / 2;
+            const int nmid = s_nmid, r_me = two ? tid & (kPlanThreads / 2 - 1) : tid, half = two ? tid / (kPlanThreads / 2) : 0;
             const bool active = r_me < msel;
             long long s_me = 0;
             int l0 = 0, l1 = -1;
@@ -691,7 +718,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
 #pragma unroll 1
                 for (int n0 = 0; n0 < nmid; n0 += kSpSort) {
                     if (n0) __syncthreads();                                        // (the sorted tiles are free)
-                    if (n0 + warp < nmid) {
+                    if (warp < kSpSort && n0 + warp < nmid) {
                         const int lt = (int)t_mid[n0 + warp], t0 = (lt * G + c) * kSpTile, n = K - t0 < kSpTile ? K - t0 : kSpTile;
                         SpSorted &q = sorted[warp];
                         const long long o = off[lt];
@@ -740,7 +767,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
                     if (active) {
                         const int more = nmid - n0 < kSpSort ? nmid - n0 : kSpSort;
 #pragma unroll 1
-                        for (int m = half; m < more; m += kPlanThreads / kSpRound) {
+                        for (int m = half; m < more; m += two ? 2 : 1) {
                             const SpSorted &q = sorted[m];
                             if (q.lt < l0 || q.lt > l1) continue;
                             int j = 0;                                              // slots less than s above capacity
@@ -768,7 +795,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
                 const int r = r_me;
                 u128 v = sum_me;
 #pragma unroll
-                for (int q = 0; q < kSpLimbs; ++q) v += (u128)r_acc[q * kSpRound + r] << (16 * q);
+                for (int q = 0; q < kSpLimbs; ++q) v += (u128)r_acc[q * kSpRound + r] << (21 * q);
                 ull *dst = S.partials + (size_t)pp * 2 * kSpRound + r;
                 const ull lo = (ull)v & 0xfffffffffffull, hi = (ull)(v >> 44);
                 if (lo) asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(dst), "l"(lo) : "memory");
@@ -782,16 +809,16 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
             x.ben = 0; x.cost = 1; x.idx = -1; x.dest = -1;
             unsigned key = 0;
             if (tid < msel) {
-                const int i = r_p[tid], p = i >> 1;
+                const int i = own, p = i >> 1;
                 const ull *src = S.partials + (size_t)pp * 2 * kSpRound + tid;
                 const u128 tot = ((u128)__ldcg(src + kSpRound) << 44) + __ldcg(src);
-                x.ben = tot; x.cost = r_cost[tid]; x.idx = tot == 0 ? -1 : p; x.dest = i & 1;
+                x.ben = tot; x.cost = cost; x.idx = tot == 0 ? -1 : p; x.dest = i & 1;
                 key = sp_key(tot, x.cost);
                 const int e = owner_entry(p);
                 if (e >= 0) {
                     S.c_ben_lo[p] = (ull)tot; S.c_ben_hi[p] = (ull)(tot >> 64);
                     uint4 q = hot[e];
-                    q.x = key; q.w |= 1u << 23;
+                    q.x = key; q.w |= kSpFresh;
                     hot[e] = q;
                 }
             }
