@@ -258,32 +258,30 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
             const int p = e * G + c;
             const bool exact = (q.w & kSpFresh) != 0u;
             if (exact) { f2 = q.x > fk ? fk : q.x > f2 ? q.x : f2; fe = q.x > fk ? e : fe; fk = q.x > fk ? q.x : fk; }
-            bool take = !exact && q.x >= least;
+            bool take = !exact & (q.x >= least);
             if (with_floor && take) take = sp_may_beat(S, p, q.x, bar, gBest);
             list(take, q, p);
         };
-        constexpr int kAhead = 4;                                   // runs whose periods are read together
+        // (a short loop, the next run's periods on the way: unrolled four times it took longer, for its instructions)
         unsigned touched = 0;                                       // (the warp has at most 32 runs)
+        uint4 next = warp < my_runs ? hot[warp * 32 + lane] : make_uint4(0, 0, 0, 0);
 #pragma unroll 1
-        for (int r0 = 0; warp + r0 * kPlanWarps < my_runs; r0 += kAhead) {
-            uint4 ahead[kAhead];
-#pragma unroll
-            for (int h = 0; h < kAhead; ++h) { const int r = warp + (r0 + h) * kPlanWarps; ahead[h] = r < my_runs ? hot[r * 32 + lane] : make_uint4(0, 0, 0, 0); }
-#pragma unroll
-            for (int h = 0; h < kAhead; ++h) {
-                const int e = (warp + (r0 + h) * kPlanWarps) * 32 + lane;
-                uint4 q = ahead[h];
-                if (classify) {
-                    // does the commit concern the period at all?  Its channel windows meet those of the commit (rarely: these runs come
-                    // after the others); an exact score's absent range meets it
-                    // (out: a < w.ap and w.a < ap; in: bp < w.b and w.bp < b)
-                    bool meets = (q.w & kSpDest) == w_tag && ((q.y < w_ap && q.w >= w_a1) || (q.z >= w_bp1 && sp_bp(q) < w.b));
-                    if (host_fills) meets = meets || ((q.w & kSpDest) == G10_DEST_HOST + 1 && q.y >> 11 <= (unsigned)w.b && (unsigned)w.a <= q.z >> 11);
-                    if ((q.w & kSpFresh) && q.w < w_bp1 && w.ap <= sp_bp(q)) { q.w &= ~kSpFresh; hot[e].w = q.w; }
-                    if (__any_sync(0xffffffffu, meets)) { touched |= 1u << (r0 + h); continue; }
-                }
-                look(q, e);
+        for (int r = warp, n_run = 0; r < my_runs; r += kPlanWarps, ++n_run) {
+            const int e = r * 32 + lane;
+            uint4 q = next;
+            if (r + kPlanWarps < my_runs) next = hot[e + kPlanWarps * 32];
+            if (classify) {
+                // does the commit concern the period at all?  Its channel windows meet those of the commit (rarely: these runs come
+                // after the others); an exact score's absent range meets it
+                // (out: a < w.ap and w.a < ap; in: bp < w.b and w.bp < b)
+                const int bp = sp_bp(q);
+                bool meets = ((q.w & kSpDest) == w_tag) & (((q.y < w_ap) & (q.w >= w_a1)) | ((q.z >= w_bp1) & (bp < w.b)));     // (no branches)
+                if (host_fills) meets = meets || ((q.w & kSpDest) == G10_DEST_HOST + 1 && q.y >> 11 <= (unsigned)w.b && (unsigned)w.a <= q.z >> 11);
+                const bool stale = ((q.w & kSpFresh) != 0u) & (q.w < w_bp1) & (w.ap <= bp);
+                if (stale) { q.w &= ~kSpFresh; hot[e].w = q.w; }
+                if (__any_sync(0xffffffffu, meets)) { touched |= 1u << n_run; continue; }
             }
+            look(q, e);
         }
         if (classify) {
             __syncwarp();
