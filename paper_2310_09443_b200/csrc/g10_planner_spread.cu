@@ -108,7 +108,7 @@ __device__ __forceinline__ bool sp_may_beat(const SpreadArgs &S, int p, unsigned
 // A tile's slots in order of their pressure, for the periods of a round that cover it all and find some of its slots less than their
 // size above capacity: with prefix sums of the durations and of pressure x duration, a period's benefit is a binary search
 // instead of 64 slots (a round's periods mostly overlap: the same few tiles near capacity are wanted a hundred times).
-struct SpSorted {
+struct __align__(16) SpSorted {
     long long v[kSpTile];                       // pressure above capacity, at least 0 and at most 2^40 (tensors are smaller), ascending
     ull lo[kSpTile + 1], hi[kSpTile + 1];       // sums of (v mod 2^20) x duration and of (v >> 20) x duration over the first n
     unsigned d[kSpTile + 1];                    // sums of the durations (a tile's total is below 2^32 ns)
@@ -703,6 +703,14 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
                     if (eb > tb && (eb != ea || ea >= ta) && eb % G == c && mm[eb / G].y > 0) s_edge[atomicAdd(&s_nedge, 1)] = (unsigned)r_me << 20 | (unsigned)(eb / G);
                 }
             }
+            __syncthreads();
+            // (the last warps first: the others sort meanwhile)
+#pragma unroll 1
+            for (int x = kPlanWarps - 1 - warp, nedge = s_nedge; x < nedge; x += kPlanWarps) {
+                const int r = (int)(s_edge[x] >> 20);
+                const u128 v = warp_sum_u128(slots(r, (int)(s_edge[x] & 0xfffffu)));
+                if (lane == 0) add(r, v);
+            }
             const bool direct = msel * nmid <= kSpDirect;
             if (direct) {
 #pragma unroll 1
@@ -727,20 +735,22 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
                         for (int h = 0; h < 2; ++h) {
                             const int x = h * 32 + lane;
                             d[h] = x < n ? (unsigned)(A.start[t0 + x + 1] - A.start[t0 + x]) : 0u;
-                            v[h] = x < n ? ex[lt * kSpTile + x] : 0x7fffffffffffffffll;
+                            const long long e = x < n ? ex[lt * kSpTile + x] + o : 0;
+                            // (with the slot as the lowest bits: no two are equal)
+                            v[h] = x < n ? (e < 0 ? 0 : e > ((long long)1 << 40) ? (long long)1 << 40 : e) << 6 | x : (long long)1 << 62;
+                            q.v[x] = v[h];
                         }
+                        __syncwarp();
+                        const longlong2 *all = reinterpret_cast<const longlong2 *>(q.v);
 #pragma unroll 4
-                        for (int j = 0; j < n; ++j) {                               // position of each: how many come before it
-                            const long long y = ex[lt * kSpTile + j];
+                        for (int j = 0; j < kSpTile / 2; ++j) {                     // position of each: how many come before it
+                            const longlong2 y = all[j];
 #pragma unroll
-                            for (int h = 0; h < 2; ++h) rank[h] += y < v[h] || (y == v[h] && j < h * 32 + lane) ? 1 : 0;
+                            for (int h = 0; h < 2; ++h) rank[h] += (y.x < v[h] ? 1 : 0) + (y.y < v[h] ? 1 : 0);
                         }
+                        __syncwarp();
 #pragma unroll
-                        for (int h = 0; h < 2; ++h) if (h * 32 + lane < n) {
-                            long long e = v[h] + o;
-                            e = e < 0 ? 0 : e > ((long long)1 << 40) ? (long long)1 << 40 : e;
-                            q.v[rank[h]] = e; q.d[rank[h]] = d[h];
-                        }
+                        for (int h = 0; h < 2; ++h) if (h * 32 + lane < n) { q.v[rank[h]] = v[h] >> 6; q.d[rank[h]] = d[h]; }
                         __syncwarp();
                         // prefix sums: two consecutive entries per lane
                         const bool i0 = 2 * lane < n, i1 = 2 * lane + 1 < n;
@@ -779,13 +789,6 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
                 }
             }
             if (half != 0 && sum_me != 0) add(r_me, sum_me);
-            if (direct || nmid == 0) __syncthreads();                              // (the list of the ends; otherwise a barrier has passed)
-#pragma unroll 1
-            for (int x = kPlanWarps - 1 - warp, nedge = s_nedge; x < nedge; x += kPlanWarps) {
-                const int r = (int)(s_edge[x] >> 20);
-                const u128 v = warp_sum_u128(slots(r, (int)(s_edge[x] & 0xfffffu)));
-                if (lane == 0) add(r, v);
-            }
             __syncthreads();
             // this block's shares go into the grid-wide sums: the low 44 bits and the rest on their own, so that neither needs a carry
             // and no block waits for an answer
