@@ -31,7 +31,7 @@ struct EmitArgs {
     int bw, nb;                           // boundaries per bucket, buckets
     ull magic;                            // ceil(2^64 / bw) (0 when bw == 1): the bucket of boundary x is the high half of x * magic
     unsigned *bucket_count, *bucket_cursor;
-    unsigned *block_count;                // [nb][G] per bucket: what each block of the counting kernel saw, then the running sums
+    unsigned *block_count;                // [G][nb] what each block of the counting kernel saw of every bucket, then the running sums
     int G;                                // blocks of the counting and of the scatter kernel (the same items go to the same block)
     ull *keys;
     int32_t *payload;
@@ -39,33 +39,82 @@ struct EmitArgs {
     ull *status;
 };
 
-// item -> (boundary, opcode, tensor, record); false if the item does not exist
-__device__ __forceinline__ bool emit_item(const EmitArgs &A, int64_t item, int64_t *boundary, int *opcode, int *tensor, int *record)
+// A pre-eviction (item < n) or a prefetch of a plan record -> boundary, opcode, record
+__device__ __forceinline__ void emit_record(const EmitArgs &A, int64_t item, int64_t *boundary, int *opcode, int *record)
 {
-    *record = -1;
-    if (item < 2 * A.N) {
-        const int64_t i = item < A.N ? item : item - A.N;
-        const int f = A.first_use[i];
-        if (f < 0) return false;
-        const bool g = A.glob != nullptr && A.glob[i] != 0;
-        *tensor = (int)i;
-        if (item < A.N) { *opcode = kOpAlloc; *boundary = g ? 0 : f; return true; }
-        if (g) return false;
-        *opcode = kOpFree; *boundary = (int64_t)A.last_use[i] + 1;
-        return true;
-    }
-    const int64_t r = item - 2 * A.N < A.n ? item - 2 * A.N : item - 2 * A.N - A.n;
-    const bool evict = item - 2 * A.N < A.n;
-    *record = (int)r; *tensor = A.mig[r].tensor;
+    const bool evict = item < A.n;
+    const int64_t r = evict ? item : item - A.n;
     int64_t t = evict ? A.mig[r].evict_issue_ns : (A.new_issue ? A.new_issue[r] : A.mig[r].prefetch_issue_ns);
     // (a steady-state plan: the prefetch of a wrap-around period may lie in the next iteration; it stands at the same
     // moment of this one)
     if (!evict && t >= A.start[A.K]) t -= A.start[A.K];
-    // last boundary b in [0, K] with start[b] <= t (for a pre-eviction start[b] == t_r exactly)
+    // last boundary b in [0, K] with start[b] <= t (for a pre-eviction start[b] == t_r exactly).  Seven probes a step, all on their
+    // way together: a third of the round trips of a binary search
     int lo = 0, hi = (int)A.K;
-    while (lo < hi) { const int mid = lo + (hi - lo + 1) / 2; if (A.start[mid] <= t) lo = mid; else hi = mid - 1; }
-    *boundary = lo; *opcode = evict ? kOpPreEvict : kOpPrefetch;
-    return true;
+    while (lo < hi) {
+        const int step = (hi - lo) / 8 + 1;
+        int c = 0;
+#pragma unroll
+        for (int j = 1; j < 8; ++j) { const int64_t x = (int64_t)lo + (int64_t)j * step; c += x <= hi && A.start[x <= hi ? x : hi] <= t ? 1 : 0; }
+        lo += c * step;
+        if (c < 7 && lo + step - 1 < hi) hi = lo + step - 1;
+    }
+    *boundary = lo; *opcode = evict ? kOpPreEvict : kOpPrefetch; *record = (int)r;
+}
+
+// Calls put(valid, boundary, opcode, tensor, record), whole warps at a time, for the instructions of the block's share of the work:
+// the plan's records (first: their searches take longest), then every tensor's allocation and release.  The same items go to the
+// same block in every kernel.
+template <typename F>
+__device__ __forceinline__ void emit_items(const EmitArgs &A, F &&put)
+{
+    constexpr int kBatch = 4;                 // tensors a thread reads together
+    const int lane = threadIdx.x & 31;
+    const int64_t stride = (int64_t)gridDim.x * kEmitThreads, total = 2 * A.n + A.N;
+    for (int64_t w0 = (int64_t)blockIdx.x * kEmitThreads + (threadIdx.x - lane); w0 < total; w0 += kBatch * stride) {
+        int f[kBatch], la[kBatch];
+        bool g[kBatch];
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) {
+            const int64_t i = w0 + lane + u * stride - 2 * A.n;
+            const bool in = i >= 0 && i < A.N;
+            f[u] = in ? A.first_use[i] : -1;
+            la[u] = in ? A.last_use[i] : 0;
+            g[u] = in && A.glob != nullptr && A.glob[i] != 0;
+        }
+#pragma unroll 1
+        for (int64_t r0 = w0; r0 < 2 * A.n && r0 < w0 + kBatch * stride; r0 += stride) {
+            int64_t bd = 0;
+            int op = 0, rc = -1, tn = 0;
+            const bool in = r0 + lane < 2 * A.n;
+            if (in) { emit_record(A, r0 + lane, &bd, &op, &rc); tn = A.mig[rc].tensor; }
+            put(in, bd, op, tn, rc);
+        }
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) {
+            if (w0 + u * stride >= total) break;
+            const int i = (int)(w0 + lane + u * stride - 2 * A.n);
+            put(f[u] >= 0, (int64_t)(g[u] ? 0 : f[u]), (int)kOpAlloc, i, -1);
+            put(f[u] >= 0 && !g[u], (int64_t)la[u] + 1, (int)kOpFree, i, -1);
+        }
+    }
+}
+
+// The next free place of every lane's bucket (shared-memory counters).  Neighbouring tensors are born and die at neighbouring
+// kernels: most lanes of a warp want the same bucket, and one lane counts for those that want the first one's (32 atomics on one
+// word take turns; sorting out all of a warp's buckets with match.any took as long).
+__device__ __forceinline__ unsigned emit_take(unsigned *next, bool valid, int b)
+{
+    const int lane = threadIdx.x & 31;
+    const unsigned on = __ballot_sync(0xffffffffu, valid);
+    if (on == 0u) return 0u;
+    const int first = __ffs(on) - 1, b0 = __shfl_sync(0xffffffffu, b, first);
+    const unsigned same = __ballot_sync(0xffffffffu, valid && b == b0);
+    unsigned at = 0;
+    if (lane == first) at = atomicAdd(&next[b0], (unsigned)__popc(same));
+    else if (valid && b != b0) at = atomicAdd(&next[b], 1u);
+    const unsigned run = __shfl_sync(0xffffffffu, at, first) + __popc(same & ((1u << lane) - 1u));
+    return b == b0 ? run : at;
 }
 
 // Bucket of a boundary.  With magic = (2^64 + e) / bw, 0 <= e < bw, the product x * magic / 2^64 exceeds x / bw by less than
@@ -85,35 +134,33 @@ __global__ void __launch_bounds__(kEmitThreads) k_emit_hist(EmitArgs A)
     extern __shared__ unsigned s_hist[];
     for (int b = threadIdx.x; b < A.nb; b += kEmitThreads) s_hist[b] = 0;
     __syncthreads();
-    const int64_t total = 2 * A.N + 2 * A.n;
-    for (int64_t item = (int64_t)blockIdx.x * kEmitThreads + threadIdx.x; item < total; item += (int64_t)gridDim.x * kEmitThreads) {
-        int64_t bd; int op, tn, rc;
-        if (emit_item(A, item, &bd, &op, &tn, &rc)) atomicAdd(&s_hist[emit_bucket(A, bd)], 1u);
-    }
+    emit_items(A, [&](bool valid, int64_t bd, int, int, int) { emit_take(s_hist, valid, emit_bucket(A, bd)); });
     __syncthreads();
     // what this block saw of every bucket: the scatter kernel, whose blocks walk the same items, gets from it the block's own
     // run inside every bucket's slice and needs no global cursor
-    for (int b = threadIdx.x; b < A.nb; b += kEmitThreads) A.block_count[(size_t)b * A.G + blockIdx.x] = s_hist[b];
+    for (int b = threadIdx.x; b < A.nb; b += kEmitThreads) A.block_count[(size_t)blockIdx.x * A.nb + b] = s_hist[b];
 }
 
-// Per bucket: running sums over the blocks (in place) and the bucket's total.  One warp per bucket.
-__global__ void __launch_bounds__(kEmitThreads) k_emit_block_offsets(EmitArgs A)
+// Per bucket: running sums over the blocks (in place) and the bucket's total.  A block takes 32 buckets, a lane each (rows of
+// consecutive buckets: whole sectors); its warps split the counting blocks among them and add up their shares before they write.
+constexpr int kOffWarps = 32, kOffRows = (kEmitMaxBlocks + kOffWarps - 1) / kOffWarps;
+__global__ void __launch_bounds__(kOffWarps * 32) k_emit_block_offsets(EmitArgs A)
 {
-    const int lane = threadIdx.x & 31;
-    const int b = (int)(blockIdx.x * (kEmitThreads / 32) + (threadIdx.x >> 5));
-    if (b >= A.nb) return;
-    unsigned *row = A.block_count + (size_t)b * A.G;
-    unsigned carry = 0;
-    for (int j0 = 0; j0 < A.G; j0 += 32) {
-        const int j = j0 + lane;
-        const unsigned v = j < A.G ? row[j] : 0u;
-        unsigned incl = v;
+    __shared__ unsigned s_sum[kOffWarps][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, b = blockIdx.x * 32 + lane;
+    const int rows = (A.G + kOffWarps - 1) / kOffWarps, r0 = warp * rows;       // (rows <= kOffRows)
+    unsigned v[kOffRows], sum = 0;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) { const unsigned y = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += y; }
-        if (j < A.G) row[j] = carry + incl - v;
-        carry += __shfl_sync(0xffffffffu, incl, 31);
-    }
-    if (lane == 0) A.bucket_count[b] = carry;
+    for (int q = 0; q < kOffRows; ++q) { v[q] = q < rows && r0 + q < A.G && b < A.nb ? A.block_count[(size_t)(r0 + q) * A.nb + b] : 0u; sum += v[q]; }
+    s_sum[warp][lane] = sum;
+    __syncthreads();
+    unsigned run = 0, all = 0;
+#pragma unroll
+    for (int x = 0; x < kOffWarps; ++x) { const unsigned y = s_sum[x][lane]; if (x < warp) run += y; all += y; }
+    if (b >= A.nb) return;
+#pragma unroll
+    for (int q = 0; q < kOffRows; ++q) if (q < rows && r0 + q < A.G) { A.block_count[(size_t)(r0 + q) * A.nb + b] = run; run += v[q]; }
+    if (warp == 0) A.bucket_count[b] = all;
 }
 
 // exclusive scan of the bucket counts (nb <= 4096) into s_base[0..nb]
@@ -144,19 +191,17 @@ __global__ void __launch_bounds__(kEmitThreads) k_emit_scatter(EmitArgs A)
     __shared__ long long s_w[kEmitThreads / 32];
     emit_scan_buckets(A.bucket_count, A.nb, s_base, s_w);
     unsigned *s_next = (unsigned *)(s_base + A.nb + 1);
-    for (int b = threadIdx.x; b < A.nb; b += kEmitThreads) s_next[b] = A.block_count[(size_t)b * A.G + blockIdx.x];
+    for (int b = threadIdx.x; b < A.nb; b += kEmitThreads) s_next[b] = A.block_count[(size_t)blockIdx.x * A.nb + b];
     __syncthreads();
-    const int64_t total = 2 * A.N + 2 * A.n;
-    for (int64_t item = (int64_t)blockIdx.x * kEmitThreads + threadIdx.x; item < total; item += (int64_t)gridDim.x * kEmitThreads) {
-        int64_t bd; int op, tn, rc;
-        if (emit_item(A, item, &bd, &op, &tn, &rc)) {
-            const int b = emit_bucket(A, bd);
-            const long long pos = s_base[b] + atomicAdd(&s_next[b], 1u);       // (shared memory: the block's own run of the bucket)
-            A.keys[pos] = emit_key(bd, op, tn);
-            if (rc >= 0) A.payload[pos] = rc;          // (only the few instructions that come from a plan record carry one: the
-                                                       // others' payload is never read, which spares a scattered store per tensor)
-        }
-    }
+    emit_items(A, [&](bool valid, int64_t bd, int op, int tn, int rc) {
+        const int b = emit_bucket(A, bd);
+        const unsigned at = emit_take(s_next, valid, b);                   // (shared memory: the block's own run of the bucket)
+        if (!valid) return;
+        const long long pos = s_base[b] + at;
+        A.keys[pos] = emit_key(bd, op, tn);
+        if (rc >= 0) A.payload[pos] = rc;          // (only the few instructions that come from a plan record carry one: the
+                                                   // others' payload is never read, which spares a scattered store per tensor)
+    });
 }
 
 // bitonic network over (key, payload) pairs; arbitrary n (values only ever move up)
@@ -336,23 +381,36 @@ __global__ void __launch_bounds__(kEmitThreads, 2) k_emit_write(EmitArgs A, int6
         {
             const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
             ull *st = s_stage + warp * (4 * kEmitStageStride);
-            for (int j0 = 0; j0 < n; j0 += kEmitThreads) {
-                const int j = j0 + threadIdx.x;
+            constexpr int kBatch = 4;                                      // rounds whose sizes and times are read together
+            for (int j1 = 0; j1 < n; j1 += kBatch * kEmitThreads) {
+            ull size[kBatch];
+            int64_t when[kBatch];
+#pragma unroll
+            for (int u = 0; u < kBatch; ++u) {
+                const int j = j1 + u * kEmitThreads + threadIdx.x;
+                const bool in = j < n && base + j < inst_cap;
+                const ull key = in ? kp[j] : 0;
+                size[u] = in ? (ull)A.bytes[key & 0x7fffffffu] : 0;
+                when[u] = in ? A.start[key >> 33] : 0;
+            }
+#pragma unroll
+            for (int u = 0; u < kBatch; ++u) {
+                const int j0 = j1 + u * kEmitThreads, j = j0 + threadIdx.x;
+                if (j0 >= n) break;
                 ull w0 = 0, w1 = 0, w2 = 0, w3 = 0;
                 if (j < n && base + j < inst_cap) {
                     const ull key = kp[j];
-                    const int64_t boundary = (int64_t)(key >> 33);
                     const int opcode = (int)((key >> 31) & 3u), tensor = (int)(key & 0x7fffffffu), record = (opcode & 1) ? pp[j] : -1;
                     int target = -1;
-                    int64_t time_ns = A.start[boundary];
+                    int64_t time_ns = when[u];
                     if (opcode == kOpPreEvict) { target = A.mig[record].dest; time_ns = A.mig[record].evict_issue_ns; }
                     if (opcode == kOpPrefetch) {
                         time_ns = A.new_issue ? A.new_issue[record] : A.mig[record].prefetch_issue_ns;
-                        if (time_ns >= A.start[A.K]) time_ns -= A.start[A.K];      // (steady-state plans: see emit_item)
+                        if (time_ns >= A.start[A.K]) time_ns -= A.start[A.K];      // (steady-state plans: see emit_record)
                     }
                     w0 = (ull)(unsigned)opcode | ((ull)(unsigned)tensor << 32);
                     w1 = (ull)(unsigned)target | ((ull)(unsigned)record << 32);
-                    w2 = (ull)A.bytes[tensor];
+                    w2 = size[u];
                     w3 = (ull)time_ns;
                 }
                 st[0 * kEmitStageStride + lane] = w0; st[1 * kEmitStageStride + lane] = w1;
@@ -369,6 +427,7 @@ __global__ void __launch_bounds__(kEmitThreads, 2) k_emit_write(EmitArgs A, int6
                     if ((i >> 2) < nrec) dst[i] = st[(i & 3) * kEmitStageStride + (i >> 2)];
                 }
                 __syncwarp();
+            }
             }
         }
     }
@@ -406,14 +465,14 @@ cudaError_t launch_emit(const EmitLaunch &L, cudaStream_t s)
     const int sms = current_sm_count();
     if (sms <= 0) return cudaErrorInvalidDevice;
     if (!emit_choose_buckets(L.K, 2 * L.N + 2 * L.n, sms, &A.bw, &A.nb, &A.magic)) return cudaErrorInvalidValue;
-    const int64_t total = 2 * L.N + 2 * L.n;
+    const int64_t total = L.N + 2 * L.n;
     int64_t g = (total + kEmitThreads - 1) / kEmitThreads;
     if (g > 4 * (int64_t)sms) g = 4 * (int64_t)sms;
     if (g > kEmitMaxBlocks) g = kEmitMaxBlocks;
     if (g < 1) g = 1;
     A.block_count = L.block_count; A.G = (int)g;
     k_emit_hist<<<(int)g, kEmitThreads, sizeof(unsigned) * (size_t)A.nb, s>>>(A); count_launch();
-    k_emit_block_offsets<<<(A.nb + kEmitThreads / 32 - 1) / (kEmitThreads / 32), kEmitThreads, 0, s>>>(A); count_launch();
+    k_emit_block_offsets<<<(A.nb + 31) / 32, kOffWarps * 32, 0, s>>>(A); count_launch();
     const size_t sm2 = sizeof(long long) * (size_t)(A.nb + 1) + sizeof(unsigned) * (size_t)A.nb;
     cudaError_t e2 = cudaFuncSetAttribute(k_emit_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2);
     if (e2 != cudaSuccess) return e2;

@@ -437,9 +437,10 @@ constexpr unsigned kPpGaveUp = 0xffffffffu;       // (in place of a record's wor
 
 // Visiting order by counting: the position of a record is the number of records that come before it -- earlier
 // moment of the prefetch inside the iteration, or the same moment and a lower index.  Every (record, record) pair is
-// compared once, by a grid of blocks that each hold one run of 2048 keys in shared memory: for the few ten thousand
+// compared once, by a grid of blocks that each hold one run of 256 keys in shared memory (2000 records: 64 blocks, 6 us; with runs
+// of 2048 keys 8 blocks were at it for 28 us): for the few ten thousand
 // records of a plan this is a few microseconds of the whole GPU, where a sorting network in one block takes hundreds.
-constexpr int kRankNT = 256, kRankChunk = 2048;
+constexpr int kRankNT = 256, kRankChunk = 256;
 __global__ void __launch_bounds__(kRankNT) k_pf_rank(int64_t n, const g10_migration *__restrict__ mig, const int64_t *__restrict__ start,
                                                     int64_t K, unsigned *rank)
 {
@@ -598,38 +599,46 @@ __global__ void __launch_bounds__(NT) k_pf_pipe(int64_t K, int64_t n, int L, con
         // ---- their visits, one after the other
         int e = 0;
         while (e < cnt) {
-            unsigned st = s_st[e];
-            if (st == 1u) { ++e; continue; }
+            unsigned st;
+            {                                                    // (finished ones are passed over 32 at a time)
+                const unsigned v = e + lane < cnt ? s_st[e + lane] : 1u, open = __ballot_sync(0xffffffffu, v != 1u);
+                if (open == 0u) { e += 32; continue; }
+                const int skip = __ffs(open) - 1;
+                st = __shfl_sync(0xffffffffu, v, skip);
+                e += skip;
+            }
             const int q = s_lq[e], ua = s_la[e], ub = s_lb[e];
             const bool own = ub < s1;
             if (!own && st != here) {
-                // under way when last polled: poll this one and those behind it again, all at once
+                // under way when last polled: one warp waits for it, and watches those behind it meanwhile (when this one is
+                // settled, so are usually the next few: one trip to the L2 instead of one for each)
                 __syncthreads();                                 // (every thread has read s_st[e])
-                for (int x = e + (int)threadIdx.x; x < cnt; x += NT)
-                    if (s_lb[x] >= s1 && s_st[x] != 1u) s_st[x] = ld_relaxed_u32(&w.word[s_lq[x]]);
-                __syncthreads();
-                st = s_st[e];
-                if (st != 1u && st != here) {                    // still under way: thread 0 waits for it
-                    __syncthreads();
-                    if (threadIdx.x == 0) {
-                        const ull t0 = global_timer_ns();
-                        unsigned polls = 0, v;
-                        while (true) {
-                            v = ld_relaxed_u32(&w.word[q]);
-                            if (v == 1u || v == here) break;
-                            // (every so often: out of time, or another block has given up -- then this wait is in vain too)
-                            if ((++polls & 255u) == 0u && (global_timer_ns() - t0 > wait_ns || *(volatile ull *)w.status != 0)) {
-                                raise_status(w.status, G10_DEV_TIMEOUT);
-                                v = kPpGaveUp;
+                if (warp == 0) {
+                    const int x = e + lane;
+                    bool under_way = x < cnt && s_lb[x] >= s1 && s_st[x] != 1u && s_st[x] != here;
+                    const unsigned *at = &w.word[s_lq[x < cnt ? x : e]];
+                    ull t0 = 0;
+                    unsigned polls = 0;
+                    while (true) {
+                        if (under_way) {
+                            const unsigned v = ld_relaxed_u32(at);
+                            if (v == 1u || v == here) { s_st[x] = v; under_way = false; }
+                        }
+                        if (!(__ballot_sync(0xffffffffu, under_way) & 1u)) break;
+                        // (every so often: out of time, or another block has given up -- then this wait is in vain too)
+                        if ((++polls & 255u) == 0u) {
+                            const ull now = global_timer_ns();
+                            if (t0 == 0) t0 = now;
+                            if (__any_sync(0xffffffffu, now - t0 > wait_ns || *(volatile ull *)w.status != 0)) {
+                                if (lane == 0) { raise_status(w.status, G10_DEV_TIMEOUT); s_st[e] = kPpGaveUp; }
                                 break;
                             }
                         }
-                        s_st[e] = v;
                     }
-                    __syncthreads();
-                    st = s_st[e];
-                    if (st == kPpGaveUp) { dead = true; break; }
                 }
+                __syncthreads();
+                st = s_st[e];
+                if (st == kPpGaveUp) { dead = true; break; }
                 if (st == 1u) { ++e; continue; }
             }
             // ---- the record is this block's to visit
