@@ -1,23 +1,25 @@
-// Algorithm 1 for long timelines whose state fits the shared memory of the whole GPU (about 150 SMs, 30 MB: a million slots and a
+// Algorithm 1 for long timelines whose state fits the shared memory of the whole GPU (148 SMs, 32 MB: a million slots and a
 // million periods): the lazy evaluation of g10_planner_lazy.cu with every piece of hot state in some SM's shared memory.
-//   - The timeline is cut into tiles of 64 slots, tile t in block t mod G: pressure above capacity and duration per slot; smallest
-//     and largest value, a pending offset and the total duration per tile.  A range of slots, however long, is thus spread evenly
-//     over all blocks, and so are the tiles that have to be read slot by slot, which cluster where the pressure is near capacity.
-//   - Runs of 32 periods are dealt out the same way.  A period is 16 bytes: rounded score, inactive and absent slots, destination,
-//     and whether the score is FRESH (exact) or a bound (pressure only falls, so an earlier score is one).
+//   - The timeline is cut into tiles of 64 slots, tile t in block t mod G: pressure above capacity per slot; smallest and largest
+//     value, a pending offset and the total duration per tile.  A range of slots, however long, is thus spread evenly over all
+//     blocks, and so are the tiles near capacity, which cluster.
+//   - Period p is kept by block p mod G, in 16 bytes: rounded score, inactive and absent slots, destination, and whether the score is
+//     FRESH (exact) or a bound (pressure only falls, so an earlier score is one).
 // Per iteration:
 //  A  every block applies the last commit to its tiles, compares its periods with it (absent ranges that meet: no longer FRESH;
 //     transfer windows on the same channel that meet: is the destination still possible?  Channels only fill up: SSD -> host ->
-//     erased) and publishes its best FRESH score and its four best bounds; grid barrier;
+//     erased) and publishes its best FRESH score and its eight best bounds; grid barrier;
 //  R  rounds: the published bounds that may beat the best exact score are rescored by all blocks together, each over its own
 //     tiles, with the shares added into grid-wide sums; grid barrier; the best exact score is updated.  A block whose published
 //     bounds are used up while the last may still beat the best score publishes more;
 //  D  no bound left that may beat it: commit.
 // All decisions are taken from data every block has, so the control flow is the same in every block.  Rounded scores steer the
 // search; anything within kNear of a decision is settled by exact 128-bit comparison.
-// What bounds it: grid barriers (three to four an iteration) and waiting in them for the block with the most to rescore.
-// With slots and periods in global memory (g10_planner_lazy.cu) an iteration on a million kernels read 140 MB through the L2: 1.02 s for its plan,
-// 0.90 s here (200 k kernels: 1.4 to 1.5 times faster).
+// What bounds it: a chain of block-wide phases, 62 k cycles an iteration on a million kernels (pass over the periods 14 k, rescoring
+// 20 k in 1.45 rounds of 230 periods each, choice of what to rescore 8 k, 2.7 grid barriers 15 k with the wait for the slowest block).
+// With slots and periods in global memory (g10_planner_lazy.cu) an iteration there read 140 MB through the L2: 1.02 s for the plan,
+// 0.45 s here.  Durations are read from global memory when a tile is sorted or a range's end scored: in
+// shared memory they cost 4 bytes a slot and saved nothing.
 #include "g10_planner.cuh"
 
 namespace g10 {
@@ -27,7 +29,10 @@ constexpr int kSpRound = 512;                   // periods rescored together, at
 constexpr int kSpEdge = 2 * kSpRound;           // pairs in which the period covers the tile in part
 constexpr int kSpSort = 12;                     // tiles sorted together (one warp each; a round has about four in a block)
 constexpr int kSpDirect = 2 * kPlanWarps;       // up to this many (period, tile) pairs are read slot by slot rather than sorted
-constexpr float kFirst = 0.97f;
+constexpr float kFirst = 0.97f;                 // the first round takes bounds down to this share of the best one (0.6 to 0.998: the same time)
+// Bounds below kLikely of the lowest of the last kSpPast winners are not listed at first.  (Scores go up and down from winner to winner:
+// with the last one alone every third iteration had to publish again, with four every hundredth; eight winners or 0.6 list more than
+// they spare.)
 constexpr float kLikely = 0.8f;
 constexpr int kSpPast = 4;
 constexpr double kNear = 1e-6;                  // (scores are kept as floats, rounded up: 2^-23)
@@ -135,7 +140,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
     __shared__ int s_ti[kSpTop], s_cnt[kPlanWarps];
     constexpr int kChunks = (kSpPool + kPlanThreads - 1) / kPlanThreads;        // entries of the pool a thread looks at
     __shared__ Cand s_fin[32];
-    __shared__ int s_nfin, s_nmid, s_nedge, s_wcnt[kChunks * kPlanWarps];
+    __shared__ int s_nfin, s_nmid, s_nedge;
     __shared__ Cand s_one;
     __shared__ ull s_full[32];                                                  // [group of 32 tiles]
     __shared__ unsigned char s_refresh[kLazyMaxBlocks];
@@ -229,8 +234,8 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
     else if (__ldcg(S.flag) != 0u) return;                   // (nothing changed: the planner queued behind this one takes over)
 
     struct { int idx, dest, a, ap, bp, b; int64_t s, t, t_r, t_end; } w = {-1, -1, 0, 0, -1, -1, 0, 0, 0, 0};     // the pending commit
-    unsigned likely = 0;                                     // bounds below this (four fifths of the last winner's score) are not listed at first
-    float last_key = 0.0f, won[kSpPast] = {};                // the last winner's score; lowest and those of the last few
+    unsigned likely = 0;                                     // bounds below this are not listed at first
+    float last_key = 0.0f, won[kSpPast] = {};                // the last winner's score, and those of the last few
     bool pending = false;
     Cand gBest;                                              // best exactly scored period known to the grid
     gBest.ben = 0; gBest.cost = 1; gBest.idx = -1; gBest.dest = -1;
@@ -466,12 +471,13 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
         if (__syncthreads_count(near) <= 1) return s_one;    // (nobody: thread 0's, which is none)
         return block_best_fast(x, &s_best, s_cand);
     };
+    unsigned best_bound = 0;                                 // the largest published bound of the iteration
     // Reads publications of buffer `buf` into the pool of bounds (all, or those of the blocks that published again); returns the best
     // exactly scored one, and whether anything is above capacity.
     auto load = [&](int buf, bool only_flagged, bool *over) {
         Cand x;
         x.ben = 0; x.cost = 1; x.idx = -1; x.dest = -1;
-        unsigned key = 0;
+        unsigned key = 0, bound = 0;
         bool above = false;
         for (int j = tid; j < G; j += kPlanThreads) {        // (G <= kPlanThreads: one block's values per thread)
             if (only_flagged && !s_refresh[j]) continue;
@@ -481,10 +487,16 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
             for (int q = 0; q < (int)sizeof(SpProp) / 16; ++q) u.v[q] = __ldcg(src + q);
             if (u.o.idx >= 0) { x.ben = ((u128)u.o.ben_hi << 64) | u.o.ben_lo; x.cost = u.o.cost; x.idx = u.o.idx >> 1; x.dest = u.o.idx & 1; key = u.o.key; }
             above = u.o.peak > 0;
+            bound = u.o.skey[0];
 #pragma unroll
             for (int q = 0; q < kSpTop; ++q) { pkey[q * G + j] = u.o.skey[q]; pidx[q * G + j] = u.o.sidx[q]; pdone[q * G + j] = 0; }
         }
-        if (over != nullptr) *over = __syncthreads_or(above) != 0;
+        if (over != nullptr) {
+            bound = __reduce_max_sync(0xffffffffu, bound);
+            if (lane == 0) s_wm[warp] = bound;
+            *over = __syncthreads_or(above) != 0;
+            best_bound = __reduce_max_sync(0xffffffffu, lane < kPlanWarps ? s_wm[lane] : 0u);
+        }
         const Cand b = best_of(x, key);
         __syncthreads();
         return b;
@@ -553,54 +565,38 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
 #pragma unroll 1
         for (;;) {
             const SpBar bar = sp_bar(gBest);
-            // which published bounds are rescored now (the same choice in every block, in publication order): every unused one that
-            // may beat the best exact score -- in the first round only those within 10 % of the best bound (the winner is usually
+            // which published bounds are rescored now (the same choice in every block, in the same order): every unused one that
+            // may beat the best exact score -- in the first round only those near the best bound (kFirst; the winner is usually
             // among them, and a strong exact score spares the rest)
-            int msel = 0;
+            int msel;
             {
-                unsigned k = 0;                               // the best unused bound
-                for (int e = tid; e < n_pool; e += kPlanThreads) if (!pdone[e] && pidx[e] >= 0 && pkey[e] > k) k = pkey[e];
-                k = __reduce_max_sync(0xffffffffu, k);
-                if (lane == 0) s_fk[warp] = k;
-                __syncthreads();
-                k = __reduce_max_sync(0xffffffffu, lane < kPlanWarps ? s_fk[lane] : 0u);
-                if (k >= bar.lo) {
-                    const unsigned floor0 = round_no == 0 ? __float_as_uint(fminf(__uint_as_float(k), last_key > 0.0f ? last_key : __uint_as_float(k)) * kFirst) : 0u;
-                    unsigned took = 0;                        // (bit j: the thread's j-th entry)
-                    int j = 0;
-                    for (int e0 = 0; e0 < n_pool; e0 += kPlanThreads, ++j) {
-                        const int e = e0 + tid;
-                        bool take = false;
-                        if (e < n_pool && !pdone[e] && pidx[e] >= 0 && pkey[e] >= floor0) {
-                            take = sp_may_beat(S, pidx[e] >> 1, pkey[e], bar, gBest);
-                            if (!take) pdone[e] = 2;
-                        }
-                        const unsigned mk = __ballot_sync(0xffffffffu, take);
-                        if (take) took |= 1u << j;
-                        if (lane == 0) s_wcnt[j * kPlanWarps + warp] = __popc(mk);
-                    }
-                    const int n_cnt = j * kPlanWarps;
-                    __syncthreads();
-                    // entries taken before this warp's, chunk by chunk (every warp adds them up for itself)
-                    for (int x = 0, y = 0; x < n_cnt; x += 32, y += 2) {
-                        const int v = x + lane < n_cnt ? s_wcnt[x + lane] : 0;
-                        int incl = v;
+                const unsigned floor0 = round_no == 0 ? __float_as_uint(fminf(__uint_as_float(best_bound), last_key > 0.0f ? last_key : __uint_as_float(best_bound)) * kFirst) : 0u;
+                int mine = 0, at[kChunks];                    // the warp's, and for each of the thread's entries those before it in the warp (-1: not taken)
 #pragma unroll
-                        for (int o = 1; o < 32; o <<= 1) { const int z = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += z; }
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            if (y + h >= j) break;
-                            const int before = msel + __shfl_sync(0xffffffffu, incl - v, h * kPlanWarps + warp);
-                            const bool t = (took >> (y + h) & 1u) != 0u;
-                            const int pos = before + __popc(__ballot_sync(0xffffffffu, t) & ((1u << lane) - 1u));
-                            const int e = (y + h) * kPlanThreads + tid;
-                            if (t && pos < kSpRound) { r_e[pos] = e; pdone[e] = 1; }      // (beyond the cap: next round)
-                        }
-                        msel += __shfl_sync(0xffffffffu, incl, 31);
+                for (int j = 0; j < kChunks; ++j) {
+                    const int e = j * kPlanThreads + tid;
+                    bool take = false;
+                    if (e < n_pool && !pdone[e] && pidx[e] >= 0 && pkey[e] >= floor0) {
+                        take = sp_may_beat(S, pidx[e] >> 1, pkey[e], bar, gBest);
+                        if (!take) pdone[e] = 2;
                     }
-                    msel = msel < kSpRound ? msel : kSpRound;
-                    __syncthreads();
+                    const unsigned mk = __ballot_sync(0xffffffffu, take);
+                    at[j] = take ? mine + __popc(mk & ((1u << lane) - 1u)) : -1;
+                    mine += __popc(mk);
                 }
+                if (lane == 0) s_cnt[warp] = mine;
+                __syncthreads();
+                const int v = lane < kPlanWarps ? s_cnt[lane] : 0;
+                int incl = v;
+#pragma unroll
+                for (int o = 1; o < kPlanWarps; o <<= 1) { const int z = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += z; }
+                const int before = __shfl_sync(0xffffffffu, incl - v, warp);
+                msel = __shfl_sync(0xffffffffu, incl, kPlanWarps - 1);
+#pragma unroll
+                for (int j = 0; j < kChunks; ++j)
+                    if (at[j] >= 0 && before + at[j] < kSpRound) { const int e = j * kPlanThreads + tid; r_e[before + at[j]] = e; pdone[e] = 1; }      // (beyond the cap: next round)
+                msel = msel < kSpRound ? msel : kSpRound;
+                __syncthreads();
             }
             if (msel == 0) {
                 if (round_no == 0) round_no = 1;
