@@ -70,6 +70,15 @@ __device__ __forceinline__ void small_add64(long long *p, long long v)
     if (up) atomicAdd(&w[1], up);
 }
 
+// Largest value of the lanes and its lowest slot (slot < 0: the lane has none), in every lane.
+__device__ __forceinline__ void small_peak(long long &mx, int &sl)
+{
+    const unsigned hi = sl >= 0 ? (unsigned)((ull)mx >> 32) ^ 0x80000000u : 0u, lo = sl >= 0 ? (unsigned)mx : 0u;
+    const unsigned mh = __reduce_max_sync(0xffffffffu, hi), ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
+    const unsigned s = __reduce_min_sync(0xffffffffu, sl >= 0 && hi == mh && lo == ml ? (unsigned)sl : 0xffffffffu);
+    mx = (long long)((ull)(mh ^ 0x80000000u) << 32 | ml); sl = (int)s;              // (all ones: -1)
+}
+
 // Bitonic sort of n entries by `nt` threads (a warp or the block); arbitrary n: the network only moves values up.
 template <bool kBlock>
 __device__ void small_sort(u16 *a, int n, int me, int nt)
@@ -127,22 +136,44 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(SmallArgs A)
     const bool clock = A.start != nullptr;
     unsigned bad = 0;
 
-    // ---- tensor ids, durations, kernels of the events
+    // ---- tensor ids, durations, kernels of the events.  The first batch of all three arrays (all of them, up to 4096 kernels and
+    // 16 384 events) is on its way before anything is used: one round trip instead of three -- a microsecond each from a cold L2,
+    // 1.5 from host memory.  (All loads of a batch before the first use: the stores in between would keep the compiler from it.)
+    constexpr int kIn = 4;
+    const int E4 = ((uintptr_t)A.t.kernel_tensors & 15) == 0 ? E / 4 : 0;        // events taken four at a time
+    long long dur[kIn];
+    int4 ids[kIn];
+    int64_t first[kIn], next[kIn];
+    auto load_dur = [&](int k0) {
+#pragma unroll
+        for (int q = 0; q < kIn; ++q) dur[q] = k0 + q * kSmThreads < K ? A.t.kernel_ns[k0 + q * kSmThreads] : 1;
+    };
+    auto load_ids = [&](int e0) {
+#pragma unroll
+        for (int q = 0; q < kIn; ++q) ids[q] = e0 + q * kSmThreads < E4 ? reinterpret_cast<const int4 *>(A.t.kernel_tensors)[e0 + q * kSmThreads] : make_int4(0, 0, 0, 0);
+    };
+    auto load_ptr = [&](int k0) {                   // (k0: of the warp's first lane)
+#pragma unroll
+        for (int q = 0; q < kIn; ++q) {
+            const int k = k0 + q * kSmThreads + lane;
+            first[q] = k <= K ? A.t.kernel_ptr[k] : E;
+            next[q] = lane == 31 && k < K ? A.t.kernel_ptr[k + 1] : E;
+        }
+    };
+    if (clock) load_dur(tid);
+    load_ids(tid);
+    load_ptr(warp * 32);
     if (tid == 0) { s_bits = 0; s_nmid = 0; s_nheavy = 0; }
 #pragma unroll 4
     for (int t = tid; t <= N; t += kSmThreads) off[t] = 0;
     __syncthreads();
-    // (loads in batches, all of a batch before the first use: the stores in between would keep the compiler from doing that, and
-    // from host memory a load takes 1.5 us)
     if (clock)
-        for (int k0 = tid; k0 < K; k0 += 4 * kSmThreads) {
-            long long d[4];
+        for (int k0 = tid; k0 < K; k0 += kIn * kSmThreads) {
+            if (k0 != tid) load_dur(k0);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) d[q] = k0 + q * kSmThreads < K ? A.t.kernel_ns[k0 + q * kSmThreads] : 1;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                if (d[q] < 1 || d[q] >= ((long long)1 << 44)) { bad |= G10_DEV_BAD_DURATION; d[q] = 1; }
-                if (k0 + q * kSmThreads < K) s_ns[k0 + q * kSmThreads] = d[q];
+            for (int q = 0; q < kIn; ++q) {
+                if (dur[q] < 1 || dur[q] >= ((long long)1 << 44)) { bad |= G10_DEV_BAD_DURATION; dur[q] = 1; }
+                if (k0 + q * kSmThreads < K) s_ns[k0 + q * kSmThreads] = dur[q];
             }
         }
     auto event = [&](int e, int id) {
@@ -150,15 +181,12 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(SmallArgs A)
         if (ok) atomicAdd(&off[id], 1u); else bad |= G10_DEV_BAD_TENSOR_ID;
         s_id[e] = ok ? (u16)id : (u16)0xffff;
     };
-    const int E4 = ((uintptr_t)A.t.kernel_tensors & 15) == 0 ? E / 4 : 0;        // events taken four at a time
-    for (int e0 = tid; e0 < E4; e0 += 4 * kSmThreads) {
-        int4 id[4];
+    for (int e0 = tid; e0 < E4; e0 += kIn * kSmThreads) {
+        if (e0 != tid) load_ids(e0);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) id[q] = e0 + q * kSmThreads < E4 ? reinterpret_cast<const int4 *>(A.t.kernel_tensors)[e0 + q * kSmThreads] : make_int4(0, 0, 0, 0);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
+        for (int q = 0; q < kIn; ++q) {
             const int e = 4 * (e0 + q * kSmThreads);
-            if (e < 4 * E4) { event(e, id[q].x); event(e + 1, id[q].y); event(e + 2, id[q].z); event(e + 3, id[q].w); }
+            if (e < 4 * E4) { event(e, ids[q].x); event(e + 1, ids[q].y); event(e + 2, ids[q].z); event(e + 3, ids[q].w); }
         }
     }
     for (int e = 4 * E4 + tid; e < E; e += kSmThreads) event(e, A.t.kernel_tensors[e]);
@@ -177,16 +205,10 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(SmallArgs A)
         __syncthreads();
     }
     // (a kernel_ptr that is no monotone map onto [0, E] leaves every tensor unused; the walk stays inside the events in any case)
-    for (int k0 = warp * 32; k0 < K; k0 += 4 * kSmThreads) {
-        int64_t first[4], next[4];
+    for (int k0 = warp * 32; k0 < K; k0 += kIn * kSmThreads) {
+        if (k0 != warp * 32) load_ptr(k0);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int k = k0 + q * kSmThreads + lane;
-            first[q] = k <= K ? A.t.kernel_ptr[k] : E;
-            next[q] = lane == 31 && k < K ? A.t.kernel_ptr[k + 1] : E;
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
+        for (int q = 0; q < kIn; ++q) {
             const int kq = k0 + q * kSmThreads, k = kq + lane;
             if (kq >= K) break;
             const int64_t p0 = first[q], down = __shfl_down_sync(0xffffffffu, first[q], 1), p1 = lane == 31 ? next[q] : down;
@@ -294,6 +316,19 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(SmallArgs A)
         if (warp == 0) { const unsigned r = small_compact_warp(seg, m, lane); if (lane == 0) dp[t] = r; }
     }
     __syncthreads();
+    // (the sizes of the first tensors are on their way meanwhile)
+    constexpr int kBook = 4;
+    long long size[kBook];
+    bool global[kBook];
+    auto load_size = [&](int t00) {
+#pragma unroll
+        for (int q = 0; q < kBook; ++q) {
+            const int t = t00 + q * kSmThreads + tid;
+            size[q] = t < N ? A.t.tensor_bytes[t] : 1;
+            global[q] = t < N && A.t.tensor_global != nullptr && A.t.tensor_global[t] != 0;
+        }
+    };
+    if (clock) load_size(0);
     // ---- offsets of every tensor's uses and periods (16 bits each: both sums are at most E)
     const unsigned total = small_prefix<unsigned>(dp, N, s_w32);
     if (tid == 0) dp[N] = total;
@@ -306,23 +341,24 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(SmallArgs A)
     const int raw = none ? 0 : (int)off[N - 1];
     const bool dense = D == raw;                    // no repeats: ks is the use list as it stands
     u16 *s_pos = s_id, *s_ten = s_krel;             // of every period: where its first use stands in ks, its tensor
-    for (int t0 = tid; t0 < N; t0 += 2 * kSmThreads) {
-        unsigned x[2], y[2];
-        int o[2], f[2], la[2];
+    constexpr int kOut = 3;                         // tensors of a thread whose tables are read together
+    for (int t0 = tid; t0 < N; t0 += kOut * kSmThreads) {
+        unsigned x[kOut], y[kOut];
+        int o[kOut], f[kOut], la[kOut];
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
+        for (int q = 0; q < kOut; ++q) {
             const int t = t0 + q * kSmThreads;
             const bool in = t < N;
             x[q] = in ? dp[t] : 0u; y[q] = in ? dp[t + 1] : 0u;
             o[q] = in && t > 0 ? (int)off[t - 1] : 0;
         }
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
+        for (int q = 0; q < kOut; ++q) {
             const int d = (int)((y[q] - x[q]) & 0xffffu);
             f[q] = d > 0 ? (int)ks[o[q]] : -1; la[q] = d > 0 ? (int)ks[o[q] + d - 1] : -1;
         }
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
+        for (int q = 0; q < kOut; ++q) {
             const int t = t0 + q * kSmThreads;
             if (t >= N) break;
             const int d = (int)((y[q] - x[q]) & 0xffffu), uo = (int)(x[q] & 0xffffu), p0 = (int)(x[q] >> 16);
@@ -352,21 +388,10 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(SmallArgs A)
         // ---- pressure: sizes where the tensors are born and where they die, prefix sum, peak and its lowest slot
         long long everywhere = 0;                   // bytes of the global tensors
         int wrap_base = PC;
-        const uint8_t *glob = A.t.tensor_global;
-        constexpr int kBook = 4;
+        for (int k = tid; k <= K; k += kSmThreads) s_diff[k] = 0;
+        __syncthreads();
         for (int t00 = 0; t00 < N; t00 += kBook * kSmThreads) {
-            long long size[kBook];
-            bool global[kBook];
-#pragma unroll
-            for (int q = 0; q < kBook; ++q) {
-                const int t = t00 + q * kSmThreads + tid;
-                size[q] = t < N ? A.t.tensor_bytes[t] : 1;
-                global[q] = t < N && glob != nullptr && glob[t] != 0;
-            }
-            if (t00 == 0) {                         // (cleared while the first sizes come in)
-                for (int k = tid; k <= K; k += kSmThreads) s_diff[k] = 0;
-                __syncthreads();
-            }
+            if (t00 != 0) load_size(t00);
 #pragma unroll
             for (int q = 0; q < kBook; ++q) {
                 const int t = t00 + q * kSmThreads + tid;
@@ -414,12 +439,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(SmallArgs A)
             s_diff[k] = run;
             if (sl < 0 || run > mx) { mx = run; sl = k; }
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const long long ym = __shfl_down_sync(0xffffffffu, mx, o);
-            const int ys = __shfl_down_sync(0xffffffffu, sl, o);
-            if (ys >= 0 && (sl < 0 || ym > mx || (ym == mx && ys < sl))) { mx = ym; sl = ys; }
-        }
+        small_peak(mx, sl);
         __syncthreads();
         if (lane == 0) { s_w64[warp] = mx; s_sl[warp] = sl; }
 #pragma unroll 4
@@ -427,12 +447,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(SmallArgs A)
         __syncthreads();
         if (warp == 0) {
             mx = s_w64[lane]; sl = s_sl[lane];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const long long ym = __shfl_down_sync(0xffffffffu, mx, o);
-                const int ys = __shfl_down_sync(0xffffffffu, sl, o);
-                if (ys >= 0 && (sl < 0 || ym > mx || (ym == mx && ys < sl))) { mx = ym; sl = ys; }
-            }
+            small_peak(mx, sl);
             if (lane == 0) { *A.peak_bytes = mx; *A.peak_slot = sl; }
         }
     }
