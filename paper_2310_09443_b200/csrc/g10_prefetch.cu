@@ -86,8 +86,12 @@ template <int kPfThreads>
 __global__ void __launch_bounds__(kPfThreads) k_schedule_prefetch(int64_t K, int64_t n, const g10_migration *__restrict__ mig,
                                                                   const int64_t *__restrict__ start, const int64_t *__restrict__ bytes,
                                                                   int64_t cap, int64_t *P, int32_t *order, int32_t *new_last,
-                                                                  int64_t *new_issue, int64_t *summary, int p_in_smem, int sort_in_smem)
+                                                                  int64_t *new_issue, int64_t *summary, int p_in_smem, int sort_in_smem,
+                                                                  const unsigned *only_if, int presorted)
 {
+    // (launched behind the many-block form, which leaves the records alone and sets *only_if when they need this one;
+    // `order` is then already there)
+    if (only_if != nullptr && *only_if == 0u) return;
     extern __shared__ long long s_dyn[];   // the pressure curve, when the launch gave it room
     __shared__ int s_wstop[2][kPfThreads / 32];   // per warp: smallest offset below hi of a slot of the current chunk that cannot take the tensor;
                                                   // two copies used in turn, so that one barrier per chunk is enough
@@ -105,7 +109,7 @@ __global__ void __launch_bounds__(kPfThreads) k_schedule_prefetch(int64_t K, int
     int64_t n2 = 1;
     while (n2 < n) n2 <<= 1;
     const int64_t T = K > 0 ? start[K] : 1;
-    pf_order_records(n, n2, mig, order, s_dyn + (p_in_smem ? K : 0), sort_in_smem, kPfThreads, T);
+    if (!presorted) pf_order_records(n, n2, mig, order, s_dyn + (p_in_smem ? K : 0), sort_in_smem, kPfThreads, T);
     // ---- visit the records in that order, a batch of kPfThreads at a time: the batch's fields are fetched together
     // (one thread per record), the visits read them from shared memory; the pressure curve sits in shared memory
     // too when it fits (Pw), else in global memory
@@ -433,6 +437,7 @@ __global__ void __launch_bounds__(kPfNT) k_schedule_prefetch_tiled(int64_t K, in
 // ---------------------------------------------------------------------------------------------
 constexpr int kPpBatch = 512;                    // records fetched together
 constexpr int kPpResults = 256;                  // finished records a block keeps before it writes them out
+constexpr int64_t kPfLeastSlice = 64;            // slots (short timelines: 256 took 118 us where 64 takes 89)
 constexpr unsigned kPpGaveUp = 0xffffffffu;       // (in place of a record's word: the wait for it ran out)
 
 // Visiting order by counting: the position of a record is the number of records that come before it -- earlier
@@ -785,7 +790,7 @@ static bool pf_pipe_geometry(int64_t K, int *blocks, int *slice, int *per_sm_out
         int64_t G = (int64_t)sms * per_sm;
         if (G > kPfMaxBlocks) continue;
         int64_t L = ((K + G - 1) / G + 31) / 32 * 32;
-        if (L < 256) L = 256;
+        if (L < kPfLeastSlice) L = kPfLeastSlice;
         G = (K + L - 1) / L;
         const size_t dyn = (size_t)L * 8;
         if (dyn > 200 * 1024) continue;
@@ -816,21 +821,15 @@ cudaError_t launch_schedule_prefetch(int64_t K, int64_t n, const g10_migration *
     int sort_smem = 0;
     if (n > 0 && (size_t)n2 * 12 <= 64 * 1024) { dyn += (size_t)n2 * 12; sort_smem = 1; }
     const int64_t tiles = (K + kPfTile - 1) / kPfTile;
-    if (in_smem || n == 0) {
-        if (dyn > 0) {
-            const cudaError_t e = cudaFuncSetAttribute(k_schedule_prefetch<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-            if (e != cudaSuccess) return e;
-        }
-        k_schedule_prefetch<256><<<1, 256, dyn, s>>>(K, n, mig, start, bytes, cap, P, order, new_last, new_issue, summary, in_smem, sort_smem); count_launch();
-        return cudaGetLastError();
-    }
     int G = 0, L = 0, per_sm = 0;
     const unsigned *only_if = nullptr;
     int presorted = 0;
     // (the visiting order by counting compares all pairs of records: fine for the tens of thousands of a plan, too slow
     // far beyond that)
     constexpr int64_t kPfMaxRanked = 262144;
-    if (scratch.word != nullptr && n <= kPfMaxRanked && tiles <= kPfMaxTiles && pf_pipe_geometry(K, &G, &L, &per_sm)) {
+    // (Timelines of four slices and more: a one-block pass takes 0.6 us a record.  Prefetch pass and emission of 200 / 300 / 1000 /
+    // 2794 / 15 300 kernels: 82 / 103 / 205 / 283 / 504 us with one block, 84 / 76 / 95 / 88 / 97 us with slices.)
+    if (scratch.word != nullptr && n > 0 && n <= kPfMaxRanked && K >= 4 * kPfLeastSlice && tiles <= kPfMaxTiles && pf_pipe_geometry(K, &G, &L, &per_sm)) {
         // many blocks, one slice of the timeline each; behind them the one-block form, which runs only if the records ask for it
         k_pf_rank<<<dim3((unsigned)((n + kRankNT - 1) / kRankNT), (unsigned)((n + kRankChunk - 1) / kRankChunk)), kRankNT, 0, s>>>(n, mig, start, K, scratch.rank); count_launch();
         k_pf_prepare<<<(unsigned)((n + kRankNT - 1) / kRankNT), kRankNT, 0, s>>>(K, n, mig, bytes, order, scratch, summary); count_launch();
@@ -848,6 +847,14 @@ cudaError_t launch_schedule_prefetch(int64_t K, int64_t n, const g10_migration *
         only_if = scratch.fallback;
         presorted = 1;
     }
+    if (in_smem || n == 0) {
+        if (dyn > 0) {
+            const cudaError_t e = cudaFuncSetAttribute(k_schedule_prefetch<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+            if (e != cudaSuccess) return e;
+        }
+        k_schedule_prefetch<256><<<1, 256, dyn, s>>>(K, n, mig, start, bytes, cap, P, order, new_last, new_issue, summary, in_smem, sort_smem, only_if, presorted); count_launch();
+        return cudaGetLastError();
+    }
     if (tiles <= kPfMaxTiles) {
         sort_smem = (!presorted && (size_t)n2 * 12 + (size_t)tiles * 16 <= 200 * 1024) ? 1 : 0;   // (this kernel has most of the SM's shared memory to itself)
         dyn = (sort_smem ? ((size_t)n2 * 12 + 7) / 8 * 8 : 0) + (size_t)tiles * 16;
@@ -859,7 +866,7 @@ cudaError_t launch_schedule_prefetch(int64_t K, int64_t n, const g10_migration *
             const cudaError_t e = cudaFuncSetAttribute(k_schedule_prefetch<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
             if (e != cudaSuccess) return e;
         }
-        k_schedule_prefetch<1024><<<1, 1024, dyn, s>>>(K, n, mig, start, bytes, cap, P, order, new_last, new_issue, summary, in_smem, sort_smem); count_launch();
+        k_schedule_prefetch<1024><<<1, 1024, dyn, s>>>(K, n, mig, start, bytes, cap, P, order, new_last, new_issue, summary, in_smem, sort_smem, nullptr, 0); count_launch();
     }
     return cudaGetLastError();
 }

@@ -834,6 +834,18 @@ def test_prefetch_pass_in_slices(gpu, oracle):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("K,n", [(255, 30), (256, 30), (257, 300), (319, 1), (2000, 700), (9473, 500), (15360, 900)])
+def test_prefetch_short_timelines(gpu, oracle, K, n):
+    """The sliced pass on timelines that one block could hold: below and at four slices of 64 slots, a ragged last slice, more
+    records than a batch; records that wrap, which the one-block form behind it takes."""
+    rng = np.random.default_rng(K + n)
+    for wrap in (False, True):
+        mig, start, nbytes, P = synthetic_prefetch_records(gpu, rng, K, n, wrap=wrap, long_share=0.3)
+        for cap in (int(1 << 22), 0, int(1 << 62)):
+            check_prefetch_records(gpu, oracle, K, mig, start, nbytes, cap, P)
+
+
+@pytest.mark.gpu
 def test_cyclic_planning(gpu, oracle):
     import json, os, torch
     ex = json.load(open(os.path.join(os.path.dirname(__file__), "golden", "cyclic_example.json")))
