@@ -180,7 +180,7 @@ int32_t check_ws(int32_t which, const g10_trace *t, void *ws, size_t ws_bytes)
 // Prepares the workspace and returns the device view of the trace (staging it first in host mode).
 enum { kZeroCounts = 1, kZeroDiff = 2, kZeroState = 4, kZeroPairs = 8, kZeroDiffPoint = 16, kZeroNothing = 32 };
 
-int32_t begin_call(int32_t which, const g10_trace *t, void *ws, Workspace &w, DeviceTrace &d, cudaStream_t s, int zero_mask)
+int32_t begin_call(int32_t which, const g10_trace *t, void *ws, Workspace &w, DeviceTrace &d, cudaStream_t s, int zero_mask, bool staged = false)
 {
     Sizes z{t->num_kernels, t->num_tensors, t->num_events, t->mem == G10_MEM_HOST};
     carve(ws, z, w, which);
@@ -198,12 +198,14 @@ int32_t begin_call(int32_t which, const g10_trace *t, void *ws, Workspace &w, De
         d.kernel_ptr = t->kernel_ptr; d.kernel_tensors = t->kernel_tensors; d.tensor_bytes = t->tensor_bytes;
         d.kernel_ns = t->kernel_ns; d.tensor_global = t->tensor_global;
     } else {
+        if (!staged) {                                     // (staged: the caller brings the arrays in itself)
         CU(cudaMemcpyAsync(w.s_kernel_ptr, t->kernel_ptr, sizeof(int64_t) * (size_t)(z.K + 1), cudaMemcpyHostToDevice, s));
         if (z.E) CU(cudaMemcpyAsync(w.s_kernel_tensors, t->kernel_tensors, sizeof(int32_t) * (size_t)z.E, cudaMemcpyHostToDevice, s));
         if (z.N) CU(cudaMemcpyAsync(w.s_tensor_bytes, t->tensor_bytes, sizeof(int64_t) * (size_t)z.N, cudaMemcpyHostToDevice, s));
         if (z.K) CU(cudaMemcpyAsync(w.s_kernel_ns, t->kernel_ns, sizeof(int64_t) * (size_t)z.K, cudaMemcpyHostToDevice, s));
         if (z.N && t->tensor_global)
             CU(cudaMemcpyAsync(w.s_tensor_global, t->tensor_global, (size_t)z.N, cudaMemcpyHostToDevice, s));
+        }
         d.kernel_ptr = w.s_kernel_ptr; d.kernel_tensors = w.s_kernel_tensors; d.tensor_bytes = w.s_tensor_bytes;
         d.kernel_ns = w.s_kernel_ns; d.tensor_global = t->tensor_global ? w.s_tensor_global : nullptr;
     }
@@ -251,6 +253,60 @@ bool pinned_small(const g10_trace *t, const g10_vitality_out *out, SmallArgs &A)
     if (!ok) return false;
     A.status_counts = A.v.counts + 2;
     return true;
+}
+
+// Arrays that one kernel copies between pinned host memory and the workspace.
+struct CopyList {
+    const void *src[16];
+    void *dst[16];
+    int64_t bytes[16];               // (with `count`: the most)
+    const int64_t *count[16];        // not null: how many 4-byte elements there are is on the device
+    int first[17];                   // first block of each array
+    int n;
+};
+// Up to this many events the kernel copies (trace and results of 12 k / 37 k / 100 k / 200 k kernels through host pointers: 205 / 278 /
+// 516 / 922 us with the copy engine, 114 / 200 / 438 / 892 so); beyond, the copy engine (1 M kernels, 5 M events: 4.40 ms against 4.64).
+constexpr int64_t kDirectMost = (int64_t)1 << 20;
+constexpr int kCopyThreads = 256, kCopyItems = 4, kCopyChunk = kCopyThreads * kCopyItems * 16;
+
+// A block per 16 KB, four 16-byte accesses of a thread on their way together.  A trace of 37 k kernels and its results are 19 arrays:
+// with a copy for each, and a wait in the middle because the host had to know the number of uses, they took longer than the kernels.
+__global__ void __launch_bounds__(kCopyThreads) k_copy_list(CopyList L)
+{
+    int a = 0;
+    while (a + 1 < L.n && (int)blockIdx.x >= L.first[a + 1]) ++a;
+    int64_t bytes = L.bytes[a];
+    if (L.count[a] != nullptr) { const int64_t c = *L.count[a] * 4; bytes = c < bytes ? c : bytes; }
+    const int64_t lo = (int64_t)((int)blockIdx.x - L.first[a]) * kCopyChunk, hi = lo + kCopyChunk < bytes ? lo + kCopyChunk : bytes;
+    const char *src = (const char *)L.src[a];
+    char *dst = (char *)L.dst[a];
+    int64_t at = lo;
+    if ((((uintptr_t)src | (uintptr_t)dst) & 15) == 0) {
+        const int64_t whole = hi > lo ? (hi - lo) / 16 : 0;
+        uint4 v[kCopyItems];
+#pragma unroll
+        for (int q = 0; q < kCopyItems; ++q) { const int64_t i = threadIdx.x + q * kCopyThreads; if (i < whole) v[q] = ((const uint4 *)(src + lo))[i]; }
+#pragma unroll
+        for (int q = 0; q < kCopyItems; ++q) { const int64_t i = threadIdx.x + q * kCopyThreads; if (i < whole) ((uint4 *)(dst + lo))[i] = v[q]; }
+        at += whole * 16;
+    }
+    for (int64_t i = at + threadIdx.x; i < hi; i += kCopyThreads) dst[i] = src[i];
+}
+
+void copy_add(CopyList &L, const void *src, void *dst, size_t bytes, const int64_t *count = nullptr)
+{
+    if (bytes == 0 || src == nullptr || dst == nullptr) return;
+    if (L.n == 0) L.first[0] = 0;
+    L.src[L.n] = src; L.dst[L.n] = dst; L.bytes[L.n] = (int64_t)bytes; L.count[L.n] = count;
+    L.first[L.n + 1] = L.first[L.n] + (int)((bytes + kCopyChunk - 1) / kCopyChunk);
+    L.n += 1;
+}
+
+cudaError_t copy_launch(const CopyList &L, cudaStream_t s)
+{
+    if (L.n == 0) return cudaSuccess;
+    k_copy_list<<<L.first[L.n], kCopyThreads, 0, s>>>(L); count_launch();
+    return cudaGetLastError();
 }
 
 // The analysis of a planner call in one launch, into the workspace (pressure: where the planner wants it).
@@ -389,11 +445,22 @@ int32_t g10_vitality(const g10_trace *trace, g10_vitality_out *out, void *ws, si
     }
     Workspace w;
     DeviceTrace d;
+    SmallArgs P;                                           // (host trace: the device's addresses of its arrays, if all are pinned)
+    const bool direct = trace->mem == G10_MEM_HOST && trace->num_events > 0 && trace->num_events <= kDirectMost && pinned_small(trace, out, P);
     const bool buckets = vitality_buckets_supported(trace->num_tensors, trace->num_events);
     // (bucketed formulation with the timeline: its counting kernel clears the difference array and the point masses itself)
-    rc = begin_call(wsk, trace, ws, w, d, s, (buckets ? 0 : kZeroCounts) | (to && !buckets ? kZeroDiffPoint : 0));
+    rc = begin_call(wsk, trace, ws, w, d, s, (buckets ? 0 : kZeroCounts) | (to && !buckets ? kZeroDiffPoint : 0), direct);
     if (rc != G10_OK) return rc;
     const bool host = trace->mem == G10_MEM_HOST;
+    if (direct) {
+        CopyList in{};
+        copy_add(in, P.t.kernel_ptr, w.s_kernel_ptr, sizeof(int64_t) * (size_t)(d.K + 1));
+        copy_add(in, P.t.kernel_tensors, w.s_kernel_tensors, sizeof(int32_t) * (size_t)d.E);
+        copy_add(in, P.t.tensor_bytes, w.s_tensor_bytes, sizeof(int64_t) * (size_t)d.N);
+        copy_add(in, P.t.kernel_ns, w.s_kernel_ns, sizeof(int64_t) * (size_t)d.K);
+        copy_add(in, P.t.tensor_global, w.s_tensor_global, (size_t)d.N);
+        CU(copy_launch(in, s));
+    }
     VitalityBuffers vb;
     if (!host) {
         vb = VitalityBuffers{out->first_use, out->last_use, out->num_uses, out->use_ptr, out->uses, out->uses_cap, out->period_ptr,
@@ -422,7 +489,29 @@ int32_t g10_vitality(const g10_trace *trace, g10_vitality_out *out, void *ws, si
         CU(launch_publish_status(w, vb.counts + 2, s));
         if (to) CU(launch_timeline_given(d, w, tl_start, vb.first_use, vb.last_use, w.tl_point, tl_P, tl_pk, tl_ps, tl_st, s));
     }
-    if (host) {
+    if (direct) {
+        const size_t N = (size_t)d.N;
+        CopyList o{};
+        copy_add(o, w.first_use, P.v.first_use, sizeof(int32_t) * N);
+        copy_add(o, w.last_use, P.v.last_use, sizeof(int32_t) * N);
+        copy_add(o, w.num_uses, P.v.num_uses, sizeof(int32_t) * N);
+        copy_add(o, w.use_ptr, P.v.use_ptr, sizeof(int64_t) * (N + 1));
+        copy_add(o, w.period_ptr, P.v.period_ptr, sizeof(int64_t) * (N + 1));
+        copy_add(o, w.uses, P.v.uses, sizeof(int32_t) * (size_t)vb.uses_cap, w.counts);
+        copy_add(o, w.period_tensor, P.v.period_tensor, sizeof(int32_t) * (size_t)vb.periods_cap, w.counts + 1);
+        copy_add(o, w.period_prev_use, P.v.period_prev_use, sizeof(int32_t) * (size_t)vb.periods_cap, w.counts + 1);
+        copy_add(o, w.period_next_use, P.v.period_next_use, sizeof(int32_t) * (size_t)vb.periods_cap, w.counts + 1);
+        copy_add(o, w.counts, P.v.counts, 3 * sizeof(int64_t));
+        if (to) {
+            copy_add(o, w.start, P.start, sizeof(int64_t) * (size_t)(d.K + 1));
+            copy_add(o, w.pressure, P.pressure, sizeof(int64_t) * (size_t)d.K);
+            copy_add(o, w.peak_bytes, P.peak_bytes, sizeof(int64_t));
+            copy_add(o, w.peak_slot, P.peak_slot, sizeof(int32_t));
+            copy_add(o, w.counts + 3, P.status_timeline, sizeof(int64_t));
+        }
+        CU(copy_launch(o, s));
+        CU(cudaStreamSynchronize(s));
+    } else if (host) {
         int64_t counts[3];
         CU(cudaMemcpyAsync(counts, w.counts, sizeof(counts), cudaMemcpyDeviceToHost, s));
         CU(cudaStreamSynchronize(s));

@@ -982,6 +982,34 @@ def test_on_chip_planner_edges(gpu, oracle, K, chains):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("K,N,E", [(2047, 301, 65536), (2048, 4096, 69632), (33001, 70001, 200003)])
+def test_host_analysis_middle_sizes(gpu, K, N, E):
+    """Traces in pinned host memory that do not fit one SM: arrays of whole and ragged 16 KB pieces, few and many uses and periods,
+    an output array that is not 16-byte aligned, one that is too small; the device call's results bit for bit (pageable too)."""
+    rng = np.random.default_rng(K + N)
+    ptr = np.sort(np.concatenate([[0, E], rng.integers(0, E + 1, size=K - 1)])).astype(np.int64)
+    tr = traces.Trace(name="edges", kernel_ptr=ptr, kernel_tensors=rng.integers(0, N, size=E).astype(np.int32),
+                      tensor_bytes=rng.integers(1, 1 << 39, size=N).astype(np.int64), kernel_ns=rng.integers(1, 1 << 20, size=K).astype(np.int64),
+                      tensor_global=(rng.random(N) < 0.3).astype(np.uint8), capacity_frac=(1, 2))
+    ref = gpu.g10_vitality(gpu.upload(tr), timeline=True)
+    nu, npd = int(ref.counts[0].item()), int(ref.counts[1].item())
+    pinned = gpu.pin(tr)
+    pageable = gpu.TraceBuffers(*(t.clone() for t in (pinned.kernel_ptr, pinned.kernel_tensors, pinned.tensor_bytes, pinned.kernel_ns, pinned.tensor_global)))
+    for host, cap in ((pinned, None), (pageable, None), (pinned, npd - 5)):
+        first = gpu.g10_vitality(host, timeline=True, periods_cap=cap)
+        first.last_use = first.last_use.new_empty(N + 1).pin_memory()[1:]
+        h = gpu.g10_vitality(host, timeline=first.timeline, out=first, periods_cap=cap)
+        m = npd if cap is None else cap
+        for a, b, n in ((h.first_use, ref.first_use, N), (h.last_use, ref.last_use, N), (h.num_uses, ref.num_uses, N), (h.use_ptr, ref.use_ptr, N + 1),
+                        (h.uses, ref.uses, nu), (h.period_ptr, ref.period_ptr, N + 1), (h.period_tensor, ref.period_tensor, m),
+                        (h.period_prev_use, ref.period_prev_use, m), (h.period_next_use, ref.period_next_use, m), (h.counts, ref.counts, 2),
+                        (h.timeline.pressure, ref.timeline.pressure, K), (h.timeline.kernel_start_ns, ref.timeline.kernel_start_ns, K + 1),
+                        (h.timeline.peak_bytes, ref.timeline.peak_bytes, 1), (h.timeline.peak_slot, ref.timeline.peak_slot, 1)):
+            assert np.array_equal(a[:n].numpy(), _np(b)[:n])
+        assert int(h.counts[2]) == int(h.timeline.status[0]) == (0 if cap is None else 0x20)
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("K,n,ns", [(1, 8, 1 << 20), (63, 300, 1 << 20), (64, 3000, 1 << 12), (65, 3000, 1 << 20), (9471, 400, 1 << 20),
                                     (9473, 3000, 1 << 10), (19000, 200, 1 << 25), (300, 400, 1 << 27)])
 def test_spread_planner_edges(gpu, oracle, K, n, ns):
