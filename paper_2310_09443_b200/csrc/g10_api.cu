@@ -352,6 +352,7 @@ size_t carve_prefetch(void *base, int64_t n, PrefetchScratch &p, size_t *zero_by
     p.size = c.take<int64_t>((size_t)n);
     p.block_max = c.take<int64_t>(kPfMaxBlocks);
     p.block_slot = c.take<int32_t>(kPfMaxBlocks);
+    p.slice_max = c.take<int64_t>(kPfMaxBlocks);
     return align_up(c.off);
 }
 

@@ -240,6 +240,7 @@ struct PrefetchScratch {
     int64_t *size;            // [n] tensor size in visiting order
     int64_t *block_max;       // [kPfMaxBlocks] largest pressure of each block's slice ...
     int32_t *block_slot;      // [kPfMaxBlocks] ... and its lowest slot
+    int64_t *slice_max;       // [kPfMaxBlocks] largest pressure of each block's slice before the pass
 };
 cudaError_t launch_schedule_prefetch(int64_t K, int64_t n, const g10_migration *mig, const int64_t *start, const int64_t *bytes,
                                      uint64_t gpu_capacity_bytes, int64_t *P, int32_t *order, int32_t *new_last, int64_t *new_issue,

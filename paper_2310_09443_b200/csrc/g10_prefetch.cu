@@ -467,13 +467,28 @@ __global__ void __launch_bounds__(kRankNT) k_pf_rank(int64_t n, const g10_migrat
     if (c) atomicAdd(&rank[i], c);
 }
 
-// The records' fields, in visiting order, for every block of the pass.
-__global__ void __launch_bounds__(kRankNT) k_pf_prepare(int64_t K, int64_t n, const g10_migration *__restrict__ mig,
+// The records' fields, in visiting order, for every block of the pass; the blocks behind those take the largest pressure of a slice
+// of L slots each.
+__global__ void __launch_bounds__(kRankNT) k_pf_prepare(int64_t K, int64_t n, int L, const int64_t *__restrict__ P, const g10_migration *__restrict__ mig,
                                                         const int64_t *__restrict__ bytes, int32_t *order, PrefetchScratch w,
                                                         int64_t *summary)
 {
     const int64_t i = (int64_t)blockIdx.x * kRankNT + threadIdx.x;
     if (blockIdx.x == 0 && threadIdx.x < 5) summary[threadIdx.x] = 0;
+    if (const int64_t b = (int64_t)blockIdx.x - (n + kRankNT - 1) / kRankNT; b >= 0) {
+        __shared__ long long s_m[kRankNT / 32];
+        long long m = -0x7fffffffffffffffll - 1;
+        for (int64_t k = b * L + threadIdx.x; k < (b + 1) * L && k < K; k += kRankNT) m = P[k] > m ? P[k] : m;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) { const long long x = __shfl_xor_sync(0xffffffffu, m, o); m = x > m ? x : m; }
+        if ((threadIdx.x & 31) == 0) s_m[threadIdx.x >> 5] = m;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int x = 1; x < kRankNT / 32; ++x) m = s_m[x] > m ? s_m[x] : m;
+            w.slice_max[b] = m;
+        }
+        return;
+    }
     if (i >= n) return;
     const unsigned q = w.rank[i];
     const int a = mig[i].absent_first, b = mig[i].absent_last;
@@ -491,6 +506,9 @@ __global__ void __launch_bounds__(kRankNT) k_pf_prepare(int64_t K, int64_t n, co
 // Where the records of a batch stand is polled for the whole batch at a time (a thread per record) and kept in shared
 // memory; "finished" never changes again, so the walk skips such records without touching global memory and polls again
 // only when it comes to a record that was still under way at the last poll.
+// Pressure only rises in this pass: a slice that held a slot too full for a record before the pass never lets it through.  A block
+// therefore leaves out every record that such a slice keeps away from it (`beyond`: running maxima of the slices to its right)
+// instead of waiting to hear that its search has ended (200 k kernels, 2000 records, with the emission: 222 -> 199 us).
 template <int NT>
 __global__ void __launch_bounds__(NT) k_pf_pipe(int64_t K, int64_t n, int L, const g10_migration *__restrict__ mig,
                                                 const int64_t *__restrict__ start, int64_t cap, int64_t *P,
@@ -502,10 +520,12 @@ __global__ void __launch_bounds__(NT) k_pf_pipe(int64_t K, int64_t n, int L, con
     // test build: block `hook - 1` keeps every record it should hand over or finish to itself, and waits last a millisecond
     const bool mute = hook != 0 && (int)blockIdx.x == hook - 1;
     const ull wait_ns = hook != 0 ? 1000000ull : kBarrierTimeoutNs;
+    const bool all_ways = hook == 0;             // (else every record is waited for)
 #else
     (void)hook;
     constexpr bool mute = false;
     constexpr ull wait_ns = kBarrierTimeoutNs;
+    constexpr bool all_ways = true;
 #endif
     extern __shared__ long long Ps[];            // this block's slice of the pressure curve (raw values)
     __shared__ int s_lq[kPpBatch], s_la[kPpBatch], s_lb[kPpBatch];      // the batch's records that concern this block, in order
@@ -524,6 +544,24 @@ __global__ void __launch_bounds__(NT) k_pf_pipe(int64_t K, int64_t n, int L, con
     const int s0 = b * L, s1 = (int)((int64_t)(b + 1) * L < K ? (int64_t)(b + 1) * L : K);   // slice [s0, s1)
     const unsigned here = 2u + (unsigned)b;
     long long off = 0, rmax = -0x7fffffffffffffffll - 1;
+    long long *beyond = Ps + L;                  // [G] largest of slices (b, c], for c > b
+    {
+        const int cnt = G - 1 - b, per = (cnt + NT - 1) / NT, x0 = (int)threadIdx.x * per < cnt ? (int)threadIdx.x * per : cnt, x1 = x0 + per < cnt ? x0 + per : cnt;
+        for (int x = threadIdx.x; x < cnt; x += NT) beyond[b + 1 + x] = w.slice_max[b + 1 + x];
+        __syncthreads();
+        long long m = rmax;
+        for (int x = x0; x < x1; ++x) m = beyond[b + 1 + x] > m ? beyond[b + 1 + x] : m;
+        long long incl = m;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const long long y = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o && y > incl) incl = y; }
+        if (lane == 31) s_wmax[warp] = incl;
+        m = __shfl_up_sync(0xffffffffu, incl, 1);
+        if (lane == 0) m = rmax;
+        __syncthreads();
+        for (int x = 0; x < warp; ++x) m = s_wmax[x] > m ? s_wmax[x] : m;
+        for (int x = x0; x < x1; ++x) { const long long v = beyond[b + 1 + x]; m = v > m ? v : m; beyond[b + 1 + x] = m; }
+        __syncthreads();
+    }
     {
         long long m = rmax;
         for (int k = s0 + (int)threadIdx.x; k < s1; k += NT) { const long long v = P[k]; Ps[k - s0] = v; m = v > m ? v : m; }
@@ -573,8 +611,12 @@ __global__ void __launch_bounds__(NT) k_pf_pipe(int64_t K, int64_t n, int L, con
             if (keep[u]) {
                 qs[u] = w.size[q];
                 if (qb[u] >= s1) {
-                    qw[u] = ld_relaxed_u32(&w.word[q]);
-                    if (qw[u] == 1u) keep[u] = false;            // finished before it came here
+                    const int c = qb[u] / L - 1;                 // the slices up to this one it has to cross whole
+                    if (c > b && all_ways && beyond[c] > cap - qs[u]) keep[u] = false;
+                    else {
+                        qw[u] = ld_relaxed_u32(&w.word[q]);
+                        if (qw[u] == 1u) keep[u] = false;        // finished before it came here
+                    }
                 }
             }
         }
@@ -775,11 +817,22 @@ __global__ void __launch_bounds__(NT) k_pf_pipe(int64_t K, int64_t n, int L, con
 
 // Blocks, block width and slice length of the many-block form for a timeline of K slots, or false if no choice keeps
 // every slice in shared memory with all blocks resident at once (the blocks wait for one another: a cooperative launch).
-// Many short slices are tried first (four blocks per SM measured fastest on the stress trace: a visit that has to look at
+// Many short slices are tried first (pf_slice: a visit that has to look at
 // the slots costs time in proportion to the slice, a hand-over to the next block only a round trip through the L2).
 static const void *pf_pipe_kernel(int per_sm)
 {
     return per_sm == 1 ? (const void *)k_pf_pipe<512> : per_sm == 2 ? (const void *)k_pf_pipe<256> : (const void *)k_pf_pipe<128>;
+}
+// Slots per slice.  Short slices make a visit cheap, few slices make few hand-overs.  Measured over slices of 64 to 1024 slots and four
+// traces of each size (us, prefetch pass and emission): 64 slots are best up to 15 k kernels (101; 256 slots 116), about K / 296 for 25 k
+// to 60 k (143 and 152 at 192 slots; 155 and 171 at 64), K / 444 for 100 k to 400 k (200 k kernels: 208 at K / 592, 194 at K / 444; 400 k: 397
+// and 383), K / 592 for a million (404 and 408; with 12 000 records 884 and 931).
+static int64_t pf_slice(int64_t K, int64_t sms)
+{
+    auto share = [&](int64_t blocks) { return ((K + blocks - 1) / blocks + 31) / 32 * 32; };
+    int64_t L = share(2 * sms) < 256 ? share(2 * sms) : 256;
+    if (L < share(3 * sms)) L = share(3 * sms) <= 1024 ? share(3 * sms) : share(4 * sms);
+    return L < kPfLeastSlice ? kPfLeastSlice : L;
 }
 static bool pf_pipe_geometry(int64_t K, int *blocks, int *slice, int *per_sm_out)
 {
@@ -790,9 +843,9 @@ static bool pf_pipe_geometry(int64_t K, int *blocks, int *slice, int *per_sm_out
         int64_t G = (int64_t)sms * per_sm;
         if (G > kPfMaxBlocks) continue;
         int64_t L = ((K + G - 1) / G + 31) / 32 * 32;
-        if (L < kPfLeastSlice) L = kPfLeastSlice;
+        if (per_sm == 4) L = pf_slice(K, sms);
         G = (K + L - 1) / L;
-        const size_t dyn = (size_t)L * 8;
+        const size_t dyn = (size_t)(L + G) * 8;
         if (dyn > 200 * 1024) continue;
         const void *f = pf_pipe_kernel(per_sm);
         if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess) return false;
@@ -832,7 +885,7 @@ cudaError_t launch_schedule_prefetch(int64_t K, int64_t n, const g10_migration *
     if (scratch.word != nullptr && n > 0 && n <= kPfMaxRanked && K >= 4 * kPfLeastSlice && tiles <= kPfMaxTiles && pf_pipe_geometry(K, &G, &L, &per_sm)) {
         // many blocks, one slice of the timeline each; behind them the one-block form, which runs only if the records ask for it
         k_pf_rank<<<dim3((unsigned)((n + kRankNT - 1) / kRankNT), (unsigned)((n + kRankChunk - 1) / kRankChunk)), kRankNT, 0, s>>>(n, mig, start, K, scratch.rank); count_launch();
-        k_pf_prepare<<<(unsigned)((n + kRankNT - 1) / kRankNT), kRankNT, 0, s>>>(K, n, mig, bytes, order, scratch, summary); count_launch();
+        k_pf_prepare<<<(unsigned)((n + kRankNT - 1) / kRankNT + G), kRankNT, 0, s>>>(K, n, L, P, mig, bytes, order, scratch, summary); count_launch();
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         int Li = L;
@@ -842,7 +895,7 @@ cudaError_t launch_schedule_prefetch(int64_t K, int64_t n, const g10_migration *
         if (const char *h = getenv("G10_TEST_PREFETCH_MUTE_BLOCK")) hook = atoi(h) + 1;
 #endif
         void *args[] = {&K, &n, &Li, &mig, &start, &cap, &P, &order, &new_last, &new_issue, &summary, &w, &hook};
-        e = cudaLaunchCooperativeKernel(pf_pipe_kernel(per_sm), dim3(G), dim3(per_sm == 1 ? 512 : per_sm == 2 ? 256 : 128), args, (size_t)L * 8, s);
+        e = cudaLaunchCooperativeKernel(pf_pipe_kernel(per_sm), dim3(G), dim3(per_sm == 1 ? 512 : per_sm == 2 ? 256 : 128), args, (size_t)(L + G) * 8, s);
         if (e != cudaSuccess) return e;
         only_if = scratch.fallback;
         presorted = 1;
