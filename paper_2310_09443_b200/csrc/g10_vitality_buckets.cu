@@ -580,7 +580,7 @@ __global__ void __launch_bounds__(kBkThreads, 2) k_bk_emit(BucketArgs B, Vitalit
                 }
                 if (pending) {
                     if (++polls > kSpinLimit) { raise_status(B.status, G10_DEV_TIMEOUT); break; }
-                    __nanosleep(100);
+                    __nanosleep(20);
                 }
             }
 #pragma unroll
