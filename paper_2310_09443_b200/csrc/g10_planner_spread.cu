@@ -120,13 +120,40 @@ struct __align__(16) SpSorted {
     int n, lt, pad;
 };
 
-__host__ __device__ inline size_t sp_round16(size_t x) { return (x + 15) / 16 * 16; }
-__host__ __device__ inline size_t sp_smem(int64_t K, int64_t Pn, int G)
+// Where a block's dynamic shared memory goes: byte offsets of its arrays, and what they take together (the same function measures
+// and lays out, so that a trace is never taken on that the arrays have no room for).
+struct SpreadLayout {
+    // (tiles: of slots, a block, at most; runs: of 32 periods, likewise)
+    size_t mm;                                  // [tiles] longlong2
+    size_t hot;                                 // [runs * 32] uint4
+    size_t r_acc, r_s, r_e, r_ap, r_bp;         // a round: [kSpLimbs][kSpRound] unsigned; [kSpRound] long long, int, int, int
+    size_t edge;                                // [kSpEdge] unsigned
+    size_t sorted;                              // [kSpSort] SpSorted
+    size_t mid, full;                           // [tiles] unsigned, ull
+    size_t pkey, pidx, pdone;                   // [kSpTop * G] unsigned, int, unsigned char
+    size_t ex;                                  // [tiles * kSpTile] long long
+    size_t off, tsum;                           // [tiles] long long, unsigned
+    size_t total;
+};
+__host__ __device__ inline SpreadLayout spread_layout(int64_t K, int64_t Pn, int G)
 {
+    SpreadLayout l;
+    size_t at = 0;
+    auto take = [&](size_t bytes) { const size_t p = at; at += (bytes + 15) / 16 * 16; return p; };
     const size_t tiles = (size_t)(((K + kSpTile - 1) / kSpTile + G - 1) / G), runs = (size_t)(((Pn + G - 1) / G + 31) / 32);
-    return tiles * kSpTile * 8 + tiles * 36 + runs * 32 * 16 + kSpSort * sizeof(SpSorted) + kSpEdge * 4 +                                     // slots, tiles, periods
-           sp_round16((size_t)G * kSpTop * 4) * 2 + sp_round16((size_t)G * kSpTop) +                              // published bounds
-           (size_t)kSpRound * (4 * kSpLimbs + 8 + 3 * 4) + 128;                      // a round
+    l.mm = take(tiles * 16);
+    l.hot = take(runs * 32 * 16);
+    l.r_acc = take((size_t)kSpRound * 4 * kSpLimbs);
+    l.r_s = take((size_t)kSpRound * 8); l.r_e = take((size_t)kSpRound * 4);
+    l.r_ap = take((size_t)kSpRound * 4); l.r_bp = take((size_t)kSpRound * 4);
+    l.edge = take((size_t)kSpEdge * 4);
+    l.sorted = take(kSpSort * sizeof(SpSorted));
+    l.mid = take(tiles * 4); l.full = take(tiles * 8);
+    l.pkey = take((size_t)G * kSpTop * 4); l.pidx = take((size_t)G * kSpTop * 4); l.pdone = take((size_t)G * kSpTop);
+    l.ex = take(tiles * kSpTile * 8);
+    l.off = take(tiles * 8); l.tsum = take(tiles * 4);
+    l.total = at;
+    return l;
 }
 
 __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, SpreadArgs S)
@@ -147,29 +174,29 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
     if (*S.done) return;                                     // (same answer in every thread of the grid: written by an earlier launch)
     const int G = gridDim.x, c = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t Pn64 = *A.Pn_dev < A.geo_stride ? *A.Pn_dev : A.geo_stride;
-    if (A.K < 1 || A.K > kSpMaxSlots || Pn64 > 0x3fffffff || sp_smem(A.K, Pn64, G) > (size_t)S.smem_bytes) return;     // (the same answer in all blocks)
+    if (A.K < 1 || A.K > kSpMaxSlots || Pn64 > 0x3fffffff) return;               // (the same answer in all blocks)
+    const SpreadLayout l = spread_layout(A.K, Pn64, G);
+    if (l.total > (size_t)S.smem_bytes) return;                                 // (here too)
     const int K = (int)A.K, Pn = (int)Pn64;
     const int64_t limit = (A.max_iterations <= 0 || A.max_iterations > Pn64) ? Pn64 : A.max_iterations;
-    const int NT = (K + kSpTile - 1) / kSpTile, tiles = (NT + G - 1) / G, runs = ((Pn + G - 1) / G + 31) / 32;
+    const int NT = (K + kSpTile - 1) / kSpTile;
     const int my_tiles = NT > c ? (NT - c + G - 1) / G : 0, my_runs = Pn > c ? ((Pn - c + G - 1) / G + 31) / 32 : 0;
-    unsigned char *at = s_raw;
-    auto take = [&](size_t bytes) { unsigned char *p = at; at += sp_round16(bytes); return p; };
-    longlong2 *mm = (longlong2 *)take((size_t)tiles * 16);                      // [tiles] smallest / largest, offset included
-    uint4 *hot = (uint4 *)take((size_t)runs * 32 * 16);
-    unsigned *r_acc = (unsigned *)take((size_t)kSpRound * 4 * kSpLimbs);        // [limb][period] (sums of far fewer than 2^11 limbs)
-    long long *r_s = (long long *)take((size_t)kSpRound * 8);
-    int *r_e = (int *)take((size_t)kSpRound * 4);                               // pool entry
-    int *r_ap = (int *)take((size_t)kSpRound * 4), *r_bp = (int *)take((size_t)kSpRound * 4);
-    unsigned *s_edge = (unsigned *)take((size_t)kSpEdge * 4);      // period of the round << 20 | local tile
-    SpSorted *sorted = (SpSorted *)take(kSpSort * sizeof(SpSorted));
-    unsigned *t_mid = (unsigned *)take((size_t)tiles * 4);                      // tiles of a round that are near capacity
-    ull *t_full = (ull *)take((size_t)tiles * 8);                               // duration of the tiles of this group of 32 so far that are above it for every period of the round
-    unsigned *pkey = (unsigned *)take((size_t)G * kSpTop * 4);                 // published bounds, [rank in the list][block]
-    int *pidx = (int *)take((size_t)G * kSpTop * 4);                               // period << 1 | destination, -1 = none
-    unsigned char *pdone = take((size_t)G * kSpTop);
-    long long *ex = (long long *)take((size_t)tiles * kSpTile * 8);
-    long long *off = (long long *)take((size_t)tiles * 8);
-    unsigned *tsum = (unsigned *)take((size_t)tiles * 4);
+    longlong2 *mm = (longlong2 *)(s_raw + l.mm);                                // [tiles] smallest / largest, offset included
+    uint4 *hot = (uint4 *)(s_raw + l.hot);
+    unsigned *r_acc = (unsigned *)(s_raw + l.r_acc);                            // [limb][period] (sums of far fewer than 2^11 limbs)
+    long long *r_s = (long long *)(s_raw + l.r_s);
+    int *r_e = (int *)(s_raw + l.r_e);                                          // pool entry
+    int *r_ap = (int *)(s_raw + l.r_ap), *r_bp = (int *)(s_raw + l.r_bp);
+    unsigned *s_edge = (unsigned *)(s_raw + l.edge);                            // period of the round << 20 | local tile
+    SpSorted *sorted = (SpSorted *)(s_raw + l.sorted);
+    unsigned *t_mid = (unsigned *)(s_raw + l.mid);                              // tiles of a round that are near capacity
+    ull *t_full = (ull *)(s_raw + l.full);                                      // duration of the tiles of this group of 32 so far that are above it for every period of the round
+    unsigned *pkey = (unsigned *)(s_raw + l.pkey);                              // published bounds, [rank in the list][block]
+    int *pidx = (int *)(s_raw + l.pidx);                                        // period << 1 | destination, -1 = none
+    unsigned char *pdone = s_raw + l.pdone;
+    long long *ex = (long long *)(s_raw + l.ex);
+    long long *off = (long long *)(s_raw + l.off);
+    unsigned *tsum = (unsigned *)(s_raw + l.tsum);
     auto owner_entry = [&](int p) { return p % G == c ? p / G : -1; };
 
     unsigned gen = 0;
@@ -887,7 +914,7 @@ static int spread_budget()
 bool plan_spread_possible(int64_t K, int64_t E)
 {
     const int G = current_sm_count(), budget = spread_budget();
-    return G > 0 && G <= kLazyMaxBlocks && G <= kPlanThreads && K >= 1 && K <= kSpMaxSlots && E >= 1 && budget > 0 && sp_smem(K, E < 4096 ? E : 4096, G) <= (size_t)budget;
+    return G > 0 && G <= kLazyMaxBlocks && G <= kPlanThreads && K >= 1 && K <= kSpMaxSlots && E >= 1 && budget > 0 && spread_layout(K, E < 4096 ? E : 4096, G).total <= (size_t)budget;
 }
 
 cudaError_t launch_plan_spread(const PlanArgs &A_in, const Workspace &w, cudaStream_t s)
@@ -900,5 +927,17 @@ cudaError_t launch_plan_spread(const PlanArgs &A_in, const Workspace &w, cudaStr
     void *args[] = {&A, &S};
     return cudaLaunchCooperativeKernel((const void *)k_plan_spread, dim3(current_sm_count()), dim3(kPlanThreads), args, (size_t)S.smem_bytes, s);
 }
+
+#ifdef G10_TEST_HOOKS
+// What the tests want to know of the layout: offsets of the arrays in the order of the struct, then the total.
+extern "C" int32_t g10_test_spread_layout(int64_t K, int64_t Pn, int32_t G, int64_t *out /* [18] */)
+{
+    const SpreadLayout l = spread_layout(K, Pn, G);
+    const size_t v[] = {l.mm, l.hot, l.r_acc, l.r_s, l.r_e, l.r_ap, l.r_bp, l.edge, l.sorted, l.mid, l.full, l.pkey, l.pidx, l.pdone, l.ex, l.off, l.tsum, l.total};
+    for (int j = 0; j < 18; ++j) out[j] = (int64_t)v[j];
+    return (int32_t)sizeof(SpSorted);
+}
+extern "C" int32_t g10_test_spread_budget(void) { return spread_budget(); }
+#endif
 
 }  // namespace g10

@@ -1055,3 +1055,42 @@ def test_one_launch_analysis_edges(gpu, oracle, K, N, E):
                         (h.timeline.pressure, ref.timeline.pressure, K), (h.timeline.kernel_start_ns, ref.timeline.kernel_start_ns, K + 1),
                         (h.timeline.peak_bytes, ref.timeline.peak_bytes, 1), (h.timeline.status, ref.timeline.status, 1)):
             assert np.array_equal(a[:n].numpy(), _np(b)[:n])
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("K", [1_000_000, 961_000])
+def test_spread_planner_fills_shared_memory(gpu, oracle, K):
+    """The longest traces that the planner spread over all SMs takes, and the first that it leaves to the planner behind it: as
+    many periods as fit every block's shared memory, and one run of 32 more in every block.  Each tensor is used by two kernels.
+    The first iterations bit for bit against the oracle."""
+    import ctypes as C
+    import torch
+    from paper_2310_09443_b200 import build
+    hooks = C.CDLL(build.build(hooks=True))
+    hooks.g10_test_spread_layout.argtypes = [C.c_int64, C.c_int64, C.c_int32, C.POINTER(C.c_int64)]
+    G = torch.cuda.get_device_properties(0).multi_processor_count
+    room = hooks.g10_test_spread_budget()
+    out = (C.c_int64 * 18)()
+
+    def need(periods):
+        hooks.g10_test_spread_layout(K, periods, G, out)
+        return out[17]
+
+    runs = 1
+    while need((runs + 1) * 32 * G) <= room:
+        runs += 1
+    rng = np.random.default_rng(K)
+    for n in (runs * 32 * G, (runs + 1) * 32 * G):
+        assert (need(n) <= room) == (n == runs * 32 * G)
+        u = rng.integers(0, K - 48, size=n)
+        v = u + rng.integers(2, 48, size=n)
+        k, t = np.concatenate([u, v]), np.concatenate([np.arange(n), np.arange(n)])
+        at = np.lexsort((t, k))
+        tr = traces.Trace(name="full", kernel_ptr=np.searchsorted(k[at], np.arange(K + 1)).astype(np.int64), kernel_tensors=t[at].astype(np.int32),
+                          tensor_bytes=rng.integers(1 << 16, 1 << 24, size=n).astype(np.int64), kernel_ns=rng.integers(50_000, 500_000, size=K).astype(np.int64),
+                          tensor_global=np.zeros(n, np.uint8), capacity_frac=(1, 2))
+        start, P0, peak, slot = oracle.timeline(tr)
+        cap = tr.capacity_from_peak(peak)
+        ref = oracle.plan(tr, cap, lazy=True, max_iterations=12)
+        assert len(ref.migrations) == 12
+        check_plan(gpu, tr, gpu.upload(tr), cap, ref, max_iterations=12)
