@@ -176,11 +176,14 @@ typedef struct g10_options {
                                        iteration (Algorithm 1 as printed), use lists built with global atomics
                                        instead of shared-memory buckets; identical results, slower           */
 
-#define G10_FLAG_GLOBAL_STATE 0x2   /* keep the planner state in global memory even when the timeline would fit
-                                       in shared memory (the path large traces take); same plan              */
+#define G10_FLAG_GLOBAL_STATE 0x2   /* keep the planner state in global memory even when it would fit shared memory
+                                       (the path the largest traces take); same plan                         */
 
 #define G10_FLAG_MULTI_BLOCK 0x4    /* never let a single block run the greedy loop out of its shared memory (the path
                                        the smallest traces take); same plan                                  */
+
+#define G10_FLAG_SPREAD_STATE 0x8   /* keep the planner state in the shared memory of all SMs together even when it would
+                                       fit one thread-block cluster (the path long traces take); same plan   */
 
 #ifdef G10_TEST_HOOKS
 /* Honoured only by the test build of the library (compiled with -DG10_TEST_HOOKS, never shipped): one block of the

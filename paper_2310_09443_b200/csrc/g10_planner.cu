@@ -1,7 +1,8 @@
 // Algorithm 1 (smart tensor eviction) as printed: one persistent cooperative kernel in which every
 // iteration rescores all live inactive periods in parallel, reduces the best benefit/cost ratio across the
 // grid, commits it and tests the peak -- two grid barriers per iteration, no host round trip.  Selected by
-// G10_FLAG_RESCORE_ALL; the default planner (g10_planner_lazy.cu) gives the same plan with far less work.
+// G10_FLAG_RESCORE_ALL; the other planners give the same plan with far less work: one cluster (g10_planner_chip.cu), all SMs'
+// shared memory (g10_planner_spread.cu) or global memory (g10_planner_lazy.cu), whichever the trace fits first.
 #include "g10_planner.cuh"
 
 namespace g10 {
@@ -133,7 +134,7 @@ static int chip_blocks(int64_t E, uint32_t flags) { return plan_chip_blocks(E, (
 
 bool plan_keeps_state_on_chip(int64_t K, int64_t E, bool host_cap, uint32_t flags, bool cyclic)
 {
-    if (flags & (G10_FLAG_RESCORE_ALL | G10_FLAG_GLOBAL_STATE)) return false;
+    if (flags & (G10_FLAG_RESCORE_ALL | G10_FLAG_GLOBAL_STATE | G10_FLAG_SPREAD_STATE)) return false;
     return plan_chip_possible(K, E, chip_blocks(E, flags), host_cap, cyclic) == 2;
 }
 
@@ -187,7 +188,7 @@ cudaError_t launch_plan_loop(const DeviceTrace &t, const Workspace &w, const Pla
         void *args[] = {&A, &done};
         return cudaLaunchCooperativeKernel((const void *)k_plan_loop<false>, dim3(G), dim3(kPlanThreads), args, 0, s);
     }
-    if (!(p.flags & G10_FLAG_GLOBAL_STATE)) {
+    if (!(p.flags & (G10_FLAG_GLOBAL_STATE | G10_FLAG_SPREAD_STATE))) {
         // (as in launch_plan_cyclic)
         const int C = chip_blocks(t.E, p.flags), fits = plan_chip_possible(t.K, t.E, C, p.host_capacity_bytes != 0, false);
         if (fits) {
@@ -196,7 +197,7 @@ cudaError_t launch_plan_loop(const DeviceTrace &t, const Workspace &w, const Pla
         }
     }
     // state spread over the shared memory of all SMs if it fits (the device knows), else in global memory
-    if (plan_spread_possible(t.K, t.E)) {
+    if (!(p.flags & G10_FLAG_GLOBAL_STATE) && plan_spread_possible(t.K, t.E)) {
         const cudaError_t e = launch_plan_spread(A, w, s);
         if (e != cudaSuccess) return e;
     }

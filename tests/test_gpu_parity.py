@@ -115,8 +115,9 @@ def full_parity(gpu, oracle, tr, lazy_oracle=False, repeats=1, **plan_kw):
         check_plan(gpu, tr, tb, cap, ref, **plan_kw)
     if also:
         check_plan(gpu, tr, tb, cap, ref, flags=gpu.FLAG_RESCORE_ALL, **plan_kw)      # Algorithm 1 as printed
-        check_plan(gpu, tr, tb, cap, ref, flags=gpu.FLAG_GLOBAL_STATE, **plan_kw)     # the large-trace planner
-        check_plan(gpu, tr, tb, cap, ref, flags=gpu.FLAG_MULTI_BLOCK, **plan_kw)      # never the single-block planner
+        check_plan(gpu, tr, tb, cap, ref, flags=gpu.FLAG_GLOBAL_STATE, **plan_kw)     # the planner in global memory
+        check_plan(gpu, tr, tb, cap, ref, flags=gpu.FLAG_SPREAD_STATE, **plan_kw)     # the planner spread over all SMs
+        check_plan(gpu, tr, tb, cap, ref, flags=gpu.FLAG_MULTI_BLOCK, **plan_kw)      # never one block alone
     return ref
 
 
@@ -410,6 +411,7 @@ def test_full_size_stress_dag_passes(gpu, oracle):
     tl, (start, P0, peak, slot) = check_timeline(gpu, oracle, tr, tb)
     cap = tr.capacity_from_peak(peak)
     ref = oracle.plan(tr, cap, lazy=True, max_iterations=1000)
+    check_plan(gpu, tr, tb, cap, ref, max_iterations=1000, flags=gpu.FLAG_GLOBAL_STATE)      # (the default is the planner spread over all SMs)
     plan = check_plan(gpu, tr, tb, cap, ref, max_iterations=1000)
     helpers.check_plan_invariants(tr, cap, start, P0, ov, gpu.migrations_numpy(plan), _np(plan.final_pressure),
                                   gpu.STATUS[int(plan.summary[2].item())], tr.host_bw, tr.ssd_bw, check_area=False)
@@ -450,6 +452,11 @@ def test_full_size_stress_plan_digest(gpu):
     h = hashlib.sha256()
     h.update(mig.tobytes()); h.update(_np(plan.final_pressure)[:tr.K].tobytes()); h.update(summary[:7].tobytes())
     assert h.hexdigest() == gold["plan_sha256"]
+    # the same plan with the planner's state in global memory
+    other = gpu.g10_plan_migrations(tb, cap, tr.host_bw, tr.ssd_bw, flags=gpu.FLAG_GLOBAL_STATE)
+    torch.cuda.synchronize()
+    assert torch.equal(other.summary, plan.summary) and torch.equal(other.final_pressure, plan.final_pressure)
+    assert np.array_equal(gpu.migrations_numpy(other), mig)
     # the eager prefetch pass over the same plan
     n = int(summary[0])
     pf = gpu.g10_schedule_prefetch(tr.K, n, plan.migrations, tl.kernel_start_ns, tb.tensor_bytes, cap, plan.final_pressure)
@@ -914,7 +921,7 @@ def test_crowded_ties_and_conflicts(gpu, oracle):
         cap = tr.capacity_from_peak(peak)
         ref = oracle.plan(tr, cap, lazy=True)
         assert np.array_equal(ref.migrations, oracle.plan(tr, cap).migrations) and len(ref.migrations) > 100
-        for flags in (0, gpu.FLAG_GLOBAL_STATE, gpu.FLAG_MULTI_BLOCK, gpu.FLAG_RESCORE_ALL):
+        for flags in (0, gpu.FLAG_GLOBAL_STATE, gpu.FLAG_SPREAD_STATE, gpu.FLAG_MULTI_BLOCK, gpu.FLAG_RESCORE_ALL):
             check_plan(gpu, tr, tb, cap, ref, flags=flags)
         check_cyclic(gpu, oracle, tr, cap)
 
@@ -1028,7 +1035,8 @@ def test_spread_planner_edges(gpu, oracle, K, n, ns):
     cap = tr.capacity_from_peak(peak)
     for host in (0, 3 << 24):
         ref = oracle.plan(tr, cap, lazy=True, host_capacity_bytes=host)
-        check_plan(gpu, tr, tb, cap, ref, host_capacity=host, flags=gpu.FLAG_GLOBAL_STATE)
+        for flags in (gpu.FLAG_SPREAD_STATE, gpu.FLAG_GLOBAL_STATE):
+            check_plan(gpu, tr, tb, cap, ref, host_capacity=host, flags=flags)
 
 
 @pytest.mark.gpu
@@ -1094,3 +1102,21 @@ def test_spread_planner_fills_shared_memory(gpu, oracle, K):
         ref = oracle.plan(tr, cap, lazy=True, max_iterations=12)
         assert len(ref.migrations) == 12
         check_plan(gpu, tr, gpu.upload(tr), cap, ref, max_iterations=12)
+
+
+@pytest.mark.gpu
+def test_flags_reach_their_planners(gpu):
+    """What a flag keeps away is not launched: the planner in global memory alone; that one behind the planner spread over all
+    SMs (it returns at once if the plan is there); one cluster alone for a trace that fits it."""
+    tr = traces.config1_resnet152()
+    tb = gpu.upload(tr)
+
+    def launches(flags):
+        before = gpu.g10_launch_count()
+        gpu.g10_plan_migrations(tb, tr.capacity_bytes, tr.host_bw, tr.ssd_bw, flags=flags)
+        return gpu.g10_launch_count() - before
+
+    alone = launches(gpu.FLAG_GLOBAL_STATE)
+    assert launches(gpu.FLAG_SPREAD_STATE) == alone + 1
+    assert launches(gpu.FLAG_GLOBAL_STATE | gpu.FLAG_SPREAD_STATE) == alone
+    assert launches(0) == launches(gpu.FLAG_MULTI_BLOCK) < alone
