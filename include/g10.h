@@ -191,6 +191,9 @@ typedef struct g10_options {
    millisecond, so that the give-up path of the bounded waits can be exercised: the call returns with
    G10_DEV_TIMEOUT in summary[7].  The product build ignores the bit. */
 #define G10_FLAG_TEST_SKIP_ARRIVAL 0x40000000
+/* Likewise: one block of the grid comes 50 us late to every choice of what to rescore, so that whatever the others write
+   too early is there when it reads.  The plan is the same. */
+#define G10_FLAG_TEST_LATE_BLOCK 0x20000000
 #endif
 
 #define G10_WS_VITALITY 0

@@ -830,6 +830,10 @@ int32_t g10_plan_migrations(const g10_trace *trace, uint64_t gpu_capacity_bytes,
         static const unsigned hook = 2u;
         CU(cudaMemcpyAsync(&((GridBarrier *)w.barrier)->pad, &hook, sizeof(hook), cudaMemcpyHostToDevice, s));
     }
+    if (flags & G10_FLAG_TEST_LATE_BLOCK) {
+        static const unsigned hook = 2u;
+        for (void *b : {w.barrier, w.barrier2}) CU(cudaMemcpyAsync(&((GridBarrier *)b)->late, &hook, sizeof(hook), cudaMemcpyHostToDevice, s));
+    }
 #endif
     VitalityBuffers vb{w.first_use, w.last_use, w.num_uses, w.use_ptr, w.uses, d.E, w.period_ptr,
                        w.period_tensor, w.period_prev_use, w.period_next_use, d.E, w.counts};

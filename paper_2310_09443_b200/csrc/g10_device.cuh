@@ -246,7 +246,7 @@ __device__ __forceinline__ void period_geometry(const int64_t *start, int u, int
 // ---------------------------------------------------------------------------------------------
 struct GridBarrier {
     unsigned count;
-    unsigned unused;
+    unsigned late;                                 // (test build: this block - 1 comes late to choices)
     unsigned error;
     unsigned pad;
 };
@@ -292,6 +292,19 @@ __device__ __forceinline__ bool grid_barrier(GridBarrier *b, unsigned nblocks, u
     my_gen += 1u;
     __syncthreads();
     return s_ok != 0u;
+}
+
+// Test build: the block named by the barrier's `late` word waits 50 us (G10_FLAG_TEST_LATE_BLOCK).
+__device__ __forceinline__ void test_come_late(const GridBarrier *b)
+{
+#ifdef G10_TEST_HOOKS
+    if (blockIdx.x + 1u == *(const volatile unsigned *)&b->late) {
+        const ull t0 = global_timer_ns();
+        while (global_timer_ns() - t0 < 50000ull) __nanosleep(1000);
+    }
+#else
+    (void)b;
+#endif
 }
 
 }  // namespace g10

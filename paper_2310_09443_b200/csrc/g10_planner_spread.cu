@@ -586,7 +586,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
         }
         pending = false;
         // ---------------- R: rounds of joint rescoring
-        bool failed = false;
+        bool failed = false, compared = false;
         int round_no = 0;
         const int n_pool = G * kSpTop;
 #pragma unroll 1
@@ -596,7 +596,9 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
             // may beat the best exact score -- in the first round only those near the best bound (kFirst; the winner is usually
             // among them, and a strong exact score spares the rest)
             int msel;
+            test_come_late(A.bar);
             {
+                bool near = false;
                 const unsigned floor0 = round_no == 0 ? __float_as_uint(fminf(__uint_as_float(best_bound), last_key > 0.0f ? last_key : __uint_as_float(best_bound)) * kFirst) : 0u;
                 int mine = 0, at[kChunks];                    // the warp's, and for each of the thread's entries those before it in the warp (-1: not taken)
 #pragma unroll
@@ -605,6 +607,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
                     bool take = false;
                     if (e < n_pool && !pdone[e] && pidx[e] >= 0 && pkey[e] >= floor0) {
                         take = sp_may_beat(S, pidx[e] >> 1, pkey[e], bar, gBest);
+                        near = near || (pkey[e] >= bar.lo && pkey[e] <= bar.hi);
                         if (!take) pdone[e] = 2;
                     }
                     const unsigned mk = __ballot_sync(0xffffffffu, take);
@@ -612,7 +615,8 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
                     mine += __popc(mk);
                 }
                 if (lane == 0) s_cnt[warp] = mine;
-                __syncthreads();
+                // (other blocks' periods were compared exactly: see the barrier before the decision)
+                compared = __syncthreads_or(near) != 0;
                 const int v = lane < kPlanWarps ? s_cnt[lane] : 0;
                 int incl = v;
 #pragma unroll
@@ -852,7 +856,11 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
             __syncthreads();
         }
         if (failed) { status = -2; break; }
-        if (!barrier_since_booking) { if (!grid_barrier(A.bar, G, gen)) { status = -2; break; } }
+        // The bookings have to be there before the next pass.  And where the last choice compared other blocks' periods exactly, by the
+        // benefits and costs in global memory, nobody may restart a period (begin_period in the next pass) before all blocks have
+        // read them: a block that comes late would choose otherwise than the rest.  (`compared` is the same in all blocks: they see
+        // the same bounds and the same best score.  Rare, and a barrier is a tenth of an iteration.)
+        if (!barrier_since_booking || compared) { if (!grid_barrier(A.bar, G, gen)) { status = -2; break; } }
         // ---------------- D: decide
         if (gBest.idx < 0) { status = G10_EXHAUSTED; break; }
         {
