@@ -398,7 +398,10 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
                 }
         }
         // more bounds than the lists hold: the lowest score that at least kSpTop of them reach and the lists hold, by bisection (if too
-        // many share one score, any of those: what is not listed is no larger than what is)
+        // many share one score, any of those: what is not listed is no larger than what is).  Under a floor only bounds that may beat it
+        // count, here as above: with those that share its score but lose the exact comparison the lists could be full of bounds that
+        // nobody rescores, publication after publication.
+        auto counts = [&](uint4 q, int p) { return !(q.w & kSpFresh) && (!with_floor || sp_may_beat(S, p, q.x, bar, gBest)); };
         if (__any_sync(0xffffffffu, lane < kPlanWarps && s_cnt[lane] > kSpSeg)) {
             unsigned lo = least, hi = 0x7f800000u;                  // too many; too few (or just right, which ends the search)
             bool fits = false;
@@ -406,8 +409,8 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
             while (!fits && hi - lo > 1u) {
                 const unsigned mid = lo + (hi - lo) / 2;
                 unsigned m = 0;
-#pragma unroll 4
-                for (int r = warp; r < my_runs; r += kPlanWarps) { const uint4 q = hot[r * 32 + lane]; m += !(q.w & kSpFresh) && q.x >= mid ? 1u : 0u; }
+#pragma unroll 1
+                for (int r = warp; r < my_runs; r += kPlanWarps) { const uint4 q = hot[r * 32 + lane]; m += q.x >= mid && counts(q, (r * 32 + lane) * G + c) ? 1u : 0u; }
                 m = __reduce_add_sync(0xffffffffu, m);
                 __syncthreads();
                 if (lane == 0) s_cnt[warp] = (int)m;
@@ -423,7 +426,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
 #pragma unroll 1
                 for (int r = warp; r < my_runs; r += kPlanWarps) {
                     const uint4 q = hot[r * 32 + lane];
-                    list(!(q.w & kSpFresh) && (pass == 0 ? q.x >= hi : q.x == lo), q, (r * 32 + lane) * G + c);
+                    list((pass == 0 ? q.x >= hi : q.x == lo) && counts(q, (r * 32 + lane) * G + c), q, (r * 32 + lane) * G + c);
                 }
             __syncwarp();
             mine = lane < n ? s_seg[warp][lane] : make_uint2(0, 0);
@@ -586,7 +589,8 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
         }
         pending = false;
         // ---------------- R: rounds of joint rescoring
-        bool failed = false, compared = false;
+        // (compared: other blocks' periods, in the last choice; again_published: bounds were published again and none has been taken since)
+        bool failed = false, compared = false, again_published = false;
         int round_no = 0;
         const int n_pool = G * kSpTop;
 #pragma unroll 1
@@ -641,6 +645,8 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
                     s_refresh[tid] = again ? 1 : 0;
                 }
                 if (!__syncthreads_or(again)) break;
+                if (again_published) { failed = true; break; }       // (cannot be: what is published under a floor may beat it)
+                again_published = true;
                 if (unlikely) likely = 0;
                 if (s_refresh[c]) scan(false, true);
                 if (!grid_barrier(A.bar, G, gen)) { failed = true; break; }
@@ -650,6 +656,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
                 continue;
             }
             round_no += 1;
+            again_published = false;
             long long sz = 0;
             ull cost = 1;
             int own = -1;                                                           // the thread's period << 1 | destination

@@ -1120,3 +1120,32 @@ def test_flags_reach_their_planners(gpu):
     assert launches(gpu.FLAG_SPREAD_STATE) == alone + 1
     assert launches(gpu.FLAG_GLOBAL_STATE | gpu.FLAG_SPREAD_STATE) == alone
     assert launches(0) == launches(gpu.FLAG_MULTI_BLOCK) < alone
+
+
+@pytest.mark.gpu
+def test_more_near_ties_than_the_lists_hold(gpu, oracle):
+    """Every warp of the planner spread over all SMs keeps three runs of 32 periods of one and the same inactive period, all with
+    the same rounded score: the first run's lose the exact comparison (a transfer time that has to be rounded up), the others' win
+    it.  The lists of bounds hold 32 a warp; what is published again has to be bounds that may win, or the search would not end."""
+    import torch
+    G = torch.cuda.get_device_properties(0).multi_processor_count
+    K, n = 300, G * 16 * 3 * 32
+    rng = np.random.default_rng(8)
+    size = (1 << 33) + 16 * rng.integers(0, 1 << 18, size=n) + (np.arange(n) < G * 512)     # 16 B take 5 ns to the SSD, 1 ns to the host
+    deg = np.zeros(K, np.int64)
+    deg[2] = deg[K - 3] = n
+    tr = traces.Trace(name="ties", kernel_ptr=np.concatenate([[0], np.cumsum(deg)]), kernel_tensors=np.tile(np.arange(n, dtype=np.int32), 2),
+                      tensor_bytes=size.astype(np.int64), kernel_ns=np.full(K, 50_000_001, np.int64), tensor_global=np.zeros(n, np.uint8),
+                      host_bw=16_000_000_000, ssd_bw=3_200_000_000, capacity_frac=(1, 2))
+    tb = gpu.upload(tr)
+    start, P0, peak, slot = oracle.timeline(tr)
+    cap = tr.capacity_from_peak(peak)
+    ref = oracle.plan(tr, cap, lazy=True)
+    for m in ref.migrations:                             # (benefit / cost as the planner rounds it, upwards to a float)
+        t = -(-size * 10 ** 9 // (tr.ssd_bw, tr.host_bw)[m["dest"]])
+        ratio = size / (2.0 * t) * float(start[m["absent_last"] + 1] - start[m["absent_first"]])
+        key = ratio.astype(np.float32)
+        assert len(set(np.where(key < ratio, np.nextafter(key, np.float32(np.inf)), key).tolist())) == 1 and len(set((size / t).tolist())) > 1
+    assert ref.migrations["period"].tolist() == [G * 512, G * 512 + 1] and ref.migrations["dest"].tolist() == [0, 1]
+    for flags in (gpu.FLAG_SPREAD_STATE, gpu.FLAG_GLOBAL_STATE, gpu.FLAG_RESCORE_ALL):
+        check_plan(gpu, tr, tb, cap, ref, flags=flags)
