@@ -741,12 +741,14 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_lazy(PlanArgs A, LazyA
         }
 
         // ---------------- R: rounds of joint rescoring
-        bool failed = false;
+        bool failed = false, compared = false;
         int round_no = 0;
 #pragma unroll 1
         for (;;) {
             const double gkey = gBest.idx >= 0 ? cand_key(gBest) : -1.0;
             int msel = 0;
+            bool near = false;                                      // a bound of another block's period was compared exactly
+            test_come_late(A.bar);
             {
                 // which published bounds are rescored now (same choice in every block, in publication order):
                 // every unused one that may beat the best exact score -- in the first round of an iteration only those
@@ -768,6 +770,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_lazy(PlanArgs A, LazyA
                     bool take = false;
                     if (e < n_pool && !s_pdone[e] && s_pidx[e] >= 0 && s_pkey[e] >= floor0) {
                         take = bound_may_beat(L, s_pidx[e], s_pkey[e], gkey, &gBest);
+                        near = near || (gBest.idx >= 0 && may_beat(s_pkey[e], gBest) && s_pkey[e] <= gkey * (1.0 + 1e-10));
                         if (!take) s_pdone[e] = 4;
                     }
                     const unsigned mk = __ballot_sync(0xffffffffu, take);
@@ -791,7 +794,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_lazy(PlanArgs A, LazyA
                     s_it_cost[r] = 2ull * (ull)A.geo_t[d * A.geo_stride + p];
                 }
             }
-            __syncthreads();
+            compared = __syncthreads_or(near) != 0;
             if (msel == 0) {
                 if (round_no == 0) { round_no = 1; continue; }      // (the first round only looks at the best bounds)
                 // nothing published may beat the best score.  A block that has used all its bounds may hold more.
@@ -910,7 +913,11 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_lazy(PlanArgs A, LazyA
             __syncthreads();
         }
         if (failed) { status = -2; break; }
-        if (!barrier_since_booking) { if (!grid_barrier(A.bar, G, gen)) { status = -2; break; } }
+        // The bookings have to be there before the next pass.  And where the last choice compared other blocks' periods exactly, by the
+        // benefits and costs in global memory, nobody may re-choose a period's destination (dest_warp behind the next pass) before all
+        // blocks have read them: a block that comes late would choose otherwise than the rest.  (`compared` is the same in all
+        // blocks: they see the same bounds and the same best score.)
+        if (!barrier_since_booking || compared) { if (!grid_barrier(A.bar, G, gen)) { status = -2; break; } }
 
         // ---------------- D: decide
         if (gBest.idx < 0) { status = G10_EXHAUSTED; break; }

@@ -11,7 +11,7 @@ from paper_2310_09443_b200 import traces
 
 pytestmark = pytest.mark.gpu
 
-FLAG_SPREAD_STATE = 0x8
+FLAG_GLOBAL_STATE, FLAG_SPREAD_STATE = 0x2, 0x8
 FLAG_TEST_LATE_BLOCK = 0x20000000
 
 
@@ -29,7 +29,7 @@ def near_ties(groups=3, K=300, n=7000):
                         host_bw=16_000_000_000, ssd_bw=3_200_000_000, capacity_frac=(1, 2))
 
 
-@pytest.mark.parametrize("flags", [FLAG_SPREAD_STATE])
+@pytest.mark.parametrize("flags", [FLAG_SPREAD_STATE, FLAG_GLOBAL_STATE])
 def test_a_late_block_decides_as_the_others(oracle, flags):
     import torch
     from paper_2310_09443_b200 import binding, build
