@@ -122,6 +122,9 @@ __global__ void __launch_bounds__(kPeakThreads) __cluster_dims__(kPeakBlocks, 1,
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     auto better = [](long long m, long long a, long long &mx, long long &at) { if (m > mx || (m == mx && a < at)) { mx = m; at = a; } };
     long long mx = -1, at = kNone;
+    // (a block's shared memory may be written by others once it has started, not before: all say that they have, and wait for it
+    // where the first remote store stands)
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
     for (int64_t k0 = (int64_t)blockIdx.x * kPeakThreads + threadIdx.x; k0 < K; k0 += 8 * (int64_t)kPeakBlocks * kPeakThreads) {
         long long v[8];
@@ -137,6 +140,7 @@ __global__ void __launch_bounds__(kPeakThreads) __cluster_dims__(kPeakBlocks, 1,
     }
     if (lane == 0) { s_mx[warp] = mx; s_at[warp] = at; }
     __syncthreads();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     if (warp == 0) {
         mx = s_mx[lane]; at = s_at[lane];
 #pragma unroll

@@ -1149,3 +1149,31 @@ def test_more_near_ties_than_the_lists_hold(gpu, oracle):
     assert ref.migrations["period"].tolist() == [G * 512, G * 512 + 1] and ref.migrations["dest"].tolist() == [0, 1]
     for flags in (gpu.FLAG_SPREAD_STATE, gpu.FLAG_GLOBAL_STATE, gpu.FLAG_RESCORE_ALL):
         check_plan(gpu, tr, tb, cap, ref, flags=flags)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("K", [1, 16, 3000])
+def test_characterisation_on_a_busy_gpu(gpu, oracle, K):
+    """The maximum over the kernels is taken by a cluster whose blocks write into the first one's shared memory: they may start at
+    different times, which other work on the GPU brings about, and on a short trace the first is done at once.  Many calls beside
+    a stream full of other kernels, every one's results."""
+    import torch
+    tr = traces.random_toy(np.random.default_rng(K), K, 40, max_deg=5)
+    tb = gpu.upload(tr)
+    v = gpu.g10_vitality(tb, timeline=True)
+    Pn = int(v.counts[1].item())
+    ov = oracle.vitality(tr.kernel_ptr, tr.kernel_tensors, tr.N)
+    oc = oracle.characterize(tr.K, ov, tr.tensor_bytes, oracle.slot_clock(tr.kernel_ns), tr.host_bw, tr.ssd_bw)
+    other = torch.cuda.Stream()
+    x = torch.zeros(1 << 22, device="cuda")
+    torch.cuda.synchronize()
+    results = []
+    for _ in range(100):
+        with torch.cuda.stream(other):
+            for _ in range(3):
+                x.add_(1.0)
+        results.append(gpu.g10_characterize(tr.K, tr.N, v.use_ptr, v.uses, tb.tensor_bytes, v.timeline.kernel_start_ns, Pn, v.period_tensor,
+                                            v.period_prev_use, v.period_next_use, tr.host_bw, tr.ssd_bw))
+    torch.cuda.synchronize()
+    for st in results:
+        assert np.array_equal(_np(st.active_bytes)[:tr.K], oc.active_bytes) and np.array_equal(_np(st.summary), oc.summary)
