@@ -736,11 +736,13 @@ int32_t g10_plan_batch(const g10_trace *trace, int32_t V, const g10_variant *var
     if (out->migrations_cap < 0 || (out->migrations_cap > 0 && !out->migrations)) return G10_ERR_ARG;
     if (trace->num_kernels > 0 && !out->final_pressure) return G10_ERR_ARG;
     std::vector<BatchVariant> bv((size_t)V);
+    uint64_t most_host = 0;
     for (int32_t v = 0; v < V; ++v) {
         if (variants[v].host_bw == 0 || variants[v].ssd_bw == 0) return G10_ERR_ARG;
         bv[v].kernel_ns = variants[v].kernel_ns ? variants[v].kernel_ns : trace->kernel_ns;
         bv[v].cap = variants[v].gpu_capacity_bytes; bv[v].host_bw = variants[v].host_bw; bv[v].ssd_bw = variants[v].ssd_bw;
         bv[v].host_capacity = variants[v].host_capacity_bytes;
+        if (bv[v].host_capacity > most_host) most_host = bv[v].host_capacity;
     }
     rc = check_ws(G10_WS_BATCH, trace, ws, ws_bytes);
     if (rc != G10_OK) return rc;
@@ -755,7 +757,7 @@ int32_t g10_plan_batch(const g10_trace *trace, int32_t V, const g10_variant *var
     VitalityBuffers vb{w.first_use, w.last_use, w.num_uses, w.use_ptr, w.uses, d.E, w.period_ptr,
                        w.period_tensor, w.period_prev_use, w.period_next_use, d.E, w.counts};
     PlanParams pp;
-    pp.gpu_capacity_bytes = 0; pp.host_bw = 1; pp.ssd_bw = 1; pp.host_capacity_bytes = 0;      // per variant, on the device
+    pp.gpu_capacity_bytes = 0; pp.host_bw = 1; pp.ssd_bw = 1; pp.host_capacity_bytes = most_host;      // per variant, on the device
     pp.max_iterations = max_iterations; pp.flags = 0;
     pp.migrations = out->migrations; pp.migrations_cap = out->migrations_cap;
     pp.final_pressure = out->final_pressure; pp.summary = out->summary;

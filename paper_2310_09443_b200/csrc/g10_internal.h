@@ -75,6 +75,7 @@ struct BatchArgs {
     const BatchVariant *variants;     // [V]
     const int64_t *P0;                // [K] unplanned pressure, shared by all variants
     int64_t *P_out;                   // [V][K]
+    int host_cap;                     // some variant has finite host memory: room is asked for accordingly in all of them
 };
 constexpr int kMaxVariants = 1024;
 

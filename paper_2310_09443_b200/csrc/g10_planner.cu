@@ -145,7 +145,7 @@ cudaError_t launch_plan_variants(const DeviceTrace &t, const Workspace &w, const
     PlanArgs A;
     fill_plan_args(t, w, p, A);
     BatchArgs B;
-    B.variants = w.batch_variants; B.P0 = w.pressure; B.P_out = p.final_pressure;
+    B.variants = w.batch_variants; B.P0 = w.pressure; B.P_out = p.final_pressure; B.host_cap = p.host_capacity_bytes != 0 ? 1 : 0;
     return launch_plan_batch(A, w, V, C, B, stability, s);
 }
 

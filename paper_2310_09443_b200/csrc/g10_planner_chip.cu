@@ -353,11 +353,12 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_plan_chip(PlanArgs A, ChipA
     const bool host_cap = A.host_capacity != 0;
     unsigned dev_bits = 0;                              // device status bits of this plan
     const int64_t per_block = (Pn64 + C - 1) / C;
-    // Does it fit?  (The answer is the same in all blocks.)
+    // Does it fit?  (The answer is the same in all blocks, and in all variants of a batch: the host asks variant 0.)
+    const bool host_room = kBatch ? B.host_cap != 0 : host_cap;
     bool fits = (kCyclic ? 2 * A.K : A.K) < (int64_t)kSlotTop && per_block <= kChipMaxPeriods, busy_smem = false;
     if (fits) {
-        const size_t core = chip_smem_core(A.K, per_block, C, host_cap, kCyclic);
-        busy_smem = core + chip_smem_busy(A.K, host_cap) <= (size_t)O.smem_bytes;
+        const size_t core = chip_smem_core(A.K, per_block, C, host_room, kCyclic);
+        busy_smem = core + chip_smem_busy(A.K, host_room) <= (size_t)O.smem_bytes;
         fits = core <= (size_t)O.smem_bytes && (busy_smem || (O.busy_global && A.K <= kChipMaxSlots));
     }
     if (!fits) {
@@ -930,7 +931,7 @@ cudaError_t launch_plan_chip(const PlanArgs &A, const Workspace &w, int C, bool 
 {
     const int which = cyclic ? kOneCycle : kOnePlan;
     BatchArgs B;
-    B.variants = nullptr; B.P0 = nullptr; B.P_out = nullptr;
+    B.variants = nullptr; B.P0 = nullptr; B.P_out = nullptr; B.host_cap = 0;
     ChipArgs O = chip_args(which, w);
     O.alone = alone ? 1 : 0;
     return launch_chip(which, A, O, B, 1, C, s);

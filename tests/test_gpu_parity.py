@@ -1177,3 +1177,21 @@ def test_characterisation_on_a_busy_gpu(gpu, oracle, K):
     torch.cuda.synchronize()
     for st in results:
         assert np.array_equal(_np(st.active_bytes)[:tr.K], oc.active_bytes) and np.array_equal(_np(st.summary), oc.summary)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("K", [3600, 4200])
+def test_batch_of_mixed_host_capacities(gpu, oracle, K):
+    """Finite host memory takes two more arrays in shared memory.  At 4200 kernels a variant without it fits a cluster and one with
+    it does not: the batch as a whole is planned one after the other then, whatever variant 0 is (at 3600 all fit)."""
+    rng = np.random.default_rng(K)
+    n = 400
+    lists = [[] for _ in range(K)]
+    for i in range(n):
+        for k in sorted(set(int(x) for x in rng.integers(0, K, size=2))):
+            lists[k].append(i)
+    tr = traces.from_lists("mixed", lists, rng.integers(1 << 16, 1 << 24, size=n), rng.integers(10_000, 300_000, size=K), capacity_frac=(2, 5))
+    start, P0, peak, slot = oracle.timeline(tr)
+    base = dict(gpu_capacity_bytes=tr.capacity_from_peak(peak), host_bw=tr.host_bw, ssd_bw=tr.ssd_bw)
+    ref = check_batch(gpu, oracle, tr, [base, dict(base, host_capacity_bytes=3 << 24), dict(base, host_capacity_bytes=1 << 40)])
+    assert len(ref.plans[1].migrations) > 20
