@@ -496,6 +496,14 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_plan_chip(PlanArgs A, ChipA
 #pragma unroll 1
         for (int k = tid; k < K; k += kChipThreads) hocc[k] = 0;
     __syncthreads();                                   // (the clock is complete)
+    if (kBatch && T.start[K] >= ((int64_t)1 << 44)) {
+        // (transfer times of the periods have to fit 44 bits; a trace's own clock is checked where it is made)
+        if (tid == 0 && rank == 0) {
+            for (int j = 0; j < 7; ++j) A.summary[j] = j == 2 || j == 4 ? -1 : 0;
+            A.summary[7] = G10_DEV_BAD_DURATION;
+        }
+        return;
+    }
 #pragma unroll 1
     for (int li = tid; li < np; li += kChipThreads) {
         ckey[li] = 0; cwin[li] = make_uint2(0, 0); chost[li] = kNoRange;

@@ -707,6 +707,18 @@ def test_batched_replanning(gpu, oracle):
     torch.cuda.synchronize()
     s7 = _np(got.summary)[:, 7]
     assert s7[0] == 0 and (s7[1] & 0x8) and s7[2] == 0
+    # ... and so does one whose durations are valid but add up to 2^44 ns or more (2^44 - 1 is still planned)
+    long = np.full(tr.K, (1 << 44) // tr.K, np.int64)
+    long[0] += (1 << 44) - int(long.sum())
+    most = long.copy(); most[0] -= 1
+    got = gpu.g10_plan_batch(tb, [base] + [dict(base, kernel_ns=torch.from_numpy(ns).cuda()) for ns in (long, most, 4 * long)] + [base])
+    torch.cuda.synchronize()
+    s = _np(got.summary)
+    assert s[:, 7].tolist() == [0, 0x8, 0, 0x8, 0] and s[1, 2] == s[3, 2] == -1 and np.array_equal(s[0], s[4])
+    assert _np(got.stability)[[1, 3]].tolist() == [[-1, -1], [-1, -1]]
+    ref = oracle.plan_batch(tr, [base, dict(base, kernel_ns=most)])
+    for j, v in ((0, 0), (1, 2)):
+        assert np.array_equal(gpu.batch_migrations_numpy(got, v), ref.plans[j].migrations)
     # a trace too large for one SM: the variants are planned one after the other by the planners that use the whole GPU
     tr = traces.make_config(3)
     start, P0, peak, slot = oracle.timeline(tr)
