@@ -400,17 +400,34 @@ def g10_plan_batch(tb: TraceBuffers, variants, max_iterations=0, migrations_cap=
     return out
 
 
+_AHEAD_VARIANTS, _AHEAD_BYTES = 256, 8 << 20
+
+
 def batch_migrations_numpy(batch, v) -> np.ndarray:
-    """Committed migration records of variant v of a finished batch (synchronises).  The first call brings the records of all
-    variants over in two copies: a study reads them all, and a copy each costs some 40 us."""
-    host = getattr(batch, "_host", None)
-    if host is None:
-        counts = batch.summary[:, 0].cpu().numpy().clip(0, batch.migrations_cap)
-        most = int(counts.max()) if counts.size else 0
-        records = torch.empty((counts.size, most * 48), dtype=torch.uint8, pin_memory=True)
-        records.copy_(batch.migrations[:, : most * 48])
-        host = batch._host = (counts, records.numpy())
-    return host[1][v, : int(host[0][v]) * 48].view(MIGRATION_DTYPE).copy()
+    """Committed migration records of variant v of a finished batch (synchronises).
+
+    A study reads variant after variant, and a copy from the device costs some 50 us whatever its size: the call brings over the
+    records of the variants behind v as well (at most 8 MB) and keeps them on `batch`.  What is kept is handed out once, and only
+    while nothing can have changed the tensors since: they are the same ones, torch has not written to them and the library has
+    launched no kernel.  Asking for the same variant again reads it again."""
+    mig, summary = batch.migrations, batch.summary
+    ahead = getattr(batch, "_ahead", None)
+    if ahead is not None and ahead[0] is mig and ahead[1] is summary and ahead[2:5] == (mig._version, summary._version, _lib.g10_launch_count()):
+        found = ahead[5].pop(v, None)
+        if found is not None:
+            return found.view(MIGRATION_DTYPE).copy()
+    v = range(summary.shape[0])[v]
+    keep = not (mig.is_inference() or summary.is_inference())        # (torch does not count the writes to those)
+    state = (mig._version, summary._version, g10_launch_count()) if keep else ()
+    counts = summary[v:v + (_AHEAD_VARIANTS if keep else 1), 0].cpu().numpy().clip(0, batch.migrations_cap).tolist()
+    counts = counts[:max(1, _AHEAD_BYTES // max(max(counts) * 48, 1))]
+    most = max(counts) * 48
+    records = torch.empty((len(counts), most), dtype=torch.uint8, pin_memory=True)
+    records.copy_(mig[v:v + len(counts), :most])
+    host = records.numpy()
+    if keep:
+        batch._ahead = (mig, summary) + state + ({v + j: host[j, :counts[j] * 48] for j in range(1, len(counts))},)
+    return host[0, :counts[0] * 48].view(MIGRATION_DTYPE).copy()
 
 
 def g10_schedule_prefetch(K, num_migrations, migrations, kernel_start_ns, tensor_bytes, gpu_capacity_bytes, pressure,

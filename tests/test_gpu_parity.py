@@ -1207,3 +1207,53 @@ def test_batch_of_mixed_host_capacities(gpu, oracle, K):
     base = dict(gpu_capacity_bytes=tr.capacity_from_peak(peak), host_bw=tr.host_bw, ssd_bw=tr.ssd_bw)
     ref = check_batch(gpu, oracle, tr, [base, dict(base, host_capacity_bytes=3 << 24), dict(base, host_capacity_bytes=1 << 40)])
     assert len(ref.plans[1].migrations) > 20
+
+
+@pytest.mark.gpu
+def test_batch_records_are_those_on_the_device(gpu):
+    """batch_migrations_numpy reads ahead: what it hands out has to be what the tensors hold when it is called, also after they
+    were written to, exchanged, or filled by another call of the library; in any order; without reading a large batch whole."""
+    import ctypes as C
+    import torch
+    tr = traces.config1_resnet152()
+    tb = gpu.upload(tr)
+    base = dict(gpu_capacity_bytes=tr.capacity_bytes, host_bw=tr.host_bw, ssd_bw=tr.ssd_bw)
+    variants = [dict(base, gpu_capacity_bytes=tr.capacity_bytes * (20 + j) // 24) for j in range(6)]
+    batch = gpu.g10_plan_batch(tb, variants)
+
+    def now(b, v):
+        return b.migrations[v, : int(b.summary[v, 0].item()) * 48].cpu().numpy().view(gpu.MIGRATION_DTYPE)
+
+    def check(b, order=range(6)):
+        for v in order:
+            assert np.array_equal(gpu.batch_migrations_numpy(b, v), now(b, v)), v
+
+    check(batch, (0, 1, 2, 3, 4, 5, 0, 0, 5, 3, -1, -6))
+    assert len({len(now(batch, v)) for v in range(6)}) > 3
+    with pytest.raises(IndexError):
+        gpu.batch_migrations_numpy(batch, 6)
+    gpu.batch_migrations_numpy(batch, 0)
+    batch.migrations[3, 0] += 1                              # the records, then the counts
+    batch.summary[4, 0] -= 7
+    check(batch, (3, 4, 5))
+    gpu.batch_migrations_numpy(batch, 0)
+    batch.migrations = batch.migrations.flip(0).contiguous()          # other tensors
+    batch.summary = batch.summary.flip(0).contiguous()
+    check(batch)
+    # the library itself fills them again, by their addresses
+    gpu.batch_migrations_numpy(batch, 0)
+    before = now(batch, 1).copy()
+    lib = gpu.load_library()
+    arr = (gpu._Variant * 6)(*[gpu._Variant(None, v["gpu_capacity_bytes"], tr.host_bw, 2 * tr.ssd_bw, 0) for v in variants])
+    out = gpu._BatchOut(batch.migrations.data_ptr(), batch.migrations_cap, batch.final_pressure.data_ptr(), batch.summary.data_ptr(), batch.stability.data_ptr())
+    ws = torch.empty(gpu.g10_workspace_bytes(gpu.WS_BATCH, tb.K, tb.N, tb.E), dtype=torch.uint8, device="cuda")
+    assert lib.g10_plan_batch(C.byref(tb.c_struct()), 6, arr, 0, C.byref(out), ws.data_ptr(), ws.numel(), torch.cuda.current_stream().cuda_stream) == 0
+    torch.cuda.synchronize()
+    assert not np.array_equal(now(batch, 1), before)
+    check(batch, (1, 2, 3, 4, 5, 0))
+    with torch.inference_mode():
+        check(gpu.g10_plan_batch(tb, variants))
+    # a large batch is not brought over whole
+    many = gpu.g10_plan_batch(tb, [dict(base, gpu_capacity_bytes=tr.capacity_bytes * 20 // 24)] * 500)
+    first = gpu.batch_migrations_numpy(many, 7)
+    assert 100 < len(many._ahead[5]) < 256 and (len(many._ahead[5]) + 1) * first.nbytes <= 8 << 20
