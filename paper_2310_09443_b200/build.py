@@ -17,7 +17,7 @@ LIB_PLAIN, LIB_HOOKS = os.path.join(HERE, "libg10.so"), os.path.join(HERE, "libg
 LIB = LIB_PLAIN
 SOURCES = ["g10_api.cu", "g10_passes.cu", "g10_planner.cu", "g10_planner_lazy.cu", "g10_planner_spread.cu",
            "g10_planner_chip.cu", "g10_small.cu", "g10_vitality_buckets.cu", "g10_prefetch.cu", "g10_emit.cu", "g10_stats.cu", "g10_cyclic.cu",
-           "g10_static.cu"]
+           "g10_static.cu", "g10_limits.cu"]
 HEADERS = ["g10_device.cuh", "g10_internal.h", "g10_planner.cuh"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17", "-Xcompiler", "-fPIC"]
 

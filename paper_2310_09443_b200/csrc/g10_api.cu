@@ -772,15 +772,16 @@ int32_t g10_plan_batch(const g10_trace *trace, int32_t V, const g10_variant *var
     // can tell (the number of periods is counted there).  Variant 0 says so: if it could not be planned, more blocks get a try;
     // if that does not help, the variants are planned one after the other by the planners that use the whole GPU.  Asking costs
     // one small copy and a synchronisation.
+    const int most = plan_batch_most_blocks();
     int C = 1;
-    while (C < kChipMaxCluster && 2 * C * V <= current_sm_count()) C *= 2;
-    for (;; C *= 2) {
+    while (2 * C <= most && 2 * C * V <= current_sm_count()) C *= 2;
+    for (; C <= most; C *= 2) {
         CU(launch_plan_variants(d, w, pp, V, C, out->stability, s));
         int64_t first[8];
         CU(cudaMemcpyAsync(first, out->summary, sizeof(first), cudaMemcpyDeviceToHost, s));
         CU(cudaStreamSynchronize(s));
         if (!(first[2] == -1 && (first[7] & G10_DEV_BATCH_UNFIT))) return G10_OK;
-        if (C >= kChipMaxCluster || d.K > kChipMaxSlots) break;
+        if (d.K > kChipMaxSlots) break;
     }
     CU(launch_publish_status(w, w.counts + 3, s));              // what trace validation found: folded into every variant at the end
     for (int32_t v = 0; v < V; ++v) {

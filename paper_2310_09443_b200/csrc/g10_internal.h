@@ -185,6 +185,7 @@ struct SmallArgs {
     ull *status_word = nullptr;  // planner calls: the call's own status word and "the plan is done" flag, set up here
     unsigned *done = nullptr;
 };
+int largest_cluster(const void *const *kernels, bool one_each, int threads, size_t smem, int *known /* [kMaxDevices] */);
 bool small_analysis_fits(int64_t K, int64_t N, int64_t E);
 cudaError_t launch_small(const SmallArgs &A, cudaStream_t s);
 
@@ -280,6 +281,7 @@ cudaError_t launch_plan_variants(const DeviceTrace &t, const Workspace &w, const
 // stability pairs of V finished plans against plan 0; ORs *status_word into every plan's summary[7]
 cudaError_t launch_batch_finish(const DeviceTrace &t, const Workspace &w, const PlanParams &p, int V, int64_t *stability, const ull *status_word,
                                 cudaStream_t s);
+int plan_batch_most_blocks();        // largest C
 int plan_loop_max_blocks();
 bool plan_keeps_state_on_chip(int64_t K, int64_t E, bool host_cap, uint32_t flags, bool cyclic);   // true: no other planner will be needed
 cudaError_t launch_publish_status(const Workspace &w, int64_t *dst, cudaStream_t s);

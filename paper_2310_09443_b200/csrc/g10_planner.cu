@@ -126,16 +126,16 @@ cudaError_t launch_plan_lazy(const PlanArgs &A, const Workspace &w, int G, cudaS
 int plan_lazy_blocks();
 bool plan_spread_possible(int64_t K, int64_t E);
 cudaError_t launch_plan_spread(const PlanArgs &A, const Workspace &w, cudaStream_t s);
-int plan_chip_blocks(int64_t E, bool several);
+int plan_chip_blocks(int64_t E, bool several, bool cyclic);
 int plan_chip_possible(int64_t K, int64_t E, int C, bool host_cap, bool cyclic);
 cudaError_t launch_plan_chip(const PlanArgs &A, const Workspace &w, int C, bool cyclic, bool alone, cudaStream_t s);
 
-static int chip_blocks(int64_t E, uint32_t flags) { return plan_chip_blocks(E, (flags & G10_FLAG_MULTI_BLOCK) != 0); }
+static int chip_blocks(int64_t E, uint32_t flags, bool cyclic) { return plan_chip_blocks(E, (flags & G10_FLAG_MULTI_BLOCK) != 0, cyclic); }
 
 bool plan_keeps_state_on_chip(int64_t K, int64_t E, bool host_cap, uint32_t flags, bool cyclic)
 {
     if (flags & (G10_FLAG_RESCORE_ALL | G10_FLAG_GLOBAL_STATE | G10_FLAG_SPREAD_STATE)) return false;
-    return plan_chip_possible(K, E, chip_blocks(E, flags), host_cap, cyclic) == 2;
+    return plan_chip_possible(K, E, chip_blocks(E, flags, cyclic), host_cap, cyclic) == 2;
 }
 
 cudaError_t launch_plan_batch(const PlanArgs &A, const Workspace &w, int V, int C, const BatchArgs &B, int64_t *stability, cudaStream_t s);
@@ -156,7 +156,7 @@ cudaError_t launch_plan_cyclic(const DeviceTrace &t, const Workspace &w, const P
     A.start = w.start2;
     // one cluster plans when everything fits its shared memory; where only the device can tell, the planner that uses the whole
     // GPU is queued behind it and does the work otherwise
-    const int C = chip_blocks(t.E, 0), fits = plan_chip_possible(t.K, t.E, C, p.host_capacity_bytes != 0, true);
+    const int C = chip_blocks(t.E, 0, true), fits = plan_chip_possible(t.K, t.E, C, p.host_capacity_bytes != 0, true);
     if (fits) {
         const cudaError_t e = launch_plan_chip(A, w, C, true, fits == 2, s);
         if (e != cudaSuccess || fits == 2) return e;
@@ -190,7 +190,7 @@ cudaError_t launch_plan_loop(const DeviceTrace &t, const Workspace &w, const Pla
     }
     if (!(p.flags & (G10_FLAG_GLOBAL_STATE | G10_FLAG_SPREAD_STATE))) {
         // (as in launch_plan_cyclic)
-        const int C = chip_blocks(t.E, p.flags), fits = plan_chip_possible(t.K, t.E, C, p.host_capacity_bytes != 0, false);
+        const int C = chip_blocks(t.E, p.flags, false), fits = plan_chip_possible(t.K, t.E, C, p.host_capacity_bytes != 0, false);
         if (fits) {
             const cudaError_t e = launch_plan_chip(A, w, C, false, fits == 2, s);
             if (e != cudaSuccess || fits == 2) return e;

@@ -897,6 +897,15 @@ static int chip_smem_budget(int which)
     return room;
 }
 
+// Blocks of the largest cluster that can be placed with that memory.
+static int chip_largest(int which)
+{
+    static int known[3][kMaxDevices];
+    const int room = chip_smem_budget(which);
+    const void *kernel = chip_kernel(which);
+    return room > 0 ? largest_cluster(&kernel, false, kChipThreads, (size_t)room, known[which]) : 0;
+}
+
 // Launches `plans` clusters of C blocks (one per plan).
 static cudaError_t launch_chip(int which, PlanArgs A, ChipArgs O, BatchArgs B, int plans, int C, cudaStream_t s)
 {
@@ -923,12 +932,18 @@ static ChipArgs chip_args(int which, const Workspace &w)
 // periods) 3.7 / 3.1 / 2.9 with 1 / 8 / 16; four ViT-H steps (6692 kernels, 13 875 periods) do not fit fewer than 16.  A block
 // more takes work off the others' lanes in every iteration, an exchange costs 500-700 cycles whatever the size: one block only
 // where there is next to nothing to share (E bounds the periods).
-int plan_chip_blocks(int64_t E, bool several) { return E <= 1024 && !several ? 1 : kChipMaxCluster; }
+// (0: none can be placed)
+int plan_chip_blocks(int64_t E, bool several, bool cyclic)
+{
+    const int most = chip_largest(cyclic ? kOneCycle : kOnePlan);
+    return E <= 1024 && !several && most > 1 ? 1 : most;
+}
+int plan_batch_most_blocks() { return chip_largest(kManyPlans); }
 
 // Worth launching (0: no; 1: the device decides, from the number of periods that it counted; 2: fits whatever their number).
 int plan_chip_possible(int64_t K, int64_t E, int C, bool host_cap, bool cyclic)
 {
-    if (E < 1 || K > kChipMaxSlots || (cyclic ? 2 * K : K) >= (int64_t)kSlotTop) return 0;
+    if (E < 1 || C < 1 || K > kChipMaxSlots || (cyclic ? 2 * K : K) >= (int64_t)kSlotTop) return 0;
     const int64_t room = chip_smem_budget(cyclic ? kOneCycle : kOnePlan), most = (E + C - 1) / C;
     if (most <= kChipMaxPeriods && (int64_t)chip_smem_core(K, most, C, host_cap, cyclic) <= room) return 2;
     return (int64_t)chip_smem_core(K, most < 64 ? most : 64, C, host_cap, cyclic) <= room ? 1 : 0;

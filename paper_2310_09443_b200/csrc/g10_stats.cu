@@ -16,7 +16,7 @@ namespace g10 {
 constexpr int kStatThreads = 256;
 constexpr int kLenBins = 64, kSizeBins = 41, kLen2Bins = 45;
 
-constexpr int kPeakThreads = 1024, kPeakBlocks = 16;
+constexpr int kPeakThreads = 1024;
 constexpr long long kNone = 0x7fffffffffffffffll;
 
 struct StatsOut {
@@ -114,24 +114,27 @@ __global__ void __launch_bounds__(kStatThreads) k_stats(int64_t N, const int64_t
     if (threadIdx.x < 2 && s_hide[threadIdx.x]) atomicAdd(&out.hide[threadIdx.x], (ull)s_hide[threadIdx.x]);
 }
 
-// summary = largest active bytes, its lowest kernel (0, -1 for an empty trace).  One cluster; every block reads every 16th run.
-__global__ void __launch_bounds__(kPeakThreads) __cluster_dims__(kPeakBlocks, 1, 1) k_active_peak(int64_t K, const long long *__restrict__ active, long long *summary)
+// summary = largest active bytes, its lowest kernel (0, -1 for an empty trace).  One cluster, the largest that the
+// device can place; every block reads every kBlocks-th run.  (One kernel with its size given at launch: a microsecond more.)
+template <int kBlocks>
+__global__ void __launch_bounds__(kPeakThreads) __cluster_dims__(kBlocks, 1, 1) k_active_peak(int64_t K, const long long *__restrict__ active, long long *summary)
 {
     __shared__ long long s_mx[kPeakThreads / 32], s_at[kPeakThreads / 32];
-    __shared__ longlong2 s_all[kPeakBlocks];
+    __shared__ longlong2 s_all[kBlocks];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int64_t step = (int64_t)kBlocks * kPeakThreads;
     auto better = [](long long m, long long a, long long &mx, long long &at) { if (m > mx || (m == mx && a < at)) { mx = m; at = a; } };
     long long mx = -1, at = kNone;
     // (a block's shared memory may be written by others once it has started, not before: all say that they have, and wait for it
     // where the first remote store stands)
     asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    for (int64_t k0 = (int64_t)blockIdx.x * kPeakThreads + threadIdx.x; k0 < K; k0 += 8 * (int64_t)kPeakBlocks * kPeakThreads) {
+    for (int64_t k0 = (int64_t)blockIdx.x * kPeakThreads + threadIdx.x; k0 < K; k0 += 8 * step) {
         long long v[8];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) { const int64_t k = k0 + q * (int64_t)kPeakBlocks * kPeakThreads; v[q] = k < K ? __ldcg(&active[k]) : -1; }
+        for (int q = 0; q < 8; ++q) { const int64_t k = k0 + q * step; v[q] = k < K ? __ldcg(&active[k]) : -1; }
 #pragma unroll
-        for (int q = 0; q < 8; ++q) if (v[q] > mx) { mx = v[q]; at = k0 + q * (int64_t)kPeakBlocks * kPeakThreads; }    // (k ascending: the first stays)
+        for (int q = 0; q < 8; ++q) if (v[q] > mx) { mx = v[q]; at = k0 + q * step; }    // (k ascending: the first stays)
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -156,7 +159,7 @@ __global__ void __launch_bounds__(kPeakThreads) __cluster_dims__(kPeakBlocks, 1,
     }
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
     if (blockIdx.x == 0 && threadIdx.x == 0) {
-        for (int b = 1; b < kPeakBlocks; ++b) better(s_all[b].x, s_all[b].y, mx, at);
+        for (int b = 1; b < kBlocks; ++b) better(s_all[b].x, s_all[b].y, mx, at);
         summary[0] = K > 0 ? mx : 0; summary[1] = K > 0 ? at : -1;
     }
 }
@@ -172,12 +175,12 @@ cudaError_t launch_characterize(int64_t K, int64_t N, const int64_t *use_ptr, co
                                 int64_t Pn, const int32_t *per_t, const int32_t *per_u, const int32_t *per_v, uint64_t host_bw, uint64_t ssd_bw,
                                 int64_t *active, int64_t *len_hist, int64_t *size_len_hist, int64_t *hide, int64_t *summary, cudaStream_t s)
 {
-    static int allowed[kMaxDevices];                      // clusters of 16 have to be allowed once per device
+    static int allowed[kMaxDevices], known[kMaxDevices];  // clusters of 16 have to be allowed once per device
     int dev = 0;
     cudaError_t e;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if (dev < 0 || dev >= kMaxDevices || !__atomic_load_n(&allowed[dev], __ATOMIC_ACQUIRE)) {
-        if ((e = cudaFuncSetAttribute((const void *)k_active_peak, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess) return e;
+        if ((e = cudaFuncSetAttribute((const void *)k_active_peak<16>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess) return e;
         if (dev >= 0 && dev < kMaxDevices) __atomic_store_n(&allowed[dev], 1, __ATOMIC_RELEASE);
     }
     StatsOut out{(ull *)active, (ull *)len_hist, (ull *)size_len_hist, (ull *)hide, (long long *)summary};
@@ -193,8 +196,13 @@ cudaError_t launch_characterize(int64_t K, int64_t N, const int64_t *use_ptr, co
         cfg.gridDim = dim3((unsigned)(pb + tb));
         if ((e = cudaLaunchKernelEx(&cfg, k_stats, N, use_ptr, uses, bytes, start, Pn, per_t, per_u, per_v, host_bw, ssd_bw, pb, out)) != cudaSuccess) return e;
     }
-    cfg.gridDim = dim3(kPeakBlocks); cfg.blockDim = dim3(kPeakThreads);
-    return cudaLaunchKernelEx(&cfg, k_active_peak, K, (const long long *)active, (long long *)summary);
+    void (*const peak[])(int64_t, const long long *, long long *) = {k_active_peak<16>, k_active_peak<8>, k_active_peak<4>, k_active_peak<2>, k_active_peak<1>};
+    const void *const any[] = {(const void *)peak[0], (const void *)peak[1], (const void *)peak[2], (const void *)peak[3], (const void *)peak[4]};
+    const int most = largest_cluster(any, true, kPeakThreads, 0, known);
+    int j = 0;
+    while (j < 4 && 16 >> j > most) ++j;
+    cfg.gridDim = dim3(16u >> j); cfg.blockDim = dim3(kPeakThreads);
+    return cudaLaunchKernelEx(&cfg, peak[j], K, (const long long *)active, (long long *)summary);
 }
 
 }  // namespace g10
