@@ -21,8 +21,6 @@
  *     dependencies between them) and may be captured in a CUDA graph, after one ordinary call of the same
  *     entry point (which sets kernel attributes).  The planner calls launch cooperative kernels and
  *     g10_plan_batch may synchronise: they are not meant for capture.
- *   - Devices: what the library asks and sets once per device (shared memory its kernels may use) is remembered for the life
- *     of the process: after cudaDeviceReset() no call may be made again in that process.
  *   - Errors: the return value is 0 (enqueued) or a negative G10_ERR_* found on the host before any
  *     launch.  Errors that depend on the data (tensor id out of range, non-monotone kernel_ptr,
  *     sizes or durations outside their limits, an output array too small, a grid barrier that timed

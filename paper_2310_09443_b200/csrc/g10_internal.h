@@ -185,6 +185,8 @@ struct SmallArgs {
     ull *status_word = nullptr;  // planner calls: the call's own status word and "the plan is done" flag, set up here
     unsigned *done = nullptr;
 };
+int dynamic_smem_room(const void *kernel, int *known /* [kMaxDevices] */);
+cudaError_t allow_launch(const void *kernel, size_t smem, int cluster);
 int largest_cluster(const void *const *kernels, bool one_each, int threads, size_t smem, int *known /* [kMaxDevices] */);
 bool small_analysis_fits(int64_t K, int64_t N, int64_t E);
 cudaError_t launch_small(const SmallArgs &A, cudaStream_t s);

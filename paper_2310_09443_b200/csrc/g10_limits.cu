@@ -5,6 +5,32 @@
 
 namespace g10 {
 
+// Dynamic shared memory that a block of `kernel` can be given on the current device (the most a block can opt in to, minus the kernel's
+// static part; 0 if a query fails).  `known` [kMaxDevices] remembers it.
+int dynamic_smem_room(const void *kernel, int *known)
+{
+    int dev = 0, optin = 0;
+    cudaFuncAttributes fa;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return 0;
+    if (dev < kMaxDevices) if (const int b = __atomic_load_n(&known[dev], __ATOMIC_ACQUIRE)) return b;
+    if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) return 0;
+    if (cudaFuncGetAttributes(&fa, kernel) != cudaSuccess) return 0;
+    const int room = optin - (int)fa.sharedSizeBytes;
+    if (room <= 0) return 0;
+    if (dev < kMaxDevices) __atomic_store_n(&known[dev], room, __ATOMIC_RELEASE);
+    return room;
+}
+
+// Allows `kernel` so much dynamic shared memory, and clusters of so many blocks, on the current device.  For every launch: what was
+// allowed once is gone after cudaDeviceReset.  (The same amount each time, not what one launch needs: threads may launch side by side.)
+cudaError_t allow_launch(const void *kernel, size_t smem, int cluster)
+{
+    cudaError_t e = cudaSuccess;
+    if (smem != 0) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess && cluster > 8) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    return e;
+}
+
 // Can the current device place a cluster of so many blocks of `kernel` with so much dynamic shared memory each?
 static bool places_cluster(const void *kernel, int blocks, int threads, size_t smem)
 {
@@ -14,7 +40,7 @@ static bool places_cluster(const void *kernel, int blocks, int threads, size_t s
     at[0].val.clusterDim.x = (unsigned)blocks; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
     cfg.gridDim = dim3((unsigned)blocks); cfg.blockDim = dim3((unsigned)threads); cfg.dynamicSmemBytes = smem; cfg.attrs = at; cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n >= 1) return true;
+    if (allow_launch(kernel, smem, blocks) == cudaSuccess && cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n >= 1) return true;
     cudaGetLastError();
     return false;
 }
@@ -38,5 +64,17 @@ int largest_cluster(const void *const *kernels, bool one_each, int threads, size
 #endif
     return most;
 }
+
+#ifdef G10_TEST_HOOKS
+// For a test that resets the device under the library: the reset, and device memory of the library's own runtime.
+extern "C" int32_t g10_test_device_reset(void) { return (int32_t)cudaDeviceReset(); }
+extern "C" void *g10_test_upload(const void *src, size_t bytes)
+{
+    void *p = nullptr;
+    if (cudaMalloc(&p, bytes) != cudaSuccess || (src != nullptr && cudaMemcpy(p, src, bytes, cudaMemcpyHostToDevice) != cudaSuccess)) return nullptr;
+    return p;
+}
+extern "C" int32_t g10_test_download(void *dst, const void *src, size_t bytes) { return (int32_t)cudaMemcpy(dst, src, bytes, cudaMemcpyDeviceToHost); }
+#endif
 
 }  // namespace g10

@@ -878,23 +878,11 @@ static const void *chip_kernel(int which)
     return which == kOnePlan ? (const void *)k_plan_chip<false, false> : which == kOneCycle ? (const void *)k_plan_chip<false, true> : (const void *)k_plan_chip<true, false>;
 }
 
-// Shared memory a launch can offer (opt-in maximum minus the kernel's static part; 0 if a query fails), and that and the largest
-// cluster allowed on the current device: asked once per kernel and device.
+// Shared memory a launch can offer (0 if a query fails).
 static int chip_smem_budget(int which)
 {
     static int known[3][kMaxDevices];
-    int dev = 0, optin = 0;
-    cudaFuncAttributes fa;
-    const void *kernel = chip_kernel(which);
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return 0;
-    if (dev < kMaxDevices) if (const int b = __atomic_load_n(&known[which][dev], __ATOMIC_ACQUIRE)) return b;
-    if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) return 0;
-    if (cudaFuncGetAttributes(&fa, kernel) != cudaSuccess) return 0;
-    const int room = optin - (int)fa.sharedSizeBytes;
-    if (room <= 0 || cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, room) != cudaSuccess ||
-        cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return 0;
-    if (dev < kMaxDevices) __atomic_store_n(&known[which][dev], room, __ATOMIC_RELEASE);
-    return room;
+    return dynamic_smem_room(chip_kernel(which), known[which]);
 }
 
 // Blocks of the largest cluster that can be placed with that memory.
@@ -916,6 +904,7 @@ static cudaError_t launch_chip(int which, PlanArgs A, ChipArgs O, BatchArgs B, i
     at[0].val.clusterDim.x = (unsigned)C; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
     cfg.attrs = at; cfg.numAttrs = 1;
     void *args[] = {&A, &O, &B};
+    if (const cudaError_t e = allow_launch(chip_kernel(which), (size_t)O.smem_bytes, C); e != cudaSuccess) return e;
     return cudaLaunchKernelExC(&cfg, chip_kernel(which), args);
 }
 

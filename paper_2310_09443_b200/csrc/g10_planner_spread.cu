@@ -909,20 +909,11 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_spread(PlanArgs A, Spr
     plan_epilogue(A, c, G, gen, status, peak, n_mig, rounds, bytes_ssd, bytes_host);
 }
 
-// Shared memory that the kernel may use on the current device (allowed once per device); 0 if a query fails.
+// Shared memory a launch can offer (0 if a query fails).
 static int spread_budget()
 {
     static int known[kMaxDevices];
-    int dev = 0, optin = 0;
-    cudaFuncAttributes fa;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return 0;
-    if (dev < kMaxDevices) if (const int b = __atomic_load_n(&known[dev], __ATOMIC_ACQUIRE)) return b;
-    if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) return 0;
-    if (cudaFuncGetAttributes(&fa, (const void *)k_plan_spread) != cudaSuccess) return 0;
-    const int room = optin - (int)fa.sharedSizeBytes;
-    if (room <= 0 || cudaFuncSetAttribute((const void *)k_plan_spread, cudaFuncAttributeMaxDynamicSharedMemorySize, room) != cudaSuccess) return 0;
-    if (dev < kMaxDevices) __atomic_store_n(&known[dev], room, __ATOMIC_RELEASE);
-    return room;
+    return dynamic_smem_room((const void *)k_plan_spread, known);
 }
 
 // Worth launching: the timeline leaves room for at least some periods (their number is counted on the device, which decides).
@@ -940,6 +931,7 @@ cudaError_t launch_plan_spread(const PlanArgs &A_in, const Workspace &w, cudaStr
     S.c_ben_lo = w.c_ben_lo; S.c_ben_hi = w.c_ben_hi; S.c_cost = w.c_cost; S.props = (SpProp *)w.lazy_props; S.partials = w.lazy_partials;
     S.flag = w.spread_flag; S.done = w.one_done; S.smem_bytes = spread_budget();
     void *args[] = {&A, &S};
+    if (const cudaError_t e = allow_launch((const void *)k_plan_spread, (size_t)S.smem_bytes, 1); e != cudaSuccess) return e;
     return cudaLaunchCooperativeKernel((const void *)k_plan_spread, dim3(current_sm_count()), dim3(kPlanThreads), args, (size_t)S.smem_bytes, s);
 }
 

@@ -465,21 +465,10 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(SmallArgs A)
     }
 }
 
-// Shared memory the kernel may use (the most that a block can opt in to, minus its static part), allowed on the current device:
-// asked once per device.
 static size_t small_budget()
 {
-    static int known[kMaxDevices];                  // 0: not asked yet
-    int dev = 0, optin = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return 0;
-    if (dev < kMaxDevices) if (const int b = __atomic_load_n(&known[dev], __ATOMIC_ACQUIRE)) return (size_t)b;
-    cudaFuncAttributes fa;
-    if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) return 0;
-    if (cudaFuncGetAttributes(&fa, (const void *)k_small) != cudaSuccess) return 0;
-    const int room = optin - (int)fa.sharedSizeBytes;
-    if (room <= 0 || cudaFuncSetAttribute((const void *)k_small, cudaFuncAttributeMaxDynamicSharedMemorySize, room) != cudaSuccess) return 0;
-    if (dev < kMaxDevices) __atomic_store_n(&known[dev], room, __ATOMIC_RELEASE);
-    return (size_t)room;
+    static int known[kMaxDevices];
+    return (size_t)dynamic_smem_room((const void *)k_small, known);
 }
 
 bool small_analysis_fits(int64_t K, int64_t N, int64_t E)
@@ -491,6 +480,7 @@ bool small_analysis_fits(int64_t K, int64_t N, int64_t E)
 cudaError_t launch_small(const SmallArgs &A, cudaStream_t s)
 {
     const size_t smem = small_layout(A.t.K, A.t.N, A.t.E).total;
+    if (const cudaError_t e = allow_launch((const void *)k_small, small_budget(), 1); e != cudaSuccess) return e;
     k_small<<<1, kSmThreads, smem, s>>>(A); count_launch();
     return cudaGetLastError();
 }

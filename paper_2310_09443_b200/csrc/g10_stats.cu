@@ -175,14 +175,8 @@ cudaError_t launch_characterize(int64_t K, int64_t N, const int64_t *use_ptr, co
                                 int64_t Pn, const int32_t *per_t, const int32_t *per_u, const int32_t *per_v, uint64_t host_bw, uint64_t ssd_bw,
                                 int64_t *active, int64_t *len_hist, int64_t *size_len_hist, int64_t *hide, int64_t *summary, cudaStream_t s)
 {
-    static int allowed[kMaxDevices], known[kMaxDevices];  // clusters of 16 have to be allowed once per device
-    int dev = 0;
+    static int known[kMaxDevices];
     cudaError_t e;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if (dev < 0 || dev >= kMaxDevices || !__atomic_load_n(&allowed[dev], __ATOMIC_ACQUIRE)) {
-        if ((e = cudaFuncSetAttribute((const void *)k_active_peak<16>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess) return e;
-        if (dev >= 0 && dev < kMaxDevices) __atomic_store_n(&allowed[dev], 1, __ATOMIC_RELEASE);
-    }
     StatsOut out{(ull *)active, (ull *)len_hist, (ull *)size_len_hist, (ull *)hide, (long long *)summary};
     k_stats_clear<<<stat_grid(K > 2 * kSizeBins * kLen2Bins ? K : 2 * kSizeBins * kLen2Bins, 2 * kStatThreads), kStatThreads, 0, s>>>(K, out); count_launch();
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -202,6 +196,7 @@ cudaError_t launch_characterize(int64_t K, int64_t N, const int64_t *use_ptr, co
     int j = 0;
     while (j < 4 && 16 >> j > most) ++j;
     cfg.gridDim = dim3(16u >> j); cfg.blockDim = dim3(kPeakThreads);
+    if ((e = allow_launch(any[j], 0, 16 >> j)) != cudaSuccess) return e;
     return cudaLaunchKernelEx(&cfg, peak[j], K, (const long long *)active, (long long *)summary);
 }
 
