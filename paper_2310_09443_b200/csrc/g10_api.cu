@@ -219,17 +219,14 @@ cudaError_t d2h(T *dst, const T *src, size_t count, cudaStream_t s)
     return cudaMemcpyAsync(dst, src, sizeof(T) * count, cudaMemcpyDeviceToHost, s);
 }
 
-// The device's address of pinned host memory (null if `p` is not pinned; a null p with nothing behind it stays null).
+// The device's address of pinned host memory; false if not all of it is pinned (a null p with nothing behind it stays null).
 template <typename T>
 bool pinned(T *p, size_t count, T **out)
 {
     *out = nullptr;
     if (p == nullptr || count == 0) return true;
-    cudaPointerAttributes at;
-    if (cudaPointerGetAttributes(&at, (const void *)p) != cudaSuccess) { cudaGetLastError(); return false; }
-    if (at.type != cudaMemoryTypeHost || at.devicePointer == nullptr) return false;
-    *out = (T *)at.devicePointer;
-    return true;
+    *out = (T *)pinned_address((const void *)p, count * sizeof(T));
+    return *out != nullptr;
 }
 
 // A host trace that fits one SM, every array pinned: the kernel reads and writes host memory itself (20 copies of 3-5 us each cost

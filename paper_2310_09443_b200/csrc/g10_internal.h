@@ -185,6 +185,7 @@ struct SmallArgs {
     ull *status_word = nullptr;  // planner calls: the call's own status word and "the plan is done" flag, set up here
     unsigned *done = nullptr;
 };
+void *pinned_address(const void *p, size_t bytes);
 int dynamic_smem_room(const void *kernel, int *known /* [kMaxDevices] */);
 cudaError_t allow_launch(const void *kernel, size_t smem, int cluster);
 int largest_cluster(const void *const *kernels, bool one_each, int threads, size_t smem, int *known /* [kMaxDevices] */);

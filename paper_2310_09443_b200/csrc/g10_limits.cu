@@ -1,4 +1,6 @@
 // What the current device lets a kernel have.
+#include <cuda.h>
+
 #include <cstdlib>
 
 #include "g10_internal.h"
@@ -65,7 +67,37 @@ int largest_cluster(const void *const *kernels, bool one_each, int threads, size
     return most;
 }
 
+// The device's address of pinned host memory if all `bytes` from p on lie in ONE pinned range, else null: memory may be registered in
+// pieces, and a kernel that reads past one faults where a copy returns an error.
+void *pinned_address(const void *p, size_t bytes)
+{
+    typedef CUresult (*Query)(unsigned, CUpointer_attribute *, void **, CUdeviceptr);
+    static void *known = nullptr;                    // (the driver's function: the same in every thread)
+    void *f = __atomic_load_n(&known, __ATOMIC_ACQUIRE);
+    if (f == nullptr) {
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPoint("cuPointerGetAttributes", &f, cudaEnableDefault, &found) != cudaSuccess || found != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        __atomic_store_n(&known, f, __ATOMIC_RELEASE);
+    }
+    CUmemorytype type = (CUmemorytype)0;
+    CUdeviceptr start = 0;
+    void *device = nullptr;
+    size_t size = 0;
+    int managed = 0;
+    CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_DEVICE_POINTER, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                  CU_POINTER_ATTRIBUTE_RANGE_SIZE, CU_POINTER_ATTRIBUTE_IS_MANAGED};
+    void *to[] = {&type, &device, &start, &size, &managed};
+    if (((Query)f)(5, what, to, (CUdeviceptr)(uintptr_t)p) != CUDA_SUCCESS || type != CU_MEMORYTYPE_HOST || managed) return nullptr;
+    const uintptr_t at = (uintptr_t)p;
+    if ((uintptr_t)device != at || start == 0 || at < start || bytes > size || at - start > size - bytes) return nullptr;
+    return device;
+}
+
 #ifdef G10_TEST_HOOKS
+extern "C" int32_t g10_test_reads_in_place(const void *p, size_t bytes) { return pinned_address(p, bytes) != nullptr; }
 // For a test that resets the device under the library: the reset, and device memory of the library's own runtime.
 extern "C" int32_t g10_test_device_reset(void) { return (int32_t)cudaDeviceReset(); }
 extern "C" void *g10_test_upload(const void *src, size_t bytes)

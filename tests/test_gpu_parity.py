@@ -1257,3 +1257,33 @@ def test_batch_records_are_those_on_the_device(gpu):
     many = gpu.g10_plan_batch(tb, [dict(base, gpu_capacity_bytes=tr.capacity_bytes * 20 // 24)] * 500)
     first = gpu.batch_migrations_numpy(many, 7)
     assert 100 < len(many._ahead[5]) < 256 and (len(many._ahead[5]) + 1) * first.nbytes <= 8 << 20
+
+
+@pytest.mark.gpu
+def test_only_wholly_pinned_memory_is_read_in_place(gpu):
+    """A kernel reads host arrays where they are only if all of each lies in one pinned range.  (The question is put to the test
+    build of the library; no kernel runs.)"""
+    import ctypes as C
+    import mmap
+    import torch
+    from paper_2310_09443_b200 import build
+    hooks = C.CDLL(build.build(hooks=True))
+    hooks.g10_test_reads_in_place.argtypes = [C.c_void_p, C.c_size_t]
+    in_place = lambda p, n: hooks.g10_test_reads_in_place(p, n) == 1
+    t = torch.empty(100_000, dtype=torch.uint8).pin_memory()
+    assert in_place(t.data_ptr(), 100_000) and in_place(t.data_ptr() + 1, 99_999) and not in_place(t.data_ptr(), 1 << 30)
+    page, half = 4096, 1 << 16
+    buf = np.frombuffer(mmap.mmap(-1, 2 * half), dtype=np.uint8)
+    p = buf.ctypes.data
+    assert p % page == 0 and not in_place(p, page) and not in_place(torch.empty(page, device="cuda", dtype=torch.uint8).data_ptr(), page)
+    rt = torch.cuda.cudart()
+    assert int(rt.cudaHostRegister(p, half, 0)) == 0
+    try:
+        assert in_place(p, half) and in_place(p + half - 8, 8)
+        assert not in_place(p, half + 1) and not in_place(p, 2 * half) and not in_place(p + half - 8, 16)
+        assert int(rt.cudaHostRegister(p + half, half, 0)) == 0           # two ranges side by side are not one
+        assert not in_place(p, 2 * half) and in_place(p + half, half)
+        assert int(rt.cudaHostUnregister(p + half)) == 0
+    finally:
+        assert int(rt.cudaHostUnregister(p)) == 0
+    assert not in_place(p, half)
