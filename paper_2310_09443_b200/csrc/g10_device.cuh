@@ -237,6 +237,38 @@ __device__ __forceinline__ void period_geometry(const int64_t *start, int u, int
 }
 
 // ---------------------------------------------------------------------------------------------
+// Sorting in place.
+// ---------------------------------------------------------------------------------------------
+// Eight values in registers: Batcher's network of 19 comparators.
+template <typename T>
+__device__ __forceinline__ void sort_eight(T (&v)[8])
+{
+    auto ce = [&](int a, int b) { const T lo = min(v[a], v[b]), hi = max(v[a], v[b]); v[a] = lo; v[b] = hi; };
+    ce(0, 1); ce(2, 3); ce(4, 5); ce(6, 7); ce(0, 2); ce(1, 3); ce(4, 6); ce(5, 7); ce(1, 2); ce(5, 6);
+    ce(0, 4); ce(1, 5); ce(2, 6); ce(3, 7); ce(2, 4); ce(3, 5); ce(1, 2); ce(3, 4); ce(5, 6);
+}
+// n entries by `nt` threads, a warp or (kBlock) the whole block, of which this is number `me`: a bitonic network whose merges
+// begin mirrored, so that it only ever moves values up and partners behind the end are left out.
+template <bool kBlock, typename T>
+__device__ __forceinline__ void bitonic_sort(T *a, int n, int me, int nt)
+{
+    int n2 = 1;
+    while (n2 < n) n2 <<= 1;
+    for (int k = 2; k <= n2; k <<= 1)
+        for (int j = k >> 1, lj = 31 - __clz(k >> 1); j > 0; j >>= 1, --lj) {
+            const bool mirror = j == (k >> 1);
+            for (int t = me; t < n2 / 2; t += nt) {
+                const int blk = t >> lj, f = t & (j - 1), i = blk * 2 * j + f, p = mirror ? blk * 2 * j + 2 * j - 1 - f : i + j;
+                if (p < n) {
+                    const T x = a[i], y = a[p];
+                    if (x > y) { a[i] = y; a[p] = x; }
+                }
+            }
+            if (kBlock) __syncthreads(); else __syncwarp();
+        }
+}
+
+// ---------------------------------------------------------------------------------------------
 // Grid barrier for the persistent planner kernel (launched cooperatively, so all blocks are
 // resident).  One counter that only grows: barrier n is complete when n * blocks have arrived.  (148
 // blocks: 2460 cycles; with a count that is reset and a generation to poll, one trip to the L2 more,

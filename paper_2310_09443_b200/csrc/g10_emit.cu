@@ -389,51 +389,51 @@ __global__ void __launch_bounds__(kEmitThreads, 2) k_emit_write(EmitArgs A, int6
             ull *st = s_stage + warp * (4 * kEmitStageStride);
             constexpr int kBatch = 4;                                      // rounds whose sizes and times are read together
             for (int j1 = 0; j1 < n; j1 += kBatch * kEmitThreads) {
-            ull size[kBatch];
-            int64_t when[kBatch];
+                ull size[kBatch];
+                int64_t when[kBatch];
 #pragma unroll
-            for (int u = 0; u < kBatch; ++u) {
-                const int j = j1 + u * kEmitThreads + threadIdx.x;
-                const bool in = j < n && base + j < inst_cap;
-                const ull key = in ? kp[j] : 0;
-                size[u] = in ? (ull)A.bytes[key & 0x7fffffffu] : 0;
-                when[u] = in ? A.start[key >> 33] : 0;
-            }
+                for (int u = 0; u < kBatch; ++u) {
+                    const int j = j1 + u * kEmitThreads + threadIdx.x;
+                    const bool in = j < n && base + j < inst_cap;
+                    const ull key = in ? kp[j] : 0;
+                    size[u] = in ? (ull)A.bytes[key & 0x7fffffffu] : 0;
+                    when[u] = in ? A.start[key >> 33] : 0;
+                }
 #pragma unroll
-            for (int u = 0; u < kBatch; ++u) {
-                const int j0 = j1 + u * kEmitThreads, j = j0 + threadIdx.x;
-                if (j0 >= n) break;
-                ull w0 = 0, w1 = 0, w2 = 0, w3 = 0;
-                if (j < n && base + j < inst_cap) {
-                    const ull key = kp[j];
-                    const int opcode = (int)((key >> 31) & 3u), tensor = (int)(key & 0x7fffffffu), record = (opcode & 1) ? pp[j] : -1;
-                    int target = -1;
-                    int64_t time_ns = when[u];
-                    if (opcode == kOpPreEvict) { target = A.mig[record].dest; time_ns = A.mig[record].evict_issue_ns; }
-                    if (opcode == kOpPrefetch) {
-                        time_ns = A.new_issue ? A.new_issue[record] : A.mig[record].prefetch_issue_ns;
-                        if (time_ns >= A.start[A.K]) time_ns -= A.start[A.K];      // (steady-state plans: see emit_record)
+                for (int u = 0; u < kBatch; ++u) {
+                    const int j0 = j1 + u * kEmitThreads, j = j0 + threadIdx.x;
+                    if (j0 >= n) break;
+                    ull w0 = 0, w1 = 0, w2 = 0, w3 = 0;
+                    if (j < n && base + j < inst_cap) {
+                        const ull key = kp[j];
+                        const int opcode = (int)((key >> 31) & 3u), tensor = (int)(key & 0x7fffffffu), record = (opcode & 1) ? pp[j] : -1;
+                        int target = -1;
+                        int64_t time_ns = when[u];
+                        if (opcode == kOpPreEvict) { target = A.mig[record].dest; time_ns = A.mig[record].evict_issue_ns; }
+                        if (opcode == kOpPrefetch) {
+                            time_ns = A.new_issue ? A.new_issue[record] : A.mig[record].prefetch_issue_ns;
+                            if (time_ns >= A.start[A.K]) time_ns -= A.start[A.K];      // (steady-state plans: see emit_record)
+                        }
+                        w0 = (ull)(unsigned)opcode | ((ull)(unsigned)tensor << 32);
+                        w1 = (ull)(unsigned)target | ((ull)(unsigned)record << 32);
+                        w2 = size[u];
+                        w3 = (ull)time_ns;
                     }
-                    w0 = (ull)(unsigned)opcode | ((ull)(unsigned)tensor << 32);
-                    w1 = (ull)(unsigned)target | ((ull)(unsigned)record << 32);
-                    w2 = size[u];
-                    w3 = (ull)time_ns;
-                }
-                st[0 * kEmitStageStride + lane] = w0; st[1 * kEmitStageStride + lane] = w1;
-                st[2 * kEmitStageStride + lane] = w2; st[3 * kEmitStageStride + lane] = w3;
-                __syncwarp();
-                const long long first = base + j0 + warp * 32;              // the warp's first record
-                long long nrec = n - (j0 + warp * 32);
-                if (inst_cap - first < nrec) nrec = inst_cap - first;
-                if (nrec > 32) nrec = 32;
-                ull *dst = reinterpret_cast<ull *>(inst + first);
+                    st[0 * kEmitStageStride + lane] = w0; st[1 * kEmitStageStride + lane] = w1;
+                    st[2 * kEmitStageStride + lane] = w2; st[3 * kEmitStageStride + lane] = w3;
+                    __syncwarp();
+                    const long long first = base + j0 + warp * 32;              // the warp's first record
+                    long long nrec = n - (j0 + warp * 32);
+                    if (inst_cap - first < nrec) nrec = inst_cap - first;
+                    if (nrec > 32) nrec = 32;
+                    ull *dst = reinterpret_cast<ull *>(inst + first);
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int i = q * 32 + lane;                          // 8-byte word of the warp's 1024 bytes
-                    if ((i >> 2) < nrec) dst[i] = st[(i & 3) * kEmitStageStride + (i >> 2)];
+                    for (int q = 0; q < 4; ++q) {
+                        const int i = q * 32 + lane;                          // 8-byte word of the warp's 1024 bytes
+                        if ((i >> 2) < nrec) dst[i] = st[(i & 3) * kEmitStageStride + (i >> 2)];
+                    }
+                    __syncwarp();
                 }
-                __syncwarp();
-            }
             }
         }
     }

@@ -496,28 +496,6 @@ cudaError_t launch_first_last(const DeviceTrace &t, const Workspace &w, int32_t 
 constexpr int kHeavyThreads = 256;
 constexpr int kHeavySmem = 8192;   // ints sorted in shared memory; longer segments are sorted in global memory
 
-__device__ void block_bitonic_sort(int32_t *a, int n)
-{
-    int n2 = 1;
-    while (n2 < n) n2 <<= 1;
-    for (int k = 2; k <= n2; k <<= 1) {
-        // first stage of each merge mirrors the upper half, the others are plain half-cleaners
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            const bool mirror = (j == (k >> 1));
-            for (int t = threadIdx.x; t < n2 / 2; t += blockDim.x) {
-                const int blk = t / j, off = t % j;
-                const int i = blk * 2 * j + off;
-                const int p = mirror ? (blk * 2 * j + 2 * j - 1 - off) : (i + j);
-                if (p < n) {
-                    const int32_t x = a[i], y = a[p];
-                    if (x > y) { a[i] = y; a[p] = x; }
-                }
-            }
-            __syncthreads();
-        }
-    }
-}
-
 __global__ void __launch_bounds__(kHeavyThreads) k_sort_heavy(const unsigned *heavy_count, const int32_t *__restrict__ heavy_list,
                                                               const int32_t *__restrict__ raw_ptr, int32_t *__restrict__ raw_uses,
                                                               int32_t *__restrict__ cnt, int32_t *__restrict__ heavy_info)
@@ -536,7 +514,7 @@ __global__ void __launch_bounds__(kHeavyThreads) k_sort_heavy(const unsigned *he
             for (int t = threadIdx.x; t < n; t += blockDim.x) s_buf[t] = seg[t];
         }
         __syncthreads();
-        block_bitonic_sort(a, n);
+        bitonic_sort<true>(a, n, (int)threadIdx.x, kHeavyThreads);
         // in-place compaction of the distinct values, chunk by chunk, in order (read chunk, sync, write)
         if (threadIdx.x == 0) { s_total = 0; s_periods = 0; }
         __syncthreads();

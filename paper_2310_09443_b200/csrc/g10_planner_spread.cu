@@ -15,10 +15,10 @@
 //  D  no bound left that may beat it: commit.
 // All decisions are taken from data every block has, so the control flow is the same in every block.  Rounded scores steer the
 // search; anything within kNear of a decision is settled by exact 128-bit comparison.
-// What bounds it: a chain of block-wide phases, 62 k cycles an iteration on a million kernels (pass over the periods 14 k, rescoring
-// 20 k in 1.45 rounds of 230 periods each, choice of what to rescore 8 k, 2.7 grid barriers 15 k with the wait for the slowest block).
-// With slots and periods in global memory (g10_planner_lazy.cu) an iteration there read 140 MB through the L2: 1.02 s for the plan,
-// 0.45 s here.  Durations are read from global memory when a tile is sorted or a range's end scored: in
+// What bounds it: a chain of block-wide phases, 28 us an iteration on a million kernels, 0.40 s for the plan.  When it was 70 k cycles
+// the pass over the periods took 14 k, rescoring 27 k (1.45 rounds of 230 periods each), the choice of what to rescore 8 k (less since),
+// 2.7 grid barriers 15 k with the wait for the slowest block.  With slots and periods in global memory (g10_planner_lazy.cu) an
+// iteration reads 140 MB through the L2: 0.97 s for the plan.  Durations are read from global memory when a tile is sorted or a range's end scored: in
 // shared memory they cost 4 bytes a slot and saved nothing.
 #include "g10_planner.cuh"
 

@@ -79,26 +79,6 @@ __device__ __forceinline__ void small_peak(long long &mx, int &sl)
     mx = (long long)((ull)(mh ^ 0x80000000u) << 32 | ml); sl = (int)s;              // (all ones: -1)
 }
 
-// Bitonic sort of n entries by `nt` threads (a warp or the block); arbitrary n: the network only moves values up.
-template <bool kBlock>
-__device__ void small_sort(u16 *a, int n, int me, int nt)
-{
-    int n2 = 1;
-    while (n2 < n) n2 <<= 1;
-    for (int k = 2; k <= n2; k <<= 1)
-        for (int j = k >> 1, lj = 31 - __clz(k >> 1); j > 0; j >>= 1, --lj) {
-            const bool mirror = j == (k >> 1);
-            for (int t = me; t < n2 / 2; t += nt) {
-                const int blk = t >> lj, f = t & (j - 1), i = blk * 2 * j + f, p = mirror ? blk * 2 * j + 2 * j - 1 - f : i + j;
-                if (p < n) {
-                    const u16 x = a[i], y = a[p];
-                    if (x > y) { a[i] = y; a[p] = x; }
-                }
-            }
-            if (kBlock) __syncthreads(); else __syncwarp();
-        }
-}
-
 // Removes the repeats of a sorted segment and counts its periods (one warp); distinct uses | periods << 16.
 __device__ unsigned small_compact_warp(u16 *seg, int m, int lane)
 {
@@ -271,10 +251,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(SmallArgs A)
             int v[8];
 #pragma unroll
             for (int j = 0; j < 8; ++j) v[j] = j < m ? seg[j] : 0x10000;
-#define G10_CE(a, b) { const int lo = min(v[a], v[b]), hi = max(v[a], v[b]); v[a] = lo; v[b] = hi; }
-            G10_CE(0, 1) G10_CE(2, 3) G10_CE(4, 5) G10_CE(6, 7) G10_CE(0, 2) G10_CE(1, 3) G10_CE(4, 6) G10_CE(5, 7) G10_CE(1, 2) G10_CE(5, 6)
-            G10_CE(0, 4) G10_CE(1, 5) G10_CE(2, 6) G10_CE(3, 7) G10_CE(2, 4) G10_CE(3, 5) G10_CE(1, 2) G10_CE(3, 4) G10_CE(5, 6)
-#undef G10_CE
+            sort_eight(v);
             prev = v[0];
             seg[0] = (u16)prev;
 #pragma unroll
@@ -303,7 +280,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(SmallArgs A)
         int m;
         u16 *seg = segment(t, &m);
         if (m > kSmWarpSort) continue;
-        small_sort<false>(seg, m, lane, 32);
+        bitonic_sort<false>(seg, m, lane, 32);
         const unsigned r = small_compact_warp(seg, m, lane);
         if (lane == 0) dp[t] = r;
     }
@@ -312,7 +289,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small(SmallArgs A)
         int m;
         u16 *seg = segment(t, &m);
         if (m <= kSmWarpSort) continue;
-        small_sort<true>(seg, m, tid, kSmThreads);
+        bitonic_sort<true>(seg, m, tid, kSmThreads);
         if (warp == 0) { const unsigned r = small_compact_warp(seg, m, lane); if (lane == 0) dp[t] = r; }
     }
     __syncthreads();
