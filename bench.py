@@ -563,8 +563,8 @@ def run_ours(args):
         "plan_ms": plan1["plan_ms"], "plan_workload": PLAN_WORKLOAD,
         "plan_greedy_loop": {"kernel": "k_plan_chip", "bound": "latency", "ms": plan1.get("greedy_loop_ms"),
                              "us_per_iteration": plan1.get("greedy_loop_us_per_iteration"), "iterations": plan1["iterations"],
-                             "note": "the planner state of this workload lives in the shared memory of one SM: a chain of dependent "
-                                     "iterations (search, rescore, commit); reported per iteration, an HBM fraction would mean nothing"},
+                             "note": "the planner state of this workload lives in the shared memory of a cluster of 16 SMs: a chain of dependent "
+                                     "iterations (search, exchange, commit); reported per iteration, an HBM fraction would mean nothing"},
         "plans": plans,
         "passes": passes,
         "e2e": {"value": e2e_value, "unit": "events/s", "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,

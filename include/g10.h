@@ -62,7 +62,7 @@ extern "C" {
 #define G10_DEV_PLAN_OVERFLOW 0x40   /* migrations_cap too small (summary[0] holds the need)      */
 #define G10_DEV_TIMEOUT 0x80         /* an internal wait gave up; the kernel returned early       */
 #define G10_DEV_BAD_FIRST_LAST 0x200 /* first_use / last_use handed to g10_pressure_timeline: last < first or last >= K (tensor skipped) */
-#define G10_DEV_BATCH_UNFIT 0x100    /* internal: the trace does not fit one SM (g10_plan_batch then plans the variants one by one) */
+#define G10_DEV_BATCH_UNFIT 0x100    /* internal: the trace does not fit one cluster (g10_plan_batch then plans the variants one by one) */
 
 /* exit status of the planner (summary[2]) */
 #define G10_ALREADY_FITS 0      /* unplanned peak pressure <= capacity, empty plan                 */
@@ -239,9 +239,9 @@ int32_t g10_plan_migrations(const g10_trace *trace, uint64_t gpu_capacity_bytes,
    its lowest slot, device status word (0, or G10_DEV_TIMEOUT when a wait between thread blocks ran out: the other
    outputs are then not valid).
    `ws` (optional; G10_WS_PREFETCH, with the number of migrations in place of E; contents are scratch): with it, a
-   timeline too long for one SM's shared memory (more than 15 360 slots, up to about 25 000 slots per SM of the GPU;
-   at most 262 144 migrations) is cut into slices, one per thread block of a cooperative launch, and every block walks the records in visiting
-   order, waiting only for the records that can still reach its slice; the result is that of the sequential pass.
+   timeline of 256 slots or more (up to about 25 000 per SM of the GPU; at most 262 144 migrations) is cut into slices, one per
+   thread block of a cooperative launch, and every block walks the records in visiting order, waiting only for the records
+   that can still reach its slice; the result is that of the sequential pass.
    With ws == NULL (ws_bytes ignored) one block does the whole pass, record by record.
    Records of g10_plan_cyclic are accepted as they are: a slot beyond K stands for the same slot of the cycle (the
    pressure curve has K slots), a moved prefetch is issued at the unrolled time of its first regained slot, and the
@@ -319,10 +319,12 @@ int32_t g10_plan_cyclic(const g10_trace *trace, uint64_t gpu_capacity_bytes, uin
    stability [V][2] = (|M_v & M_0|, |M_v | M_0|) over the sets of migrated periods of variant v and variant 0 (their
    quotient is the Jaccard index; (-1, -1) when a plan is missing).
    Limits: the trace has to be device resident (G10_MEM_DEVICE); 1 <= V <= 1024.
-   One cluster per variant requires that pressure, clock, bookings and the periods of the trace fit its shared memory (the DNN-shaped traces of a few thousand kernels do).  Only the device can tell, so the call reads variant
-   0's summary back (one small copy and a synchronisation of `stream`: unlike the other calls this one returns with
-   its kernels finished); if the trace did not fit, the variants are then planned one after the other by the planners
-   that use the whole GPU -- the same results, V times the time of one plan.
+   One cluster per variant requires that pressure, clock, bookings and the periods of the trace fit its shared memory (the
+   DNN-shaped traces of a few thousand kernels do; finite host memory in any variant takes a sixth more for all).  Only the
+   device can tell, so the call reads variant 0's summary back (one small copy and a synchronisation of `stream`: unlike the
+   other calls this one returns with its kernels finished); if the trace did not fit, the variants are then planned one
+   after the other by the planners that use the whole GPU -- the same results, V times the time of one plan.  A variant whose
+   durations add up to 2^44 ns or more gets G10_DEV_BAD_DURATION.
    Workspace: G10_WS_BATCH. */
 typedef struct g10_variant {
     const int64_t *kernel_ns;       /* [K] device pointer, or NULL: the trace's own durations */

@@ -371,7 +371,7 @@ def g10_plan_cyclic(tb: TraceBuffers, gpu_capacity_bytes, host_bw, ssd_bw, host_
 
 
 def g10_plan_batch(tb: TraceBuffers, variants, max_iterations=0, migrations_cap=None, ws=None, stream=None):
-    """Plans the device-resident trace under every variant at once (one thread block each).  A variant is a dict with
+    """Plans the device-resident trace under every variant at once (one thread-block cluster each).  A variant is a dict with
     gpu_capacity_bytes, host_bw, ssd_bw and optionally kernel_ns (int64 device tensor [K]) and host_capacity_bytes.
     Returns migrations [V, migrations_cap * 48] (uint8), final_pressure [V, K], summary [V, 8], stability [V, 2]."""
     lib = load_library()

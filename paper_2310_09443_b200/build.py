@@ -27,8 +27,8 @@ def _newer(path: str, than: float) -> bool:
 
 
 def build(force: bool = False, verbose: bool = False, hooks: bool = False) -> str:
-    """hooks=True builds libg10_hooks.so instead: the same sources with -DG10_TEST_HOOKS (used by one test that makes a
-    bounded device wait run out; never loaded by the binding)."""
+    """hooks=True builds libg10_hooks.so instead: the same sources with -DG10_TEST_HOOKS (used by the tests that need
+    a wait that runs out, a late block, a smaller device and the like; never loaded by the binding)."""
     nvcc = os.environ.get("NVCC", "nvcc")
     OBJ, LIB = (OBJ_HOOKS, LIB_HOOKS) if hooks else (OBJ_PLAIN, LIB_PLAIN)
     flags = NVCC_FLAGS + (["-DG10_TEST_HOOKS"] if hooks else [])

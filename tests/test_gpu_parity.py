@@ -719,7 +719,7 @@ def test_batched_replanning(gpu, oracle):
     ref = oracle.plan_batch(tr, [base, dict(base, kernel_ns=most)])
     for j, v in ((0, 0), (1, 2)):
         assert np.array_equal(gpu.batch_migrations_numpy(got, v), ref.plans[j].migrations)
-    # a trace too large for one SM: the variants are planned one after the other by the planners that use the whole GPU
+    # a trace too large for a cluster per variant: the variants are planned one after the other by the planners that use the whole GPU
     tr = traces.make_config(3)
     start, P0, peak, slot = oracle.timeline(tr)
     base = dict(gpu_capacity_bytes=tr.capacity_from_peak(peak), host_bw=tr.host_bw, ssd_bw=tr.ssd_bw)
@@ -892,7 +892,7 @@ def test_cyclic_planning(gpu, oracle):
     for lists, nb in (([], []), ([[], []], []), ([[0], [0], [0]], [9])):
         tr = traces.from_lists("e", lists, nb, [3] * len(lists), [1] * len(nb), capacity_bytes=0)
         check_cyclic(gpu, oracle, tr, 0)
-    # too large for one SM: the multi-block planner behind the single-block one takes over (Algorithm 1 as printed, on
+    # too large for one cluster on the unrolled clock (232 KB a block): the planner behind it takes over (Algorithm 1 as printed, on
     # the cycle).  The oracle's plain tier needs most of a minute for the whole plan of this trace, so the first 400
     # iterations are compared record by record, and a shorter ViT-shaped trace (two iterations) to the end.
     tr = traces.make_config(3)
