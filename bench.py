@@ -41,8 +41,8 @@ L2_FLUSH_BYTES = 512 << 20
 # caches alone between launches, as this program does: the write-back of the L2 flush's dirty lines is part of it).
 # "sources_sha256" is the hash of the kernel sources at the time of the capture: when the sources have changed since, the
 # bench line says so ("traffic_stale") instead of passing old traffic off as current, and a CPU test warns.
-TRAFFIC = {"vitality": 227_100_000, "timeline": 117_800_000, "timeline_given": 135_500_000, "fused": 337_200_000, "captured_at": "2026-11-25",
-           "sources_sha256": "ebb78cb31457e2e2a3b2906af1e995c64e1459826260a1eb9c5a0bb878efadf8"}
+TRAFFIC = {"vitality": 227_400_000, "timeline": 124_000_000, "timeline_given": 135_600_000, "fused": 338_400_000, "captured_at": "2026-12-03",
+           "sources_sha256": "e80a3701fe0f96906ce0d2e5a297bc0c24356e407b607c519daf1ba290351278"}
 
 
 PASS_SOURCES = ("g10_passes.cu", "g10_vitality_buckets.cu")     # the kernels of g10_vitality and g10_pressure_timeline
