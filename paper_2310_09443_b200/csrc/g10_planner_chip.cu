@@ -17,8 +17,8 @@
 //      its periods' transfer windows with the winner's (one subtraction per pair of ranges); where they meet on the same channel, a
 //      destination is lost if a slot it needs wholly has been booked, or if the one slot it needs in part has too little left.
 //      Channels only fill up, so a destination that failed is out for good: SSD -> host (if its windows are free) -> erased.
-// What bounds it: a chain of on-chip latencies, one iteration after the other: about 800 instructions of one warp at 7.7 cycles each
-// (2.6 of them fixed latency, 1.3 shared memory and reductions, 0.9 branches, 0.8 instruction fetch), an exchange between 16 blocks (550-680 cycles) among them.
+// What bounds it: a chain of on-chip latencies, one iteration after the other: about 900 instructions of one warp at 7 cycles each
+// (2.7 of them fixed latency, 1.5 shared memory, 0.8 instruction fetch), an exchange between 16 blocks (550-680 cycles) among them.
 // Measured (whole plans, before / now): 96-kernel chain 191 / 154 us, ResNet-152 step 2.98 / 2.53 ms, four ViT-H steps 14.1 / 12.2 ms,
 // DAG of 4000 kernels 2.61 / 1.85 ms.  Several winners per exchange (each block goes through a list of 32 candidates and applies those whose
 // score and destination the ones before leave alone) took 4.7 ms for the ResNet-152 step: only 1.4 to 2 of them stand, because a period
