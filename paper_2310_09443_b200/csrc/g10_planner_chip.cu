@@ -19,8 +19,8 @@
 //      Channels only fill up, so a destination that failed is out for good: SSD -> host (if its windows are free) -> erased.
 // What bounds it: a chain of on-chip latencies, one iteration after the other: about 900 instructions of one warp at 7 cycles each
 // (2.7 of them fixed latency, 1.5 shared memory, 0.8 instruction fetch), an exchange between 16 blocks (550-680 cycles) among them.
-// Measured (whole plans, before / now): 96-kernel chain 191 / 154 us, ResNet-152 step 2.98 / 2.53 ms, four ViT-H steps 14.1 / 12.2 ms,
-// DAG of 4000 kernels 2.61 / 1.85 ms.  Several winners per exchange (each block goes through a list of 32 candidates and applies those whose
+// Measured (before / now): 96-kernel chain 208 / 150 us, ResNet-152 step 2.92 / 2.5 ms, four ViT-H steps 14.1 / 12.3 ms, DAG of 4000
+// kernels 2.6 / 1.9 ms.  Several winners per exchange (each block goes through a list of 32 candidates and applies those whose
 // score and destination the ones before leave alone) took 4.7 ms for the ResNet-152 step: only 1.4 to 2 of them stand, because a period
 // that loses the SSD to a winner and goes to the host comes before the next one every second time, and finding that out costs three
 // iterations' worth of instructions.
@@ -41,7 +41,6 @@ constexpr int kChipMaxPeriods = 4096;        // per block (32 groups of at most 
 // the last place off.  The exactly best candidate is therefore never more than 8 below the largest key.
 constexpr ull kBand = 10;
 constexpr int kAlone = 3;                    // periods warp 0 rescores in an iteration before it asks the other warps for help
-static_assert(kAlone > 0, "with none, those asked for help would give up before their first, and be asked again");
 constexpr unsigned kNoRange = 0xffffffffu;   // (destination unusable)
 
 struct ChipArgs {
@@ -251,26 +250,20 @@ __device__ __noinline__ int contest(bool in, ull ben_hi, ull ben_lo, ull cost, i
     return f;
 }
 
-// The lane with the best candidate (-1: no lane has a key; load: a lane's benefit, cost, period).  The upper halves of the keys
-// nearly always tell; keys that are as close as that are compared whole, and those within the band exactly.  (One reduction instead
-// of two, three times an iteration: ResNet-152 step 2.70 / 2.68 ms, batch of 96 one-block plans 2.97 / 2.91 ms.)
+// Of the lanes with a key within the band of the largest, M: the one with the exactly best candidate (load: a lane's benefit, cost, period).
 template <class Load>
-__device__ __forceinline__ int front_lane(ull key, Load load)
+__device__ __forceinline__ int front_lane(ull key, ull M, Load load)
 {
-    const unsigned high = (unsigned)(key >> 32), most = __reduce_max_sync(0xffffffffu, high);
-    unsigned b = __ballot_sync(0xffffffffu, high + 1u >= most && key != 0);
+    const bool in = key != 0 && key + kBand >= M;
+    const unsigned b = __ballot_sync(0xffffffffu, in);
+    int l = b ? __ffs(b) - 1 : 0;
     if (b & (b - 1u)) {
-        const ull m = warp_max_u64(key);
-        const bool in = key != 0 && key + kBand >= m;
-        b = __ballot_sync(0xffffffffu, in);
-        if (b & (b - 1u)) {
-            ull hi = 0, lo = 0, cost = 1;
-            int idx = 0x7fffffff;
-            if (in) load(&hi, &lo, &cost, &idx);
-            return contest(in, hi, lo, cost, idx);
-        }
+        ull hi = 0, lo = 0, cost = 1;
+        int idx = 0x7fffffff;
+        if (in) load(&hi, &lo, &cost, &idx);
+        l = contest(in, hi, lo, cost, idx);
     }
-    return __ffs(b) - 1;
+    return l;
 }
 
 // ---- a period's slot ranges --------------------------------------------------------------------------------------------
@@ -463,8 +456,9 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_plan_chip(PlanArgs A, ChipA
                 if (take) { k = kn; li = ln; }
             }
         }
-        const int l = front_lane(k, [&](ull *hi, ull *lo, ull *cost, int *idx) { *hi = cben_hi[li]; *lo = cben[li]; *cost = 2ull * (ull)data_time(cdata[li]); *idx = li; });
-        if (lane == (l < 0 ? 0 : l)) { s_gkey[g] = k; s_gtop[g] = li; }
+        const ull m = warp_max_u64(k);
+        const int l = front_lane(k, m, [&](ull *hi, ull *lo, ull *cost, int *idx) { *hi = cben_hi[li]; *lo = cben[li]; *cost = 2ull * (ull)data_time(cdata[li]); *idx = li; });
+        if (lane == l) { s_gkey[g] = k; s_gtop[g] = li; }
         __syncwarp();
     };
 
@@ -641,16 +635,14 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_plan_chip(PlanArgs A, ChipA
                 for (;;) {
                     ull k = lane < NG ? s_gkey[lane] : 0ull;
                     if (help && (lane & (kChipWarps - 1)) != warp) k = 0;
-                    const int l = front_lane(k, [&](ull *hi, ull *lo, ull *cost, int *idx) {
-                        const int q = s_gtop[lane];
-                        *hi = cben_hi[q]; *lo = cben[q]; *cost = 2ull * (ull)data_time(cdata[q]); *idx = q;
-                    });
+                    const ull m = warp_max_u64(k);
                     top = -1;
                     fresh = true;
-                    if (l < 0) break;
-                    const ull m = s_gkey[l];
-                    if (help && m + kBand < s_floor) break;
-                    top = s_gtop[l];
+                    if (m == 0 || (help && m + kBand < s_floor)) break;
+                    top = s_gtop[front_lane(k, m, [&](ull *hi, ull *lo, ull *cost, int *idx) {
+                        const int q = s_gtop[lane];
+                        *hi = cben_hi[q]; *lo = cben[q]; *cost = 2ull * (ull)data_time(cdata[q]); *idx = q;
+                    })];
                     const unsigned r = cabs[top];
                     const int64_t s = data_size(cdata[top]);
                     if (!stale(cstamp[top], r, s, it)) break;
@@ -693,20 +685,18 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_plan_chip(PlanArgs A, ChipA
                         if (!__all_sync(0xffffffffu, here)) what = kGaveUp;
                         else {
                             const ChipCand &y = from[lane < C ? lane : 0];
-                            const ull k = lane < C ? y.key : 0ull;
+                            const ull k = lane < C ? y.key : 0ull, m = warp_max_u64(k);
                             const bool exact = (y.rec.x >> 31) != 0u;
-                            const int l = front_lane(k, [&](ull *hi, ull *lo2, ull *cost, int *idx) {
-                                *hi = y.rec.w; *lo2 = y.ben_lo; *cost = 2ull * (ull)data_time(y.data); *idx = (int)data_rest(y.data);
-                            });
-                            what = l < 0 ? kNone : kFound;
-                            const ull m = l < 0 ? 0ull : from[l].key;
+                            what = m == 0 ? kNone : kFound;
                             if (__any_sync(0xffffffffu, k != 0 && k + kBand >= m && !exact)) {
                                 // a bound is in front: the blocks whose bound may beat the best exact key make it exact
                                 least = warp_max_u64(exact ? k : 0ull);
                                 least = least > kBand ? least - kBand : 1ull;
                                 continue;
                             }
-                            src = (int)buf * C + (l < 0 ? 0 : l);
+                            src = (int)buf * C + front_lane(k, m, [&](ull *hi, ull *lo2, ull *cost, int *idx) {
+                                *hi = y.rec.w; *lo2 = y.ben_lo; *cost = 2ull * (ull)data_time(y.data); *idx = (int)data_rest(y.data);
+                            });
                             if (lane == 0) s_likely = m - (1ull << 47);      // (2 to 3 per cent less)
                         }
                     }
@@ -830,8 +820,6 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_plan_chip(PlanArgs A, ChipA
         while (check) {
             const int j = __ffs(check) - 1, li = entry(j);
             check &= check - 1;
-            // (the winner itself; on its own: 2.68 / 2.63 ms for the ResNet-152 step)
-            if (li * C + rank == widx) { cwin[li] = make_uint2(0, 0); ckey[li] = 0; groups |= 1u << (j >> lq); continue; }
             const uint2 q = cwin[li];
             const ulonglong2 d = cdata[li];
             const int a = range_lo(q.x), b = range_hi(q.y);
@@ -839,7 +827,7 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_plan_chip(PlanArgs A, ChipA
             unsigned r = cabs[li];
             int64_t t = data_time(d);
             int D = X;
-            bool free = true;
+            bool free = li * C + rank != widx;
 #pragma unroll 1
             for (;;) {
 #pragma unroll 1
@@ -878,7 +866,7 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_plan_chip(PlanArgs A, ChipA
                         }
                     }
                 }
-                if (free || D == G10_DEST_HOST || chost[li] == kNoRange) break;
+                if (free || D == G10_DEST_HOST || chost[li] == kNoRange || li * C + rank == widx) break;
                 r = chost[li];
                 D = G10_DEST_HOST; t = (int64_t)data_rest(d); free = true;
             }
@@ -976,8 +964,7 @@ static ChipArgs chip_args(int which, const Workspace &w)
 }
 
 // Blocks of the cluster.  Measured (ms): 96-kernel chain 0.18 with one block, 0.21 with 16; ResNet-152 step (1652 kernels, 2020
-// periods) 2.67 / 2.68 with 8 / 16, one ViT-H step 4.0 / 2.9, DAG of 4000 kernels 2.6 / 1.9; four ViT-H steps (6692 kernels, 13 875
-// periods) do not fit fewer than 16.  A block
+// periods) 3.7 / 3.1 / 2.9 with 1 / 8 / 16; four ViT-H steps (6692 kernels, 13 875 periods) do not fit fewer than 16.  A block
 // more takes work off the others' lanes in every iteration, an exchange costs 500-700 cycles whatever the size: one block only
 // where there is next to nothing to share (E bounds the periods).
 // (0: none can be placed)
