@@ -7,23 +7,17 @@
 // it had when it was last scored (an upper bound of the present one, because pressure only falls) and when that was.  The periods
 // of a block lie in at most 32 groups with their best kept, so that one warp finds the block's best with one look.  One iteration:
 //   S  warp 0 takes the best period by bound.  Its score is exact if no tile of its absent range has changed since it was scored
-//      (or only tiles that are still at least the tensor's size above capacity throughout); else it is rescored from the tiles, and
-//      if it has fallen the warp looks again (four times out of five it has not, and the period stays the best without another
-//      look).  Where there is a warp for every group, each has rescored its group's best before.  The block's best goes to all blocks
-//      of the cluster as asynchronous stores into their shared memory, counted by a transaction barrier there; a bound that lies
-//      well below the last winner's score goes out as it is after one attempt, and only if it turns out in front is it made exact.
+//      (or only tiles that are still at least the tensor's size above capacity throughout); else it is rescored from the tiles and
+//      the warp looks again.  The block's best goes to all blocks of the cluster as asynchronous stores into their shared memory,
+//      counted by a transaction barrier there; a bound that lies well below the last winner's score goes out as it is, and only if
+//      it turns out in front is it made exact.
 //   C  the winner is applied to every block's copy of the timeline: tiles wholly inside the absent range only change their offset,
 //      the two tiles at its ends are rewritten; the transfer windows set bits, and one booked amount each.  Every thread compares
 //      its periods' transfer windows with the winner's (one subtraction per pair of ranges); where they meet on the same channel, a
 //      destination is lost if a slot it needs wholly has been booked, or if the one slot it needs in part has too little left.
 //      Channels only fill up, so a destination that failed is out for good: SSD -> host (if its windows are free) -> erased.
-// What bounds it: a chain of on-chip latencies, one iteration after the other: about 900 instructions of one warp at 7 cycles each
-// (2.7 of them fixed latency, 1.5 shared memory, 0.8 instruction fetch), an exchange between 16 blocks (550-680 cycles) among them.
-// Measured (before / now): 96-kernel chain 208 / 150 us, ResNet-152 step 2.92 / 2.5 ms, four ViT-H steps 14.1 / 12.3 ms, DAG of 4000
-// kernels 2.6 / 1.9 ms.  Several winners per exchange (each block goes through a list of 32 candidates and applies those whose
-// score and destination the ones before leave alone) took 4.7 ms for the ResNet-152 step: only 1.4 to 2 of them stand, because a period
-// that loses the SSD to a winner and goes to the host comes before the next one every second time, and finding that out costs three
-// iterations' worth of instructions.
+// What bounds it: a chain of on-chip latencies (shared memory 40 cycles, a warp reduction 26, a barrier of 8 warps 28, an exchange
+// between 16 blocks 550-680), one iteration after the other.
 //
 // Scores are compared as rounded 64-bit ratios; candidates within kBand units in the last place of the best are told apart by
 // the exact 128-bit cross products (lowest period index on ties).
@@ -60,6 +54,10 @@ struct __align__(16) ChipCand {
 static_assert(sizeof(ChipCand) == 48, "three 16-byte stores per block");
 // What warp 0 tells the other warps.
 enum { kFound, kNone, kHelp, kGaveUp };
+struct __align__(16) ChipWinner {
+    ChipCand c;
+    int what, idx;           // period
+};
 
 // ---- thread-block clusters ---------------------------------------------------------------------------------------------
 __device__ __forceinline__ unsigned cluster_rank() { unsigned r; asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
@@ -221,11 +219,12 @@ __device__ __forceinline__ u128 benefit_warp(const ChipTimeline &T, int64_t s, i
             while (m) {
                 const int tt = t0 + __ffs(m) - 1, k = tt * kTileO + lane;
                 m &= m - 1;
-                const int kk = k < K ? k : K - 1;            // (loads without a branch)
-                int64_t e = T.ex[kk] + T.off[tt];
-                const ull dur = k >= lo && k <= hi ? (ull)(T.start[kk + 1] - T.start[kk]) : 0ull;
-                e = e > s ? s : e < 0 ? 0 : e;
-                sum += (u128)(ull)e * (u128)dur;
+                if (k >= lo && k <= hi) {
+                    int64_t e = T.ex[k] + T.off[tt];
+                    const ull dur = (ull)(T.start[k + 1] - T.start[k]);
+                    e = e > s ? s : e < 0 ? 0 : e;
+                    sum += (u128)(ull)e * (u128)dur;
+                }
             }
         }
     }
@@ -248,22 +247,6 @@ __device__ __noinline__ int contest(bool in, ull ben_hi, ull ben_lo, ull cost, i
         b = __ballot_sync(0xffffffffu, (threadIdx.x & 31) != (unsigned)f && cand_beats(x, best));
     }
     return f;
-}
-
-// Of the lanes with a key within the band of the largest, M: the one with the exactly best candidate (load: a lane's benefit, cost, period).
-template <class Load>
-__device__ __forceinline__ int front_lane(ull key, ull M, Load load)
-{
-    const bool in = key != 0 && key + kBand >= M;
-    const unsigned b = __ballot_sync(0xffffffffu, in);
-    int l = b ? __ffs(b) - 1 : 0;
-    if (b & (b - 1u)) {
-        ull hi = 0, lo = 0, cost = 1;
-        int idx = 0x7fffffff;
-        if (in) load(&hi, &lo, &cost, &idx);
-        l = contest(in, hi, lo, cost, idx);
-    }
-    return l;
 }
 
 // ---- a period's slot ranges --------------------------------------------------------------------------------------------
@@ -338,8 +321,7 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_plan_chip(PlanArgs A, ChipA
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ ull s_bar[2];
-    __shared__ int s_what, s_src;                       // what warp 0 tells the others; where in s_block the winner stands
-    __shared__ ull s_likely;                            // a little less than the last winner's key
+    __shared__ ChipWinner s_win;
     __shared__ ull s_gkey[32];                          // of each group of periods: the best, and its key
     __shared__ int s_gtop[32];
     __shared__ int64_t s_moved[2];                      // bytes sent to the SSD and to host memory
@@ -457,49 +439,18 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_plan_chip(PlanArgs A, ChipA
             }
         }
         const ull m = warp_max_u64(k);
-        const int l = front_lane(k, m, [&](ull *hi, ull *lo, ull *cost, int *idx) { *hi = cben_hi[li]; *lo = cben[li]; *cost = 2ull * (ull)data_time(cdata[li]); *idx = li; });
+        const bool in = k + kBand >= m && k != 0;
+        const unsigned b = __ballot_sync(0xffffffffu, in);
+        int l = b ? __ffs(b) - 1 : 0;
+        if (b & (b - 1u)) l = contest(in, (ull)cben_hi[li], cben[li], 2ull * (ull)data_time(cdata[li]), li);
         if (lane == l) { s_gkey[g] = k; s_gtop[g] = li; }
         __syncwarp();
     };
 
-    // Is the score of a period a bound?  It is exact if no tile of its absent range has changed since it was found (never, for the first
-    // bound) -- or if the tile is still at least the tensor's size above capacity throughout, so that it was before and counts the
-    // same.  One warp.
-    auto stale = [&](int stamp, unsigned r, int64_t s, int now) {
-        if (stamp == now) return false;
-        bool hit = false;
-#pragma unroll 1
-        for (int part = 0; part < (kCyclic ? 2 : 1); ++part) {
-            int lo, hi;
-            if (!phys_part<kCyclic>(part, range_lo(r), range_hi(r), K, &lo, &hi)) break;
-#pragma unroll 1
-            for (int t = (lo >> 5) + lane; t <= hi >> 5; t += 32) hit |= T.stamp[t] > stamp && T.mm[t].x < s;
-        }
-        return __any_sync(0xffffffffu, hit) != 0;
-    };
-    // Scores the best period of its group anew; false if its benefit is what it was (it is still the best, then).
-    auto rescore = [&](int li, unsigned r, int64_t s, int now, ull &floor) {
-        const ull was_lo = cben[li];
-        const unsigned was_hi = cben_hi[li];
-        const u128 ben = benefit_warp<kCyclic>(T, s, range_lo(r), range_hi(r), K, lane);
-        if ((ull)ben == was_lo && (unsigned)(ben >> 64) == was_hi) {
-            if (lane == 0) cstamp[li] = now;
-            __syncwarp();
-            return false;
-        }
-        const ull key = chip_key(ben, cinv[li]);
-        if (key > floor) floor = key;
-        if (lane == 0) { cben[li] = (ull)ben; cben_hi[li] = (unsigned)(ben >> 64); ckey[li] = key; cstamp[li] = now; }
-        __syncwarp();
-        update_group(li >> (5 + lq));
-        return true;
-    };
-
     // ---------------- the timeline and the periods
     if (tid == 0) {
-        s_over = 0; s_bits = 0; s_moved[0] = s_moved[1] = 0; s_likely = 0;
+        s_over = 0; s_bits = 0; s_moved[0] = s_moved[1] = 0;
         bar_init(smem_addr(&s_bar[0]), 1); bar_init(smem_addr(&s_bar[1]), 1);
-        bar_expect(smem_addr(&s_bar[0]), (unsigned)(C * sizeof(ChipCand)));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
 #pragma unroll 1
@@ -588,38 +539,18 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_plan_chip(PlanArgs A, ChipA
     unsigned groups = 0xffffffffu;                     // groups of this warp (bit i: its i-th) whose best has to be found again
     int64_t n_mig = 0, rounds = 0;
     int status = -1;
+    ull likely = 0;                                    // a little less than the last winner's key
     unsigned sent = 0;                                 // exchanges with the other blocks so far
 #pragma unroll 1
     for (int64_t it64 = 0;; ++it64) {
-        // The groups' best.  Where there is a warp for each, one that may win is made exact at once (alone in its block: all are), and the
-        // search below finds that done (its score is as of this iteration).  Measured: 96-kernel chain (3 groups) 248 / 205 us; with
-        // more groups than warps the passes after the first cost more than they spare (batch of one-block plans, 28 groups: 3.14 / 3.38 ms).
-        if (kBatch || NG > kChipWarps) {
 #pragma unroll 1
-            for (int g = warp; g < NG; g += kChipWarps, groups >>= 1) if (groups & 1u) update_group(g);
-        } else if (warp < NG) {
-            if (groups & 1u) update_group(warp);
-            const ull least = C == 1 ? 0ull : s_likely;
-            const int now = (int)it64;
-#pragma unroll 1
-            for (;;) {
-                const ull k = s_gkey[warp];
-                if (k == 0 || k < least) break;
-                const int top = s_gtop[warp];
-                const unsigned r = cabs[top];
-                const int64_t s = data_size(cdata[top]);
-                if (!stale(cstamp[top], r, s, now)) { if (lane == 0) cstamp[top] = now; break; }
-                ull key = 0;
-                if (!rescore(top, r, s, now, key)) break;
-            }
-        }
+        for (int g = warp; g < NG; g += kChipWarps, groups >>= 1) if (groups & 1u) update_group(g);
         if (it64 == 0 && C > 1) cluster_sync_all();    // (the transaction barriers are set up everywhere)
         else __syncthreads();
         if (A.fits_always || s_over == 0) { status = n_mig == 0 ? G10_ALREADY_FITS : G10_FIT; break; }
         if (it64 >= limit) { status = limit < Pn64 ? G10_ITERATION_LIMIT : G10_EXHAUSTED; break; }
         rounds += 1;
         const int it = (int)it64;
-        const ull likely = s_likely;
         // ---------------- S: the winner.  Warp 0 takes the best period by bound; if its score is not exact any more it rescores it
         // and looks again.  After a few of those it asks the other warps for help: each rescores the best of its own groups, as
         // long as they may beat the best exact score.
@@ -639,85 +570,107 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_plan_chip(PlanArgs A, ChipA
                     top = -1;
                     fresh = true;
                     if (m == 0 || (help && m + kBand < s_floor)) break;
-                    top = s_gtop[front_lane(k, m, [&](ull *hi, ull *lo, ull *cost, int *idx) {
-                        const int q = s_gtop[lane];
-                        *hi = cben_hi[q]; *lo = cben[q]; *cost = 2ull * (ull)data_time(cdata[q]); *idx = q;
-                    })];
+                    const bool in = k + kBand >= m && k != 0;
+                    const unsigned b = __ballot_sync(0xffffffffu, in);
+                    int l = __ffs(b) - 1;
+                    if ((b & (b - 1u)) != 0u && !help) {
+                        const int q = in ? s_gtop[lane] : 0;
+                        l = contest(in, (ull)cben_hi[q], cben[q], 2ull * (ull)data_time(cdata[q]), q);
+                    }
+                    top = s_gtop[l];
+                    if (m < least) { fresh = false; break; }  // (far from winning, in all likelihood: it goes out as a bound)
+                    // Is its score exact?  It is if no tile of its absent range has changed since it was found (never, for the first
+                    // bound) -- or if the tile is still at least the tensor's size above capacity throughout, so that it was before
+                    // and counts the same.
+                    const int stamp = cstamp[top];
                     const unsigned r = cabs[top];
                     const int64_t s = data_size(cdata[top]);
-                    if (!stale(cstamp[top], r, s, it)) break;
-                    // (far from winning, in all likelihood: what is a bound still after one attempt goes out as one.  Another block rescores in
-                    // nearly every iteration anyway, and a bound that turns out in front costs an exchange)
-                    if (m < least && (done > 0 || help)) { fresh = false; break; }
+                    const int ra = range_lo(r), rb = range_hi(r);
+                    bool hit = false;
+                    if (stamp != it)
+#pragma unroll 1
+                        for (int part = 0; part < (kCyclic ? 2 : 1); ++part) {
+                            int lo, hi;
+                            if (!phys_part<kCyclic>(part, ra, rb, K, &lo, &hi)) break;
+#pragma unroll 1
+                            for (int t = (lo >> 5) + lane; t <= hi >> 5; t += 32) hit |= T.stamp[t] > stamp && T.mm[t].x < s;
+                        }
+                    if (!__any_sync(0xffffffffu, hit)) break;
                     if (done == kAlone) { top = -2; break; }
                     ++done;
-                    if (!rescore(top, r, s, it, floor)) break;
+                    const u128 ben = benefit_warp<kCyclic>(T, s, ra, rb, K, lane);
+                    const ull key = chip_key(ben, cinv[top]);
+                    if (key > floor) floor = key;
+                    if (lane == 0) { cben[top] = (ull)ben; cben_hi[top] = (unsigned)(ben >> 64); ckey[top] = key; cstamp[top] = it; }
+                    __syncwarp();
+                    update_group(top >> (5 + lq));
                 }
             }
             if (warp == 0 && !help) {
-                int what = top == -2 ? kHelp : top < 0 ? kNone : kFound, src = 0;
+                if (lane == 0) s_floor = floor;
+                int what = top == -2 ? kHelp : top < 0 ? kNone : kFound;
                 if (top != -2) {
                     const int li = top < 0 ? 0 : top;
                     const uint2 win = cwin[li];
-                    ulonglong2 d = cdata[li];
-                    // (the period goes where the transfer time to the host was; the top bit of the first range says that the key is exact)
-                    d.y = (d.y & 0xfffffull) | (ull)(unsigned)(top * C + rank) << 20;
-                    const ull key = top < 0 ? 0ull : ckey[li], lo = cben[li];
-                    const uint4 v0 = make_uint4((unsigned)key, (unsigned)(key >> 32), (unsigned)lo, (unsigned)(lo >> 32));
-                    const uint4 v1 = make_uint4((unsigned)d.x, (unsigned)(d.x >> 32), (unsigned)d.y, (unsigned)(d.y >> 32));
-                    const uint4 v2 = make_uint4((win.x & 0x7fffffffu) | (fresh ? 0x80000000u : 0u), win.y, cabs[li], cben_hi[li]);
-                    if (C == 1) {
-                        uint4 *to = (uint4 *)s_block;
-                        if (lane == 0) { to[0] = v0; to[1] = v1; to[2] = v2; }
-                    } else {
-                        // to all blocks of the cluster (two lanes per block), and the best of theirs
-                        const unsigned buf = sent & 1u;
-                        ChipCand *from = s_block + buf * C;
-                        const unsigned bar = smem_addr(&s_bar[buf]), peer = (unsigned)lane & 15u, half = (unsigned)lane >> 4;
-                        if (peer < (unsigned)C) {
-                            const unsigned to = peer_addr(smem_addr(&from[rank]), peer), their = peer_addr(bar, peer);
-                            st_async_v4(to + 16 * half, half ? v1 : v0, their);
-                            if (!half) st_async_v4(to + 32, v2, their);
-                        }
+                    ChipCand w;
+                    w.key = top < 0 ? 0ull : ckey[li]; w.ben_lo = cben[li]; w.data = cdata[li];
+                    w.rec = make_uint4(win.x, win.y, cabs[li], cben_hi[li]);
+                    int idx = top * C + rank;
+                    if (C > 1) {
+                        // to all blocks of the cluster, and the best of theirs (the period goes where the transfer time to the
+                        // host was; the top bit of the first range says that the key is exact)
+                        ChipCand *from = s_block + (sent & 1u) * C;
+                        const unsigned bar = smem_addr(&s_bar[sent & 1u]);
+                        if (lane == 0) bar_expect(bar, (unsigned)(C * sizeof(ChipCand)));
+                        w.data.y = (w.data.y & 0xfffffull) | (ull)(unsigned)idx << 20;
+                        w.rec.x = (w.rec.x & 0x7fffffffu) | (fresh ? 0x80000000u : 0u);
+                        const unsigned part = (unsigned)lane % 3u;
+                        uint4 v = w.rec;
+                        if (part == 0) v = make_uint4((unsigned)w.key, (unsigned)(w.key >> 32), (unsigned)w.ben_lo, (unsigned)(w.ben_lo >> 32));
+                        if (part == 1) v = make_uint4((unsigned)w.data.x, (unsigned)(w.data.x >> 32), (unsigned)w.data.y, (unsigned)(w.data.y >> 32));
+#pragma unroll 1
+                        for (int j = lane; j < 3 * C && lane < 30; j += 30)
+                            st_async_v4(peer_addr(smem_addr(&from[rank]) + 16 * part, (unsigned)(j / 3)), v, peer_addr(bar, (unsigned)(j / 3)));
                         const bool here = bar_wait(bar, sent >> 1 & 1u);
                         sent += 1;
-                        if (lane == 0) bar_expect(smem_addr(&s_bar[sent & 1u]), (unsigned)(C * sizeof(ChipCand)));      // (for the next)
                         if (!__all_sync(0xffffffffu, here)) what = kGaveUp;
                         else {
-                            const ChipCand &y = from[lane < C ? lane : 0];
+                            const ChipCand y = from[lane < C ? lane : 0];
                             const ull k = lane < C ? y.key : 0ull, m = warp_max_u64(k);
-                            const bool exact = (y.rec.x >> 31) != 0u;
+                            const bool in = k + kBand >= m && k != 0, exact = (y.rec.x >> 31) != 0u;
+                            const unsigned b = __ballot_sync(0xffffffffu, in);
                             what = m == 0 ? kNone : kFound;
-                            if (__any_sync(0xffffffffu, k != 0 && k + kBand >= m && !exact)) {
+                            int l = b ? __ffs(b) - 1 : 0;
+                            if (__any_sync(0xffffffffu, in && !exact)) {
                                 // a bound is in front: the blocks whose bound may beat the best exact key make it exact
                                 least = warp_max_u64(exact ? k : 0ull);
                                 least = least > kBand ? least - kBand : 1ull;
                                 continue;
                             }
-                            src = (int)buf * C + front_lane(k, m, [&](ull *hi, ull *lo2, ull *cost, int *idx) {
-                                *hi = y.rec.w; *lo2 = y.ben_lo; *cost = 2ull * (ull)data_time(y.data); *idx = (int)data_rest(y.data);
-                            });
-                            if (lane == 0) s_likely = m - (1ull << 47);      // (2 to 3 per cent less)
+                            if (b & (b - 1u)) l = contest(in, (ull)y.rec.w, y.ben_lo, 2ull * (ull)data_time(y.data), (int)data_rest(y.data));
+                            w = from[l];
+                            idx = (int)data_rest(w.data);
+                            w.rec.x &= 0x7fffffffu;
+                            likely = (ull)__double_as_longlong(__longlong_as_double((long long)w.key) * 0.97);
                         }
                     }
+                    if (lane == 0) { s_win.c = w; s_win.idx = idx; }
                 }
-                if (lane == 0) { s_what = what; s_src = src; s_floor = floor; }
+                if (lane == 0) s_win.what = what;
             }
             __syncthreads();
             if (help) help = false;
-            else if (s_what != kHelp) break;
+            else if (s_win.what != kHelp) break;
             else { help = true; floor = s_floor; }
         }
         // ---------------- C: the winner is applied
-        const int what = s_what;
-        const ChipCand &won = s_block[C == 1 ? 0 : s_src];
+        const int what = s_win.what;
         if (what == kGaveUp) { status = -2; break; }
         if (what == kNone) { status = G10_EXHAUSTED; break; }
-        const uint4 wr = won.rec;
+        const uint4 wr = s_win.c.rec;
         const int wa = range_lo(wr.x), wap = range_lo(wr.z), wbp = range_hi(wr.z), wb = range_hi(wr.y), X = (int)(wr.x >> 15 & 1u);
         const ChipProbe<kCyclic> p_out(wa, wap - 1, K), p_in(wbp + 1, wb, K);
-        const ulonglong2 wd = won.data;
-        const int widx = (int)data_rest(wd);
+        const ulonglong2 wd = s_win.c.data;
         const int64_t ws = data_size(wd);
         // pressure falls by its size in the absent slots: whole tiles by their offset, the tiles at the ends slot by slot
 #pragma unroll 1
@@ -790,7 +743,7 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_plan_chip(PlanArgs A, ChipA
             const int64_t t = data_time(wd);
             if (rank == 0 && n_mig < A.out_cap) {
                 g10_migration m;
-                m.period = widx; m.tensor = 0; m.dest = X; m.absent_first = wap; m.absent_last = wbp; m.iteration = it;
+                m.period = s_win.idx; m.tensor = 0; m.dest = X; m.absent_first = wap; m.absent_last = wbp; m.iteration = it;
                 m.evict_issue_ns = T.start[wa]; m.prefetch_issue_ns = T.start[wb + 1] - t; m.transfer_ns = t;
                 A.out[n_mig] = m;
             } else if (rank == 0) dev_bits |= G10_DEV_PLAN_OVERFLOW;
@@ -816,6 +769,7 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_plan_chip(PlanArgs A, ChipA
         // ---------------- those periods (the winner is among them, in its block): is their destination still possible?  Not if a
         // slot that a window needs wholly has been booked, or if the slot it needs in part has too little left.  Then the host, if
         // its windows are free.
+        const int widx = s_win.idx;
 #pragma unroll 1
         while (check) {
             const int j = __ffs(check) - 1, li = entry(j);
