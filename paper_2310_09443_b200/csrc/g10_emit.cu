@@ -489,14 +489,14 @@ cudaError_t launch_emit(const EmitLaunch &L, cudaStream_t s)
     if (e1 != cudaSuccess) return e1;
     cfg.blockDim = dim3(kEmitThreads);
     const size_t sm2 = sizeof(long long) * (size_t)(A.nb + 1) + sizeof(unsigned) * (size_t)A.nb;
-    cudaError_t e2 = cudaFuncSetAttribute(k_emit_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2);
+    cudaError_t e2 = allow_any<k_emit_scatter>();
     if (e2 != cudaSuccess) return e2;
     cfg.gridDim = dim3((unsigned)g); cfg.dynamicSmemBytes = sm2;
     e1 = cudaLaunchKernelEx(&cfg, k_emit_scatter, A);
     if (e1 != cudaSuccess) return e1;
     const size_t sm3 = sizeof(long long) * (size_t)(A.nb + 1) + sizeof(int) * (size_t)(2 * A.bw + 2) + 8 +
                        (sizeof(ull) + sizeof(int32_t)) * kEmitCap + sizeof(ull) * (kEmitThreads / 32) * 4 * kEmitStageStride;
-    cudaError_t e = cudaFuncSetAttribute(k_emit_write, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm3);
+    cudaError_t e = allow_any<k_emit_write>();
     if (e != cudaSuccess) return e;
     const int g3 = A.nb < 2 * sms ? A.nb : 2 * sms;
     cfg.gridDim = dim3(g3); cfg.dynamicSmemBytes = sm3;

@@ -188,6 +188,15 @@ struct SmallArgs {
 void *pinned_address(const void *p, size_t bytes);
 int dynamic_smem_room(const void *kernel, int *known /* [kMaxDevices] */);
 cudaError_t allow_launch(const void *kernel, size_t smem, int cluster);
+// Allows kKernel all the dynamic shared memory that a block of it can have, for launches that ask for more or less with the size of
+// the trace: allowing what one launch needs takes away what another thread has just been allowed for a larger one.
+template <auto kKernel>
+cudaError_t allow_any()
+{
+    static int known[kMaxDevices];
+    const int room = dynamic_smem_room((const void *)kKernel, known);
+    return room > 0 ? allow_launch((const void *)kKernel, (size_t)room, 1) : cudaErrorInvalidDevice;
+}
 int largest_cluster(const void *const *kernels, bool one_each, int threads, size_t smem, int *known /* [kMaxDevices] */);
 bool small_analysis_fits(int64_t K, int64_t N, int64_t E);
 cudaError_t launch_small(const SmallArgs &A, cudaStream_t s);

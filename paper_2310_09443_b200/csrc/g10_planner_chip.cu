@@ -994,7 +994,7 @@ static cudaError_t run_batch_finish(int64_t geo_stride, const int64_t *Pn_dev, c
 {
     const int64_t bound = geo_stride < batch_max_periods() ? geo_stride : batch_max_periods();
     const size_t smem = (size_t)((bound + 31) / 32) * 4;
-    cudaError_t e = cudaFuncSetAttribute((const void *)k_batch_finish, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_any<k_batch_finish>();
     if (e != cudaSuccess) return e;
     k_batch_finish<<<V, 256, smem, s>>>(bound, Pn_dev, mig, out_cap, summary, stability, status_word); count_launch();
     return cudaGetLastError();

@@ -847,8 +847,7 @@ static bool pf_pipe_geometry(int64_t K, int *blocks, int *slice, int *per_sm_out
         G = (K + L - 1) / L;
         const size_t dyn = (size_t)(L + G) * 8;
         if (dyn > 200 * 1024) continue;
-        const void *f = pf_pipe_kernel(per_sm);
-        if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess) return false;
+        if ((per_sm == 1 ? allow_any<k_pf_pipe<512>>() : per_sm == 2 ? allow_any<k_pf_pipe<256>>() : allow_any<k_pf_pipe<128>>()) != cudaSuccess) return false;
         int occ = 0;
         const int nt = per_sm == 1 ? 512 : per_sm == 2 ? 256 : 128;
         cudaError_t e = per_sm == 1   ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_pf_pipe<512>, nt, dyn)
@@ -902,7 +901,7 @@ cudaError_t launch_schedule_prefetch(int64_t K, int64_t n, const g10_migration *
     }
     if (in_smem || n == 0) {
         if (dyn > 0) {
-            const cudaError_t e = cudaFuncSetAttribute(k_schedule_prefetch<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+            const cudaError_t e = allow_any<k_schedule_prefetch<256>>();
             if (e != cudaSuccess) return e;
         }
         k_schedule_prefetch<256><<<1, 256, dyn, s>>>(K, n, mig, start, bytes, cap, P, order, new_last, new_issue, summary, in_smem, sort_smem, only_if, presorted); count_launch();
@@ -911,12 +910,12 @@ cudaError_t launch_schedule_prefetch(int64_t K, int64_t n, const g10_migration *
     if (tiles <= kPfMaxTiles) {
         sort_smem = (!presorted && (size_t)n2 * 12 + (size_t)tiles * 16 <= 200 * 1024) ? 1 : 0;   // (this kernel has most of the SM's shared memory to itself)
         dyn = (sort_smem ? ((size_t)n2 * 12 + 7) / 8 * 8 : 0) + (size_t)tiles * 16;
-        const cudaError_t e = cudaFuncSetAttribute(k_schedule_prefetch_tiled, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+        const cudaError_t e = allow_any<k_schedule_prefetch_tiled>();
         if (e != cudaSuccess) return e;
         k_schedule_prefetch_tiled<<<1, kPfNT, dyn, s>>>(K, n, mig, start, bytes, cap, P, order, new_last, new_issue, summary, sort_smem, only_if, presorted); count_launch();
     } else {
         if (dyn > 0) {
-            const cudaError_t e = cudaFuncSetAttribute(k_schedule_prefetch<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+            const cudaError_t e = allow_any<k_schedule_prefetch<1024>>();
             if (e != cudaSuccess) return e;
         }
         k_schedule_prefetch<1024><<<1, 1024, dyn, s>>>(K, n, mig, start, bytes, cap, P, order, new_last, new_issue, summary, in_smem, sort_smem, nullptr, 0); count_launch();

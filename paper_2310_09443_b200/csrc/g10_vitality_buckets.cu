@@ -761,8 +761,7 @@ static cudaError_t launch_bucket_pass(BucketArgs B, const DeviceTrace &t, const 
         const int64_t ktiles = (t.K + tk - 1) / tk;
         const int g2 = (int)(ktiles < g2max ? ktiles : g2max);
         const size_t sm2 = tables + (sizeof(ull) + sizeof(unsigned short)) * (size_t)cap;
-        cudaError_t e = multi ? cudaFuncSetAttribute(k_bk_scatter<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2)
-                              : cudaFuncSetAttribute(k_bk_scatter<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm2);
+        cudaError_t e = multi ? allow_any<k_bk_scatter<true>>() : allow_any<k_bk_scatter<false>>();
         if (e != cudaSuccess) return e;
         cfg.gridDim = dim3((unsigned)g2);
         cfg.dynamicSmemBytes = sm2;
@@ -773,8 +772,7 @@ static cudaError_t launch_bucket_pass(BucketArgs B, const DeviceTrace &t, const 
     }
     const size_t sm3 = sizeof(int) * (size_t)(bk_pad(B.nb) + 3 * bk_pad(B.bt) + kBkCap) + sizeof(unsigned short) * (size_t)B.bt;
     const bool fused = out.tl_diff != nullptr;
-    cudaError_t e = fused ? cudaFuncSetAttribute(k_bk_emit<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm3)
-                          : cudaFuncSetAttribute(k_bk_emit<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm3);
+    cudaError_t e = fused ? allow_any<k_bk_emit<true>>() : allow_any<k_bk_emit<false>>();
     if (e != cudaSuccess) return e;
     const int g3 = B.nb < 2 * sms ? B.nb : 2 * sms;
     cfg.gridDim = dim3((unsigned)g3);
