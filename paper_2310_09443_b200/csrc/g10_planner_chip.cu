@@ -35,6 +35,7 @@ constexpr int kChipMaxPeriods = 4096;        // per block (32 groups of at most 
 // the last place off.  The exactly best candidate is therefore never more than 8 below the largest key.
 constexpr ull kBand = 10;
 constexpr int kAlone = 3;                    // periods warp 0 rescores in an iteration before it asks the other warps for help
+static_assert(kAlone > 0, "with none, those asked for help would give up before their first, and be asked again");
 constexpr unsigned kNoRange = 0xffffffffu;   // (destination unusable)
 
 struct ChipArgs {
@@ -539,7 +540,11 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_plan_chip(PlanArgs A, ChipA
     unsigned groups = 0xffffffffu;                     // groups of this warp (bit i: its i-th) whose best has to be found again
     int64_t n_mig = 0, rounds = 0;
     int status = -1;
-    ull likely = 0;                                    // a little less than the last winner's key
+    // A little less than the last winner's key.  Warp 0's alone: in the others it stays 0, and with it `least` below.  They have to
+    // rescore whatever may win when they are asked for help: warp 0 lowers its own `least` when a bound turns out in front, and
+    // helpers that kept a higher one would leave everything to it (a variant of this search, three ViT-H steps at half their peak:
+    // 25.6 ms with such helpers, 15.7 without).
+    ull likely = 0;
     unsigned sent = 0;                                 // exchanges with the other blocks so far
 #pragma unroll 1
     for (int64_t it64 = 0;; ++it64) {
