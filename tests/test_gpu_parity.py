@@ -1001,6 +1001,28 @@ def test_on_chip_planner_edges(gpu, oracle, K, chains):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("periods", [256, 257, 4096, 4097])
+def test_on_chip_planner_group_per_warp(gpu, oracle, periods):
+    """As many groups of 32 periods as a block has warps (a group for each), and one more (one warp has two, updated, checked and
+    searched in turn), in one block and in each of a cluster of 16 (every tensor is used twice, at least three kernels apart, so
+    that it has one period).  Bit for bit against the oracle."""
+    K = 64
+    rng = np.random.default_rng(periods)
+    lists = [[] for _ in range(K)]
+    for i in range(periods):
+        a = int(rng.integers(0, K - 3))
+        lists[a].append(i)
+        lists[int(rng.integers(a + 3, K))].append(i)
+    tr = traces.from_lists("groups", lists, rng.integers(1 << 16, 1 << 22, size=periods), rng.integers(100_000, 3_000_000, size=K),
+                           np.zeros(periods, np.uint8), capacity_frac=(2, 5))
+    tb = gpu.upload(tr)
+    cap = tr.capacity_from_peak(oracle.timeline(tr)[2])
+    ref = oracle.plan(tr, cap, lazy=True)
+    for flags in (0, gpu.FLAG_MULTI_BLOCK):
+        check_plan(gpu, tr, tb, cap, ref, flags=flags)
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("K,N,E", [(2047, 301, 65536), (2048, 4096, 69632), (33001, 70001, 200003)])
 def test_host_analysis_middle_sizes(gpu, K, N, E):
     """Traces in pinned host memory that do not fit one SM: arrays of whole and ragged 16 KB pieces, few and many uses and periods,
