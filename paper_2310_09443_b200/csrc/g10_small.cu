@@ -448,6 +448,12 @@ static size_t small_budget()
     return (size_t)dynamic_smem_room((const void *)k_small, known);
 }
 
+// This kernel for whatever fits it.  Measured against the general passes (us, whole calls; trace on the device: here / there, in
+// pinned host memory: here / there): 96 kernels and 320 events 13 / 28, 30 / 58; 1652 and 5268: 18.5 / 36.9, 38 / 69; 3346 and 12 600:
+// 26.7 / 40.0, 49 / 77; 6692 and 25 200 (7721 tensors): 43.1 / 50.6, 77 / 95.  With many tensors of few uses the general passes draw level
+// on the device, and only there: 2000 kernels, 8000 tensors, 9860 events 24.6 / 39.5, 48 / 77; 3000, 12 000, 14 819: 32.8 / 32.0, 59 / 72;
+// 6000, 12 000, 14 891: 36.9 / 33.1, 70 / 77; 7000, 10 500, 13 047: 35.8 / 34.9, 69 / 77.  What a line below the shared memory's end could
+// give is a tenth on a few device traces between 12 000 tensors and that end.
 bool small_analysis_fits(int64_t K, int64_t N, int64_t E)
 {
     if (K < 1 || N < 1 || E < 1 || K >= 65535 || N >= 65535 || E >= 65535) return false;
