@@ -37,12 +37,12 @@ WORKLOAD = "config4_stress_dag"
 PLAN_WORKLOAD = "config1_resnet152_b256"
 L2_FLUSH_BYTES = 512 << 20
 # DRAM bytes per call on the stress trace (dram__bytes_read.sum + dram__bytes_write.sum summed over the call's kernels), from
-# the one-pass ncu capture whose command and table are in profiles/passes_config4_stress.md (the capture that leaves the
-# caches alone between launches, as this program does: the write-back of the L2 flush's dirty lines is part of it).
+# a one-pass ncu capture of `bench.py --passes-only` that leaves the caches alone between launches, as this program does (the
+# write-back of the L2 flush's dirty lines is part of it).
 # "sources_sha256" is the hash of the kernel sources at the time of the capture: when the sources have changed since, the
 # bench line says so ("traffic_stale") instead of passing old traffic off as current, and a CPU test warns.
-TRAFFIC = {"vitality": 227_400_000, "timeline": 124_000_000, "timeline_given": 135_600_000, "fused": 338_400_000, "captured_at": "2026-12-03",
-           "sources_sha256": "e80a3701fe0f96906ce0d2e5a297bc0c24356e407b607c519daf1ba290351278"}
+TRAFFIC = {"vitality": 227_600_000, "timeline": 124_100_000, "timeline_given": 135_600_000, "fused": 339_200_000, "captured_at": "2026-12-03",
+           "sources_sha256": "de7b10fd4df099399f3e7879be4c029f565b10b0dad9429ae900ff42a21b1302"}
 
 
 PASS_SOURCES = ("g10_passes.cu", "g10_vitality_buckets.cu")     # the kernels of g10_vitality and g10_pressure_timeline

@@ -61,4 +61,4 @@ def test_traffic_constants_carry_the_hash_of_the_sources_they_were_captured_on()
     assert bench.TRAFFIC["vitality"] > 0 and bench.TRAFFIC["timeline"] > 0
     if now != bench.TRAFFIC["sources_sha256"]:
         warnings.warn("kernel sources changed since the DRAM traffic in bench.py was captured: re-capture it "
-                      "(profiles/passes_config4_stress.md has the command)")
+                      "(one pass of dram__bytes_read.sum and dram__bytes_write.sum over bench.py --passes-only)")
