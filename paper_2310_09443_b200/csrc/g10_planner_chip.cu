@@ -16,8 +16,11 @@
 //      its periods' transfer windows with the winner's (one subtraction per pair of ranges); where they meet on the same channel, a
 //      destination is lost if a slot it needs wholly has been booked, or if the one slot it needs in part has too little left.
 //      Channels only fill up, so a destination that failed is out for good: SSD -> host (if its windows are free) -> erased.
-// What bounds it: a chain of on-chip latencies (shared memory 40 cycles, a warp reduction 26, a barrier of 8 warps 28, an exchange
-// between 16 blocks 550-680), one iteration after the other.
+// What bounds it: the instructions of one warp, one after the other, and the slowest of the blocks.  An iteration of the ResNet-152
+// step takes 7.2 k cycles: 660 for the groups' best and a barrier, 1260-1550 for the search, 625 to send, 2600-2800 of waiting for
+// the block that has to rescore, 1000 to decide, 810 to apply and check.  Outside the block barrier an instruction takes 7.7 cycles
+// (2.5 fixed latency, 1.2 shared memory and reductions, 1.2 other loads and waits, 1.0 branches, 1.0 issue, 0.6 fetch); the exchange
+// itself is 550-680 cycles.
 //
 // Scores are compared as rounded 64-bit ratios; candidates within kBand units in the last place of the best are told apart by
 // the exact 128-bit cross products (lowest period index on ties).
